@@ -137,7 +137,7 @@ def _points(case, g, n=None, d=None, comps=None):
     if aniso:
         w = -torch.log(torch.rand(c, generator=g, device=DEV, dtype=torch.float64).clamp_(1e-12))
         cdf = torch.cumsum(w / w.sum(), 0).float()
-        axes = torch.linalg.qr(torch.randn(c, d, d, generator=g, device=DEV))[0]
+        axes = torch.linalg.qr(torch.randn(c, d, d, generator=g, device=DEV).cpu())[0].to(DEV)
         axes = axes * (torch.rand(c, 1, d, generator=g, device=DEV) * 1.5 + 0.5)
     off = case.get("offset", 0.0)
     for a in range(0, n, 1 << 23):
