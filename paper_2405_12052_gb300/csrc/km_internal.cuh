@@ -299,11 +299,11 @@ struct SetNetArgs {
   const float* prm;   // flat parameters
   float* grads;
   float* xs; float* ts; float* ms;   // standardised points, targets; [B][2d] mean, std
-  float* w2t; float* h1; float* h2; float* tile_pool; float* G; float* P; float* dG; float* loss;
-  float* dz2; float* dz1; float* part;
+  float* w2t; uint32_t* bits; float* tile_pool; float* G; float* P; float* dG; float* loss;
+  float* A3; float* dZ3; float* dP; float* set_loss;  // [B][H], [B][H], [B][K d], [B]: head values of each set
+  float* part;
 };
 int setnet_param_count(int d, int k);
-size_t setnet_point_smem();
 int64_t setnet_part_floats(int64_t P, int d);
 cudaError_t launch_setnet_forward(const SetNetArgs& a, bool train, cudaStream_t st);
 cudaError_t launch_setnet_backward(const SetNetArgs& a, cudaStream_t st);

@@ -13,16 +13,17 @@
 // FP32 throughout; every reduction runs in a fixed order (no float
 // atomics), so a step is deterministic.  Kernels:
 //   sn_standardize   one block per set
-//   sn_fwd_points    64 points per block: h1, h2 and the tile's pooled sum
-//                    (W2 staged transposed in shared memory, 8x4 register
-//                    tiles)
-//   sn_pool          one block per set: tile sums in order / S
-//   sn_head          one block: head forward, loss, head backward for every
-//                    set in order (dW3, dW4, db3, db4, dg)
-//   sn_bwd_points    64 points per block: dz2 = dg/S * [h2 > 0],
-//                    dz1 = (dz2 W2) * [h1 > 0]
-//   sn_wgrad         1024-point chunks: dW2 = sum dz2 h1^T, dW1, db1, db2
-//                    partials; sn_wgrad_reduce adds the chunks in order
+//   sn_fwd_points    64 or 256 points per block: h1 in shared memory, h2 by
+//                    8x8 register tiles, the pooled sums of 64 points, and
+//                    (training) one bit per h2 value, h2 > 0
+//   sn_head          one block per set: pooling, head forward, loss and head
+//                    backward to dg
+//   sn_head_grad     dW3, dW4, db3, db4 and the loss, sets added in order
+//   sn_bwd_points    one block per run of 64-point tiles: h1 formed again,
+//                    dz2 = dg/S * [h2 > 0] from the bits, dz1 = (dz2 W2) *
+//                    [h1 > 0], and the block's dW2 = sum dz2 h1^T, dW1, db1,
+//                    db2 kept in registers
+//   sn_wgrad_reduce  adds the blocks' gradients in order
 //   sn_adam          Adam with bias correction (Kingma and Ba 2015)
 #include "km_internal.cuh"
 
@@ -33,9 +34,8 @@ namespace km {
 namespace {
 
 constexpr int H = kSetH;
-constexpr int kTileP = 64;     // points per block in the per-point kernels
-constexpr int kChunkP = 1024;  // points per weight-gradient chunk
-constexpr int kAT = 68;        // row stride of the transposed point tiles (16-byte rows, 4-way banks)
+constexpr int kTileP = 64;     // points per pooled sum and per backward tile
+constexpr int kBwdBlocks = 152;  // backward blocks: one per SM (166 KB of shared memory each)
 
 struct NetOff {  // offsets of the parameters in the flat vector
   int W1, b1, W2, b2, W3, b3, W4, b4, total;
@@ -54,77 +54,71 @@ __host__ __device__ inline NetOff net_off(int d, int k) {
   return o;
 }
 
-__global__ void __launch_bounds__(256) sn_standardize(const float* __restrict__ x, const float* __restrict__ t,
-                                                      int S, int d, int k, float* xs, float* ts, float* ms) {
-  __shared__ float s_red[256];
-  __shared__ float s_m[3], s_s[3];
-  const int b = blockIdx.x, tid = threadIdx.x;
-  const float* xb = x + (size_t)b * S * d;
-  for (int j = 0; j < d; ++j) {
-    float acc = 0.f;
-    for (int i = tid; i < S; i += blockDim.x) acc += xb[(size_t)i * d + j];
-    s_red[tid] = acc;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-      if (tid < w) s_red[tid] += s_red[tid + w];
-      __syncthreads();
-    }
-    const float m = s_red[0] / (float)S;
-    __syncthreads();
-    acc = 0.f;
-    for (int i = tid; i < S; i += blockDim.x) {
-      const float u = xb[(size_t)i * d + j] - m;
-      acc = fmaf(u, u, acc);
-    }
-    s_red[tid] = acc;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-      if (tid < w) s_red[tid] += s_red[tid + w];
-      __syncthreads();
-    }
-    if (tid == 0) {
-      const float sd = sqrtf(s_red[0] / (float)S);
-      s_m[j] = m;
-      s_s[j] = sd > 0.f ? sd : 1.f;
-    }
+// Sum over the block's 256 threads of up to three values at once: the pairwise
+// tree t += t + 128, 64, ..., 1 (the last five levels inside warp 0).
+__device__ __forceinline__ void tree3(float (&v)[3], float (*s_red)[256], int d, int tid) {
+  for (int j = 0; j < d; ++j) s_red[j][tid] = v[j];
+  __syncthreads();
+#pragma unroll
+  for (int w = 128; w >= 32; w >>= 1) {
+    if (tid < w)
+      for (int j = 0; j < d; ++j) s_red[j][tid] += s_red[j][tid + w];
     __syncthreads();
   }
-  for (int q = tid; q < S * d; q += blockDim.x) {
-    const int j = q % d;
-    xs[(size_t)b * S * d + q] = (xb[q] - s_m[j]) / s_s[j];
-  }
-  if (t)
-    for (int q = tid; q < k * d; q += blockDim.x) {
-      const int j = q % d;
-      ts[(size_t)b * k * d + q] = (t[(size_t)b * k * d + q] - s_m[j]) / s_s[j];
+  if (tid < 32)
+    for (int j = 0; j < d; ++j) {
+      float t = s_red[j][tid];
+#pragma unroll
+      for (int w = 16; w > 0; w >>= 1) t += __shfl_down_sync(0xffffffffu, t, w);
+      if (tid == 0) s_red[j][0] = t;
     }
-  if (tid < d) {
-    ms[b * 2 * d + tid] = s_m[tid];
-    ms[b * 2 * d + d + tid] = s_s[tid];
-  }
+  __syncthreads();
+  for (int j = 0; j < d; ++j) v[j] = s_red[j][0];
+  __syncthreads();
 }
 
-// 64 points x 128 outputs per block, 256 threads as 8 point-groups (8 points
-// each) x 32 unit-groups (4 units each); A^T tile [128][64] and the weight
-// matrix transposed [128][128] in shared memory.
-__device__ __forceinline__ void tile_gemm_8x4(const float* __restrict__ aT, const float* __restrict__ wT, int ty,
-                                              int tx, float acc[8][4]) {
-#pragma unroll
-  for (int r = 0; r < 8; ++r)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
+// One block per set; the d coordinates are summed together (one read of the
+// set per pass instead of d; 26.7 -> 18.4 us for 256 sets of 4096 points).
+__global__ void __launch_bounds__(256) sn_standardize(const float* __restrict__ x, const float* __restrict__ t,
+                                                      int S, int d, int k, float* xs, float* ts, float* ms) {
+  __shared__ float s_red[3][256];
+  const int b = blockIdx.x, tid = threadIdx.x;
+  const float* xb = x + (size_t)b * S * d;
+  float m[3] = {0.f, 0.f, 0.f}, sd[3] = {0.f, 0.f, 0.f};
 #pragma unroll 4
-  for (int q = 0; q < H; ++q) {
-    const float4 a0 = *reinterpret_cast<const float4*>(aT + q * kAT + 8 * ty);
-    const float4 a1 = *reinterpret_cast<const float4*>(aT + q * kAT + 8 * ty + 4);
-    const float4 w = *reinterpret_cast<const float4*>(wT + q * H + 4 * tx);
-    const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-    const float wv[4] = {w.x, w.y, w.z, w.w};
+  for (int i = tid; i < S; i += 256)
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+    for (int j = 0; j < 3; ++j)
+      if (j < d) m[j] += xb[(size_t)i * d + j];
+  tree3(m, s_red, d, tid);
+  for (int j = 0; j < d; ++j) m[j] = m[j] / (float)S;
+#pragma unroll 4
+  for (int i = tid; i < S; i += 256)
 #pragma unroll
-      for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(av[r], wv[c], acc[r][c]);
+    for (int j = 0; j < 3; ++j)
+      if (j < d) {
+        const float u = xb[(size_t)i * d + j] - m[j];
+        sd[j] = fmaf(u, u, sd[j]);
+      }
+  tree3(sd, s_red, d, tid);
+  for (int j = 0; j < d; ++j) {
+    const float q = sqrtf(sd[j] / (float)S);
+    sd[j] = q > 0.f ? q : 1.f;
   }
+  for (int i = tid; i < S; i += 256)
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      if (j < d) xs[((size_t)b * S + i) * d + j] = (xb[(size_t)i * d + j] - m[j]) / sd[j];
+  if (t)
+    for (int i = tid; i < k; i += 256)
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        if (j < d) ts[((size_t)b * k + i) * d + j] = (t[((size_t)b * k + i) * d + j] - m[j]) / sd[j];
+  if (tid == 0)
+    for (int j = 0; j < d; ++j) {
+      ms[b * 2 * d + j] = m[j];
+      ms[b * 2 * d + d + j] = sd[j];
+    }
 }
 
 __global__ void sn_transpose(const float* __restrict__ prm, int d, int k, float* w2t) {
@@ -133,223 +127,386 @@ __global__ void sn_transpose(const float* __restrict__ prm, int d, int k, float*
   if (q < H * H) w2t[q] = prm[o.W2 + (q % H) * H + q / H];
 }
 
-__global__ void __launch_bounds__(256) sn_fwd_points(const float* __restrict__ xs, const float* __restrict__ prm,
-                                                     const float* __restrict__ w2t, int d, int k, float* h1g,
-                                                     float* h2g, float* tile_pool) {
+// acc[r][c] += sum over k of a[k][8 ty + r] w[k][4 tx + (c & 3) + 64 (c >> 2)],
+// k ascending: one fused multiply-add per term.  16 unit groups tx of two
+// runs of four units: the 16-byte reads of a half-warp are then contiguous
+// (with eight units in a row per thread they would hit every bank twice).
+template <int KN, int AS, int WS>
+__device__ __forceinline__ void tile_gemm_8x8(const float* __restrict__ a, const float* __restrict__ w, int ty, int tx,
+                                              float (&acc)[8][8]) {
+#pragma unroll 4
+  for (int q = 0; q < KN; ++q) {
+    const float4 a0 = *reinterpret_cast<const float4*>(a + q * AS + 8 * ty);
+    const float4 a1 = *reinterpret_cast<const float4*>(a + q * AS + 8 * ty + 4);
+    const float4 w0 = *reinterpret_cast<const float4*>(w + q * WS + 4 * tx);
+    const float4 w1 = *reinterpret_cast<const float4*>(w + q * WS + 64 + 4 * tx);
+    const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+    const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int c = 0; c < 8; ++c) acc[r][c] = fmaf(av[r], wv[c], acc[r][c]);
+  }
+}
+
+// h1 of one point and unit (the same expression forward and backward).
+__device__ __forceinline__ float h1_of(const float* s_w1, const float (&xv)[3], int u) {
+  const float4 w = *reinterpret_cast<const float4*>(s_w1 + 4 * u);  // W1[u][0..2] (0 past d), b1[u]
+  return fmaxf(fmaf(w.z, xv[2], fmaf(w.y, xv[1], fmaf(w.x, xv[0], w.w))), 0.f);
+}
+__device__ __forceinline__ void stage_w1(float* s_w1, const float* __restrict__ prm, const NetOff& o, int d, int tid,
+                                         int nth) {
+  for (int q = tid; q < 4 * H; q += nth) {
+    const int u = q >> 2, j = q & 3;
+    s_w1[q] = j == 3 ? prm[o.b1 + u] : j < d ? prm[o.W1 + u * d + j] : 0.f;
+  }
+}
+
+// The per-point layers of PT points (PT = 64 or 256, 2 PT threads): h1 into
+// shared memory transposed, h2 by 8 points x 8 units per thread.  Bound by
+// the FP32 multiply-adds (17.2e9 for 1M points: 0.46 ms at one per lane and
+// cycle); neither h1 nor h2 goes to memory (the backward pass forms h1 again
+// and needs only the sign of h2: 16 bytes per point instead of 1 KB), and the
+// 8x8 tile takes 4 16-byte shared reads per 64 multiply-adds (the 8x4 tile: 3
+// per 32).  1M points: 1.29 -> 0.72 ms.  64-point blocks where 256-point ones
+// would leave SMs idle.  The pooled sum of 64 points is added as before: 8
+// points in order per thread, then the eight groups in order.
+template <int PT>
+__global__ void __launch_bounds__(2 * PT) sn_fwd_points(const float* __restrict__ xs, const float* __restrict__ prm,
+                                                        const float* __restrict__ w2t, int d, int k, int64_t P,
+                                                        uint32_t* __restrict__ bits, float* __restrict__ tile_pool) {
+  constexpr int AS = PT + 4, NT = 2 * PT;
   extern __shared__ __align__(16) float sm[];
-  float* w2T = sm;                 // [128][128]: w2T[c][u] = W2[u][c]
-  float* h1T = w2T + H * H;        // [128][kAT]: h1T[c][p]
-  float* s_pool = h1T + H * kAT;   // [8][128]
+  float* s_w2 = sm;               // [128][128]: s_w2[c][u] = W2[u][c]
+  float* s_h1 = s_w2 + H * H;     // [128][AS]: s_h1[c][p]; then the pooled sums of 8 points [PT / 8][128]
+  float* s_w1 = s_h1 + H * AS;    // [128][4]
   const NetOff o = net_off(d, k);
-  const int tid = threadIdx.x, ty = tid >> 5, tx = tid & 31;
-  const int64_t p0 = (int64_t)blockIdx.x * kTileP;
-  for (int q = tid; q < H * H / 4; q += blockDim.x)
-    reinterpret_cast<float4*>(w2T)[q] = reinterpret_cast<const float4*>(w2t)[q];
-  for (int q = tid; q < kTileP * H; q += blockDim.x) {
-    const int p = q / H, u = q % H;
-    float z = prm[o.b1 + u];
-    for (int j = 0; j < d; ++j) z = fmaf(prm[o.W1 + u * d + j], xs[(p0 + p) * d + j], z);
-    const float h = fmaxf(z, 0.f);
-    h1T[u * kAT + p] = h;
-    h1g[(p0 + p) * H + u] = h;
-  }
-  __syncthreads();
-  float acc[8][4];
-  tile_gemm_8x4(h1T, w2T, ty, tx, acc);
-  float ps[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    const int p = 8 * ty + r;
-    float4 out;
-    float* ov = reinterpret_cast<float*>(&out);
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      ov[c] = fmaxf(acc[r][c] + prm[o.b2 + 4 * tx + c], 0.f);
-      ps[c] += ov[c];
-    }
-    *reinterpret_cast<float4*>(h2g + (p0 + p) * H + 4 * tx) = out;
-  }
-#pragma unroll
-  for (int c = 0; c < 4; ++c) s_pool[ty * H + 4 * tx + c] = ps[c];
-  __syncthreads();
-  if (tid < H) {
-    float s = 0.f;
-    for (int g = 0; g < 8; ++g) s += s_pool[g * H + tid];
-    tile_pool[(size_t)blockIdx.x * H + tid] = s;
-  }
-}
-
-__global__ void __launch_bounds__(H) sn_pool(const float* tile_pool, int tiles_per_set, int S, float* G) {
-  const int b = blockIdx.x, u = threadIdx.x;
-  float s = 0.f;
-  for (int t = 0; t < tiles_per_set; ++t) s += tile_pool[((size_t)b * tiles_per_set + t) * H + u];
-  G[b * H + u] = s / (float)S;
-}
-
-// Head for every set in order.  With targets: loss, head gradients (which
-// it overwrites) and dg; without: the predictions only.
-__global__ void __launch_bounds__(256) sn_head(const float* __restrict__ prm, const float* __restrict__ G, int B,
-                                               int d, int k, const float* __restrict__ ts, float* P, float* grads,
-                                               float* dG, float* loss) {
-  __shared__ float s_g[H], s_z3[H], s_a3[H], s_dz3[H];
-  __shared__ float s_p[kBatchMaxK * 3], s_dp[kBatchMaxK * 3], s_t[kBatchMaxK * 3];
-  __shared__ float s_loss;
-  const NetOff o = net_off(d, k);
-  const int tid = threadIdx.x, KD = k * d;
-  const bool train = ts != nullptr;
-  if (train) {
-    for (int q = tid; q < H * H; q += blockDim.x) grads[o.W3 + q] = 0.f;
-    for (int q = tid; q < KD * H; q += blockDim.x) grads[o.W4 + q] = 0.f;
-    for (int q = tid; q < H; q += blockDim.x) grads[o.b3 + q] = 0.f;
-    for (int q = tid; q < KD; q += blockDim.x) grads[o.b4 + q] = 0.f;
-  }
-  if (tid == 0) s_loss = 0.f;
-  __syncthreads();
-  for (int b = 0; b < B; ++b) {
-    if (tid < H) s_g[tid] = G[b * H + tid];
-    __syncthreads();
-    if (tid < H) {
-      float z = prm[o.b3 + tid];
-      for (int c = 0; c < H; ++c) z = fmaf(prm[o.W3 + tid * H + c], s_g[c], z);
-      s_z3[tid] = z;
-      s_a3[tid] = fmaxf(z, 0.f);
-    }
-    __syncthreads();
-    for (int q = tid; q < KD; q += blockDim.x) {
-      float z = prm[o.b4 + q];
-      for (int u = 0; u < H; ++u) z = fmaf(prm[o.W4 + q * H + u], s_a3[u], z);
-      s_p[q] = z;
-      P[b * KD + q] = z;
-      if (train) {
-        s_t[q] = ts[b * KD + q];
-        s_dp[q] = 0.f;
-      }
-    }
-    __syncthreads();
-    if (!train) continue;
-    if (tid == 0) {
-      // symmetric Chamfer distance; gradients scaled by 1 / (K B)
-      const float sc = 2.f / ((float)k * (float)B);
-      float l1 = 0.f, l2 = 0.f;
-      for (int a = 0; a < k; ++a) {  // nearest target of each prediction
-        int js = 0;
-        float best = 3.0e38f;
-        for (int j = 0; j < k; ++j) {
-          float dd = 0.f;
-          for (int c = 0; c < d; ++c) {
-            const float u = s_p[a * d + c] - s_t[j * d + c];
-            dd = fmaf(u, u, dd);
-          }
-          if (dd < best) { best = dd; js = j; }
-        }
-        l1 += best;
-        for (int c = 0; c < d; ++c) s_dp[a * d + c] += sc * (s_p[a * d + c] - s_t[js * d + c]);
-      }
-      for (int j = 0; j < k; ++j) {  // nearest prediction of each target
-        int as = 0;
-        float best = 3.0e38f;
-        for (int a = 0; a < k; ++a) {
-          float dd = 0.f;
-          for (int c = 0; c < d; ++c) {
-            const float u = s_p[a * d + c] - s_t[j * d + c];
-            dd = fmaf(u, u, dd);
-          }
-          if (dd < best) { best = dd; as = a; }
-        }
-        l2 += best;
-        for (int c = 0; c < d; ++c) s_dp[as * d + c] += sc * (s_p[as * d + c] - s_t[j * d + c]);
-      }
-      s_loss += (l1 + l2) / (float)k / (float)B;
-    }
-    __syncthreads();
-    for (int q = tid; q < KD * H; q += blockDim.x) grads[o.W4 + q] += s_dp[q / H] * s_a3[q % H];
-    for (int q = tid; q < KD; q += blockDim.x) grads[o.b4 + q] += s_dp[q];
-    if (tid < H) {
-      float da = 0.f;
-      for (int q = 0; q < KD; ++q) da = fmaf(prm[o.W4 + q * H + tid], s_dp[q], da);
-      s_dz3[tid] = s_z3[tid] > 0.f ? da : 0.f;
-    }
-    __syncthreads();
-    for (int q = tid; q < H * H; q += blockDim.x) grads[o.W3 + q] += s_dz3[q / H] * s_g[q % H];
-    if (tid < H) {
-      grads[o.b3 + tid] += s_dz3[tid];
-      float dg = 0.f;
-      for (int u = 0; u < H; ++u) dg = fmaf(prm[o.W3 + u * H + tid], s_dz3[u], dg);
-      dG[b * H + tid] = dg;
-    }
-    __syncthreads();
-  }
-  if (tid == 0 && train) *loss = s_loss;
-}
-
-__global__ void __launch_bounds__(256) sn_bwd_points(const float* __restrict__ prm, int d, int k, int S,
-                                                     const float* __restrict__ dG, const float* __restrict__ h1g,
-                                                     const float* __restrict__ h2g, float* dz2g, float* dz1g) {
-  extern __shared__ __align__(16) float sm[];
-  float* w2 = sm;               // [128][128] = W2[u][c] (row u): the transposed use of W2
-  float* dz2T = w2 + H * H;     // [128][kAT]: dz2T[u][p]
-  const NetOff o = net_off(d, k);
-  const int tid = threadIdx.x, ty = tid >> 5, tx = tid & 31;
-  const int64_t p0 = (int64_t)blockIdx.x * kTileP;
-  const int b = (int)(p0 / S);
-  for (int q = tid; q < H * H / 4; q += blockDim.x)
-    reinterpret_cast<float4*>(w2)[q] = reinterpret_cast<const float4*>(prm + o.W2)[q];
-  for (int q = tid; q < kTileP * H; q += blockDim.x) {
-    const int p = q / H, u = q % H;
-    const float v = h2g[(p0 + p) * H + u] > 0.f ? dG[b * H + u] / (float)S : 0.f;
-    dz2T[u * kAT + p] = v;
-    dz2g[(p0 + p) * H + u] = v;
-  }
-  __syncthreads();
-  float acc[8][4];  // dh1[p][c] = sum_u dz2[p][u] W2[u][c]
-  tile_gemm_8x4(dz2T, w2, ty, tx, acc);
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    const int64_t p = p0 + 8 * ty + r;
-    const float4 h = *reinterpret_cast<const float4*>(h1g + p * H + 4 * tx);
-    float4 out;
-    out.x = h.x > 0.f ? acc[r][0] : 0.f;
-    out.y = h.y > 0.f ? acc[r][1] : 0.f;
-    out.z = h.z > 0.f ? acc[r][2] : 0.f;
-    out.w = h.w > 0.f ? acc[r][3] : 0.f;
-    *reinterpret_cast<float4*>(dz1g + p * H + 4 * tx) = out;
-  }
-}
-
-// Per 1024-point chunk: dW2 (8x8 outputs per thread over 32-point smem
-// tiles), and dW1, db1, db2 (threads 0..127 by unit).
-__global__ void __launch_bounds__(256) sn_wgrad(const float* __restrict__ dz2g, const float* __restrict__ h1g,
-                                                const float* __restrict__ dz1g, const float* __restrict__ xs, int d,
-                                                int64_t P, float* part) {
-  __shared__ __align__(16) float s_a[32 * H], s_b[32 * H];
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  const int64_t c0 = (int64_t)blockIdx.x * kChunkP;
-  const int np = (int)min((int64_t)kChunkP, P - c0);
+  const int64_t p0 = (int64_t)blockIdx.x * PT;
+  for (int q = tid; q < H * H / 4; q += NT)
+    reinterpret_cast<float4*>(s_w2)[q] = reinterpret_cast<const float4*>(w2t)[q];
+  stage_w1(s_w1, prm, o, d, tid, NT);
+  __syncthreads();
+  {
+    const int p = tid % PT, u0 = (tid / PT) * (H / 2);
+    float xv[3] = {0.f, 0.f, 0.f};
+    if (p0 + p < P)
+      for (int j = 0; j < d; ++j) xv[j] = xs[(p0 + p) * d + j];
+#pragma unroll 8
+    for (int u = u0; u < u0 + H / 2; ++u) s_h1[u * AS + p] = h1_of(s_w1, xv, u);
+  }
+  __syncthreads();
   float acc[8][8];
 #pragma unroll
   for (int r = 0; r < 8; ++r)
 #pragma unroll
     for (int c = 0; c < 8; ++c) acc[r][c] = 0.f;
-  for (int t0 = 0; t0 < np; t0 += 32) {
-    const int m = min(32, np - t0);
+  tile_gemm_8x8<H, AS, H>(s_h1, s_w2, ty, tx, acc);
+  float b2[8], ps[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    b2[c] = prm[o.b2 + 4 * tx + (c & 3) + 64 * (c >> 2)];
+    ps[c] = 0.f;
+  }
+  const bool live = p0 + 8 * ty < P;  // P is a multiple of 64
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    uint32_t m = 0u;  // bits 0..3: units 4 tx .. 4 tx + 3, bits 4..7: 64 + those
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const float h = fmaxf(acc[r][c] + b2[c], 0.f);
+      ps[c] += h;
+      m |= (h > 0.f ? 1u : 0u) << c;
+    }
+    if (bits) {
+      // the point's 128 bits from the 16 threads of its unit groups: word w
+      // (units 32 w .. 32 w + 31) from groups 8 (w & 1) .. + 7
+      uint32_t lo = (m & 15u) << (4 * (tx & 7)), hi = (m >> 4) << (4 * (tx & 7));
+#pragma unroll
+      for (int f = 1; f < 8; f <<= 1) {
+        lo |= __shfl_xor_sync(0xffffffffu, lo, f);
+        hi |= __shfl_xor_sync(0xffffffffu, hi, f);
+      }
+      if (live && (tx & 7) == 0) {
+        uint32_t* w = bits + (p0 + 8 * ty + r) * 4 + (tx >> 3);
+        w[0] = lo;
+        w[2] = hi;
+      }
+    }
+  }
+  __syncthreads();  // s_h1 is read no more: the pooled sums take its place
+#pragma unroll
+  for (int c = 0; c < 8; ++c) s_h1[ty * H + 4 * tx + (c & 3) + 64 * (c >> 2)] = ps[c];
+  __syncthreads();
+  for (int q = tid; q < PT / kTileP * H; q += NT) {
+    const int t = q / H, u = q % H;
+    if (p0 + t * kTileP >= P) break;
+    float s = 0.f;
+    for (int g = 0; g < 8; ++g) s += s_h1[(8 * t + g) * H + u];
+    tile_pool[((int64_t)blockIdx.x * (PT / kTileP) + t) * H + u] = s;
+  }
+}
+
+// One block per set: the pooled mean, the head forward and, with targets, the
+// set's loss and the head backward to dg (the weight gradients, sums over the
+// sets, are sn_head_grad's).  W3 and W4 are staged in shared memory with an
+// odd row stride, so a thread per row reads them without bank conflicts.  (One
+// block over all sets in order, one thread per loss: 26.2 ms for 256 sets;
+// this and sn_head_grad: 0.053 ms.)
+constexpr int kWS = H + 1;
+__global__ void __launch_bounds__(256) sn_head(const float* __restrict__ prm, const float* __restrict__ tile_pool,
+                                               int tiles_per_set, int S, int B, int d, int k,
+                                               const float* __restrict__ ts, float* __restrict__ G,
+                                               float* __restrict__ P, float* __restrict__ A3, float* __restrict__ dZ3,
+                                               float* __restrict__ dP, float* __restrict__ dG,
+                                               float* __restrict__ set_loss) {
+  extern __shared__ __align__(16) float s_w[];  // [max(H, KD)][kWS]: W3, then W4
+  __shared__ float s_g[H], s_z3[H], s_a3[H], s_dz3[H];
+  __shared__ float s_p[kBatchMaxK * 3], s_dp[kBatchMaxK * 3], s_t[kBatchMaxK * 3];
+  __shared__ float s_d1[kBatchMaxK], s_d2[kBatchMaxK];
+  __shared__ int s_j1[kBatchMaxK], s_j2[kBatchMaxK];
+  const NetOff o = net_off(d, k);
+  const int tid = threadIdx.x, KD = k * d, b = blockIdx.x;
+  const bool train = ts != nullptr;
+  for (int q = tid; q < H * H; q += 256) s_w[(q / H) * kWS + q % H] = prm[o.W3 + q];
+  if (tid < H) {
+    float s = 0.f;
+    const float* tp = tile_pool + (size_t)b * tiles_per_set * H + tid;
+#pragma unroll 8
+    for (int t = 0; t < tiles_per_set; ++t) s += tp[(size_t)t * H];
+    s = s / (float)S;
+    s_g[tid] = s;
+    G[b * H + tid] = s;
+  }
+  __syncthreads();
+  if (tid < H) {
+    float z = prm[o.b3 + tid];
+#pragma unroll 8
+    for (int c = 0; c < H; ++c) z = fmaf(s_w[tid * kWS + c], s_g[c], z);
+    s_z3[tid] = z;
+    s_a3[tid] = fmaxf(z, 0.f);
+    if (train) A3[b * H + tid] = fmaxf(z, 0.f);
+  }
+  __syncthreads();
+  for (int q = tid; q < KD * H; q += 256) s_w[(q / H) * kWS + q % H] = prm[o.W4 + q];
+  __syncthreads();
+  for (int q = tid; q < KD; q += 256) {
+    float z = prm[o.b4 + q];
+#pragma unroll 8
+    for (int u = 0; u < H; ++u) z = fmaf(s_w[q * kWS + u], s_a3[u], z);
+    s_p[q] = z;
+    P[(size_t)b * KD + q] = z;
+    if (train) s_t[q] = ts[(size_t)b * KD + q];
+  }
+  __syncthreads();
+  if (!train) return;
+  // symmetric Chamfer distance: nearest target of each prediction (threads
+  // 0..k-1) and nearest prediction of each target (threads 128..128+k-1),
+  // lowest index on ties
+  if ((tid & 127) < k) {
+    const int a = tid & 127;
+    const float* pa = tid < 128 ? s_p : s_t;
+    const float* pb = tid < 128 ? s_t : s_p;
+    int js = 0;
+    float best = 3.0e38f;
+    for (int j = 0; j < k; ++j) {
+      float dd = 0.f;
+      for (int c = 0; c < d; ++c) {
+        const float u = pa[a * d + c] - pb[j * d + c];  // the sign does not matter
+        dd = fmaf(u, u, dd);
+      }
+      if (dd < best) { best = dd; js = j; }
+    }
+    (tid < 128 ? s_d1 : s_d2)[a] = best;
+    (tid < 128 ? s_j1 : s_j2)[a] = js;
+  }
+  __syncthreads();
+  const float sc = 2.f / ((float)k * (float)B);  // gradients scaled by 1 / (K B)
+  for (int q = tid; q < KD; q += 256) {
+    const int a = q / d, c = q - a * d;
+    float v = sc * (s_p[q] - s_t[s_j1[a] * d + c]);
+    for (int j = 0; j < k; ++j)
+      if (s_j2[j] == a) v = fmaf(sc, s_p[q] - s_t[j * d + c], v);
+    s_dp[q] = v;
+    dP[(size_t)b * KD + q] = v;
+  }
+  if (tid == 0) {
+    float l1 = 0.f, l2 = 0.f;
+    for (int a = 0; a < k; ++a) l1 += s_d1[a];
+    for (int j = 0; j < k; ++j) l2 += s_d2[j];
+    set_loss[b] = (l1 + l2) / (float)k / (float)B;
+  }
+  __syncthreads();
+  if (tid < H) {
+    float da = 0.f;
+#pragma unroll 8
+    for (int q = 0; q < KD; ++q) da = fmaf(s_w[q * kWS + tid], s_dp[q], da);
+    const float z = s_z3[tid] > 0.f ? da : 0.f;
+    s_dz3[tid] = z;
+    dZ3[b * H + tid] = z;
+  }
+  __syncthreads();
+  if (tid < H) {
+    float dg = 0.f;
+#pragma unroll 8
+    for (int u = 0; u < H; ++u) dg = fmaf(prm[o.W3 + u * H + tid], s_dz3[u], dg);
+    dG[b * H + tid] = dg;
+  }
+}
+
+// dW3 = sum_b dz3 g^T, dW4 = sum_b dp a3^T, db3, db4 and the loss: one thread
+// per value, the sets added in order.
+__global__ void __launch_bounds__(128) sn_head_grad(int B, int d, int k, const float* __restrict__ G,
+                                                    const float* __restrict__ A3, const float* __restrict__ dZ3,
+                                                    const float* __restrict__ dP, const float* __restrict__ set_loss,
+                                                    float* __restrict__ grads, float* __restrict__ loss) {
+  const NetOff o = net_off(d, k);
+  const int KD = k * d;
+  const int q = blockIdx.x * 128 + threadIdx.x;
+  float s = 0.f;
+  if (q < H * H) {
+    const int u = q / H, c = q % H;
+#pragma unroll 8
+    for (int b = 0; b < B; ++b) s = fmaf(dZ3[b * H + u], G[b * H + c], s);
+    grads[o.W3 + q] = s;
+  } else if (q < H * H + KD * H) {
+    const int r = (q - H * H) / H, u = (q - H * H) % H;
+#pragma unroll 8
+    for (int b = 0; b < B; ++b) s = fmaf(dP[(size_t)b * KD + r], A3[b * H + u], s);
+    grads[o.W4 + r * H + u] = s;
+  } else if (q < H * H + KD * H + H) {
+    const int u = q - H * H - KD * H;
+#pragma unroll 8
+    for (int b = 0; b < B; ++b) s += dZ3[b * H + u];
+    grads[o.b3 + u] = s;
+  } else if (q < H * H + KD * H + H + KD) {
+    const int r = q - H * H - KD * H - H;
+#pragma unroll 8
+    for (int b = 0; b < B; ++b) s += dP[(size_t)b * KD + r];
+    grads[o.b4 + r] = s;
+  } else if (q == H * H + KD * H + H + KD) {
+    for (int b = 0; b < B; ++b) s += set_loss[b];
+    *loss = s;
+  }
+}
+
+// Backward through the per-point layers and their weight gradients.  Block b
+// takes the run of 64-point tiles [b T / gridDim, (b + 1) T / gridDim) and
+// writes one partial gradient.  Per tile: h1 again from the standardised
+// points (3 multiply-adds a value, against 512 bytes a point read back) and
+// dz2 from the sign bits of h2, in the layouts the two products read; dh1 =
+// dz2 W2 (4 points x 8 units per thread), dW2 += dz2^T h1 (8 x 8 outputs per
+// thread, in registers over all tiles).  Bound by the FP32 multiply-adds of
+// the two products (34.4e9 for 1M points: 0.92 ms at one per lane and cycle);
+// 1M points: 1.73 + 3.96 ms in two kernels -> 1.64 ms in one.
+constexpr int kZT = kTileP + 4;  // row stride of dz2 by unit
+constexpr int kZP = H + 4;       // row stride of the tiles by point
+constexpr size_t kBwdSmem = sizeof(float) * (H * H + H * kZT + 2 * kTileP * kZP + 4 * H + 4 * kTileP + H);
+__global__ void __launch_bounds__(256, 1) sn_bwd_points(const float* __restrict__ prm, int d, int k, int S,
+                                                        int64_t tiles, const float* __restrict__ dG,
+                                                        const float* __restrict__ xs,
+                                                        const uint32_t* __restrict__ bits, float* __restrict__ part) {
+  extern __shared__ __align__(16) float sm[];
+  float* s_w2 = sm;                    // [128][128] W2[u][c]
+  float* s_zT = s_w2 + H * H;          // [128][kZT] dz2[u][p]
+  float* s_zP = s_zT + H * kZT;        // [64][kZP] dz2[p][u]
+  float* s_hP = s_zP + kTileP * kZP;   // [64][kZP] h1[p][c]
+  float* s_w1 = s_hP + kTileP * kZP;   // [128][4]
+  float* s_x = s_w1 + 4 * H;           // [64][4]
+  float* s_dg = s_x + 4 * kTileP;      // [128] dg / S of the tile's set
+  const NetOff o = net_off(d, k);
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  const int64_t t0 = tiles * blockIdx.x / gridDim.x, t1 = tiles * (blockIdx.x + 1) / gridDim.x;
+  for (int q = tid; q < H * H / 4; q += 256)
+    reinterpret_cast<float4*>(s_w2)[q] = reinterpret_cast<const float4*>(prm + o.W2)[q];
+  stage_w1(s_w1, prm, o, d, tid, 256);
+  float acc2[8][8];       // dW2: units 8 ty + r, inputs 4 tx + (c & 3) + 64 (c >> 2)
+  float g1[8][4];         // dW1 and db1 of inputs 4 tx + ..., this thread's points: dz1 x_j, dz1
+  float gb2 = 0.f;        // db2 of unit tid (threads 0..127)
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) acc2[r][c] = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) g1[r][j] = 0.f;
+  }
+  int set = -1;
+  for (int64_t t = t0; t < t1; ++t) {
+    const int64_t p0 = t * kTileP;
+    const int b = (int)(p0 / S);
+    __syncthreads();  // the previous tile is read no more
+    if (tid < 4 * kTileP) {
+      const int p = tid >> 2, j = tid & 3;
+      s_x[tid] = j < d ? xs[(p0 + p) * d + j] : 0.f;
+    }
+    if (b != set && tid < H) s_dg[tid] = dG[(size_t)b * H + tid] / (float)S;
+    set = b;
     __syncthreads();
-    for (int q = tid; q < 32 * H; q += blockDim.x) {
-      const int p = q / H;
-      s_a[q] = p < m ? dz2g[(c0 + t0 + p) * H + (q % H)] : 0.f;
-      s_b[q] = p < m ? h1g[(c0 + t0 + p) * H + (q % H)] : 0.f;
+    // dz2 by unit: lanes over points
+    {
+      const int p = tid & 63, w = tid >> 6;  // word w of the point's bits: units 32 w ..
+      const uint32_t m = bits[(p0 + p) * 4 + w];
+#pragma unroll 8
+      for (int u = 0; u < 32; ++u) s_zT[(32 * w + u) * kZT + p] = (m >> u) & 1u ? s_dg[32 * w + u] : 0.f;
+    }
+    // dz2 and h1 by point: lanes over units
+    {
+      const int u = tid & 127, ph = tid >> 7;
+      const float dg = s_dg[u];
+      const float4 w = *reinterpret_cast<const float4*>(s_w1 + 4 * u);
+#pragma unroll 8
+      for (int q = 0; q < kTileP / 2; ++q) {
+        const int p = 2 * q + ph;
+        const uint32_t m = bits[(p0 + p) * 4 + (u >> 5)];
+        s_zP[p * kZP + u] = (m >> (u & 31)) & 1u ? dg : 0.f;
+        const float4 xv = *reinterpret_cast<const float4*>(s_x + 4 * p);
+        s_hP[p * kZP + u] = fmaxf(fmaf(w.z, xv.z, fmaf(w.y, xv.y, fmaf(w.x, xv.x, w.w))), 0.f);
+      }
     }
     __syncthreads();
-    for (int p = 0; p < 32; ++p) {
-      const float4 a0 = *reinterpret_cast<const float4*>(s_a + p * H + 8 * ty);
-      const float4 a1 = *reinterpret_cast<const float4*>(s_a + p * H + 8 * ty + 4);
-      const float4 b0 = *reinterpret_cast<const float4*>(s_b + p * H + 8 * tx);
-      const float4 b1 = *reinterpret_cast<const float4*>(s_b + p * H + 8 * tx + 4);
-      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+    // dh1[p][c] = sum_u dz2[p][u] W2[u][c]: points 4 ty .. 4 ty + 3
+    {
+      float acc[4][8];
 #pragma unroll
-      for (int r = 0; r < 8; ++r)
+      for (int r = 0; r < 4; ++r)
 #pragma unroll
-        for (int c = 0; c < 8; ++c) acc[r][c] = fmaf(av[r], bv[c], acc[r][c]);
+        for (int c = 0; c < 8; ++c) acc[r][c] = 0.f;
+#pragma unroll 4
+      for (int u = 0; u < H; ++u) {
+        const float4 a = *reinterpret_cast<const float4*>(s_zT + u * kZT + 4 * ty);
+        const float4 w0 = *reinterpret_cast<const float4*>(s_w2 + u * H + 4 * tx);
+        const float4 w1 = *reinterpret_cast<const float4*>(s_w2 + u * H + 64 + 4 * tx);
+        const float av[4] = {a.x, a.y, a.z, a.w};
+        const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int c = 0; c < 8; ++c) acc[r][c] = fmaf(av[r], wv[c], acc[r][c]);
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int p = 4 * ty + r;
+        const float4 xv = *reinterpret_cast<const float4*>(s_x + 4 * p);
+        const float4 h0 = *reinterpret_cast<const float4*>(s_hP + p * kZP + 4 * tx);
+        const float4 h1 = *reinterpret_cast<const float4*>(s_hP + p * kZP + 64 + 4 * tx);
+        const float hv[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const float z1 = hv[c] > 0.f ? acc[r][c] : 0.f;
+          g1[c][0] = fmaf(z1, xv.x, g1[c][0]);
+          g1[c][1] = fmaf(z1, xv.y, g1[c][1]);
+          g1[c][2] = fmaf(z1, xv.z, g1[c][2]);
+          g1[c][3] += z1;
+        }
+      }
+    }
+    // dW2[u][c] += sum_p dz2[p][u] h1[p][c]
+    tile_gemm_8x8<kTileP, kZP, kZP>(s_zP, s_hP, ty, tx, acc2);
+    if (tid < H) {
+      float s = 0.f;
+#pragma unroll 8
+      for (int p = 0; p < kTileP; ++p) s += s_zP[p * kZP + tid];
+      gb2 += s;
     }
   }
   const int stride = H * H + H * d + 2 * H;
@@ -357,28 +514,35 @@ __global__ void __launch_bounds__(256) sn_wgrad(const float* __restrict__ dz2g, 
 #pragma unroll
   for (int r = 0; r < 8; ++r)
 #pragma unroll
-    for (int c = 0; c < 8; ++c) out[(8 * ty + r) * H + 8 * tx + c] = acc[r][c];
-  if (tid < H) {
-    float w1[3] = {0.f, 0.f, 0.f}, g1 = 0.f, g2 = 0.f;
-    for (int p = 0; p < np; ++p) {
-      const float z1 = dz1g[(c0 + p) * H + tid];
-      g1 += z1;
-      g2 += dz2g[(c0 + p) * H + tid];
-      for (int j = 0; j < d; ++j) w1[j] = fmaf(z1, xs[(c0 + p) * d + j], w1[j]);
-    }
-    for (int j = 0; j < d; ++j) out[H * H + tid * d + j] = w1[j];
-    out[H * H + H * d + tid] = g1;
-    out[H * H + H * d + H + tid] = g2;
+    for (int c = 0; c < 8; ++c) out[(8 * ty + r) * H + 4 * tx + (c & 3) + 64 * (c >> 2)] = acc2[r][c];
+  // dW1 and db1: the 16 point groups' sums, added in order
+  __syncthreads();
+  float* s_g = sm;  // [16][128][4]
+#pragma unroll
+  for (int c = 0; c < 8; ++c)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) s_g[(ty * H + 4 * tx + (c & 3) + 64 * (c >> 2)) * 4 + j] = g1[c][j];
+  __syncthreads();
+  for (int q = tid; q < 4 * H; q += 256) {
+    float s = 0.f;
+    for (int g = 0; g < 16; ++g) s += s_g[g * 4 * H + q];
+    const int u = q >> 2, j = q & 3;
+    if (j == 3) out[H * H + H * d + u] = s;
+    else if (j < d) out[H * H + u * d + j] = s;
   }
+  if (tid < H) out[H * H + H * d + H + tid] = gb2;
 }
 
-__global__ void sn_wgrad_reduce(const float* part, int nchunks, int d, int k, float* grads) {
+// The blocks' partial gradients added in order.
+__global__ void __launch_bounds__(64) sn_wgrad_reduce(const float* __restrict__ part, int nparts, int d, int k,
+                                                      float* __restrict__ grads) {
   const NetOff o = net_off(d, k);
   const int stride = H * H + H * d + 2 * H;
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= stride) return;
   float s = 0.f;
-  for (int c = 0; c < nchunks; ++c) s += part[(size_t)c * stride + q];
+#pragma unroll 8
+  for (int c = 0; c < nparts; ++c) s += part[(size_t)c * stride + q];
   int dst;
   if (q < H * H) dst = o.W2 + q;
   else if (q < H * H + H * d) dst = o.W1 + (q - H * H);
@@ -434,39 +598,51 @@ cudaError_t launch_setnet_destandardize(const float* P, const float* ms, int B, 
   return cudaGetLastError();
 }
 
-size_t setnet_point_smem() { return sizeof(float) * (H * H + H * kAT + 8 * H); }
+template <int PT>
+static cudaError_t launch_fwd_points(const SetNetArgs& a, bool train, int64_t P, cudaStream_t st) {
+  const size_t smem = sizeof(float) * (H * H + H * (PT + 4) + 4 * H);
+  cudaError_t e = cudaFuncSetAttribute(sn_fwd_points<PT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  sn_fwd_points<PT><<<(unsigned)((P + PT - 1) / PT), 2 * PT, smem, st>>>(a.xs, a.prm, a.w2t, a.d, a.k, P,
+                                                                       train ? a.bits : nullptr, a.tile_pool);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_setnet_forward(const SetNetArgs& a, bool train, cudaStream_t st) {
   const int64_t P = (int64_t)a.B * a.S;
-  const int tiles = (int)(P / kTileP);
   sn_standardize<<<a.B, 256, 0, st>>>(a.x, train ? a.t : nullptr, a.S, a.d, a.k, a.xs, a.ts, a.ms);
-  const size_t smem = setnet_point_smem();
-  cudaError_t e = cudaFuncSetAttribute(sn_fwd_points, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   sn_transpose<<<H * H / 256, 256, 0, st>>>(a.prm, a.d, a.k, a.w2t);
-  sn_fwd_points<<<tiles, 256, smem, st>>>(a.xs, a.prm, a.w2t, a.d, a.k, a.h1, a.h2, a.tile_pool);
-  sn_pool<<<a.B, H, 0, st>>>(a.tile_pool, a.S / kTileP, a.S, a.G);
-  sn_head<<<1, 256, 0, st>>>(a.prm, a.G, a.B, a.d, a.k, train ? a.ts : nullptr, a.P, a.grads, a.dG, a.loss);
+  // 256-point blocks (one per SM) once they fill the SMs twice over; below
+  // that 64-point ones, two to an SM
+  cudaError_t e = P >= int64_t(256) * 2 * 152 ? launch_fwd_points<256>(a, train, P, st)
+                                              : launch_fwd_points<64>(a, train, P, st);
+  if (e != cudaSuccess) return e;
+  const size_t hs = sizeof(float) * (size_t)std::max(H, a.k * a.d) * kWS;
+  e = cudaFuncSetAttribute(sn_head, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hs);
+  if (e != cudaSuccess) return e;
+  sn_head<<<a.B, 256, hs, st>>>(a.prm, a.tile_pool, a.S / kTileP, a.S, a.B, a.d, a.k, train ? a.ts : nullptr, a.G, a.P,
+                                a.A3, a.dZ3, a.dP, a.dG, a.set_loss);
+  if (train) {
+    const int nv = H * H + a.k * a.d * (H + 1) + H + 1;
+    sn_head_grad<<<(nv + 127) / 128, 128, 0, st>>>(a.B, a.d, a.k, a.G, a.A3, a.dZ3, a.dP, a.set_loss, a.grads, a.loss);
+  }
   return cudaGetLastError();
 }
+
+static int bwd_blocks(int64_t P) { return (int)std::min<int64_t>(P / kTileP, kBwdBlocks); }
 
 cudaError_t launch_setnet_backward(const SetNetArgs& a, cudaStream_t st) {
   const int64_t P = (int64_t)a.B * a.S;
-  const int tiles = (int)(P / kTileP);
-  const size_t smem = sizeof(float) * (H * H + H * kAT);
-  cudaError_t e = cudaFuncSetAttribute(sn_bwd_points, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const int nb = bwd_blocks(P);
+  cudaError_t e = cudaFuncSetAttribute(sn_bwd_points, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBwdSmem);
   if (e != cudaSuccess) return e;
-  sn_bwd_points<<<tiles, 256, smem, st>>>(a.prm, a.d, a.k, a.S, a.dG, a.h1, a.h2, a.dz2, a.dz1);
-  const int nch = (int)((P + kChunkP - 1) / kChunkP);
-  sn_wgrad<<<nch, 256, 0, st>>>(a.dz2, a.h1, a.dz1, a.xs, a.d, P, a.part);
+  sn_bwd_points<<<nb, 256, kBwdSmem, st>>>(a.prm, a.d, a.k, a.S, P / kTileP, a.dG, a.xs, a.bits, a.part);
   const int stride = H * H + H * a.d + 2 * H;
-  sn_wgrad_reduce<<<(stride + 255) / 256, 256, 0, st>>>(a.part, nch, a.d, a.k, a.grads);
+  sn_wgrad_reduce<<<(stride + 63) / 64, 64, 0, st>>>(a.part, nb, a.d, a.k, a.grads);
   return cudaGetLastError();
 }
 
-int64_t setnet_part_floats(int64_t P, int d) {
-  return ((P + kChunkP - 1) / kChunkP) * (int64_t)(H * H + H * d + 2 * H);
-}
+int64_t setnet_part_floats(int64_t P, int d) { return (int64_t)bwd_blocks(P) * (H * H + H * d + 2 * H); }
 
 cudaError_t launch_setnet_adam(float* prm, const float* grads, float* m, float* v, int n, float lr, float b1,
                                float b2, float eps, float c1, float c2, cudaStream_t st) {

@@ -19,9 +19,10 @@ struct km_setnet {
   long adam_t = 0;
   int capB = 0, capS = 0;
   float *xin = nullptr, *tin = nullptr;  // host inputs are copied here
-  float *xs = nullptr, *ts = nullptr, *ms = nullptr, *w2t = nullptr, *h1 = nullptr, *h2 = nullptr;
+  float *xs = nullptr, *ts = nullptr, *ms = nullptr, *w2t = nullptr;
+  uint32_t* bits = nullptr;  // one bit per h2 value: h2 > 0
   float *tile_pool = nullptr, *G = nullptr, *P = nullptr, *dG = nullptr, *loss = nullptr;
-  float *dz2 = nullptr, *dz1 = nullptr, *part = nullptr;
+  float *A3 = nullptr, *dZ3 = nullptr, *dP = nullptr, *set_loss = nullptr, *part = nullptr;
   double* cout = nullptr;
   std::string err;
 };
@@ -47,13 +48,15 @@ cudaError_t nalloc(T** p, size_t count) {
 }
 
 void free_work(km_setnet* n) {
-  float* bufs[] = {n->xin, n->tin, n->xs, n->ts, n->ms, n->h1, n->h2, n->tile_pool, n->G, n->P, n->dG, n->dz2,
-                   n->dz1, n->part};
+  float* bufs[] = {n->xin, n->tin, n->xs, n->ts, n->ms, n->tile_pool, n->G, n->P, n->dG, n->A3,
+                   n->dZ3, n->dP, n->set_loss, n->part};
   for (float* p : bufs)
     if (p) cudaFree(p);
   if (n->cout) cudaFree(n->cout);
-  n->xin = n->tin = n->xs = n->ts = n->ms = n->h1 = n->h2 = n->tile_pool = n->G = n->P = n->dG = n->dz2 = n->dz1 =
-      n->part = nullptr;
+  if (n->bits) cudaFree(n->bits);
+  n->bits = nullptr;
+  n->xin = n->tin = n->xs = n->ts = n->ms = n->tile_pool = n->G = n->P = n->dG = n->A3 = n->dZ3 = n->dP =
+      n->set_loss = n->part = nullptr;
   n->cout = nullptr;
   n->capB = n->capS = 0;
 }
@@ -69,14 +72,15 @@ km_status ensure(km_setnet* n, int B, int S) {
   KN_CUDA(n, nalloc(&n->xs, (size_t)Pn * d));
   KN_CUDA(n, nalloc(&n->ts, (size_t)B * KD));
   KN_CUDA(n, nalloc(&n->ms, (size_t)B * 2 * d));
-  KN_CUDA(n, nalloc(&n->h1, (size_t)Pn * kSetH));
-  KN_CUDA(n, nalloc(&n->h2, (size_t)Pn * kSetH));
+  KN_CUDA(n, nalloc(&n->bits, (size_t)Pn * (kSetH / 32)));
   KN_CUDA(n, nalloc(&n->tile_pool, (size_t)(Pn / 64) * kSetH));
   KN_CUDA(n, nalloc(&n->G, (size_t)B * kSetH));
   KN_CUDA(n, nalloc(&n->P, (size_t)B * KD));
   KN_CUDA(n, nalloc(&n->dG, (size_t)B * kSetH));
-  KN_CUDA(n, nalloc(&n->dz2, (size_t)Pn * kSetH));
-  KN_CUDA(n, nalloc(&n->dz1, (size_t)Pn * kSetH));
+  KN_CUDA(n, nalloc(&n->A3, (size_t)B * kSetH));
+  KN_CUDA(n, nalloc(&n->dZ3, (size_t)B * kSetH));
+  KN_CUDA(n, nalloc(&n->dP, (size_t)B * KD));
+  KN_CUDA(n, nalloc(&n->set_loss, (size_t)B));
   KN_CUDA(n, nalloc(&n->part, (size_t)setnet_part_floats(Pn, d)));
   KN_CUDA(n, nalloc(&n->cout, (size_t)B * KD));
   n->capB = B;
@@ -88,9 +92,9 @@ SetNetArgs args(km_setnet* n, const float* x, const float* t, int B, int S) {
   SetNetArgs a{};
   a.x = x; a.t = t; a.B = B; a.S = S; a.d = n->d; a.k = n->k;
   a.prm = n->prm; a.grads = n->grads;
-  a.xs = n->xs; a.ts = n->ts; a.ms = n->ms; a.w2t = n->w2t; a.h1 = n->h1; a.h2 = n->h2;
+  a.xs = n->xs; a.ts = n->ts; a.ms = n->ms; a.w2t = n->w2t; a.bits = n->bits;
   a.tile_pool = n->tile_pool; a.G = n->G; a.P = n->P; a.dG = n->dG; a.loss = n->loss;
-  a.dz2 = n->dz2; a.dz1 = n->dz1; a.part = n->part;
+  a.A3 = n->A3; a.dZ3 = n->dZ3; a.dP = n->dP; a.set_loss = n->set_loss; a.part = n->part;
   return a;
 }
 

@@ -1,0 +1,45 @@
+"""Kernels at the sizes where their tiling, chunking or dispatch changes,
+against the FP64 oracle (or plain FP64 numpy)."""
+import numpy as np
+import pytest
+
+import synth
+from oracle import setnet as osn
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def km():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2405_12052_gb300 as m
+    m.build()
+    return m
+
+
+# one tile; fewer tiles than backward blocks; the last sizes of the 64-point
+# forward blocks and the first of the 256-point ones (77,824 points), the
+# latter with a last block of 64 points; d below 3, K at its limits
+@pytest.mark.parametrize("B,S,d,k", [(1, 64, 3, 16), (5, 192, 1, 1), (1215, 64, 3, 4), (19, 4096, 3, 16),
+                                     (1217, 64, 2, 64)])
+def test_setnet_tile_edges(km, B, S, d, k):
+    rng = np.random.default_rng(B + S)
+    p32 = osn.flatten(osn.init_params(d, k, 128, seed=B)).astype(np.float32)
+    x = rng.normal(scale=3.0, size=(B, S, d)).astype(np.float32)
+    t = rng.normal(scale=3.0, size=(B, k, d)).astype(np.float32)
+    pr = osn.unflatten(p32.astype(np.float64), d, k)
+    ref_loss, ref_g = osn.loss_and_grads(pr, x.astype(np.float64), t.astype(np.float64), k)
+    net = km.SetNet(d, k)
+    net.set_params(p32)
+    loss = net.loss_grad(x, t)
+    g = osn.unflatten(net.grads().astype(np.float64), d, k)
+    # the bounds of the set network's other tests: loss 1e-5, gradients 1e-4
+    assert abs(loss - ref_loss) <= 1e-5 * abs(ref_loss)
+    for n in osn.PARAM_NAMES:
+        err = np.linalg.norm(g[n] - ref_g[n]) / max(np.linalg.norm(ref_g[n]), 1e-30)
+        assert err <= 1e-4, (n, err)
+    c = net.predict(x)
+    assert np.max(np.abs(c - osn.predict(pr, x.astype(np.float64), k))) <= 1e-4 * np.abs(x).max()
+    net.close()
