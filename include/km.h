@@ -218,9 +218,8 @@ void* km_stream(km_ctx* ctx);
 km_status km_write_labels(km_ctx* ctx);
 
 /* The objective sum_i ||x_i - mu_{z_i}||^2 of the current labels (last step)
- * and centroids, in FP64 with the oracle's order: per point coordinates in
- * order, points in index order within 65536-point chunks, then the chunks
- * in order.  Synchronizes.  Errors: KM_ESTATE, KM_ENOMEM, KM_ECUDA. */
+ * and centroids, in FP64: per point coordinates in order, the points by
+ * fixed-order trees over 4096-point chunks, then the chunks.  Synchronizes.  Errors: KM_ESTATE, KM_ENOMEM, KM_ECUDA. */
 km_status km_objective(km_ctx* ctx, double* obj_out);
 
 /* Copy results of the last step.  mem: KM_HOST or KM_DEVICE_COPY (device

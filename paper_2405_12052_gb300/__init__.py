@@ -361,7 +361,7 @@ class KMeans:
 
     def objective(self) -> float:
         """sum_i ||x_i - mu_{z_i}||^2 of the last step's labels and the
-        current centroids (FP64, the oracle's summation order)."""
+        current centroids (FP64, summed by fixed-order trees)."""
         o = ctypes.c_double()
         self._check(self._L.km_objective(self._h, ctypes.byref(o)))
         return o.value

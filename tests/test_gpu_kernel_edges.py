@@ -43,3 +43,20 @@ def test_setnet_tile_edges(km, B, S, d, k):
     c = net.predict(x)
     assert np.max(np.abs(c - osn.predict(pr, x.astype(np.float64), k))) <= 1e-4 * np.abs(x).max()
     net.close()
+
+
+@pytest.mark.parametrize("n,d,k,label_bytes", [(1, 1, 1, 4), (255, 2, 3, 4), (4096, 3, 9, 1), (4097, 6, 9, 4),
+                                               (1_048_577 + 4096, 2, 5, 1)])
+def test_objective_edges(km, n, d, k, label_bytes):
+    x, _, _ = synth.iso_mixture(n, d, 3, sigma=1.0, box=10.0, seed=n + d)
+    mu0, _ = synth.init_distinct(x, k, seed=7)
+    g = km.KMeans(n, d, k, label_bytes=label_bytes)
+    g.set_points(x)
+    g.set_init(mu0)
+    g.step()
+    z, mu = g.labels().astype(np.int64), g.centroids()
+    ref = float(((x.astype(np.float64) - mu[z].T) ** 2).sum())
+    # two orders of n + d FP64 additions: pairwise and tree sums are each
+    # within (log2(n d) + d + 16) ulps of the sum of the (positive) terms
+    assert abs(g.objective() - ref) <= 2 * (np.log2(n * d + 1) + d + 16) * 2.0**-53 * ref
+    g.close()
