@@ -136,7 +136,7 @@ km_status km_set_init(km_ctx* ctx, const double* mu0);
  * sequential scan's except when a target lies within FP64 rounding of a
  * running-sum boundary.  Outputs (host, may be NULL): mu_out K x d doubles,
  * idx_out K point indices.  Needs km_set_points first; d <= 256; allocates
- * N + N/4096 + 4096 doubles of scratch for the call.
+ * N + N/4096 doubles of scratch for the call.
  * Errors: KM_ESTATE, KM_EINVAL (u outside [0, 1)), KM_ENOMEM, KM_ECUDA. */
 km_status km_init_kmeanspp(km_ctx* ctx, const double* u, double* mu_out, int64_t* idx_out);
 

@@ -605,24 +605,24 @@ km_status km_init_kmeanspp(km_ctx* c, const double* u, double* mu_out, int64_t* 
     if (!(u[q] >= 0.0 && u[q] < 1.0)) return fail(c, KM_EINVAL, "uniforms must lie in [0, 1)");
   const int64_t n = c->n;
   const int64_t nch = kpp_chunks(n);
-  double *du = nullptr, *dmu = nullptr, *d2 = nullptr, *cs = nullptr, *sc = nullptr;
+  double *du = nullptr, *dmu = nullptr, *d2 = nullptr, *cs = nullptr;
   int64_t* didx = nullptr;
   auto release = [&]() {
-    void* b[] = {du, dmu, d2, cs, sc, didx};
+    void* b[] = {du, dmu, d2, cs, didx};
     for (void* p : b)
       if (p) cudaFree(p);
   };
   cudaError_t e = cudaSuccess;
   if ((e = dalloc(&du, (size_t)c->k)) != cudaSuccess || (e = dalloc(&dmu, (size_t)c->k * c->d)) != cudaSuccess ||
       (e = dalloc(&d2, (size_t)n)) != cudaSuccess || (e = dalloc(&cs, (size_t)nch)) != cudaSuccess ||
-      (e = dalloc(&sc, (size_t)4096)) != cudaSuccess || (e = dalloc(&didx, (size_t)c->k)) != cudaSuccess) {
+      (e = dalloc(&didx, (size_t)c->k)) != cudaSuccess) {
     release();
     return fail(c, KM_ENOMEM, std::string("k-means++ buffers: ") + cudaGetErrorString(e));
   }
   std::vector<double> hmu((size_t)c->k * c->d);
   std::vector<int64_t> hidx((size_t)c->k);
   e = cudaMemcpyAsync(du, u, sizeof(double) * c->k, cudaMemcpyHostToDevice, c->st);
-  if (e == cudaSuccess) e = launch_kmeanspp(c->x, c->ld, n, c->d, c->k, du, dmu, didx, d2, cs, sc, c->st);
+  if (e == cudaSuccess) e = launch_kmeanspp(c->x, c->ld, n, c->d, c->k, du, dmu, didx, d2, cs, c->st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(hmu.data(), dmu, sizeof(double) * hmu.size(), cudaMemcpyDeviceToHost, c->st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(hidx.data(), didx, sizeof(int64_t) * hidx.size(), cudaMemcpyDeviceToHost, c->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);

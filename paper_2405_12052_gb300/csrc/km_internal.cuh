@@ -288,7 +288,7 @@ cudaError_t launch_batch_objective(const float* x, const BatchInst* inst, const 
 constexpr int kMaxKppD = 256;
 int64_t kpp_chunks(int64_t n);
 cudaError_t launch_kmeanspp(const float* x, int64_t ld, int64_t n, int d, int k, const double* u, double* mu,
-                            int64_t* idx, double* d2, double* chunk_sum, double* scan, cudaStream_t st);
+                            int64_t* idx, double* d2, double* chunk_sum, cudaStream_t st);
 
 // ---- learned initialiser: set network (d <= 3, K <= 64, H = 128) ----
 constexpr int kSetH = 128;

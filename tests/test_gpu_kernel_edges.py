@@ -45,6 +45,24 @@ def test_setnet_tile_edges(km, B, S, d, k):
     net.close()
 
 
+# chunk edges (4096 points), more chunks than pick threads, every d with its
+# own kernel and the general one, magnitudes near the ends of the screen
+@pytest.mark.parametrize("n,d,k,scale", [(4095, 1, 6, 1.0), (4096, 2, 9, 1.0), (4097, 3, 40, 1.0), (20_000, 4, 33, 1.0),
+                                         (20_000, 5, 12, 1.0), (9_000, 17, 20, 1.0), (4_200_001, 3, 6, 1.0),
+                                         (10_000, 3, 12, 1e-30), (10_000, 2, 12, 1e15), (10_000, 3, 12, 2e19)])
+def test_kmeanspp_edges(km, oracle, n, d, k, scale):
+    x, _, _ = synth.iso_mixture(n, d, max(k // 2, 1), sigma=1.0, box=10.0, seed=n + d)
+    x = (x.astype(np.float64) * scale).astype(np.float32)
+    x[:, n // 2:n // 2 + n // 10] = x[:, :n // 10]  # repeated points: D^2 = 0 once one of them is a centre
+    u = np.random.default_rng(n).random(k)
+    g = km.KMeans(n, d, k)
+    g.set_points(x)
+    mu, idx = g.init_kmeanspp(u)
+    mu_ref, idx_ref = oracle.kmeanspp(x, k, u)
+    assert np.array_equal(idx, idx_ref) and np.array_equal(mu, mu_ref)
+    g.close()
+
+
 @pytest.mark.parametrize("n,d,k,label_bytes", [(1, 1, 1, 4), (255, 2, 3, 4), (4096, 3, 9, 1), (4097, 6, 9, 4),
                                                (1_048_577 + 4096, 2, 5, 1)])
 def test_objective_edges(km, n, d, k, label_bytes):
