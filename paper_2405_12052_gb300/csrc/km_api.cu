@@ -235,7 +235,7 @@ cudaError_t launch_assign(km_ctx* c, bool labels_pass = false) {
     a.A_max = c->A_max; a.B_max_ptr = c->gen_bmax; a.tau = (float)(c->opt.tie_rel * (1.0 + 1e-4));
     a.store_labels = store;
     a.ignore_done = labels_pass ? 1 : 0;
-    e = launch_assign_generic(c->G, 0, c->st, a);
+    e = launch_assign_generic(c->G, c->st, a);
   }
   return e;
 }
@@ -417,7 +417,7 @@ km_status km_create(km_ctx** out, int64_t n, int32_t d, int32_t k, const km_opti
     g = std::max<int64_t>(g, (ntiles + tiles_per_block_max - 1) / tiles_per_block_max);
     c->G = (int)std::max<int64_t>(g, 1);
   } else {
-    int64_t g = std::min<int64_t>((n + kThreads - 1) / kThreads, (int64_t)c->sms * 8);
+    int64_t g = generic_grid(n, d, k, c->sms);
     g = std::max<int64_t>(g, (n + kMaxPointsPerBlock - 1) / kMaxPointsPerBlock);
     c->G = (int)std::max<int64_t>(g, 1);
   }

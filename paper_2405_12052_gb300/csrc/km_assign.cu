@@ -13,8 +13,6 @@
 // compile time (shift packing, unrolled screen); CT reads the screen table
 // from the constant bank instead of shared memory (no vector registers and
 // no shared-memory loads for the table; one context per device holds it).
-// assign_generic_kernel handles any d and K with a direct-form FP32 screen,
-// the same re-check rules and 64-bit atomics into the block's own partial row.
 #include "km_internal.cuh"
 #include "km_fast_common.cuh"
 
@@ -704,82 +702,6 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) batch_fast_kernel(BatchArgs
   }
 }
 
-// Generic path: any d, any K.  One point per thread per iteration of a
-// grid-stride loop; FP32 direct-form screen with the same bound and FP64
-// re-decision as the re-check of the fused kernel; exact integer sums with
-// 64-bit atomics into this block's own partial row.
-__global__ void __launch_bounds__(kThreads) assign_generic_kernel(GenericArgs a) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  if (a.ls->done && !a.ignore_done) return;
-  const int d = a.d, k = a.k, dp = d + 1;
-  unsigned long long* row = reinterpret_cast<unsigned long long*>(a.partials) + (size_t)blockIdx.x * k * dp;
-  for (int q = threadIdx.x; q < k * dp; q += blockDim.x) row[q] = 0ull;
-  __shared__ int n64s, nflag;
-  if (threadIdx.x == 0) { n64s = 0; nflag = 0; }
-  __syncthreads();
-  const DataConst dc = *a.dc;
-  const float B_max = *a.B_max_ptr;
-  const float sB = sqrtf(B_max);
-  int my64 = 0, myflag = 0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    float A = 0.f;
-    for (int j = 0; j < d; ++j) {
-      float t = __fsub_rn(a.x[(int64_t)j * a.ld + i], a.shift[j]);
-      A = __fmaf_rn(t, t, A);
-    }
-    A *= 1.0001f;
-    float best = 3.0e38f, second = 3.0e38f;
-    int kb = 0;
-    for (int c = 0; c < k; ++c) {
-      const float* cc = a.ctil + (size_t)c * d;
-      float dv = 0.f;
-      for (int j = 0; j < d; ++j) {
-        float xt = __fsub_rn(a.x[(int64_t)j * a.ld + i], a.shift[j]);
-        float t = __fsub_rn(xt, __ldg(cc + j));
-        dv = __fmaf_rn(t, t, dv);
-      }
-      if (dv < best) { second = best; best = dv; kb = c; }
-      else if (dv < second) { second = dv; }
-    }
-    if (k > 1) {
-      float sA = sqrtf(A), AB = A + B_max;
-      float e1 = direct_bound(best, sA, sB, AB, d), e2 = direct_bound(second, sA, sB, AB, d);
-      float lo2 = second - e2, hi1 = best + e1;
-      bool clear = (lo2 > hi1) && (lo2 - hi1 > a.tau * (second + e2));
-      if (!clear) {
-        ++myflag;
-        ++my64;
-        double bd = d64_dyn(a.x, a.ld, i, d, a.mu);
-        kb = 0;
-        for (int c = 1; c < k; ++c) {
-          double dd = d64_dyn(a.x, a.ld, i, d, a.mu + (size_t)c * d);
-          if (dd < bd) { bd = dd; kb = c; }
-        }
-      }
-    }
-    if (a.store_labels) {
-      if (a.labels8) a.labels8[i] = (uint8_t)kb;
-      else a.labels[i] = kb;
-    }
-    unsigned long long* r = row + (size_t)kb * dp;
-    for (int j = 0; j < d; ++j) {
-      uint32_t bh, bl;
-      split_limbs(a.x[(int64_t)j * a.ld + i], dc.C_hi, dc.C_lo, bh, bl);
-      long long hi = (long long)(int)(bh - dc.bits_C_hi), lo = (long long)(int)(bl - dc.bits_C_lo);
-      atomicAdd(r + j, (unsigned long long)((hi << 22) + lo));
-    }
-    atomicAdd(r + d, 1ull);
-  }
-  if (my64) atomicAdd(&n64s, my64);
-  if (myflag) atomicAdd(&nflag, myflag);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    if (nflag) atomicAdd(&a.ls->flagged, (unsigned long long)nflag);
-    if (n64s) atomicAdd(&a.ls->fp64_decided, (unsigned long long)n64s);
-  }
-}
-
 }  // namespace
 
 size_t fast_smem_bytes(int d, int kpad, int k, int nwin) {
@@ -881,13 +803,6 @@ int batch_fast_blocks_per_sm() {
   cudaFuncSetAttribute(batch_fast_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_fast_kernel, kThreads, smem) != cudaSuccess) return 1;
   return nb > 0 ? nb : 1;
-}
-
-size_t generic_smem_bytes(int, int) { return 0; }
-
-cudaError_t launch_assign_generic(int grid, size_t smem, cudaStream_t st, const GenericArgs& a) {
-  assign_generic_kernel<<<grid, kThreads, smem, st>>>(a);
-  return cudaGetLastError();
 }
 
 }  // namespace km

@@ -1,0 +1,272 @@
+// Reassignment and per-block sums for any d and K (paper, section "The
+// Lloyd's algorithm", steps 2 and 3): FP32 direct form with its rigorous
+// bound, FP64 in the oracle's order where that leaves a point open, exact
+// fixed-point sums.
+//
+// Bound by the FP32 operations of the direct form, a subtraction and a
+// multiply-add per point, centroid and coordinate (2.05e9 for N = 1e6, d = 16,
+// K = 64: 55 us at one per lane and cycle).  A block takes 128 points against
+// 64 centroids at a time, 32 coordinates of both in shared memory, 8 points x
+// 4 centroids per thread: three 16-byte shared reads per 64 operations, where
+// one point per thread reads its coordinate again for every centroid.  The
+// two smallest distances of a point are kept per thread over the centroid
+// tiles and merged over its 16 threads at the end.  Open points are decided in
+// FP64 by one warp each (lanes over centroids), not by one thread while 31
+// wait.  The sums go to 32-bit windows in shared memory (one per block,
+// flushed every 512 points) while those fit; one 64-bit global atomic per
+// coordinate and point before.  N = 1e6, d = 16, K = 64: 572 -> 214 us.
+#include "km_fast_common.cuh"
+
+namespace km {
+
+namespace {
+
+constexpr int kGP = 128;              // points per tile
+constexpr int kGC = 64;               // centroids per tile
+constexpr int kGD = 32;               // coordinates staged at a time
+constexpr int kGXS = kGP + 4;         // row strides of the staged tiles
+constexpr int kGCS = kGC + 4;
+constexpr int kGFlush = 4;            // point tiles between window flushes (512 additions per bin)
+constexpr size_t kGWinMax = 96 * 1024;   // windows above this: 64-bit global atomics instead
+constexpr size_t kGTotMax = 48 * 1024;   // int64 totals above this: in the block's partial row
+
+__device__ __forceinline__ void top2_merge(float& best, float& second, int& kb, float ob, float os, int ok) {
+  if (ob < best || (ob == best && ok < kb)) {
+    second = fminf(best, os);
+    best = ob;
+    kb = ok;
+  } else {
+    second = fminf(second, ob);
+  }
+}
+
+__global__ void __launch_bounds__(kThreads, 2) assign_generic_kernel(GenericArgs a, int use_win, int tot_sh) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  float* s_x = reinterpret_cast<float*>(smraw);       // [kGD][kGXS] x~ = fl(x - s) by coordinate
+  float* s_c = s_x + kGD * kGXS;                      // [kGD][kGCS] c~ by coordinate
+  long long* s_tot = reinterpret_cast<long long*>(s_c + kGD * kGCS);  // [k][d + 1] when tot_sh
+  const int d = a.d, k = a.k, dp = d + 1, wn = 2 * d + 1;
+  uint32_t* s_win = reinterpret_cast<uint32_t*>(s_tot + (tot_sh ? (size_t)k * dp : 0));  // [k][2 d + 1] when use_win
+  __shared__ float s_A[kGP];
+  __shared__ int s_lab[kGP], s_q[kGP];
+  __shared__ int s_qn, s_n64;
+  if (a.ls->done && !a.ignore_done) return;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31, warp = tid >> 5;
+  long long* row = a.partials + (size_t)blockIdx.x * k * dp;
+  long long* tot = tot_sh ? s_tot : row;
+  for (int q = tid; q < k * dp; q += kThreads) tot[q] = 0;
+  if (use_win)
+    for (int q = tid; q < k * wn; q += kThreads) s_win[q] = 0u;
+  if (tid == 0) { s_qn = 0; s_n64 = 0; }
+  const DataConst dc = *a.dc;
+  const float B_max = *a.B_max_ptr, sB = sqrtf(B_max);
+  const int ktiles = (k + kGC - 1) / kGC, chunks = (d + kGD - 1) / kGD;
+  const int64_t ntiles = (a.n + kGP - 1) / kGP;
+  __syncthreads();
+
+  // the windows' sums of bin q = (cluster, column) into the block's totals
+  auto flush = [&]() {
+    __syncthreads();
+    for (int q = tid; q < k * dp; q += kThreads) {
+      const int c = q / dp, j = q - c * dp;
+      const uint32_t* w = s_win + (size_t)c * wn;
+      const uint32_t cnt = w[0];
+      long long v = (long long)cnt;
+      if (j < d) {
+        const int hi = (int)(w[1 + j] - cnt * dc.bits_C_hi);  // exact: |sum| <= 2^30
+        const int lo = (int)(w[1 + d + j] - cnt * dc.bits_C_lo);
+        v = ((long long)hi << 22) + (long long)lo;
+      }
+      if (cnt) tot[q] += v;
+    }
+    __syncthreads();
+    for (int q = tid; q < k * wn; q += kThreads) s_win[q] = 0u;
+    __syncthreads();
+  };
+
+  int since = 0;
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int64_t base = tile * kGP;
+    const int np = (int)min((int64_t)kGP, a.n - base);
+    float best[8], second[8], A = 0.f;  // A: of point tid (threads below kGP)
+    int kb[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) { best[r] = 3.0e38f; second[r] = 3.0e38f; kb[r] = 0; }
+    for (int kt = 0; kt < ktiles; ++kt) {
+      float acc[8][4];
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
+      for (int ch = 0; ch < chunks; ++ch) {
+        const int j0 = ch * kGD, nj = min(kGD, d - j0);
+        __syncthreads();  // the tiles before are read no more
+        if (kt == 0 || chunks > 1)
+          for (int q = tid; q < nj * kGP; q += kThreads) {
+            const int j = q >> 7, p = q & (kGP - 1);
+            s_x[j * kGXS + p] = p < np ? __fsub_rn(a.x[(int64_t)(j0 + j) * a.ld + base + p], a.shift[j0 + j]) : 0.f;
+          }
+        if (ktiles > 1 || chunks > 1 || tile == blockIdx.x)
+          for (int q = tid; q < nj * kGC; q += kThreads) {
+            const int c = q / nj, j = q - c * nj, cc = kt * kGC + c;
+            s_c[j * kGCS + c] = cc < k ? a.ctil[(size_t)cc * d + j0 + j] : 0.f;
+          }
+        __syncthreads();
+        if (kt == 0 && tid < kGP)
+          for (int j = 0; j < nj; ++j) A = __fmaf_rn(s_x[j * kGXS + tid], s_x[j * kGXS + tid], A);
+#pragma unroll 4
+        for (int j = 0; j < nj; ++j) {
+          const float4 x0 = *reinterpret_cast<const float4*>(s_x + j * kGXS + 8 * ty);
+          const float4 x1 = *reinterpret_cast<const float4*>(s_x + j * kGXS + 8 * ty + 4);
+          const float4 cv = *reinterpret_cast<const float4*>(s_c + j * kGCS + 4 * tx);
+          const float xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+          const float cw[4] = {cv.x, cv.y, cv.z, cv.w};
+#pragma unroll
+          for (int r = 0; r < 8; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              const float t = __fsub_rn(xv[r], cw[c]);
+              acc[r][c] = __fmaf_rn(t, t, acc[r][c]);
+            }
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int cc = kt * kGC + 4 * tx + c;
+        if (cc >= k) break;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          const float dv = acc[r][c];
+          if (dv < best[r]) { second[r] = best[r]; best[r] = dv; kb[r] = cc; }
+          else if (dv < second[r]) second[r] = dv;
+        }
+      }
+    }
+    if (tid < kGP) s_A[tid] = A * 1.0001f;
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int o = 1; o < 16; o <<= 1) {
+        const float ob = __shfl_xor_sync(0xffffffffu, best[r], o), os = __shfl_xor_sync(0xffffffffu, second[r], o);
+        const int ok = __shfl_xor_sync(0xffffffffu, kb[r], o);
+        top2_merge(best[r], second[r], kb[r], ob, os, ok);
+      }
+    __syncthreads();  // s_A
+    {
+      // thread tx < 8 of the group takes point 8 ty + tx
+      float b = 0.f, s2 = 0.f;
+      int kk = 0;
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        if (tx == r) { b = best[r]; s2 = second[r]; kk = kb[r]; }
+      const int p = 8 * ty + tx;
+      if (tx < 8 && p < np) {
+        bool clear = true;
+        if (k > 1) {
+          const float Ap = s_A[p], sA = sqrtf(Ap), AB = Ap + B_max;
+          const float e1 = direct_bound(b, sA, sB, AB, d), e2 = direct_bound(s2, sA, sB, AB, d);
+          const float lo2 = s2 - e2, hi1 = b + e1;
+          clear = (lo2 > hi1) && (lo2 - hi1 > a.tau * (s2 + e2));
+        }
+        s_lab[p] = kk;
+        if (!clear) s_q[atomicAdd(&s_qn, 1)] = p;
+      }
+    }
+    __syncthreads();
+    const int qn = s_qn;
+    for (int e = warp; e < qn; e += kWarps) {
+      const int p = s_q[e];
+      double bd = 0.0;
+      int k64 = -1;
+      for (int c = lane; c < k; c += 32) {
+        const double dd = d64_dyn(a.x, a.ld, base + p, d, a.mu + (size_t)c * d);
+        if (k64 < 0 || dd < bd) { bd = dd; k64 = c; }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const double ob = __shfl_xor_sync(0xffffffffu, bd, o);
+        const int ok = __shfl_xor_sync(0xffffffffu, k64, o);
+        if (ok >= 0 && (k64 < 0 || ob < bd || (ob == bd && ok < k64))) { bd = ob; k64 = ok; }
+      }
+      if (lane == 0) s_lab[p] = k64;
+    }
+    __syncthreads();
+    if (tid == 0) { s_n64 += qn; s_qn = 0; }
+    if (a.store_labels && tid < np) {
+      if (a.labels8) a.labels8[base + tid] = (uint8_t)s_lab[tid];
+      else a.labels[base + tid] = s_lab[tid];
+    }
+    // sums: threads over (point, coordinate), coalesced along the points
+    for (int q = tid; q < dp * kGP; q += kThreads) {
+      const int j = q >> 7, p = q & (kGP - 1);
+      if (p >= np) continue;
+      const int c = s_lab[p];
+      if (j == d) {
+        if (use_win) atomicAdd(s_win + (size_t)c * wn, 1u);
+        else atomicAdd(reinterpret_cast<unsigned long long*>(row) + (size_t)c * dp + d, 1ull);
+        continue;
+      }
+      uint32_t bh, bl;
+      split_limbs(a.x[(int64_t)j * a.ld + base + p], dc.C_hi, dc.C_lo, bh, bl);
+      if (use_win) {
+        atomicAdd(s_win + (size_t)c * wn + 1 + j, bh);
+        atomicAdd(s_win + (size_t)c * wn + 1 + d + j, bl);
+      } else {
+        const long long hi = (long long)(int)(bh - dc.bits_C_hi), lo = (long long)(int)(bl - dc.bits_C_lo);
+        atomicAdd(reinterpret_cast<unsigned long long*>(row) + (size_t)c * dp + j, (unsigned long long)((hi << 22) + lo));
+      }
+    }
+    if (use_win && ++since == kGFlush) {
+      flush();
+      since = 0;
+    }
+  }
+  if (use_win && since) flush();
+  __syncthreads();
+  if (tot_sh)
+    for (int q = tid; q < k * dp; q += kThreads) row[q] = s_tot[q];
+  if (tid == 0 && s_n64) {
+    atomicAdd(&a.ls->flagged, (unsigned long long)s_n64);
+    atomicAdd(&a.ls->fp64_decided, (unsigned long long)s_n64);
+  }
+}
+
+// Where the sums go: windows while they take at most 96 KB (two blocks stay
+// resident on an SM), int64 totals beside them while those take at most 48 KB,
+// else in the block's own row (read and written by one thread each, every 512
+// points); without windows (K d beyond 12,000) 64-bit atomics into the row.
+struct GenericPlan {
+  int use_win, tot_sh;
+  size_t smem;
+};
+GenericPlan generic_plan(int d, int k) {
+  const size_t win = (size_t)k * (2 * (size_t)d + 1) * 4, tot = (size_t)k * (d + 1) * 8;
+  GenericPlan g{};
+  g.use_win = win <= kGWinMax ? 1 : 0;
+  g.tot_sh = g.use_win && tot <= kGTotMax && win + tot <= kGWinMax ? 1 : 0;
+  g.smem = sizeof(float) * kGD * (kGXS + kGCS) + (g.use_win ? win : 0) + (g.tot_sh ? tot : 0);
+  return g;
+}
+
+}  // namespace
+
+int64_t generic_grid(int64_t n, int d, int k, int sms) {
+  const GenericPlan g = generic_plan(d, k);
+  int nb = 0;
+  if (cudaFuncSetAttribute(assign_generic_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem) !=
+          cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, assign_generic_kernel, kThreads, g.smem) != cudaSuccess ||
+      nb < 1)
+    nb = 1;
+  return std::min<int64_t>((n + kGP - 1) / kGP, (int64_t)sms * nb);
+}
+
+cudaError_t launch_assign_generic(int grid, cudaStream_t st, const GenericArgs& a) {
+  const GenericPlan g = generic_plan(a.d, a.k);
+  cudaError_t e = cudaFuncSetAttribute(assign_generic_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+  if (e != cudaSuccess) return e;
+  assign_generic_kernel<<<grid, kThreads, g.smem, st>>>(a, g.use_win, g.tot_sh);
+  return cudaGetLastError();
+}
+
+}  // namespace km

@@ -332,8 +332,8 @@ size_t fast_smem_bytes(int d, int kpad, int k, int nwin);
 int fast_blocks_per_sm(int d, size_t smem, int kpad, bool ct);
 // The fused kernel has a constant-bank screen table for this shape.
 bool fast_has_const_table(int d, int kpad);
-cudaError_t launch_assign_generic(int grid, size_t smem, cudaStream_t st, const GenericArgs& a);
-size_t generic_smem_bytes(int d, int k);
+cudaError_t launch_assign_generic(int grid, cudaStream_t st, const GenericArgs& a);
+int64_t generic_grid(int64_t n, int d, int k, int sms);
 
 struct UpdateArgs {
   const long long* partials; int G; int k; int d;

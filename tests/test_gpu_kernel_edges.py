@@ -78,3 +78,32 @@ def test_objective_edges(km, n, d, k, label_bytes):
     # within (log2(n d) + d + 16) ulps of the sum of the (positive) terms
     assert abs(g.objective() - ref) <= 2 * (np.log2(n * d + 1) + d + 16) * 2.0**-53 * ref
     g.close()
+
+
+# tiles of 128 points x 64 centroids x 32 coordinates and their edges; sums in
+# shared windows with totals beside them, in the block's row, and (K d large)
+# by global atomics; more points per block than one window flush
+@pytest.mark.parametrize("n,d,k,kw", [
+    (1, 5, 1, {}), (127, 31, 3, {}), (129, 32, 64, {}), (3000, 33, 65, {}), (200_003, 5, 7, {}), (100_001, 16, 64, {}),
+    (20_000, 40, 130, {}), (5000, 70, 200, {}), (3000, 130, 257, {"label_policy": "final"}), (2000, 2, 1000, {}),
+    (50_001, 7, 256, {"label_bytes": 1}), (20_003, 64, 100, {"dist_path": "simt"})])
+def test_generic_tile_edges(km, oracle, n, d, k, kw):
+    x, _, _ = synth.iso_mixture(n, d, max(2, k // 3), sigma=1.0, box=6.0, seed=n + d)
+    x[:, n // 2:n // 2 + n // 20] = x[:, :n // 20]  # repeated points
+    mu0, _ = synth.init_distinct(x, k, seed=3)
+    if k > 2:
+        mu0[2] = mu0[1]                            # an exact tie: the lowest index takes the points
+    g = km.KMeans(n, d, k, **kw)
+    g.set_points(x)
+    mu = mu0
+    for _ in range(2):
+        g.set_init(mu)
+        g.step()
+        z, mu_ref, cnt, e2 = oracle.step(x, mu)
+        assert np.array_equal(g.counts(), cnt)
+        if kw.get("label_policy") is None:
+            assert np.array_equal(g.labels(), z)
+        assert np.allclose(g.centroids(), mu_ref, rtol=1e-6, atol=1e-6)
+        mu = mu_ref
+    assert g.stats()["path"] == 2
+    g.close()
