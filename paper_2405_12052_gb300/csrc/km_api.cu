@@ -735,7 +735,10 @@ km_status km_run(km_ctx* c, int32_t max_iter, double tol, int32_t* labels_out,
         cudaGraph_t g = nullptr;
         KM_CUDA(c, cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal));
         cudaError_t e = cudaSuccess;
-        for (int u = 0; u < c->graph_unroll && e == cudaSuccess; ++u) e = launch_step(c);
+        // the tensor-core path's steps are many kernels, so fewer of them run
+        // on past the stop
+        const int unroll = c->path == 3 ? 4 : c->graph_unroll;
+        for (int u = 0; u < unroll && e == cudaSuccess; ++u) e = launch_step(c);
         cudaError_t e2 = cudaStreamEndCapture(c->st, &g);
         KM_CUDA(c, e);
         KM_CUDA(c, e2);

@@ -120,6 +120,7 @@ __device__ __forceinline__ float bound64(float dv, float sA, float sB, float AB)
 // The oracle's distance: FP64, coordinates in order.
 __device__ __forceinline__ double d64row(const float* __restrict__ xrow, const double* __restrict__ mrow) {
   double acc = 0.0;
+#pragma unroll 16
   for (int j = 0; j < kGemmD; ++j) {
     const double t = __dsub_rn((double)xrow[j], mrow[j]);
     acc = __dadd_rn(acc, __dmul_rn(t, t));
@@ -655,24 +656,30 @@ __global__ void __launch_bounds__(256, 4) gemm_tie_kernel(GemmArgs a) {
       const float e1 = bound64(best, sA, sB, AB), e2 = bound64(second, sA, sB, AB);
       const float lo2 = second - e2, hi1 = best + e1;
       const bool need64 = !((lo2 > hi1) && (lo2 - hi1 > gc.tau * (second + e2)));
-      if (sub == 0) {
-        if (need64) {
-          // (rare) the candidates read again from the staged entry
-          const unsigned short* cl = reinterpret_cast<const unsigned short*>(&s_ent[st][grp][0]) + 4;
-          const float* xr = a.xaos + (size_t)ii * kGemmD;
-          double bd = 0.0;
-          int k64 = -1;
-          for (int q = 0; q < nc; ++q) {
-            const int c = cl[q];
-            if (c >= a.k) continue;
-            const double dd = d64row(xr, a.mu + (size_t)c * kGemmD);
-            if (k64 < 0 || dd < bd || (dd == bd && c < k64)) { bd = dd; k64 = c; }
-          }
-          lab = k64;
-          ++n64;
+      if (need64) {  // the same on the 4 threads
+        // the candidates read again from the staged entry, dealt over the 4
+        // threads (one thread took them one after another, 64 dependent FP64
+        // additions each: the tail of a small step's kernel)
+        const unsigned short* cl = reinterpret_cast<const unsigned short*>(&s_ent[st][grp][0]) + 4;
+        const float* xr = a.xaos + (size_t)ii * kGemmD;
+        double bd = 0.0;
+        int k64 = -1;
+        for (int q = sub; q < nc; q += 4) {
+          const int c = cl[q];
+          if (c >= a.k) continue;
+          const double dd = d64row(xr, a.mu + (size_t)c * kGemmD);
+          if (k64 < 0 || dd < bd || (dd == bd && c < k64)) { bd = dd; k64 = c; }
         }
-        a.labels[ii] = lab;
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+          const double ob = __shfl_xor_sync(gmask, bd, o);
+          const int ok = __shfl_xor_sync(gmask, k64, o);
+          if (ok >= 0 && (k64 < 0 || ob < bd || (ob == bd && ok < k64))) { bd = ob; k64 = ok; }
+        }
+        lab = k64;
+        n64 += sub == 0 ? 1 : 0;
       }
+      if (sub == 0) a.labels[ii] = lab;
     }
     __syncwarp(gmask);  // stage st is refilled by the next iteration's copy
   }
@@ -793,44 +800,50 @@ __global__ void __launch_bounds__(kGM) gemm_prep_points_kernel(const float* __re
   }
 }
 
-// Tables of the next step from mu, one thread per centroid: BF16 rows in the
-// swizzled layout (FP16 rows are written by the consts kernel, which knows
-// their scale), FP32 c~ rows and B_k = ||mu_k - s||^2 (FP64, coordinates in
-// order).
-__global__ void __launch_bounds__(64) gemm_tables_kernel(GemmPrepArgs a) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+// Tables of the next step from mu, one warp per centroid (two coordinates per
+// lane): BF16 rows in the swizzled layout (FP16 rows are written by the consts
+// kernel, which knows their scale), FP32 c~ rows and B_k = ||mu_k - s||^2
+// (FP64, a fixed-order tree).  One thread per centroid, its 64 coordinates one
+// after another, took 20 us.
+__global__ void __launch_bounds__(256) gemm_tables_kernel(GemmPrepArgs a) {
+  const int c = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (c >= a.kpad) return;
-  __nv_bfloat16* cb = reinterpret_cast<__nv_bfloat16*>(a.cb);
+  const int j = 2 * lane;  // coordinates j, j + 1: one 32-bit word of a BF16 row
+  float2 cv = make_float2(0.f, 0.f);
   double B = 0.0;
-  for (int j = 0; j < kGemmD; ++j) {
-    float cv = 0.f;
-    if (c < a.k) {
-      const double t = __dsub_rn(a.mu[(size_t)c * kGemmD + j], (double)a.shift[j]);
-      cv = __double2float_rn(t);
-      a.ctil[(size_t)c * kGemmD + j] = cv;
-      B = __dadd_rn(B, __dmul_rn(t, t));
-    }
-    if (!a.f16) cb[swz_index(c, j)] = __float2bfloat16_rn(cv);
+  if (c < a.k) {
+    const double2 m = *reinterpret_cast<const double2*>(a.mu + (size_t)c * kGemmD + j);
+    const float2 sv = *reinterpret_cast<const float2*>(a.shift + j);
+    const double t0 = __dsub_rn(m.x, (double)sv.x), t1 = __dsub_rn(m.y, (double)sv.y);
+    cv = make_float2(__double2float_rn(t0), __double2float_rn(t1));
+    *reinterpret_cast<float2*>(a.ctil + (size_t)c * kGemmD + j) = cv;
+    B = __dadd_rn(__dmul_rn(t0, t0), __dmul_rn(t1, t1));
   }
-  a.bnorm[c] = c < a.k ? B : 0.0;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) B = __dadd_rn(B, __shfl_xor_sync(0xffffffffu, B, o));
+  if (!a.f16)
+    *reinterpret_cast<__nv_bfloat162*>(reinterpret_cast<__nv_bfloat16*>(a.cb) + swz_index(c, j)) =
+        __nv_bfloat162(__float2bfloat16_rn(cv.x), __float2bfloat16_rn(cv.y));
+  if (lane == 0) a.bnorm[c] = B;
 }
 
-// The scale and window constants from max_k B_k (one block), then n'_k and,
-// for FP16 operands, the centre rows scaled by 2^ec.
+// The scale and window constants from max_k B_k (formed by every block for
+// itself), then n'_k and, for FP16 operands, the centre rows scaled by 2^ec,
+// dealt over the blocks (one block wrote all FP16 rows before: 23 us).
 __global__ void __launch_bounds__(256) gemm_consts_kernel(GemmPrepArgs a) {
-  __shared__ double s_max[256];
+  __shared__ long long s_max[8];
   __shared__ int s_sigma, s_ec;
   const int k = a.k, kpad = a.kpad;
-  double m = 0.0;
-  for (int c = threadIdx.x; c < k; c += blockDim.x) m = fmax(m, a.bnorm[c]);
-  s_max[threadIdx.x] = m;
+  // nonnegative doubles are ordered as integers
+  long long m = 0;
+  for (int c = threadIdx.x; c < k; c += blockDim.x) m = max(m, __double_as_longlong(a.bnorm[c]));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = m;
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) s_max[threadIdx.x] = fmax(s_max[threadIdx.x], s_max[threadIdx.x + w]);
-    __syncthreads();
-  }
   if (threadIdx.x == 0) {
-    const double bmax = s_max[0];
+    for (int w = 1; w < 8; ++w) m = max(m, s_max[w]);
+    const double bmax = __longlong_as_double(m);
     const double P = 1.02 * ((double)a.A_max + 2.0 * bmax) + 1e-300;
     const double top = 0.5;  // binade [1, 2): M = 1.5, |2^sigma (h - 2S)| < 0.5
     int sigma = ilogb(top / P);
@@ -879,17 +892,18 @@ __global__ void __launch_bounds__(256) gemm_consts_kernel(GemmPrepArgs a) {
     g.B_max = (float)(bmax * (1.0 + 1e-6));
     g.tau = (float)(a.tie_rel * (1.0 + 1e-4));
     g.pad0 = g.pad1 = 0.f;
-    *a.gc = g;
+    if (blockIdx.x == 0) *a.gc = g;
   }
   __syncthreads();
   const double tw = ldexp(1.0, s_sigma);
   // padding columns: r = 4, far above any real r < 2 plus the window
-  for (int c = threadIdx.x; c < kpad; c += blockDim.x)
+  const int t0 = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+  for (int c = t0; c < kpad; c += nt)
     a.nprime[c] = c < k ? __double2float_rn(1.5 + tw * a.bnorm[c]) : 4.0f;
   if (a.f16) {
     const float cs = ldexpf(1.f, s_ec);
     unsigned short* cb = reinterpret_cast<unsigned short*>(a.cb);
-    for (int q = threadIdx.x; q < kpad * kGemmD; q += blockDim.x) {
+    for (int q = t0; q < kpad * kGemmD; q += nt) {
       const int c = q / kGemmD, j = q - c * kGemmD;
       const float cv = c < k ? a.ctil[(size_t)c * kGemmD + j] : 0.f;
       cb[swz_index(c, j)] = __half_as_ushort(__float2half_rn(cv * cs));
@@ -957,10 +971,10 @@ cudaError_t launch_gemm_prep_points(const float* x, int64_t ld, int64_t n, const
 }
 
 cudaError_t launch_gemm_prepare(cudaStream_t st, const GemmPrepArgs& a) {
-  gemm_tables_kernel<<<(a.kpad + 63) / 64, 64, 0, st>>>(a);
+  gemm_tables_kernel<<<(a.kpad + 7) / 8, 256, 0, st>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  gemm_consts_kernel<<<1, 256, 0, st>>>(a);
+  gemm_consts_kernel<<<a.f16 ? a.kpad / 16 : 4, 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -142,6 +142,7 @@ struct GenericArgs {
 constexpr int kGemmD = 64;          // dimension of the tcgen05 path (one 128-byte BF16 row)
 constexpr int kGemmMaxK = 1024;     // centroid rows resident in shared memory
 constexpr int kChunk = 2048;        // points per chunk of the sorted mean calculation
+constexpr int kChunkSmall = 256;    // and for small sets
 
 struct GemmConst {
   float scale;   // -2^(sigma+1)

@@ -15,9 +15,14 @@ namespace km {
 
 namespace {
 
+// The kernels before the finalize take `stop` (the loop state of a step, null
+// for a shard's totals) and return at once when the loop has stopped: a graph
+// of several steps otherwise sorts and sums all points again for each step
+// after the last (0.55 ms each at N = 1e7, d = 64).
 __global__ void ms_hist_kernel(const int32_t* __restrict__ labels, int64_t n, int k,
-                               unsigned long long* counts) {
+                               unsigned long long* counts, const LoopState* stop) {
   extern __shared__ unsigned int sh[];
+  if (stop && stop->done) return;
   const bool use_sh = k <= 8192;
   if (use_sh)
     for (int c = threadIdx.x; c < k; c += blockDim.x) sh[c] = 0u;
@@ -36,17 +41,19 @@ __global__ void ms_hist_kernel(const int32_t* __restrict__ labels, int64_t n, in
 // One block: exclusive scans of the counts (point offsets) and of the
 // per-cluster chunk counts; chunk table entries (cluster, start, length).
 __global__ void ms_scan_kernel(const unsigned long long* counts, int k, int64_t* offsets, int* cfirst,
-                               unsigned long long* cursor, int4* chunks, int* nchunks, int max_chunks) {
+                               unsigned long long* cursor, int4* chunks, int* nchunks, int max_chunks, int chunk,
+                               const LoopState* stop) {
   __shared__ long long s_pt[1024];
   __shared__ int s_ch[1024];
   __shared__ long long carry_pt;
   __shared__ int carry_ch;
+  if (stop && stop->done) return;
   if (threadIdx.x == 0) { carry_pt = 0; carry_ch = 0; }
   __syncthreads();
   for (int base = 0; base < k; base += 1024) {
     const int c = base + threadIdx.x;
     const long long cnt = c < k ? (long long)counts[c] : 0;
-    const int nch = (int)((cnt + kChunk - 1) / kChunk);
+    const int nch = (int)((cnt + chunk - 1) / chunk);
     s_pt[threadIdx.x] = cnt;
     s_ch[threadIdx.x] = nch;
     __syncthreads();
@@ -65,8 +72,8 @@ __global__ void ms_scan_kernel(const unsigned long long* counts, int k, int64_t*
       cfirst[c] = cstart;
       cursor[c] = 0ull;
       for (int q = 0; q < nch && cstart + q < max_chunks; ++q) {
-        const long long a = (long long)q * kChunk;
-        chunks[cstart + q] = make_int4(c, (int)(start + a), (int)min((long long)kChunk, cnt - a), 0);
+        const long long a = (long long)q * chunk;
+        chunks[cstart + q] = make_int4(c, (int)(start + a), (int)min((long long)chunk, cnt - a), 0);
       }
     }
     __syncthreads();
@@ -77,7 +84,8 @@ __global__ void ms_scan_kernel(const unsigned long long* counts, int k, int64_t*
 }
 
 __global__ void ms_scatter_kernel(const int32_t* __restrict__ labels, int64_t n, const int64_t* offsets,
-                                  unsigned long long* cursor, int32_t* perm) {
+                                  unsigned long long* cursor, int32_t* perm, const LoopState* stop) {
+  if (stop && stop->done) return;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const int z = labels[i];
     const unsigned long long pos = atomicAdd(&cursor[z], 1ull);
@@ -93,8 +101,10 @@ constexpr int kScatterPts = 4096;
 constexpr int kScatterMaxK = 4096;
 __global__ void __launch_bounds__(256) ms_scatter_block_kernel(const int32_t* __restrict__ labels, int64_t n, int k,
                                                                const int64_t* __restrict__ offsets,
-                                                               unsigned long long* cursor, int32_t* perm) {
+                                                               unsigned long long* cursor, int32_t* perm,
+                                                               const LoopState* stop) {
   extern __shared__ unsigned long long s_base[];  // [k] run starts, then [k] u32 counts / ranks
+  if (stop && stop->done) return;
   unsigned int* s_cnt = reinterpret_cast<unsigned int*>(s_base + k);
   const int64_t i0 = (int64_t)blockIdx.x * kScatterPts;
   const int64_t i1 = min(n, i0 + kScatterPts);
@@ -122,8 +132,10 @@ __global__ void __launch_bounds__(256) ms_scatter_block_kernel(const int32_t* __
 __global__ void __launch_bounds__(256) ms_chunk_sum4_kernel(const float4* __restrict__ xa4, int d,
                                                             const int32_t* __restrict__ perm,
                                                             const int4* __restrict__ chunks, const int* nchunks,
-                                                            const DataConst* dcp, long long* chunk_sums) {
+                                                            const DataConst* dcp, long long* chunk_sums,
+                                                            const LoopState* stop) {
   extern __shared__ long long s_part4[];  // [R][d]
+  if (stop && stop->done) return;
   const int ch = blockIdx.x;
   if (ch >= *nchunks) return;
   const int4 cd = chunks[ch];
@@ -179,8 +191,9 @@ __global__ void __launch_bounds__(256) ms_chunk_sum4_kernel(const float4* __rest
 // added in order r = 0..R-1.
 __global__ void ms_chunk_sum_kernel(const float* __restrict__ xa, int d, const int32_t* __restrict__ perm,
                                     const int4* __restrict__ chunks, const int* nchunks, const DataConst* dcp,
-                                    long long* chunk_sums /* [max_chunks][d] */) {
+                                    long long* chunk_sums /* [max_chunks][d] */, const LoopState* stop) {
   extern __shared__ long long s_part[];  // [R][d]
+  if (stop && stop->done) return;
   const int ch = blockIdx.x;
   if (ch >= *nchunks) return;
   const int4 cd = chunks[ch];
@@ -242,17 +255,18 @@ __device__ __forceinline__ double ms_i128_to_double(unsigned long long lo, long 
 // written by the path's own prepare kernels afterwards.
 __global__ void __launch_bounds__(256) ms_finalize_kernel(const unsigned long long* counts, const int* cfirst,
                                                           const long long* chunk_sums, int k, int d,
-                                                          const DataConst* dcp, double* mu, long long* counts_out,
-                                                          double* df2, const LoopState* ls) {
+                                                          int chunk, const DataConst* dcp, double* mu,
+                                                          long long* counts_out, double* df2, const LoopState* ls) {
   if (ls->done) return;  // the loop already stopped (graph-driven runs)
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= k * d) return;
   const int c = q / d, j = q - c * d;
   const long long cnt = (long long)counts[c];
   const long long first = cfirst[c];  // index of the cluster's first chunk (from the scan)
-  const int nch = (int)((cnt + kChunk - 1) / kChunk);
+  const int nch = (int)((cnt + chunk - 1) / chunk);
   unsigned long long lo = 0ull;
   long long hi = 0ll;
+#pragma unroll 8
   for (int t = 0; t < nch; ++t) {
     const long long v = chunk_sums[(size_t)(first + t) * d + j];
     const unsigned long long nl = lo + (unsigned long long)v;
@@ -279,7 +293,8 @@ __global__ void __launch_bounds__(1024) ms_close_kernel(const double* df2, int k
   const int tid = threadIdx.x;
   if (tid == 0) s_empty = 0;
   double e2p = 0.0;
-  for (int q = tid; q < kd; q += blockDim.x) e2p = __dadd_rn(e2p, df2[q]);
+#pragma unroll 8
+  for (int q = tid; q < kd; q += 1024) e2p = __dadd_rn(e2p, df2[q]);
   int empty = 0;
   for (int c = tid; c < k; c += blockDim.x) empty += counts[c] == 0;
   s_red[tid] = e2p;
@@ -312,7 +327,7 @@ __global__ void __launch_bounds__(1024) ms_close_kernel(const double* df2, int k
 // sums added in chunk order, as the finalize kernel does) and its count, in
 // the sharded-step table layout [k][d+1] of (low word, high word).
 __global__ void __launch_bounds__(256) ms_shard_totals_kernel(const unsigned long long* counts, const int* cfirst,
-                                                              const long long* chunk_sums, int k, int d,
+                                                              const long long* chunk_sums, int k, int d, int chunk,
                                                               long long* out) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= k * (d + 1)) return;
@@ -324,7 +339,7 @@ __global__ void __launch_bounds__(256) ms_shard_totals_kernel(const unsigned lon
     lo = (unsigned long long)cnt;
   } else {
     const long long first = cfirst[c];
-    const int nch = (int)((cnt + kChunk - 1) / kChunk);
+    const int nch = (int)((cnt + chunk - 1) / chunk);
     for (int t = 0; t < nch; ++t) {
       const long long v = chunk_sums[(size_t)(first + t) * d + j];
       const unsigned long long nl = lo + (unsigned long long)v;
@@ -374,24 +389,30 @@ __global__ void __launch_bounds__(256) ms_shard_finalize_kernel(const long long*
 
 }  // namespace
 
-int64_t msort_max_chunks(int64_t n, int k) { return n / kChunk + k + 1; }
+// Points per chunk: 2048 where that still gives the SMs several chunks each; a
+// small set takes chunks of 256 (2e5 points in 100 clusters make 150 chunks of
+// 2048, one an SM and 128 rows after one another in each thread: 65 us, with
+// 256: 15 us).
+static int msort_chunk(int64_t n) { return n < (int64_t(1) << 21) ? kChunkSmall : kChunk; }
 
-static cudaError_t msort_sums(const MsortArgs& a, cudaStream_t st);
+int64_t msort_max_chunks(int64_t n, int k) { return n / msort_chunk(n) + k + 1; }
+
+static cudaError_t msort_sums(const MsortArgs& a, const LoopState* stop, cudaStream_t st);
 
 cudaError_t launch_msort_step(const MsortArgs& a, cudaStream_t st) {
-  cudaError_t e = msort_sums(a, st);
+  cudaError_t e = msort_sums(a, a.ls, st);
   if (e != cudaSuccess) return e;
-  ms_finalize_kernel<<<(a.k * a.d + 255) / 256, 256, 0, st>>>(a.counts_u, a.cfirst, a.chunk_sums, a.k, a.d, a.dc,
-                                                              a.mu, a.counts, a.df2, a.ls);
+  ms_finalize_kernel<<<(a.k * a.d + 255) / 256, 256, 0, st>>>(a.counts_u, a.cfirst, a.chunk_sums, a.k, a.d,
+                                                              msort_chunk(a.n), a.dc, a.mu, a.counts, a.df2, a.ls);
   ms_close_kernel<<<1, 1024, 0, st>>>(a.df2, a.k * a.d, a.counts, a.k, a.ls);
   return cudaGetLastError();
 }
 
 cudaError_t launch_msort_shard_totals(const MsortArgs& a, long long* out, cudaStream_t st) {
-  cudaError_t e = msort_sums(a, st);
+  cudaError_t e = msort_sums(a, nullptr, st);
   if (e != cudaSuccess) return e;
   ms_shard_totals_kernel<<<(a.k * (a.d + 1) + 255) / 256, 256, 0, st>>>(a.counts_u, a.cfirst, a.chunk_sums, a.k,
-                                                                        a.d, out);
+                                                                        a.d, msort_chunk(a.n), out);
   return cudaGetLastError();
 }
 
@@ -403,33 +424,32 @@ cudaError_t launch_msort_shard_update(const MsortArgs& a, const long long* table
 }
 
 // Histogram, scan, scatter and chunk sums of the sorted mean calculation.
-static cudaError_t msort_sums(const MsortArgs& a, cudaStream_t st) {
-  // callers skip the whole step once the loop has stopped: the flag is read
-  // by the finalize kernel only, so the earlier kernels run unconditionally
+static cudaError_t msort_sums(const MsortArgs& a, const LoopState* stop, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(a.counts_u, 0, sizeof(unsigned long long) * a.k, st);
   if (e != cudaSuccess) return e;
   const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((a.n + 255) / 256, 2048));
   const size_t hs = a.k <= 8192 ? sizeof(unsigned int) * a.k : 0;
-  ms_hist_kernel<<<(unsigned)blocks, 256, hs, st>>>(a.labels, a.n, a.k, a.counts_u);
-  ms_scan_kernel<<<1, 1024, 0, st>>>(a.counts_u, a.k, a.offsets, a.cfirst, a.cursor, a.chunks, a.nchunks, a.max_chunks);
+  ms_hist_kernel<<<(unsigned)blocks, 256, hs, st>>>(a.labels, a.n, a.k, a.counts_u, stop);
+  ms_scan_kernel<<<1, 1024, 0, st>>>(a.counts_u, a.k, a.offsets, a.cfirst, a.cursor, a.chunks, a.nchunks, a.max_chunks,
+                                     msort_chunk(a.n), stop);
   if (a.k <= kScatterMaxK) {
     const int64_t sb = (a.n + kScatterPts - 1) / kScatterPts;
     ms_scatter_block_kernel<<<(unsigned)std::max<int64_t>(1, sb), 256, (size_t)a.k * 12, st>>>(
-        a.labels, a.n, a.k, a.offsets, a.cursor, a.perm);
+        a.labels, a.n, a.k, a.offsets, a.cursor, a.perm, stop);
   } else {
-    ms_scatter_kernel<<<(unsigned)blocks, 256, 0, st>>>(a.labels, a.n, a.offsets, a.cursor, a.perm);
+    ms_scatter_kernel<<<(unsigned)blocks, 256, 0, st>>>(a.labels, a.n, a.offsets, a.cursor, a.perm, stop);
   }
   if (a.d % 4 == 0 && a.d <= 1024 &&
       (reinterpret_cast<uintptr_t>(a.xa) & 15u) == 0) {
     const int R = std::max(1, 256 / (a.d / 4));
     const int threads = R * (a.d / 4);
     ms_chunk_sum4_kernel<<<(unsigned)a.max_chunks, threads, sizeof(long long) * (size_t)R * a.d, st>>>(
-        reinterpret_cast<const float4*>(a.xa), a.d, a.perm, a.chunks, a.nchunks, a.dc, a.chunk_sums);
+        reinterpret_cast<const float4*>(a.xa), a.d, a.perm, a.chunks, a.nchunks, a.dc, a.chunk_sums, stop);
   } else {
     const int R = std::max(1, 256 / a.d);
     const int threads = R * a.d <= 1024 ? R * a.d : a.d;
     ms_chunk_sum_kernel<<<(unsigned)a.max_chunks, threads, sizeof(long long) * (size_t)std::max(1, threads / a.d) * a.d,
-                          st>>>(a.xa, a.d, a.perm, a.chunks, a.nchunks, a.dc, a.chunk_sums);
+                          st>>>(a.xa, a.d, a.perm, a.chunks, a.nchunks, a.dc, a.chunk_sums, stop);
   }
   return cudaGetLastError();
 }

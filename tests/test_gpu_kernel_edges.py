@@ -107,3 +107,23 @@ def test_generic_tile_edges(km, oracle, n, d, k, kw):
         mu = mu_ref
     assert g.stats()["path"] == 2
     g.close()
+
+
+# the sorted sums' small and large chunks (2^21 points), several steps past
+# the stop inside one graph, and a step after a converged run (its tables must
+# be the final centroids')
+@pytest.mark.parametrize("n,k,ops", [(5, 3, "bf16"), (20_001, 40, "f16"), (60_000, 300, "bf16"), (2_100_000, 16, "bf16")])
+def test_tensor_run_and_step_after_it(km, oracle, n, k, ops):
+    x, _, _ = synth.iso_mixture(n, 64, max(2, k // 2), sigma=1.0, box=6.0, seed=n)
+    mu0, _ = synth.init_distinct(x, k, seed=5)
+    steps = 30 if n < 1_000_000 else 3
+    ref = oracle.run(x, mu0, steps, 1e-6)
+    g = km.KMeans(n, 64, k, tc_operands=ops)
+    g.set_points(x)
+    g.set_init(mu0)
+    r = g.run(steps, 1e-6)
+    assert r["iters"] == ref["iters"] and np.array_equal(r["labels"], ref["labels"])
+    g.step()
+    z, _, cnt, _ = oracle.step(x, r["centroids"])
+    assert np.array_equal(g.labels(), z) and np.array_equal(g.counts(), cnt)
+    g.close()
