@@ -111,6 +111,16 @@ struct km_ctx {
   float A_max = 0.f;
   int tc_ex = 0;           // FP16 tensor-core operands: points scaled by 2^tc_ex
   int G0 = 0;
+  // whole-run kernel (fused path)
+  int run_state = 0;           // 0 not looked at yet, 1 in use, -1 not for this context (shape or memory)
+  int run_grid = 0, run_priv_sh = 0;
+  size_t run_smem = 0;
+  float* slack = nullptr;
+  uint8_t* zrun = nullptr;     // labels as bytes where the context keeps int32 labels
+  unsigned long long* run_delta = nullptr;
+  long long *run_tot = nullptr, *run_tot0 = nullptr;
+  float* run_cum0 = nullptr;
+  unsigned char* run_priv = nullptr;
   // loop
   cudaGraphExec_t graph = nullptr;
   int graph_unroll = 16;
@@ -149,7 +159,8 @@ void free_all(km_ctx* c) {
                   c->scan, c->scan_bad, c->xb, c->xa_pt, c->xaos, c->cbf, c->nprime, c->gc,
                   c->ms_counts, c->ms_offsets, c->ms_cfirst, c->ms_cursor, c->ms_chunks, c->ms_nchunks,
                   c->ms_chunk_sums, c->ms_perm, c->rescue_list, c->tie_list, c->rescue_count, c->ms_df2, c->bnorm,
-                  c->shard_out, c->shard_in};
+                  c->shard_out, c->shard_in, c->slack, c->zrun, c->run_delta, c->run_tot, c->run_tot0, c->run_cum0,
+                  c->run_priv};
   for (void* b : bufs)
     if (b) cudaFree(b);
   if (c->own_stream && c->st) cudaStreamDestroy(c->st);
@@ -255,6 +266,80 @@ cudaError_t launch_step(km_ctx* c) {
   cudaError_t e = launch_assign(c);
   if (e != cudaSuccess) return e;
   return launch_update_all(c);
+}
+
+// Shape and buffers of the whole-run kernel, at the context's first graph-
+// driven run.  Without the memory for them the step kernels' graph runs
+// instead, as it does for more points than a resident grid's int64 sums take.
+bool run_ready(km_ctx* c) {
+  if (c->run_state) return c->run_state > 0;
+  c->run_state = -1;
+  if (c->path != 1) return false;
+  const size_t base = fast_smem_bytes(c->d, c->kpad, c->k, c->nwin), priv = run_priv_bytes(c->d, c->k);
+  const int b0 = run_blocks_per_sm(c->d, c->kpad, base);
+  if (b0 < 1) return false;
+  // the block's own values in shared memory unless that costs a resident block
+  const bool sh = run_blocks_per_sm(c->d, c->kpad, base + priv) >= b0;
+  c->run_smem = sh ? base + priv : base;
+  c->run_priv_sh = sh ? (int)base : 0;
+  const int64_t ntiles = (c->n + kWarpTile - 1) / kWarpTile;
+  const int64_t g = std::min<int64_t>(ntiles, (int64_t)c->sms * b0);
+  const int64_t wtot = g * kWarps;
+  if ((ntiles + wtot - 1) / wtot * kWarps * kWarpTile > kMaxPointsPerBlock) return false;
+  c->run_grid = (int)g;
+  const size_t cols = (size_t)c->k * (c->d + 1);
+  if (dalloc(&c->slack, (size_t)c->n) != cudaSuccess ||
+      (!c->labels8 && dalloc(&c->zrun, (size_t)c->n) != cudaSuccess) ||
+      dalloc(&c->run_delta, run_delta_words(c->d, c->k)) != cudaSuccess ||
+      dalloc(&c->run_tot, (size_t)g * cols * 2) != cudaSuccess || dalloc(&c->run_tot0, cols * 2) != cudaSuccess ||
+      dalloc(&c->run_cum0, (size_t)c->k) != cudaSuccess ||
+      (!sh && dalloc(&c->run_priv, (size_t)g * priv) != cudaSuccess)) {
+    void* bufs[] = {c->slack, c->zrun, c->run_delta, c->run_tot, c->run_tot0, c->run_cum0, c->run_priv};
+    for (void* b : bufs)
+      if (b) cudaFree(b);
+    c->slack = nullptr; c->zrun = nullptr; c->run_delta = nullptr; c->run_tot = nullptr; c->run_tot0 = nullptr;
+    c->run_cum0 = nullptr; c->run_priv = nullptr;
+    cudaGetLastError();
+    return false;
+  }
+  c->run_state = 1;
+  return true;
+}
+
+// The steps of a run: launches of the whole-run kernel until the stop rule
+// has fired, each of at most 64 steps (so that the host keeps control of long
+// runs); then the labels.
+km_status read_state(km_ctx* c);
+km_status run_whole(km_ctx* c) {
+  RunArgs r{};
+  r.f.x = c->x; r.f.ld = c->ld; r.f.n = c->n; r.f.k = c->k; r.f.kpad = c->kpad;
+  r.f.dc = c->dc; r.f.ls = c->ls; r.f.ntiles = (c->n + kWarpTile - 1) / kWarpTile; r.f.nwin = c->nwin;
+  r.slack = c->slack;
+  r.z = c->labels8 ? c->labels8 : c->zrun;
+  r.mu = c->mu; r.counts = c->counts;
+  r.delta = c->run_delta;
+  r.bar = reinterpret_cast<unsigned int*>(c->run_delta + run_delta_words(c->d, c->k) - 1);
+  r.tot = c->run_tot; r.tot0 = c->run_tot0; r.cum0 = c->run_cum0;
+  r.priv = c->run_priv; r.priv_stride = run_priv_bytes(c->d, c->k); r.priv_sh = c->run_priv_sh;
+  r.ctil_out = c->ctil4; r.ic_out = c->ic; r.tab_out = c->tab2;
+  r.tie_rel = c->opt.tie_rel;
+  // FP64 distances are within 16 2^-53 relative of the exact ones; sqrt(D) <=
+  // 2 sqrt(A_max) + 2^20 ulps of slack for centroids outside the data's range
+  r.margin = (float)(1e-13 * (4.0 * std::sqrt((double)c->A_max) + 1e-20));
+  r.rep = run_rep(c->d, c->k);
+  r.steps = 64;
+  // one pass over the points takes far less: K N evaluations at 1e11 a second
+  r.wait_ns = 2000000000ull + (unsigned long long)((double)c->n * c->k * 0.01);
+  while (true) {
+    KM_CUDA(c, launch_run_fast(c->d, c->run_grid, c->run_smem, c->st, r));
+    r.resume = 1;
+    km_status s = read_state(c);
+    if (s != KM_OK) return s;
+    if (c->host_ls.done) break;
+  }
+  if (c->zrun && c->opt.label_policy == KM_LABELS_EVERY_STEP)
+    KM_CUDA(c, launch_widen_labels(c->zrun, c->labels, c->n, c->st));
+  return KM_OK;
 }
 
 km_status write_control(km_ctx* c, int done, int max_iter_abs, double tol) {
@@ -730,7 +815,10 @@ km_status km_run(km_ctx* c, int32_t max_iter, double tol, int32_t* labels_out,
   if (max_iter > 0) {
     s = write_control(c, 0, start + max_iter, tol);
     if (s != KM_OK) return s;
-    if (c->opt.use_graph) {
+    if (c->opt.use_graph && run_ready(c)) {
+      s = run_whole(c);
+      if (s != KM_OK) return s;
+    } else if (c->opt.use_graph) {
       if (!c->graph) {
         cudaGraph_t g = nullptr;
         KM_CUDA(c, cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal));

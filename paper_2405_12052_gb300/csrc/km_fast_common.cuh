@@ -81,10 +81,11 @@ __device__ __forceinline__ float direct_bound(float dv, float sqrtA, float sqrtB
 
 // Re-decide one flagged point: FP32 direct form with a rigorous bound, and
 // FP64 in the oracle's order when the bound (or the tie_rel rule) leaves it
-// open.  Returns the label; sets used64.
+// open.  Returns the label; sets used64, and *slack to a lower bound of
+// sqrt(D2) - sqrt(D1) (-1 when decided in FP64).
 template <int D>
 __device__ int recheck_fast(const float* xo, const float* s, const float4* ctil, const double* mu,
-                            int k, float B_max, float tau, bool& used64) {
+                            int k, float B_max, float tau, bool& used64, float* slack = nullptr) {
   float xt[D];
   float A = 0.f;
 #pragma unroll
@@ -108,12 +109,15 @@ __device__ int recheck_fast(const float* xo, const float* s, const float4* ctil,
     else if (dv < second) { second = dv; }
   }
   used64 = false;
+  if (slack) *slack = 3.0e38f;
   if (k > 1) {
     float sA = sqrtf(A), sB = sqrtf(B_max), AB = A + B_max;
     float e1 = direct_bound(best, sA, sB, AB, D);
     float e2 = direct_bound(second, sA, sB, AB, D);
     float lo2 = second - e2, hi1 = best + e1;
     bool clear = (lo2 > hi1) && (lo2 - hi1 > tau * (second + e2));
+    // lo2 <= D2 and hi1 >= D1; the factor covers the roundings here
+    if (slack) *slack = clear ? (lo2 - hi1) * 0.9999f / (__fsqrt_rn(lo2) + __fsqrt_rn(fmaxf(hi1, 0.f)) + 1e-37f) : -1.f;
     if (!clear) {
       used64 = true;
       double bd = d64_fixed<D>(xo, mu);
@@ -153,6 +157,7 @@ __device__ __forceinline__ unsigned long long fsub2(unsigned long long a, unsign
   return d;
 }
 __device__ __forceinline__ unsigned long long dup2(float v) { return pack2(v, v); }
+__device__ __forceinline__ float dup_lo(unsigned long long v) { return __uint_as_float((uint32_t)v); }
 
 // Flush the warp's windows (nwin of them) into the block's int64 totals.  acc
 // columns per centroid: 0..D-1 coordinate sums, D the count (the layout of
@@ -171,7 +176,7 @@ __device__ __forceinline__ void flush_windows(uint32_t* wwarp, long long* acc, i
       const uint32_t* w = wwarp + h * half + kk * WIN;
       const uint32_t c = w[0];
       if (j == D) {
-        v += (long long)c;
+        v += (long long)(int)c;  // the whole-run kernel takes points away too
       } else {
         const int hi = (int)(w[1 + j] - c * bias_hi);  // exact: |sum| < 2^30
         const int lo = (int)(w[1 + D + j] - c * bias_lo);

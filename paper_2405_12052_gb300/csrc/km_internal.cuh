@@ -120,6 +120,36 @@ struct FastArgs {
   int labels_unaligned;            // 1: labels + i may not be 16-byte aligned (store them one by one)
 };
 
+// A whole run in one cooperative kernel (km_run_fast.cu).
+struct RunArgs {
+  FastArgs f;                  // points, sizes, constants and loop state (labels and partials unused)
+  float* slack;                // [N]
+  uint8_t* z;                  // [N] labels
+  double* mu;                  // in/out
+  long long* counts;           // out
+  unsigned long long* delta;   // [3][rep][k (d + 1) + 2][2] changes of the column totals, flagged, FP64-decided; then
+  unsigned int* bar;           // the arrival counter (cleared together)
+  int rep;                     // copies of the table of changes
+  long long* tot;              // [grid][k (d + 1)][2] each block's running totals
+  long long* tot0;             // [k (d + 1)][2], [k]: totals and drift sums between launches
+  float* cum0;
+  unsigned char* priv;         // per-block values in global memory, priv_stride bytes each
+  size_t priv_stride;
+  int priv_sh;                 // their offset in shared memory (0: global)
+  float4* ctil_out; IterConst* ic_out; unsigned long long* tab_out;  // tables of the final centroids
+  double tie_rel;
+  float margin;                // least slack that FP64 rounding of the distances cannot turn around
+  int steps;                   // steps of this launch at most
+  int resume;                  // 1: continues the launch before (slack, labels, totals kept)
+  unsigned long long wait_ns;  // limit of one wait for the other blocks
+};
+// words of delta including the arrival counter
+int run_rep(int d, int k);
+inline size_t run_delta_words(int d, int k) { return (size_t)3 * run_rep(d, k) * ((size_t)k * (d + 1) + 2) * 2 + 1; }
+size_t run_priv_bytes(int d, int k);
+int run_blocks_per_sm(int d, int kpad, size_t smem);
+cudaError_t launch_run_fast(int d, int grid, size_t smem, cudaStream_t st, const RunArgs& a);
+
 struct GenericArgs {
   const float* x; int64_t ld; int64_t n; int d; int k;
   const float* ctil;               // [k][d] fp32 (mu - s)

@@ -9,44 +9,12 @@
 // mu_k = S_k / n_k (an empty cluster keeps mu_k), forms E^2 with a fixed-order
 // tree, tests the stop rule, and writes the next step's screen tables.
 #include "km_internal.cuh"
+#include "km_i128.cuh"
 #include "km_tables.cuh"
 
 namespace km {
 
 namespace {
-
-__device__ __forceinline__ double i128_to_double(long long lo_s, long long hi_s) {
-  // value = hi * 2^64 + (unsigned)lo, two's complement; correctly rounded.
-  unsigned long long lo = (unsigned long long)lo_s, hi = (unsigned long long)hi_s;
-  bool neg = (long long)hi < 0;
-  if (neg) {  // negate the 128-bit value
-    lo = ~lo + 1ull;
-    hi = ~hi + (lo == 0ull ? 1ull : 0ull);
-  }
-  double r;
-  if (hi == 0ull) {
-    r = __ull2double_rn(lo);
-  } else {
-    int sh = 64 - __clzll((long long)hi);  // bits used in hi
-    unsigned long long top = (hi << (64 - sh)) | (lo >> sh);
-    unsigned long long rest = lo << (64 - sh);
-    if (rest) top |= 1ull;  // sticky bit, 11 places below the rounding point
-    r = ldexp(__ull2double_rn(top), sh);
-  }
-  return neg ? -r : r;
-}
-
-__device__ __forceinline__ void add128(unsigned long long& lo, long long& hi, long long v) {
-  unsigned long long nl = lo + (unsigned long long)v;
-  hi += (v < 0 ? -1ll : 0ll) + (nl < lo ? 1ll : 0ll);
-  lo = nl;
-}
-__device__ __forceinline__ void add128p(unsigned long long& lo, long long& hi, unsigned long long vl,
-                                        long long vh) {
-  unsigned long long nl = lo + vl;
-  hi += vh + (nl < lo ? 1ll : 0ll);
-  lo = nl;
-}
 
 __device__ __forceinline__ uint32_t ordered(float f) {
   uint32_t b = __float_as_uint(f);

@@ -80,6 +80,61 @@ def test_objective_edges(km, n, d, k, label_bytes):
     g.close()
 
 
+def _run_pair(km, x, mu0, max_iter, tol, **kw):
+    """The same run by the whole-run kernel and by one host round trip per
+    step (which compares every point with every centroid in every step)."""
+    d, n = x.shape
+    out = []
+    for graph in (True, False):
+        g = km.KMeans(n, d, mu0.shape[0], use_graph=graph, **kw)
+        g.set_points(x)
+        g.set_init(mu0)
+        r = g.run(max_iter, tol)
+        r2 = g.run(3, 0.0)  # continues from the first run's state
+        out.append((r, g.stats()["empty_clusters"], r2, g.counts(), g.step(), g.labels()))
+        g.close()
+    return out
+
+
+# every d, group counts with their own instance (kpad 32 and 256 in 3-D) and
+# without, tiles at and around 256 points, fewer tiles than blocks and many per
+# warp; data in clusters (few open points), spread evenly (many, and more steps
+# than one launch takes), around an offset, on a grid (exact ties, duplicated
+# and empty centroids), and near the ends of the float range
+@pytest.mark.parametrize("kind,n,d,k,steps,kw", [
+    ("mix", 1, 1, 1, 5, {}), ("mix", 255, 2, 3, 20, {}), ("mix", 257, 3, 8, 20, {}),
+    ("even", 20_011, 1, 5, 150, {}), ("even", 30_000, 2, 11, 150, {}), ("even", 100_003, 3, 32, 100, {}),
+    ("even", 50_000, 3, 100, 40, {"label_bytes": 1}), ("mix", 60_001, 3, 256, 30, {}), ("even", 40_000, 4, 7, 80, {}),
+    ("mix", 30_000, 4, 256, 20, {"e_mode": "squared"}), ("mix", 1_300_007, 3, 17, 70, {"label_bytes": 1}),
+    ("offset", 200_000, 3, 64, 40, {}), ("grid", 6_760, 2, 6, 30, {}), ("grid", 6_760, 2, 40, 30, {"label_policy": "final"}),
+    ("tiny", 9_000, 3, 9, 40, {}), ("huge", 5_000, 3, 8, 15, {}), ("far", 30_000, 2, 9, 60, {}),
+])
+def test_whole_run_equals_step_by_step(km, oracle, kind, n, d, k, steps, kw):
+    rng = np.random.default_rng(n + k)
+    if kind == "even":
+        x = rng.random((d, n), dtype=np.float32)
+    elif kind == "grid":
+        g1 = np.arange(-6, 7, dtype=np.float32)
+        x = np.ascontiguousarray(np.tile(np.stack([m.ravel() for m in np.meshgrid(g1, g1)]), (1, 40))[:, :n])
+    else:
+        x, _, _ = synth.iso_mixture(n, d, max(2, k // 2), sigma=1.0, box=8.0, seed=n + d,
+                                    offset=1e4 if kind == "offset" else 0.0)
+        x = (x.astype(np.float64) * {"tiny": 1e-30, "huge": 1e18}.get(kind, 1.0)).astype(np.float32)
+    mu0, _ = synth.init_distinct(x, k, seed=3)
+    if kind == "grid":
+        mu0[1] = mu0[0]          # a duplicated centroid (its twin takes no point)
+    if kind == "far":
+        mu0[:4] += 1e6           # centroids far outside the data, empty at first
+    (a, ea, a2, ca, sa, za), (b, eb, b2, cb, sb, zb) = _run_pair(km, x, mu0, steps, 1e-7, **kw)
+    for p, q in ((a, b), (a2, b2)):
+        assert p["iters"] == q["iters"] and p["E"] == q["E"] and p["converged"] == q["converged"]
+        assert np.array_equal(p["labels"], q["labels"]) and np.array_equal(p["centroids"], q["centroids"])
+    assert ea == eb and np.array_equal(ca, cb) and sa == sb and np.array_equal(za, zb)
+    if n <= 60_001 and not kw.get("label_policy"):
+        ref = oracle.run(x, mu0, steps, 1e-7, e_mode=1 if kw.get("e_mode") else 0)
+        assert a["iters"] == ref["iters"] and np.array_equal(a["labels"], ref["labels"])
+
+
 # tiles of 128 points x 64 centroids x 32 coordinates and their edges; sums in
 # shared windows with totals beside them, in the block's row, and (K d large)
 # by global atomics; more points per block than one window flush
