@@ -1,43 +1,44 @@
 // Reassignment and per-block sums for any d and K (paper, section "The
-// Lloyd's algorithm", steps 2 and 3): FP32 direct form with its rigorous
-// bound, FP64 in the oracle's order where that leaves a point open, exact
-// fixed-point sums.
+// Lloyd's algorithm", steps 2 and 3): an FP32 screen ||c~||^2 - 2 x~.c~ with a
+// rigorous bound, the direct form and then FP64 in the oracle's order for the
+// points it leaves open, exact fixed-point sums.
 //
-// Bound by the FP32 operations of the direct form, a subtraction and a
-// multiply-add per point, centroid and coordinate (2.05e9 for N = 1e6, d = 16,
-// K = 64: 55 us at one per lane and cycle).  A block takes 128 points against
-// 64 centroids at a time, 32 coordinates of both in shared memory, 8 points x
-// 4 centroids per thread: three 16-byte shared reads per 64 operations, where
-// one point per thread reads its coordinate again for every centroid.  The
-// two smallest distances of a point are kept per thread over the centroid
-// tiles and merged over its 16 threads at the end.  Open points are decided in
-// FP64 by one warp each (lanes over centroids), not by one thread while 31
-// wait.  The sums go to 32-bit windows in shared memory (one per block,
-// flushed every 512 points) while those fit; one 64-bit global atomic per
-// coordinate and point before.  N = 1e6, d = 16, K = 64: 572 -> 214 us.
+// Bound by FP32 multiply-adds, one per point, centroid and coordinate (1.02e9
+// for N = 1e6, d = 16, K = 64: 27 us at one per lane and cycle; the direct
+// form takes two operations), and by what a point costs beside them: its two
+// smallest values over K and 2 d + 1 additions to the sums.  A block takes 256
+// points against 64 centroids at a time, 32 coordinates of both in shared
+// memory, 8 points x 8 centroids per thread: four 16-byte shared reads per 64
+// multiply-adds.  The two smallest values of a point are kept per thread over
+// the centroid tiles and merged over its 8 threads at the end, each exchange
+// halving the points a thread keeps.  Open points are decided by one warp each
+// (lanes over centroids).  The sums go to 32-bit windows in shared memory (one
+// per block, flushed every 512 points) while those fit, else to the block's
+// row by 64-bit global atomics.  N = 1e6, d = 16, K = 64: one point per
+// thread and 64-bit atomics 572 us, direct form in tiles of 128 points 214
+// us, this 170 us (ten steps of a run: 6.09, 2.36, 1.79 ms).
+#include <type_traits>
+
 #include "km_fast_common.cuh"
 
 namespace km {
 
 namespace {
 
-constexpr int kGP = 128;              // points per tile
+constexpr int kGP = 256;              // points per tile
 constexpr int kGC = 64;               // centroids per tile
 constexpr int kGD = 32;               // coordinates staged at a time
 constexpr int kGXS = kGP + 4;         // row strides of the staged tiles
 constexpr int kGCS = kGC + 4;
-constexpr int kGFlush = 4;            // point tiles between window flushes (512 additions per bin)
+constexpr int kGFlush = 2;            // point tiles between window flushes (512 additions per bin)
 constexpr size_t kGWinMax = 96 * 1024;   // windows above this: 64-bit global atomics instead
 constexpr size_t kGTotMax = 48 * 1024;   // int64 totals above this: in the block's partial row
 
 __device__ __forceinline__ void top2_merge(float& best, float& second, int& kb, float ob, float os, int ok) {
-  if (ob < best || (ob == best && ok < kb)) {
-    second = fminf(best, os);
-    best = ob;
-    kb = ok;
-  } else {
-    second = fminf(second, ob);
-  }
+  const bool take = ob < best || (ob == best && ok < kb);
+  second = fminf(fminf(second, os), fmaxf(best, ob));
+  best = fminf(best, ob);
+  kb = take ? ok : kb;
 }
 
 __global__ void __launch_bounds__(kThreads, 2) assign_generic_kernel(GenericArgs a, int use_win, int tot_sh) {
@@ -49,19 +50,24 @@ __global__ void __launch_bounds__(kThreads, 2) assign_generic_kernel(GenericArgs
   uint32_t* s_win = reinterpret_cast<uint32_t*>(s_tot + (tot_sh ? (size_t)k * dp : 0));  // [k][2 d + 1] when use_win
   __shared__ float s_A[kGP];
   __shared__ int s_lab[kGP], s_q[kGP];
-  __shared__ int s_qn, s_n64;
+  __shared__ int s_qn, s_nflag, s_n64;
   if (a.ls->done && !a.ignore_done) return;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3, lane = tid & 31, warp = tid >> 5;
   long long* row = a.partials + (size_t)blockIdx.x * k * dp;
   long long* tot = tot_sh ? s_tot : row;
   for (int q = tid; q < k * dp; q += kThreads) tot[q] = 0;
   if (use_win)
     for (int q = tid; q < k * wn; q += kThreads) s_win[q] = 0u;
-  if (tid == 0) { s_qn = 0; s_n64 = 0; }
+  if (tid == 0) { s_qn = 0; s_nflag = 0; s_n64 = 0; }
   const DataConst dc = *a.dc;
   const float B_max = *a.B_max_ptr, sB = sqrtf(B_max);
   const int ktiles = (k + kGC - 1) / kGC, chunks = (d + kGD - 1) / kGD;
   const int64_t ntiles = (a.n + kGP - 1) / kGP;
+  // Bound of the difference of two screen values against that of the exact
+  // distances, per unit of A + B_max.  One value: the roundings of x~ and c~
+  // (4.04 u), the d products and their sum (1.01 d u), ||c~||^2 (2.01 u), the
+  // last multiply-add (2.02 u), and the oracle's FP64 rounding.
+  const float evc = 2.04f * kU * ((float)d + 8.5f) + 2.f * kU64x * (float)(d + 1);
   __syncthreads();
 
   // the windows' sums of bin q = (cluster, column) into the block's totals
@@ -88,132 +94,169 @@ __global__ void __launch_bounds__(kThreads, 2) assign_generic_kernel(GenericArgs
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int64_t base = tile * kGP;
     const int np = (int)min((int64_t)kGP, a.n - base);
-    float best[8], second[8], A = 0.f;  // A: of point tid (threads below kGP)
+    float best[8], second[8], A = 0.f;  // A: of point tid
     int kb[8];
 #pragma unroll
     for (int r = 0; r < 8; ++r) { best[r] = 3.0e38f; second[r] = 3.0e38f; kb[r] = 0; }
     for (int kt = 0; kt < ktiles; ++kt) {
-      float acc[8][4];
+      float acc[8][8];  // points 8 ty + r, centroids 4 tx + (c & 3) + 32 (c >> 2)
 #pragma unroll
       for (int r = 0; r < 8; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
+        for (int c = 0; c < 8; ++c) acc[r][c] = 0.f;
       for (int ch = 0; ch < chunks; ++ch) {
         const int j0 = ch * kGD, nj = min(kGD, d - j0);
         __syncthreads();  // the tiles before are read no more
-        if (kt == 0 || chunks > 1)
-          for (int q = tid; q < nj * kGP; q += kThreads) {
-            const int j = q >> 7, p = q & (kGP - 1);
-            s_x[j * kGXS + p] = p < np ? __fsub_rn(a.x[(int64_t)(j0 + j) * a.ld + base + p], a.shift[j0 + j]) : 0.f;
-          }
+        if (kt == 0 || chunks > 1) {
+#pragma unroll 4
+          for (int j = 0; j < nj; ++j)
+            s_x[j * kGXS + tid] =
+                tid < np ? __fsub_rn(a.x[(int64_t)(j0 + j) * a.ld + base + tid], a.shift[j0 + j]) : 0.f;
+        }
         if (ktiles > 1 || chunks > 1 || tile == blockIdx.x)
           for (int q = tid; q < nj * kGC; q += kThreads) {
             const int c = q / nj, j = q - c * nj, cc = kt * kGC + c;
             s_c[j * kGCS + c] = cc < k ? a.ctil[(size_t)cc * d + j0 + j] : 0.f;
           }
         __syncthreads();
-        if (kt == 0 && tid < kGP)
+        if (kt == 0)
           for (int j = 0; j < nj; ++j) A = __fmaf_rn(s_x[j * kGXS + tid], s_x[j * kGXS + tid], A);
 #pragma unroll 4
         for (int j = 0; j < nj; ++j) {
           const float4 x0 = *reinterpret_cast<const float4*>(s_x + j * kGXS + 8 * ty);
           const float4 x1 = *reinterpret_cast<const float4*>(s_x + j * kGXS + 8 * ty + 4);
-          const float4 cv = *reinterpret_cast<const float4*>(s_c + j * kGCS + 4 * tx);
+          const float4 c0 = *reinterpret_cast<const float4*>(s_c + j * kGCS + 4 * tx);
+          const float4 c1 = *reinterpret_cast<const float4*>(s_c + j * kGCS + 32 + 4 * tx);
           const float xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-          const float cw[4] = {cv.x, cv.y, cv.z, cv.w};
+          const float cw[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
 #pragma unroll
           for (int r = 0; r < 8; ++r)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              const float t = __fsub_rn(xv[r], cw[c]);
-              acc[r][c] = __fmaf_rn(t, t, acc[r][c]);
-            }
+            for (int c = 0; c < 8; ++c) acc[r][c] = __fmaf_rn(xv[r], cw[c], acc[r][c]);
         }
       }
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int cc = kt * kGC + 4 * tx + c;
-        if (cc >= k) break;
+      for (int c = 0; c < 8; ++c) {
+        const int cc = kt * kGC + 4 * tx + (c & 3) + 32 * (c >> 2);
+        if (cc >= k) continue;
+        const float nc = __ldg(a.cnorm + cc);
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
-          const float dv = acc[r][c];
-          if (dv < best[r]) { second[r] = best[r]; best[r] = dv; kb[r] = cc; }
-          else if (dv < second[r]) second[r] = dv;
+          const float v = __fmaf_rn(-2.f, acc[r][c], nc);
+          const bool less = v < best[r];
+          second[r] = fminf(second[r], fmaxf(best[r], v));
+          best[r] = fminf(best[r], v);
+          kb[r] = less ? cc : kb[r];
         }
       }
     }
-    if (tid < kGP) s_A[tid] = A * 1.0001f;
+    s_A[tid] = A * 1.0001f;
+    // merge over the 8 threads of a point group: each exchange halves the
+    // points a thread keeps, so it ends with one
+    auto merge_half = [&](auto half, int bit) {
+      constexpr int H = decltype(half)::value;
+      const bool up = tx & bit;
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
-#pragma unroll
-      for (int o = 1; o < 16; o <<= 1) {
-        const float ob = __shfl_xor_sync(0xffffffffu, best[r], o), os = __shfl_xor_sync(0xffffffffu, second[r], o);
-        const int ok = __shfl_xor_sync(0xffffffffu, kb[r], o);
+      for (int r = 0; r < H; ++r) {
+        const float sb = up ? best[r] : best[r + H], ss = up ? second[r] : second[r + H];
+        const int sk = up ? kb[r] : kb[r + H];
+        const float ob = __shfl_xor_sync(0xffffffffu, sb, bit), os = __shfl_xor_sync(0xffffffffu, ss, bit);
+        const int ok = __shfl_xor_sync(0xffffffffu, sk, bit);
+        if (up) { best[r] = best[r + H]; second[r] = second[r + H]; kb[r] = kb[r + H]; }
         top2_merge(best[r], second[r], kb[r], ob, os, ok);
       }
+    };
+    merge_half(std::integral_constant<int, 4>{}, 4);
+    merge_half(std::integral_constant<int, 2>{}, 2);
+    merge_half(std::integral_constant<int, 1>{}, 1);
     __syncthreads();  // s_A
     {
-      // thread tx < 8 of the group takes point 8 ty + tx
-      float b = 0.f, s2 = 0.f;
-      int kk = 0;
-#pragma unroll
-      for (int r = 0; r < 8; ++r)
-        if (tx == r) { b = best[r]; s2 = second[r]; kk = kb[r]; }
-      const int p = 8 * ty + tx;
-      if (tx < 8 && p < np) {
+      const int p = 8 * ty + tx;  // bits 4, 2, 1 of tx chose the point's half each time
+      if (p < np) {
         bool clear = true;
         if (k > 1) {
-          const float Ap = s_A[p], sA = sqrtf(Ap), AB = Ap + B_max;
-          const float e1 = direct_bound(b, sA, sB, AB, d), e2 = direct_bound(s2, sA, sB, AB, d);
-          const float lo2 = s2 - e2, hi1 = b + e1;
-          clear = (lo2 > hi1) && (lo2 - hi1 > a.tau * (s2 + e2));
+          const float AB = s_A[p] + B_max, T0 = evc * AB + 1e-30f;  // 1e-30: underflowed products
+          clear = second[0] - best[0] > T0 + a.tau * fmaxf(s_A[p] + second[0] + T0, 0.f);
         }
-        s_lab[p] = kk;
+        s_lab[p] = kb[0];
         if (!clear) s_q[atomicAdd(&s_qn, 1)] = p;
       }
     }
     __syncthreads();
     const int qn = s_qn;
     for (int e = warp; e < qn; e += kWarps) {
+      // direct form first, then FP64 where its bound leaves the point open
       const int p = s_q[e];
-      double bd = 0.0;
-      int k64 = -1;
+      const float* xp = a.x + base + p;
+      float b1 = 3.0e38f, b2 = 3.0e38f;
+      int k1 = 0;
       for (int c = lane; c < k; c += 32) {
-        const double dd = d64_dyn(a.x, a.ld, base + p, d, a.mu + (size_t)c * d);
-        if (k64 < 0 || dd < bd) { bd = dd; k64 = c; }
+        float dv = 0.f;
+        for (int j = 0; j < d; ++j) {
+          const float t = __fsub_rn(__fsub_rn(xp[(int64_t)j * a.ld], a.shift[j]), a.ctil[(size_t)c * d + j]);
+          dv = __fmaf_rn(t, t, dv);
+        }
+        if (dv < b1) { b2 = b1; b1 = dv; k1 = c; }
+        else if (dv < b2) b2 = dv;
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
-        const double ob = __shfl_xor_sync(0xffffffffu, bd, o);
-        const int ok = __shfl_xor_sync(0xffffffffu, k64, o);
-        if (ok >= 0 && (k64 < 0 || ob < bd || (ob == bd && ok < k64))) { bd = ob; k64 = ok; }
+        const float ob = __shfl_xor_sync(0xffffffffu, b1, o), os = __shfl_xor_sync(0xffffffffu, b2, o);
+        const int ok = __shfl_xor_sync(0xffffffffu, k1, o);
+        top2_merge(b1, b2, k1, ob, os, ok);
       }
-      if (lane == 0) s_lab[p] = k64;
+      const float Ap = s_A[p], sA = sqrtf(Ap), AB = Ap + B_max;
+      const float e1 = direct_bound(b1, sA, sB, AB, d), e2 = direct_bound(b2, sA, sB, AB, d);
+      const float lo2 = b2 - e2, hi1 = b1 + e1;
+      int lab = k1;
+      if (!((lo2 > hi1) && (lo2 - hi1 > a.tau * (b2 + e2)))) {  // the same in every lane
+        double bd = 0.0;
+        int k64 = -1;
+        for (int c = lane; c < k; c += 32) {
+          const double dd = d64_dyn(a.x, a.ld, base + p, d, a.mu + (size_t)c * d);
+          if (k64 < 0 || dd < bd) { bd = dd; k64 = c; }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const double ob = __shfl_xor_sync(0xffffffffu, bd, o);
+          const int ok = __shfl_xor_sync(0xffffffffu, k64, o);
+          if (ok >= 0 && (k64 < 0 || ob < bd || (ob == bd && ok < k64))) { bd = ob; k64 = ok; }
+        }
+        lab = k64;
+        if (lane == 0) atomicAdd(&s_n64, 1);
+      }
+      if (lane == 0) s_lab[p] = lab;
     }
     __syncthreads();
-    if (tid == 0) { s_n64 += qn; s_qn = 0; }
+    if (tid == 0) { s_nflag += qn; s_qn = 0; }
     if (a.store_labels && tid < np) {
       if (a.labels8) a.labels8[base + tid] = (uint8_t)s_lab[tid];
       else a.labels[base + tid] = s_lab[tid];
     }
-    // sums: threads over (point, coordinate), coalesced along the points
-    for (int q = tid; q < dp * kGP; q += kThreads) {
-      const int j = q >> 7, p = q & (kGP - 1);
-      if (p >= np) continue;
-      const int c = s_lab[p];
-      if (j == d) {
-        if (use_win) atomicAdd(s_win + (size_t)c * wn, 1u);
-        else atomicAdd(reinterpret_cast<unsigned long long*>(row) + (size_t)c * dp + d, 1ull);
-        continue;
-      }
-      uint32_t bh, bl;
-      split_limbs(a.x[(int64_t)j * a.ld + base + p], dc.C_hi, dc.C_lo, bh, bl);
+    // sums: a thread per point, coordinate after coordinate (coalesced)
+    if (tid < np) {
+      const int c = s_lab[tid];
+      const float* xp = a.x + base + tid;
       if (use_win) {
-        atomicAdd(s_win + (size_t)c * wn + 1 + j, bh);
-        atomicAdd(s_win + (size_t)c * wn + 1 + d + j, bl);
+        uint32_t* w = s_win + (size_t)c * wn;
+        atomicAdd(w, 1u);
+#pragma unroll 4
+        for (int j = 0; j < d; ++j) {
+          uint32_t bh, bl;
+          split_limbs(xp[(int64_t)j * a.ld], dc.C_hi, dc.C_lo, bh, bl);
+          atomicAdd(w + 1 + j, bh);
+          atomicAdd(w + 1 + d + j, bl);
+        }
       } else {
-        const long long hi = (long long)(int)(bh - dc.bits_C_hi), lo = (long long)(int)(bl - dc.bits_C_lo);
-        atomicAdd(reinterpret_cast<unsigned long long*>(row) + (size_t)c * dp + j, (unsigned long long)((hi << 22) + lo));
+        unsigned long long* r = reinterpret_cast<unsigned long long*>(row) + (size_t)c * dp;
+        atomicAdd(r + d, 1ull);
+#pragma unroll 4
+        for (int j = 0; j < d; ++j) {
+          uint32_t bh, bl;
+          split_limbs(xp[(int64_t)j * a.ld], dc.C_hi, dc.C_lo, bh, bl);
+          const long long hi = (long long)(int)(bh - dc.bits_C_hi), lo = (long long)(int)(bl - dc.bits_C_lo);
+          atomicAdd(r + j, (unsigned long long)((hi << 22) + lo));
+        }
       }
     }
     if (use_win && ++since == kGFlush) {
@@ -225,9 +268,9 @@ __global__ void __launch_bounds__(kThreads, 2) assign_generic_kernel(GenericArgs
   __syncthreads();
   if (tot_sh)
     for (int q = tid; q < k * dp; q += kThreads) row[q] = s_tot[q];
-  if (tid == 0 && s_n64) {
-    atomicAdd(&a.ls->flagged, (unsigned long long)s_n64);
-    atomicAdd(&a.ls->fp64_decided, (unsigned long long)s_n64);
+  if (tid == 0) {
+    if (s_nflag) atomicAdd(&a.ls->flagged, (unsigned long long)s_nflag);
+    if (s_n64) atomicAdd(&a.ls->fp64_decided, (unsigned long long)s_n64);
   }
 }
 

@@ -102,18 +102,19 @@ __device__ void finish_update(const UpdateArgs& a, const long long* s128, int RB
   __syncthreads();
   if (tid == 0) {
     LoopState* ls = a.ls;
+    const LoopState l = *ls;  // read at once, not one field after another between the stores
     const double E2 = s_red[0];
     const double E = sqrt(E2);
     ls->E2 = E2;
     ls->E = E;
-    ls->iter += 1;
+    ls->iter = l.iter + 1;
     ls->empty = s_empty;
-    const double esel = ls->e_mode == 1 ? E2 : E;
-    if (esel < ls->tol) { ls->converged = 1; ls->done = 1; }
-    if (ls->iter >= ls->max_iter) ls->done = 1;
-    ls->last_flagged = ls->flagged;
-    ls->last_fp64 = ls->fp64_decided;
-    ls->last_overflowed = ls->overflowed;
+    const double esel = l.e_mode == 1 ? E2 : E;
+    if (esel < l.tol) { ls->converged = 1; ls->done = 1; }
+    if (l.iter + 1 >= l.max_iter) ls->done = 1;
+    ls->last_flagged = l.flagged;
+    ls->last_fp64 = l.fp64_decided;
+    ls->last_overflowed = l.overflowed;
     ls->flagged = 0ull;
     ls->fp64_decided = 0ull;
     ls->overflowed = 0ull;

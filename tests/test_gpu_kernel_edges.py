@@ -135,11 +135,11 @@ def test_whole_run_equals_step_by_step(km, oracle, kind, n, d, k, steps, kw):
         assert a["iters"] == ref["iters"] and np.array_equal(a["labels"], ref["labels"])
 
 
-# tiles of 128 points x 64 centroids x 32 coordinates and their edges; sums in
+# tiles of 256 points x 64 centroids x 32 coordinates and their edges; sums in
 # shared windows with totals beside them, in the block's row, and (K d large)
 # by global atomics; more points per block than one window flush
 @pytest.mark.parametrize("n,d,k,kw", [
-    (1, 5, 1, {}), (127, 31, 3, {}), (129, 32, 64, {}), (3000, 33, 65, {}), (200_003, 5, 7, {}), (100_001, 16, 64, {}),
+    (1, 5, 1, {}), (255, 31, 3, {}), (257, 32, 64, {}), (3000, 33, 65, {}), (200_003, 5, 7, {}), (100_001, 16, 64, {}),
     (20_000, 40, 130, {}), (5000, 70, 200, {}), (3000, 130, 257, {"label_policy": "final"}), (2000, 2, 1000, {}),
     (50_001, 7, 256, {"label_bytes": 1}), (20_003, 64, 100, {"dist_path": "simt"})])
 def test_generic_tile_edges(km, oracle, n, d, k, kw):
