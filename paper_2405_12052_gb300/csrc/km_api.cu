@@ -95,7 +95,7 @@ struct km_ctx {
   GemmConst* gc = nullptr;
   int32_t* rescue_list = nullptr;
   int4* tie_list = nullptr;
-  unsigned* rescue_count = nullptr;  // [2]: rescue and near-tie list lengths
+  unsigned* rescue_count = nullptr;  // [3]: rescue, near-tie and second rescue list lengths
   // sorted mean calculation
   unsigned long long* ms_counts = nullptr;
   int64_t* ms_offsets = nullptr;
@@ -215,7 +215,8 @@ cudaError_t launch_assign(km_ctx* c, bool labels_pass = false) {
     g.xb = c->xb; g.xa = c->xa_pt; g.xaos = c->xaos; g.cb = c->cbf; g.nprime = c->nprime; g.ctil = c->ctil;
     g.mu = c->mu; g.shift = c->shift; g.gc = c->gc; g.ls = c->ls; g.labels = c->labels;
     g.rescue_list = c->rescue_list; g.tie_list = c->tie_list;
-    g.rescue_count = c->rescue_count; g.tie_count = c->rescue_count + 1;
+    g.rescue_list2 = reinterpret_cast<int32_t*>(c->tie_list);
+    g.rescue_count = c->rescue_count; g.tie_count = c->rescue_count + 1; g.rescue_count2 = c->rescue_count + 2;
     g.n = c->n; g.k = c->k; g.kpad = c->kpad; g.ntiles = (int)((c->n + 127) / 128);
     g.f16 = c->opt.tc_operands == KM_TC_F16 ? 1 : 0;
     return launch_gemm_assign(c->G, c->st, g);
@@ -534,7 +535,7 @@ km_status km_create(km_ctx** out, int64_t n, int32_t d, int32_t k, const km_opti
     KM_CUDA(c, dalloc(&c->gc, 1));
     KM_CUDA(c, dalloc(&c->rescue_list, (size_t)n));
     KM_CUDA(c, dalloc(&c->tie_list, (size_t)gemm_tie_entries(n, c->G) * 3));
-    KM_CUDA(c, dalloc(&c->rescue_count, 2));
+    KM_CUDA(c, dalloc(&c->rescue_count, 3));
     c->ms_max_chunks = (int)msort_max_chunks(n, k);
     KM_CUDA(c, dalloc(&c->ms_counts, (size_t)k));
     KM_CUDA(c, dalloc(&c->ms_offsets, (size_t)k));

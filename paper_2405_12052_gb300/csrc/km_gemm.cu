@@ -53,6 +53,7 @@ constexpr int kHalf = 16;         // values per stored half
 constexpr int kPtStride = kSlots * kHalf * 2 + 16;  // bytes per point (padding spreads banks)
 constexpr int kTileBytes = kGM * kGemmD * 2;   // 16 KB of 16-bit operands per point tile
 constexpr int kTieMax = 20;       // candidates per near-tie list entry (48 bytes)
+constexpr int64_t kRescueTileMin = int64_t(1) << 20;  // points from which the rescue list is taken in tiles
 constexpr int kTieChunk = 64;     // near-tie entries an epilogue warp reserves at a time
 // shared-memory layout (bytes from the 1024-aligned base)
 constexpr int kOffStore = 0;                                  // [128][kPtStride] bytes
@@ -575,9 +576,22 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_assign_kernel(GemmArgs a) {
 // stride; the next entry is copied into shared memory (cp.async) while the
 // current one is ranked, so the point's row and the first candidates' rows
 // are requested as soon as an entry starts.
+// FP64 decisions: an FP64 instruction takes the pipe 17 cycles however few
+// lanes of the warp need it, so the candidates of such a point are listed and
+// taken by the block's threads side by side at the end (2000 such points
+// among 2e5: the kernel 66 -> 33 us).
+constexpr int kTieItems = 512;
 __global__ void __launch_bounds__(256, 4) gemm_tie_kernel(GemmArgs a) {
   __shared__ __align__(16) int4 s_ent[2][64][3];  // [stage][group] 48-byte entries
+  // FP64 decisions put off to the end of the block: (point, candidate) items
+  // and, per point, its first item and their number
+  __shared__ int2 s_item[kTieItems];
+  __shared__ double s_dd[kTieItems];
+  __shared__ int3 s_pt[kTieItems / 2];
+  __shared__ int s_ni, s_np;
   if (a.ls->done) return;
+  if (threadIdx.x == 0) { s_ni = 0; s_np = 0; }
+  __syncthreads();
   const unsigned cnt = *a.tie_count;
   const GemmConst gc = *a.gc;
   const int lane = threadIdx.x & 31, sub = lane & 3, grp = threadIdx.x >> 2;
@@ -656,50 +670,182 @@ __global__ void __launch_bounds__(256, 4) gemm_tie_kernel(GemmArgs a) {
       const float e1 = bound64(best, sA, sB, AB), e2 = bound64(second, sA, sB, AB);
       const float lo2 = second - e2, hi1 = best + e1;
       const bool need64 = !((lo2 > hi1) && (lo2 - hi1 > gc.tau * (second + e2)));
+      bool later = false;
       if (need64) {  // the same on the 4 threads
-        // the candidates read again from the staged entry, dealt over the 4
-        // threads (one thread took them one after another, 64 dependent FP64
-        // additions each: the tail of a small step's kernel)
         const unsigned short* cl = reinterpret_cast<const unsigned short*>(&s_ent[st][grp][0]) + 4;
-        const float* xr = a.xaos + (size_t)ii * kGemmD;
-        double bd = 0.0;
-        int k64 = -1;
-        for (int q = sub; q < nc; q += 4) {
-          const int c = cl[q];
-          if (c >= a.k) continue;
-          const double dd = d64row(xr, a.mu + (size_t)c * kGemmD);
-          if (k64 < 0 || dd < bd || (dd == bd && c < k64)) { bd = dd; k64 = c; }
+        int pos = 0, slot = kTieItems;
+        if (sub == 0) {
+          pos = atomicAdd(&s_ni, nc);
+          if (pos + nc <= kTieItems) slot = atomicAdd(&s_np, 1);
+          ++n64;
         }
+        pos = __shfl_sync(gmask, pos, lane & ~3);
+        later = __shfl_sync(gmask, slot, lane & ~3) < kTieItems;
+        if (later) {  // at most kTieItems / 2 points (two candidates or more each)
+          for (int q = sub; q < nc; q += 4) s_item[pos + q] = make_int2((int)ii, cl[q]);
+          if (sub == 0) s_pt[slot] = make_int3((int)ii, pos, nc);
+        } else {  // the list is full: here, the candidates dealt over the 4 threads
+          for (int q = pos + sub; q < min(pos + nc, kTieItems); q += 4) s_item[q] = make_int2(0, a.k);
+          const float* xr = a.xaos + (size_t)ii * kGemmD;
+          double bd = 0.0;
+          int k64 = -1;
+          for (int q = sub; q < nc; q += 4) {
+            const int c = cl[q];
+            if (c >= a.k) continue;
+            const double dd = d64row(xr, a.mu + (size_t)c * kGemmD);
+            if (k64 < 0 || dd < bd || (dd == bd && c < k64)) { bd = dd; k64 = c; }
+          }
 #pragma unroll
-        for (int o = 1; o < 4; o <<= 1) {
-          const double ob = __shfl_xor_sync(gmask, bd, o);
-          const int ok = __shfl_xor_sync(gmask, k64, o);
-          if (ok >= 0 && (k64 < 0 || ob < bd || (ob == bd && ok < k64))) { bd = ob; k64 = ok; }
+          for (int o = 1; o < 4; o <<= 1) {
+            const double ob = __shfl_xor_sync(gmask, bd, o);
+            const int ok = __shfl_xor_sync(gmask, k64, o);
+            if (ok >= 0 && (k64 < 0 || ob < bd || (ob == bd && ok < k64))) { bd = ob; k64 = ok; }
+          }
+          lab = k64;
         }
-        lab = k64;
-        n64 += sub == 0 ? 1 : 0;
       }
-      if (sub == 0) a.labels[ii] = lab;
+      if (sub == 0 && !later) a.labels[ii] = lab;
     }
     __syncwarp(gmask);  // stage st is refilled by the next iteration's copy
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  const int ni = min(s_ni, kTieItems), np = min(s_np, kTieItems / 2);
+  for (int q = threadIdx.x; q < ni; q += blockDim.x) {
+    const int2 it = s_item[q];
+    if (it.y < a.k) s_dd[q] = d64row(a.xaos + (size_t)it.x * kGemmD, a.mu + (size_t)it.y * kGemmD);
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < np; q += blockDim.x) {
+    const int3 pt = s_pt[q];
+    double bd = 0.0;
+    int k64 = -1;
+    for (int r = pt.y; r < pt.y + pt.z; ++r) {
+      const int c = s_item[r].y;
+      if (c < a.k && (k64 < 0 || s_dd[r] < bd || (s_dd[r] == bd && c < k64))) { bd = s_dd[r]; k64 = c; }
+    }
+    a.labels[pt.x] = k64;
+  }
   if (sub == 0 && n64) atomicAdd(&a.ls->fp64_decided, (unsigned long long)n64);
 }
 
-// Exact argmin over all K for the points listed by the assign kernel: one
-// warp per point, lane l takes centroids l, l + 32, ...: FP32 direct form
+// The FP32 direct form over all K for the points of the rescue list, 64 points
+// x 64 centroids at a time through shared memory (4 x 4 per thread).  In the
+// first step from new centres, without labels to start the thresholds from,
+// some percent of the points end here; a warp per point read all K rows (256
+// KB) from L2 for each: 4.67 -> 0.49 ms in that step of 1e7 points, K = 1024.
+// Points whose two nearest the bound does not separate go on to the second
+// list, for gemm_rescue_kernel.
+constexpr int kRP = 64, kRS = kRP + 4;
+__global__ void __launch_bounds__(256, 3) gemm_rescue_tile_kernel(GemmArgs a) {
+  extern __shared__ __align__(16) float s_rt[];
+  float* s_x = s_rt;                  // [64][kRS] x~ by coordinate
+  float* s_c = s_x + kGemmD * kRS;    // [64][kRS] c~ by coordinate
+  __shared__ int s_i[kRP];
+  if (a.ls->done) return;
+  const unsigned cnt = *a.rescue_count;
+  const GemmConst gc = *a.gc;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, k = a.k;
+  const float sB = sqrtf(gc.B_max);
+  for (unsigned b0 = blockIdx.x * (unsigned)kRP; b0 < cnt; b0 += gridDim.x * (unsigned)kRP) {
+    const int np = (int)min((unsigned)kRP, cnt - b0);
+    __syncthreads();  // the tile before is read no more
+    if (tid < kRP) s_i[tid] = a.rescue_list[b0 + min(tid, np - 1)];
+    __syncthreads();
+    for (int q = tid; q < kRP * (kGemmD / 4); q += 256) {
+      const int p = q & (kRP - 1), j = 4 * (q >> 6);
+      const float4 v = *reinterpret_cast<const float4*>(a.xaos + (size_t)s_i[p] * kGemmD + j);
+      const float4 sv = *reinterpret_cast<const float4*>(a.shift + j);
+      s_x[j * kRS + p] = __fsub_rn(v.x, sv.x);
+      s_x[(j + 1) * kRS + p] = __fsub_rn(v.y, sv.y);
+      s_x[(j + 2) * kRS + p] = __fsub_rn(v.z, sv.z);
+      s_x[(j + 3) * kRS + p] = __fsub_rn(v.w, sv.w);
+    }
+    float best[4], second[4];
+    int kb[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) { best[r] = 3.0e38f; second[r] = 3.0e38f; kb[r] = 0; }
+    for (int c0 = 0; c0 < k; c0 += kRP) {
+      __syncthreads();
+      for (int q = tid; q < kRP * (kGemmD / 4); q += 256) {
+        const int c = q & (kRP - 1), j = 4 * (q >> 6);
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (c0 + c < k) v = *reinterpret_cast<const float4*>(a.ctil + (size_t)(c0 + c) * kGemmD + j);
+        s_c[j * kRS + c] = v.x;
+        s_c[(j + 1) * kRS + c] = v.y;
+        s_c[(j + 2) * kRS + c] = v.z;
+        s_c[(j + 3) * kRS + c] = v.w;
+      }
+      __syncthreads();
+      float acc[4][4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
+#pragma unroll 8
+      for (int j = 0; j < kGemmD; ++j) {
+        const float4 x = *reinterpret_cast<const float4*>(s_x + j * kRS + 4 * ty);
+        const float4 c = *reinterpret_cast<const float4*>(s_c + j * kRS + 4 * tx);
+        const float xv[4] = {x.x, x.y, x.z, x.w}, cv[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const float u = __fsub_rn(xv[r], cv[q]);
+            acc[r][q] = __fmaf_rn(u, u, acc[r][q]);
+          }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int c = c0 + 4 * tx + q;
+        if (c >= k) break;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          if (acc[r][q] < best[r]) { second[r] = best[r]; best[r] = acc[r][q]; kb[r] = c; }
+          else if (acc[r][q] < second[r]) second[r] = acc[r][q];
+        }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int o = 1; o < 16; o <<= 1) {
+        const float ob = __shfl_xor_sync(0xffffffffu, best[r], o), os = __shfl_xor_sync(0xffffffffu, second[r], o);
+        const int ok = __shfl_xor_sync(0xffffffffu, kb[r], o);
+        if (ob < best[r] || (ob == best[r] && ok < kb[r])) { second[r] = fminf(best[r], os); best[r] = ob; kb[r] = ok; }
+        else second[r] = fminf(second[r], ob);
+      }
+    // thread tx < 4 of a group of 16: point 4 ty + tx
+    float bs = 0.f, sd = 0.f;
+    int kk = 0;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      if (tx == r) { bs = best[r]; sd = second[r]; kk = kb[r]; }
+    const int p = 4 * ty + tx;
+    if (tx < 4 && p < np) {
+      const int i = s_i[p];
+      const float A = a.xa[i], sA = sqrtf(A), AB = A + gc.B_max;
+      const float e1 = bound64(bs, sA, sB, AB), e2 = bound64(sd, sA, sB, AB);
+      const float lo2 = sd - e2, hi1 = bs + e1;
+      if ((lo2 > hi1) && (lo2 - hi1 > gc.tau * (sd + e2))) a.labels[i] = kk;
+      else a.rescue_list2[atomicAdd(a.rescue_count2, 1u)] = i;
+    }
+  }
+}
+
+// Exact argmin over all K for the points of the second rescue list (the first
+// one where the tile kernel is not run): one warp per point, lane l takes centroids l, l + 32, ...: FP32 direct form
 // with its bound, then FP64 in the oracle's order over every centroid whose
 // lower bound is not above the best upper bound (lowest index on ties).
 __global__ void __launch_bounds__(256) gemm_rescue_kernel(GemmArgs a) {
   __shared__ float s_x[8][kGemmD];
   if (a.ls->done) return;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const unsigned cnt = *a.rescue_count;
+  const unsigned cnt = *a.rescue_count2;
   const GemmConst gc = *a.gc;
   int n64 = 0;
   for (unsigned e = blockIdx.x * 8u + w; e < cnt; e += gridDim.x * 8u) {
-    const int64_t i = a.rescue_list[e];
+    const int64_t i = a.rescue_list2[e];
     const float* xr = a.xaos + (size_t)i * kGemmD;
     s_x[w][lane] = __fsub_rn(xr[lane], a.shift[lane]);
     s_x[w][lane + 32] = __fsub_rn(xr[lane + 32], a.shift[lane + 32]);
@@ -827,6 +973,11 @@ __global__ void __launch_bounds__(256) gemm_tables_kernel(GemmPrepArgs a) {
   if (lane == 0) a.bnorm[c] = B;
 }
 
+// 2^x, 0 or +infinity outside FP32's normal range
+__device__ __forceinline__ float gpow2(int x) {
+  return x > 127 ? __uint_as_float(0x7f800000u) : x < -126 ? 0.f : __uint_as_float((uint32_t)(x + 127) << 23);
+}
+
 // The scale and window constants from max_k B_k (formed by every block for
 // itself), then n'_k and, for FP16 operands, the centre rows scaled by 2^ec,
 // dealt over the blocks (one block wrote all FP16 rows before: 23 us).
@@ -843,65 +994,64 @@ __global__ void __launch_bounds__(256) gemm_consts_kernel(GemmPrepArgs a) {
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < 8; ++w) m = max(m, s_max[w]);
-    const double bmax = __longlong_as_double(m);
-    const double P = 1.02 * ((double)a.A_max + 2.0 * bmax) + 1e-300;
-    const double top = 0.5;  // binade [1, 2): M = 1.5, |2^sigma (h - 2S)| < 0.5
-    int sigma = ilogb(top / P);
-    if (ldexp(P, sigma) >= top) sigma -= 1;
-    sigma = max(-120, min(120, sigma));
+    // FP32 with each sum of error terms raised by 1e-3 below (an FP64 chain of
+    // roots, logarithms and a division took 5 us of one thread's time)
+    const float bmax = __double2float_ru(__longlong_as_double(m));
+    const float P = __fmul_ru(1.02f, __fadd_ru(a.A_max, 2.f * bmax));
+    // binade [1, 2): M = 1.5, |2^sigma (h - 2S)| < 0.5; P in [2^e, 2^(e+1))
+    const int e = (int)(__float_as_uint(P) >> 23) - 127;
+    const int sigma = max(-120, min(120, -2 - e));
     s_sigma = sigma;
-    const double u = 0x1p-24, tw = ldexp(1.0, sigma);
-    const double sB = sqrt(bmax);
+    const float u = 0x1p-24f, tw = gpow2(sigma), tr = (float)a.tie_rel;
+    const float sB = __fsqrt_ru(bmax);
     // FP16: every |c~_kj| <= sqrt(B_max) is scaled to at most 2^14 (FP16
     // holds up to 65504), unless that would push the epilogue's factor
     // 2^(sigma + 1 - ex - ec) below FP32's normal range
     int ec = 0;
-    double uop = 0x1p-8, ax = 0.0, ac = 0.0;
+    float uop = 0x1p-8f, ax = 0.f, ac = 0.f;
     if (a.f16) {
-      const double cm = sB * 1.001 + 1e-300;
-      ec = (int)floor(log2(0x1p14 / cm));
-      while (ec > -200 && ldexp(cm, ec) > 0x1p14) --ec;
+      const float cm = sB * 1.001f + 1e-37f;  // below 2^(e + 1)
+      ec = 13 - ((int)(__float_as_uint(cm) >> 23) - 127);
       ec = max(-100, min(ec, min(100, sigma + 126 - a.ex)));
-      uop = 0x1p-11;
-      ax = ldexp(0x1p-25, -a.ex);  // absolute rounding of a scaled value below 2^-14 (subnormal)
-      ac = ldexp(0x1p-25, -ec);
+      uop = 0x1p-11f;
+      ax = gpow2(-25 - a.ex);  // absolute rounding of a scaled value below 2^-14 (subnormal)
+      ac = gpow2(-25 - ec);
     }
     s_ec = ec;
     // one operand: |fl16(fl32(t)) - t| <= (uop + 2^-24) |t| + a; a product of
     // two: (2 v + v^2) |x||c| + (1 + v)(a_c |x| + a_x |c|) + a_x a_c with
     // v = uop + 2^-24; summed over 64 coordinates (||.||_1 <= 8 ||.||) plus
     // the FP32 accumulation of 64 products in any order (<= 2^-16 sum |p|)
-    const double v = uop + 0x1p-24;
-    const double epsS = 2.0 * v + v * v + 0x1p-16;
-    const double gam = 2.0 * 4.1 * (kGemmD + 1) * 0x1p-53;
+    const float v = uop + 0x1p-24f;
+    const float epsS = 2.f * v + v * v + 0x1p-16f;
+    const float gam = 2.f * 4.1f * (kGemmD + 1) * 0x1p-53f;
     GemmConst g;
-    g.scale = -(float)ldexp(1.0, sigma + 1 - (a.f16 ? a.ex + ec : 0));
+    g.scale = -gpow2(sigma + 1 - (a.f16 ? a.ex + ec : 0));
     g.M = 1.5f;
     // Delta(x) = c0 + ||x~|| c1 + ||x~||^2 cA (units of r): two screen errors
     // 2 (epsS ||x~|| ||c~|| + 8 (1 + v)(a_c ||x~|| + a_x ||c~||) + 64 a_x a_c) + u h
     // each, the oracle's FP64 error, tie_rel * D2 with D2 <= (||x~|| + ||c~||)^2,
     // four ulps of the binade
-    g.c0 = (float)((tw * (2.0 * u * bmax + gam * bmax + a.tie_rel * bmax + 4.0 * (8.0 * (1.0 + v) * ax * sB +
-                                                                                64.0 * ax * ac)) +
-                    8.0 * 0x1p-23) * (1.0 + 1e-3));
-    g.c1 = (float)(tw * (4.0 * epsS * sB + 2.0 * a.tie_rel * sB + 4.0 * 8.0 * (1.0 + v) * ac) * (1.0 + 1e-3));
-    g.cA = (float)(tw * (gam + a.tie_rel) * (1.0 + 1e-3));
+    const float up = 1.f + 1.01e-3f;
+    g.c0 = (tw * ((2.f * u + gam + tr) * bmax + 4.f * (8.f * (1.f + v) * ax * sB + 64.f * ax * ac)) + 8.f * 0x1p-23f) * up;
+    g.c1 = tw * ((4.f * epsS + 2.f * tr) * sB + 32.f * (1.f + v) * ac) * up;
+    g.cA = tw * (gam + tr) * up;
     // start estimate: |r_est - r_tc| <= 2^(sigma+1) (2^-16 + 2^-18) ||x_b|| ||c_b|| (two FP32
     // sums of 64 products of 16-bit operands in different orders), taken as 2^-14 per unit ||x~||
-    g.cest = (float)(2.0 * tw * 0x1p-14 * sB);
-    g.B_max = (float)(bmax * (1.0 + 1e-6));
-    g.tau = (float)(a.tie_rel * (1.0 + 1e-4));
+    g.cest = 2.f * tw * 0x1p-14f * sB * 1.0001f;
+    g.B_max = bmax * (1.f + 1.1e-6f);
+    g.tau = tr * (1.f + 1.01e-4f);
     g.pad0 = g.pad1 = 0.f;
     if (blockIdx.x == 0) *a.gc = g;
   }
   __syncthreads();
-  const double tw = ldexp(1.0, s_sigma);
+  const double tw = __hiloint2double((1023 + s_sigma) << 20, 0);  // 2^sigma
   // padding columns: r = 4, far above any real r < 2 plus the window
   const int t0 = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
   for (int c = t0; c < kpad; c += nt)
     a.nprime[c] = c < k ? __double2float_rn(1.5 + tw * a.bnorm[c]) : 4.0f;
   if (a.f16) {
-    const float cs = ldexpf(1.f, s_ec);
+    const float cs = gpow2(s_ec);
     unsigned short* cb = reinterpret_cast<unsigned short*>(a.cb);
     for (int q = t0; q < kpad * kGemmD; q += nt) {
       const int c = q / kGemmD, j = q - c * kGemmD;
@@ -944,8 +1094,8 @@ cudaError_t launch_gemm_assign(int grid, cudaStream_t st, const GemmArgs& a) {
   const size_t smem = gemm_smem_bytes(a.kpad);
   cudaError_t e = cudaFuncSetAttribute(gemm_assign_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  // rescue_count and tie_count are adjacent: one memset clears both
-  e = cudaMemsetAsync(a.rescue_count, 0, 2 * sizeof(unsigned), st);
+  // the three list lengths are adjacent: one memset clears them
+  e = cudaMemsetAsync(a.rescue_count, 0, 3 * sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
   gemm_assign_kernel<<<grid, kGThreads, smem, st>>>(a);
   e = cudaGetLastError();
@@ -955,7 +1105,18 @@ cudaError_t launch_gemm_assign(int grid, cudaStream_t st, const GemmArgs& a) {
   gemm_tie_kernel<<<grid * 4, 256, 0, st>>>(a);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  gemm_rescue_kernel<<<grid * 4, 256, 0, st>>>(a);
+  // a small set's rescue list is short: the warp-per-point kernel alone
+  GemmArgs r = a;
+  if (a.n >= kRescueTileMin) {
+    const size_t rs = sizeof(float) * 2 * kGemmD * kRS;
+    gemm_rescue_tile_kernel<<<grid * 3, 256, rs, st>>>(a);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  } else {
+    r.rescue_list2 = a.rescue_list;
+    r.rescue_count2 = a.rescue_count;
+  }
+  gemm_rescue_kernel<<<grid * 4, 256, 0, st>>>(r);
   return cudaGetLastError();
 }
 

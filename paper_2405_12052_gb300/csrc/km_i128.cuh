@@ -1,6 +1,7 @@
 // 128-bit integer sums of the mean calculation: two's complement in a low and
 // a high 64-bit word, and the correctly rounded conversion to FP64.
 #pragma once
+#include <cstdint>
 #include <cuda_runtime.h>
 
 namespace km {

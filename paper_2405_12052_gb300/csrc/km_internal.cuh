@@ -198,7 +198,9 @@ struct GemmArgs {
   int32_t* labels;       // out: labels
   int32_t* rescue_list;  // [N] points resolved over all K by the rescue kernel
   int4* tie_list;        // [gemm_tie_entries][3] near ties: point, count (0: unused), up to 20 16-bit candidates
-  unsigned* rescue_count;  // [0] rescue entries, [1] near-tie entries
+  int32_t* rescue_list2; // points the tile kernel leaves open (in the near-tie list's memory, once that is decided)
+  unsigned* rescue_count;  // [0] rescue entries, [1] near-tie entries, [2] second rescue list
+  unsigned* rescue_count2; // = rescue_count + 2
   unsigned* tie_count;     // = rescue_count + 1
   int64_t n;
   int k, kpad, ntiles;

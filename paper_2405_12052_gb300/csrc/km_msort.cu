@@ -9,6 +9,7 @@
 // divides and keeps empty centres; a one-block kernel forms E^2 by a
 // fixed-order tree.  The scatter order inside a cluster is not
 // deterministic, but integer sums do not depend on it.
+#include "km_i128.cuh"
 #include "km_internal.cuh"
 
 namespace km {
@@ -230,56 +231,50 @@ __global__ void ms_chunk_sum_kernel(const float* __restrict__ xa, int d, const i
   }
 }
 
-__device__ __forceinline__ double ms_i128_to_double(unsigned long long lo, long long hs) {
-  unsigned long long hi = (unsigned long long)hs;
-  const bool neg = hs < 0;
-  if (neg) {
-    lo = ~lo + 1ull;
-    hi = ~hi + (lo == 0ull ? 1ull : 0ull);
-  }
-  double r;
-  if (hi == 0ull) {
-    r = __ull2double_rn(lo);
-  } else {
-    const int sh = 64 - __clzll((long long)hi);
-    unsigned long long top = (hi << (64 - sh)) | (lo >> sh);
-    if (lo << (64 - sh)) top |= 1ull;
-    r = ldexp(__ull2double_rn(top), sh);
-  }
-  return neg ? -r : r;
-}
-
-// One thread per (cluster, coordinate): the cluster's chunk sums added in
-// chunk order in int128, one conversion, the divide (an empty cluster keeps
-// its centre) and the squared move.  Centroid tables for the next step are
-// written by the path's own prepare kernels afterwards.
-__global__ void __launch_bounds__(256) ms_finalize_kernel(const unsigned long long* counts, const int* cfirst,
-                                                          const long long* chunk_sums, int k, int d,
-                                                          int chunk, const DataConst* dcp, double* mu,
-                                                          long long* counts_out, double* df2, const LoopState* ls) {
+// One block per cluster, kFinGroups threads per coordinate: the cluster's
+// chunk sums added in int128 (integers: any order), one conversion, the divide
+// (an empty cluster keeps its centre) and the squared move.  (One thread per
+// coordinate walked a large cluster's chunks alone: 18 us with 40 chunks.)
+// Centroid tables for the next step are written by the path's own prepare
+// kernels afterwards.
+constexpr int kFinGroups = 8;
+__global__ void ms_finalize_kernel(const unsigned long long* counts, const int* cfirst,
+                                   const long long* __restrict__ chunk_sums, int d, int chunk, const DataConst* dcp,
+                                   double* mu, long long* counts_out, double* df2, const LoopState* ls) {
+  extern __shared__ unsigned long long s_fin[];  // [kFinGroups][w][2], w = min(d, 64) coordinates at a time
   if (ls->done) return;  // the loop already stopped (graph-driven runs)
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= k * d) return;
-  const int c = q / d, j = q - c * d;
+  const int c = blockIdx.x, w = blockDim.x / kFinGroups, g = threadIdx.x / w, jj = threadIdx.x - g * w;
   const long long cnt = (long long)counts[c];
   const long long first = cfirst[c];  // index of the cluster's first chunk (from the scan)
   const int nch = (int)((cnt + chunk - 1) / chunk);
-  unsigned long long lo = 0ull;
-  long long hi = 0ll;
-#pragma unroll 8
-  for (int t = 0; t < nch; ++t) {
-    const long long v = chunk_sums[(size_t)(first + t) * d + j];
-    const unsigned long long nl = lo + (unsigned long long)v;
-    hi += (v < 0 ? -1ll : 0ll) + (nl < lo ? 1ll : 0ll);
-    lo = nl;
+  for (int j0 = 0; j0 < d; j0 += w) {
+    const int j = j0 + jj;
+    unsigned long long lo = 0ull;
+    long long hi = 0ll;
+    if (j < d) {
+#pragma unroll 4
+      for (int t = g; t < nch; t += kFinGroups) {
+        const long long v = chunk_sums[(size_t)(first + t) * d + j];
+        add128p(lo, hi, (unsigned long long)v, v >> 63);
+      }
+    }
+    s_fin[2 * threadIdx.x] = lo;
+    s_fin[2 * threadIdx.x + 1] = (unsigned long long)hi;
+    __syncthreads();
+    if (g == 0 && j < d) {
+      for (int r = 1; r < kFinGroups; ++r)
+        add128p(lo, hi, s_fin[2 * (r * w + jj)], (long long)s_fin[2 * (r * w + jj) + 1]);
+      const size_t q = (size_t)c * d + j;
+      const double old = mu[q];
+      double nw = old;
+      if (cnt > 0) nw = __ddiv_rn(ldexp(i128_to_double((long long)lo, hi), dcp->G0), (double)cnt);
+      const double df = __dsub_rn(nw, old);
+      df2[q] = __dmul_rn(df, df);
+      mu[q] = nw;
+    }
+    __syncthreads();
   }
-  const double old = mu[q];
-  double nw = old;
-  if (cnt > 0) nw = __ddiv_rn(ldexp(ms_i128_to_double(lo, hi), dcp->G0), (double)cnt);
-  const double df = __dsub_rn(nw, old);
-  df2[q] = __dmul_rn(df, df);
-  mu[q] = nw;
-  if (j == 0) counts_out[c] = cnt;
+  if (threadIdx.x == 0) counts_out[c] = cnt;
 }
 
 // One block: E^2 = sum of the squared moves by a fixed-order tree (thread t
@@ -289,7 +284,8 @@ __global__ void __launch_bounds__(1024) ms_close_kernel(const double* df2, int k
                                                         LoopState* ls) {
   __shared__ double s_red[1024];
   __shared__ int s_empty;
-  if (ls->done) return;
+  const LoopState l = *ls;  // read at once: the fields one after another between stores took half the kernel
+  if (l.done) return;
   const int tid = threadIdx.x;
   if (tid == 0) s_empty = 0;
   double e2p = 0.0;
@@ -299,24 +295,28 @@ __global__ void __launch_bounds__(1024) ms_close_kernel(const double* df2, int k
   for (int c = tid; c < k; c += blockDim.x) empty += counts[c] == 0;
   s_red[tid] = e2p;
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+  if (empty) atomicAdd(&s_empty, empty);
+#pragma unroll
+  for (int w = 512; w >= 32; w >>= 1) {
     if (tid < w) s_red[tid] = __dadd_rn(s_red[tid], s_red[tid + w]);
     __syncthreads();
   }
-  if (empty) atomicAdd(&s_empty, empty);
-  __syncthreads();
+  if (tid >= 32) return;
+  double E2 = s_red[tid];
+#pragma unroll
+  for (int w = 16; w > 0; w >>= 1) E2 = __dadd_rn(E2, __shfl_down_sync(0xffffffffu, E2, w));
   if (tid == 0) {
-    const double E2 = s_red[0], E = sqrt(E2);
+    const double E = sqrt(E2);
     ls->E2 = E2;
     ls->E = E;
-    ls->iter += 1;
+    ls->iter = l.iter + 1;
     ls->empty = s_empty;
-    const double esel = ls->e_mode == 1 ? E2 : E;
-    if (esel < ls->tol) { ls->converged = 1; ls->done = 1; }
-    if (ls->iter >= ls->max_iter) ls->done = 1;
-    ls->last_flagged = ls->flagged;
-    ls->last_fp64 = ls->fp64_decided;
-    ls->last_overflowed = ls->overflowed;
+    const double esel = l.e_mode == 1 ? E2 : E;
+    if (esel < l.tol) { ls->converged = 1; ls->done = 1; }
+    if (l.iter + 1 >= l.max_iter) ls->done = 1;
+    ls->last_flagged = l.flagged;
+    ls->last_fp64 = l.fp64_decided;
+    ls->last_overflowed = l.overflowed;
     ls->flagged = 0ull;
     ls->fp64_decided = 0ull;
     ls->overflowed = 0ull;
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(256) ms_shard_finalize_kernel(const long long*
   const long long cnt = (long long)clo;  // counts fit in 64 bits
   const double old = mu[q];
   double nw = old;
-  if (cnt > 0) nw = __ddiv_rn(ldexp(ms_i128_to_double(lo, hi), dcp->G0), (double)cnt);
+  if (cnt > 0) nw = __ddiv_rn(ldexp(i128_to_double((long long)lo, hi), dcp->G0), (double)cnt);
   const double df = __dsub_rn(nw, old);
   df2[q] = __dmul_rn(df, df);
   mu[q] = nw;
@@ -402,8 +402,9 @@ static cudaError_t msort_sums(const MsortArgs& a, const LoopState* stop, cudaStr
 cudaError_t launch_msort_step(const MsortArgs& a, cudaStream_t st) {
   cudaError_t e = msort_sums(a, a.ls, st);
   if (e != cudaSuccess) return e;
-  ms_finalize_kernel<<<(a.k * a.d + 255) / 256, 256, 0, st>>>(a.counts_u, a.cfirst, a.chunk_sums, a.k, a.d,
-                                                              msort_chunk(a.n), a.dc, a.mu, a.counts, a.df2, a.ls);
+  const int w = std::min(a.d, 64), ft = kFinGroups * w;
+  ms_finalize_kernel<<<a.k, ft, 16 * (size_t)ft, st>>>(a.counts_u, a.cfirst, a.chunk_sums, a.d, msort_chunk(a.n), a.dc,
+                                                       a.mu, a.counts, a.df2, a.ls);
   ms_close_kernel<<<1, 1024, 0, st>>>(a.df2, a.k * a.d, a.counts, a.k, a.ls);
   return cudaGetLastError();
 }
