@@ -700,7 +700,7 @@ km_status km_init_kmeanspp(km_ctx* c, const double* u, double* mu_out, int64_t* 
   };
   cudaError_t e = cudaSuccess;
   if ((e = dalloc(&du, (size_t)c->k)) != cudaSuccess || (e = dalloc(&dmu, (size_t)c->k * c->d)) != cudaSuccess ||
-      (e = dalloc(&d2, (size_t)n)) != cudaSuccess || (e = dalloc(&cs, (size_t)nch)) != cudaSuccess ||
+      (e = dalloc(&d2, (size_t)n)) != cudaSuccess || (e = dalloc(&cs, (size_t)nch + 1)) != cudaSuccess ||
       (e = dalloc(&didx, (size_t)c->k)) != cudaSuccess) {
     release();
     return fail(c, KM_ENOMEM, std::string("k-means++ buffers: ") + cudaGetErrorString(e));
