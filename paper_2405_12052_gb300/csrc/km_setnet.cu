@@ -168,7 +168,8 @@ __device__ __forceinline__ void stage_w1(float* s_w1, const float* __restrict__ 
 // cycle); neither h1 nor h2 goes to memory (the backward pass forms h1 again
 // and needs only the sign of h2: 16 bytes per point instead of 1 KB), and the
 // 8x8 tile takes 4 16-byte shared reads per 64 multiply-adds (the 8x4 tile: 3
-// per 32).  1M points: 1.29 -> 0.72 ms.  64-point blocks where 256-point ones
+// per 32).  Resident blocks stride over the tiles, so W2 is staged once each.
+// 1M points: 1.29 -> 0.69 ms.  64-point blocks where 256-point ones
 // would leave SMs idle.  The pooled sum of 64 points is added as before: 8
 // points in order per thread, then the eight groups in order.
 template <int PT>
@@ -182,68 +183,70 @@ __global__ void __launch_bounds__(2 * PT) sn_fwd_points(const float* __restrict_
   float* s_w1 = s_h1 + H * AS;    // [128][4]
   const NetOff o = net_off(d, k);
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  const int64_t p0 = (int64_t)blockIdx.x * PT;
   for (int q = tid; q < H * H / 4; q += NT)
     reinterpret_cast<float4*>(s_w2)[q] = reinterpret_cast<const float4*>(w2t)[q];
   stage_w1(s_w1, prm, o, d, tid, NT);
-  __syncthreads();
-  {
-    const int p = tid % PT, u0 = (tid / PT) * (H / 2);
-    float xv[3] = {0.f, 0.f, 0.f};
-    if (p0 + p < P)
-      for (int j = 0; j < d; ++j) xv[j] = xs[(p0 + p) * d + j];
+  float b2[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) b2[c] = prm[o.b2 + 4 * tx + (c & 3) + 64 * (c >> 2)];
+  const int64_t ntiles = (P + PT - 1) / PT;
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int64_t p0 = tile * PT;
+    __syncthreads();  // the weights; the tile before is read no more
+    {
+      const int p = tid % PT, u0 = (tid / PT) * (H / 2);
+      float xv[3] = {0.f, 0.f, 0.f};
+      if (p0 + p < P)
+        for (int j = 0; j < d; ++j) xv[j] = xs[(p0 + p) * d + j];
 #pragma unroll 8
-    for (int u = u0; u < u0 + H / 2; ++u) s_h1[u * AS + p] = h1_of(s_w1, xv, u);
-  }
-  __syncthreads();
-  float acc[8][8];
-#pragma unroll
-  for (int r = 0; r < 8; ++r)
-#pragma unroll
-    for (int c = 0; c < 8; ++c) acc[r][c] = 0.f;
-  tile_gemm_8x8<H, AS, H>(s_h1, s_w2, ty, tx, acc);
-  float b2[8], ps[8];
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    b2[c] = prm[o.b2 + 4 * tx + (c & 3) + 64 * (c >> 2)];
-    ps[c] = 0.f;
-  }
-  const bool live = p0 + 8 * ty < P;  // P is a multiple of 64
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    uint32_t m = 0u;  // bits 0..3: units 4 tx .. 4 tx + 3, bits 4..7: 64 + those
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const float h = fmaxf(acc[r][c] + b2[c], 0.f);
-      ps[c] += h;
-      m |= (h > 0.f ? 1u : 0u) << c;
+      for (int u = u0; u < u0 + H / 2; ++u) s_h1[u * AS + p] = h1_of(s_w1, xv, u);
     }
-    if (bits) {
-      // the point's 128 bits from the 16 threads of its unit groups: word w
-      // (units 32 w .. 32 w + 31) from groups 8 (w & 1) .. + 7
-      uint32_t lo = (m & 15u) << (4 * (tx & 7)), hi = (m >> 4) << (4 * (tx & 7));
+    __syncthreads();
+    float acc[8][8], ps[8];
 #pragma unroll
-      for (int f = 1; f < 8; f <<= 1) {
-        lo |= __shfl_xor_sync(0xffffffffu, lo, f);
-        hi |= __shfl_xor_sync(0xffffffffu, hi, f);
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int c = 0; c < 8; ++c) acc[r][c] = 0.f;
+    tile_gemm_8x8<H, AS, H>(s_h1, s_w2, ty, tx, acc);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) ps[c] = 0.f;
+    const bool live = p0 + 8 * ty < P;  // P is a multiple of 64
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      uint32_t m = 0u;  // bits 0..3: units 4 tx .. 4 tx + 3, bits 4..7: 64 + those
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const float h = fmaxf(acc[r][c] + b2[c], 0.f);
+        ps[c] += h;
+        m |= (h > 0.f ? 1u : 0u) << c;
       }
-      if (live && (tx & 7) == 0) {
-        uint32_t* w = bits + (p0 + 8 * ty + r) * 4 + (tx >> 3);
-        w[0] = lo;
-        w[2] = hi;
+      if (bits) {
+        // the point's 128 bits from the 16 threads of its unit groups: word w
+        // (units 32 w .. 32 w + 31) from groups 8 (w & 1) .. + 7
+        uint32_t lo = (m & 15u) << (4 * (tx & 7)), hi = (m >> 4) << (4 * (tx & 7));
+#pragma unroll
+        for (int f = 1; f < 8; f <<= 1) {
+          lo |= __shfl_xor_sync(0xffffffffu, lo, f);
+          hi |= __shfl_xor_sync(0xffffffffu, hi, f);
+        }
+        if (live && (tx & 7) == 0) {
+          uint32_t* w = bits + (p0 + 8 * ty + r) * 4 + (tx >> 3);
+          w[0] = lo;
+          w[2] = hi;
+        }
       }
     }
-  }
-  __syncthreads();  // s_h1 is read no more: the pooled sums take its place
+    __syncthreads();  // s_h1 is read no more: the pooled sums take its place
 #pragma unroll
-  for (int c = 0; c < 8; ++c) s_h1[ty * H + 4 * tx + (c & 3) + 64 * (c >> 2)] = ps[c];
-  __syncthreads();
-  for (int q = tid; q < PT / kTileP * H; q += NT) {
-    const int t = q / H, u = q % H;
-    if (p0 + t * kTileP >= P) break;
-    float s = 0.f;
-    for (int g = 0; g < 8; ++g) s += s_h1[(8 * t + g) * H + u];
-    tile_pool[((int64_t)blockIdx.x * (PT / kTileP) + t) * H + u] = s;
+    for (int c = 0; c < 8; ++c) s_h1[ty * H + 4 * tx + (c & 3) + 64 * (c >> 2)] = ps[c];
+    __syncthreads();
+    for (int q = tid; q < PT / kTileP * H; q += NT) {
+      const int t = q / H, u = q % H;
+      if (p0 + t * kTileP >= P) break;
+      float s = 0.f;
+      for (int g = 0; g < 8; ++g) s += s_h1[(8 * t + g) * H + u];
+      tile_pool[(tile * (PT / kTileP) + t) * H + u] = s;
+    }
   }
 }
 
@@ -603,8 +606,10 @@ static cudaError_t launch_fwd_points(const SetNetArgs& a, bool train, int64_t P,
   const size_t smem = sizeof(float) * (H * H + H * (PT + 4) + 4 * H);
   cudaError_t e = cudaFuncSetAttribute(sn_fwd_points<PT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  sn_fwd_points<PT><<<(unsigned)((P + PT - 1) / PT), 2 * PT, smem, st>>>(a.xs, a.prm, a.w2t, a.d, a.k, P,
-                                                                       train ? a.bits : nullptr, a.tile_pool);
+  // resident blocks stride over the tiles: W2 (64 KB) is staged once each
+  const int64_t grid = std::min<int64_t>((P + PT - 1) / PT, 152 * (PT == 256 ? 1 : 2));
+  sn_fwd_points<PT><<<(unsigned)grid, 2 * PT, smem, st>>>(a.xs, a.prm, a.w2t, a.d, a.k, P, train ? a.bits : nullptr,
+                                                          a.tile_pool);
   return cudaGetLastError();
 }
 
