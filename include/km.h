@@ -405,7 +405,9 @@ km_status km_setnet_set_params(km_setnet* net, const float* params);
 km_status km_setnet_get_params(km_setnet* net, float* params_out);
 /* Forward, loss and backward on a batch of B sets; the gradients stay on the
  * device (km_setnet_get_grads copies them).  loss_out (host) may be NULL
- * (then nothing synchronizes). */
+ * (then nothing synchronizes).  KM_ETIMEOUT, here or from km_setnet_get_grads:
+ * a bounded wait of the backward kernel gave up; the gradients are not to be
+ * used. */
 km_status km_setnet_loss_grad(km_setnet* net, const float* x, const float* targets, int32_t B, int32_t S,
                               int32_t mem, float* loss_out);
 km_status km_setnet_get_grads(km_setnet* net, float* grads_out);

@@ -335,9 +335,13 @@ struct SetNetArgs {
   float* w2t; uint32_t* bits; float* tile_pool; float* G; float* P; float* dG; float* loss;
   float* A3; float* dZ3; float* dP; float* set_loss;  // [B][H], [B][H], [B][K d], [B]: head values of each set
   float* part;
+  int* err;           // set to 3 when a bounded wait of the backward kernel gives up
 };
+constexpr int kSetBwdBlocks = 152;  // backward blocks at most: one per SM
 int setnet_param_count(int d, int k);
-int64_t setnet_part_floats(int64_t P, int d);
+int64_t setnet_part_floats(int d);
+int setnet_bwd_blocks(int B, int S);
+cudaError_t launch_setnet_bwd_points(const SetNetArgs& a, int blocks, cudaStream_t st);
 cudaError_t launch_setnet_forward(const SetNetArgs& a, bool train, cudaStream_t st);
 cudaError_t launch_setnet_backward(const SetNetArgs& a, cudaStream_t st);
 cudaError_t launch_setnet_adam(float* prm, const float* grads, float* m, float* v, int n, float lr, float b1,

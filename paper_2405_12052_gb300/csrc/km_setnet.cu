@@ -10,7 +10,8 @@
 //   loss         mean over sets of the symmetric Chamfer distance to the
 //                standardised targets (ties: lowest index)
 //
-// FP32 throughout; every reduction runs in a fixed order (no float
+// FP32 throughout (the backward products on the tensor cores by exact three-way
+// splits of their FP32 factor); every reduction runs in a fixed order (no float
 // atomics), so a step is deterministic.  Kernels:
 //   sn_standardize   one block per set
 //   sn_fwd_points    64 or 256 points per block: h1 in shared memory, h2 by
@@ -19,40 +20,18 @@
 //   sn_head          one block per set: pooling, head forward, loss and head
 //                    backward to dg
 //   sn_head_grad     dW3, dW4, db3, db4 and the loss, sets added in order
-//   sn_bwd_points    one block per run of 64-point tiles: h1 formed again,
-//                    dz2 = dg/S * [h2 > 0] from the bits, dz1 = (dz2 W2) *
-//                    [h1 > 0], and the block's dW2 = sum dz2 h1^T, dW1, db1,
-//                    db2 kept in registers
+//   sn_bwd_points    (km_setnet_bwd.cu, tensor cores) dz2 = dg/S * [h2 > 0] from
+//                    the bits, dz1 = (dz2 W2) * [h1 > 0], and each block's dW2
+//                    = sum dz2 h1^T, dW1, db1, db2
 //   sn_wgrad_reduce  adds the blocks' gradients in order
 //   sn_adam          Adam with bias correction (Kingma and Ba 2015)
-#include "km_internal.cuh"
+#include "km_setnet.cuh"
 
 #include <algorithm>
 
 namespace km {
 
 namespace {
-
-constexpr int H = kSetH;
-constexpr int kTileP = 64;     // points per pooled sum and per backward tile
-constexpr int kBwdBlocks = 152;  // backward blocks: one per SM (166 KB of shared memory each)
-
-struct NetOff {  // offsets of the parameters in the flat vector
-  int W1, b1, W2, b2, W3, b3, W4, b4, total;
-};
-__host__ __device__ inline NetOff net_off(int d, int k) {
-  NetOff o;
-  o.W1 = 0;
-  o.b1 = o.W1 + H * d;
-  o.W2 = o.b1 + H;
-  o.b2 = o.W2 + H * H;
-  o.W3 = o.b2 + H;
-  o.b3 = o.W3 + H * H;
-  o.W4 = o.b3 + H;
-  o.b4 = o.W4 + k * d * H;
-  o.total = o.b4 + k * d;
-  return o;
-}
 
 // Sum over the block's 256 threads of up to three values at once: the pairwise
 // tree t += t + 128, 64, ..., 1 (the last five levels inside warp 0).
@@ -146,19 +125,6 @@ __device__ __forceinline__ void tile_gemm_8x8(const float* __restrict__ a, const
     for (int r = 0; r < 8; ++r)
 #pragma unroll
       for (int c = 0; c < 8; ++c) acc[r][c] = fmaf(av[r], wv[c], acc[r][c]);
-  }
-}
-
-// h1 of one point and unit (the same expression forward and backward).
-__device__ __forceinline__ float h1_of(const float* s_w1, const float (&xv)[3], int u) {
-  const float4 w = *reinterpret_cast<const float4*>(s_w1 + 4 * u);  // W1[u][0..2] (0 past d), b1[u]
-  return fmaxf(fmaf(w.z, xv[2], fmaf(w.y, xv[1], fmaf(w.x, xv[0], w.w))), 0.f);
-}
-__device__ __forceinline__ void stage_w1(float* s_w1, const float* __restrict__ prm, const NetOff& o, int d, int tid,
-                                         int nth) {
-  for (int q = tid; q < 4 * H; q += nth) {
-    const int u = q >> 2, j = q & 3;
-    s_w1[q] = j == 3 ? prm[o.b1 + u] : j < d ? prm[o.W1 + u * d + j] : 0.f;
   }
 }
 
@@ -393,149 +359,6 @@ __global__ void __launch_bounds__(128) sn_head_grad(int B, int d, int k, const f
   }
 }
 
-// Backward through the per-point layers and their weight gradients.  Block b
-// takes the run of 64-point tiles [b T / gridDim, (b + 1) T / gridDim) and
-// writes one partial gradient.  Per tile: h1 again from the standardised
-// points (3 multiply-adds a value, against 512 bytes a point read back) and
-// dz2 from the sign bits of h2, in the layouts the two products read; dh1 =
-// dz2 W2 (4 points x 8 units per thread), dW2 += dz2^T h1 (8 x 8 outputs per
-// thread, in registers over all tiles).  Bound by the FP32 multiply-adds of
-// the two products (34.4e9 for 1M points: 0.92 ms at one per lane and cycle);
-// 1M points: 1.73 + 3.96 ms in two kernels -> 1.64 ms in one.
-constexpr int kZT = kTileP + 4;  // row stride of dz2 by unit
-constexpr int kZP = H + 4;       // row stride of the tiles by point
-constexpr size_t kBwdSmem = sizeof(float) * (H * H + H * kZT + 2 * kTileP * kZP + 4 * H + 4 * kTileP + H);
-__global__ void __launch_bounds__(256, 1) sn_bwd_points(const float* __restrict__ prm, int d, int k, int S,
-                                                        int64_t tiles, const float* __restrict__ dG,
-                                                        const float* __restrict__ xs,
-                                                        const uint32_t* __restrict__ bits, float* __restrict__ part) {
-  extern __shared__ __align__(16) float sm[];
-  float* s_w2 = sm;                    // [128][128] W2[u][c]
-  float* s_zT = s_w2 + H * H;          // [128][kZT] dz2[u][p]
-  float* s_zP = s_zT + H * kZT;        // [64][kZP] dz2[p][u]
-  float* s_hP = s_zP + kTileP * kZP;   // [64][kZP] h1[p][c]
-  float* s_w1 = s_hP + kTileP * kZP;   // [128][4]
-  float* s_x = s_w1 + 4 * H;           // [64][4]
-  float* s_dg = s_x + 4 * kTileP;      // [128] dg / S of the tile's set
-  const NetOff o = net_off(d, k);
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  const int64_t t0 = tiles * blockIdx.x / gridDim.x, t1 = tiles * (blockIdx.x + 1) / gridDim.x;
-  for (int q = tid; q < H * H / 4; q += 256)
-    reinterpret_cast<float4*>(s_w2)[q] = reinterpret_cast<const float4*>(prm + o.W2)[q];
-  stage_w1(s_w1, prm, o, d, tid, 256);
-  float acc2[8][8];       // dW2: units 8 ty + r, inputs 4 tx + (c & 3) + 64 (c >> 2)
-  float g1[8][4];         // dW1 and db1 of inputs 4 tx + ..., this thread's points: dz1 x_j, dz1
-  float gb2 = 0.f;        // db2 of unit tid (threads 0..127)
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-#pragma unroll
-    for (int c = 0; c < 8; ++c) acc2[r][c] = 0.f;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) g1[r][j] = 0.f;
-  }
-  int set = -1;
-  for (int64_t t = t0; t < t1; ++t) {
-    const int64_t p0 = t * kTileP;
-    const int b = (int)(p0 / S);
-    __syncthreads();  // the previous tile is read no more
-    if (tid < 4 * kTileP) {
-      const int p = tid >> 2, j = tid & 3;
-      s_x[tid] = j < d ? xs[(p0 + p) * d + j] : 0.f;
-    }
-    if (b != set && tid < H) s_dg[tid] = dG[(size_t)b * H + tid] / (float)S;
-    set = b;
-    __syncthreads();
-    // dz2 by unit: lanes over points
-    {
-      const int p = tid & 63, w = tid >> 6;  // word w of the point's bits: units 32 w ..
-      const uint32_t m = bits[(p0 + p) * 4 + w];
-#pragma unroll 8
-      for (int u = 0; u < 32; ++u) s_zT[(32 * w + u) * kZT + p] = (m >> u) & 1u ? s_dg[32 * w + u] : 0.f;
-    }
-    // dz2 and h1 by point: lanes over units
-    {
-      const int u = tid & 127, ph = tid >> 7;
-      const float dg = s_dg[u];
-      const float4 w = *reinterpret_cast<const float4*>(s_w1 + 4 * u);
-#pragma unroll 8
-      for (int q = 0; q < kTileP / 2; ++q) {
-        const int p = 2 * q + ph;
-        const uint32_t m = bits[(p0 + p) * 4 + (u >> 5)];
-        s_zP[p * kZP + u] = (m >> (u & 31)) & 1u ? dg : 0.f;
-        const float4 xv = *reinterpret_cast<const float4*>(s_x + 4 * p);
-        s_hP[p * kZP + u] = fmaxf(fmaf(w.z, xv.z, fmaf(w.y, xv.y, fmaf(w.x, xv.x, w.w))), 0.f);
-      }
-    }
-    __syncthreads();
-    // dh1[p][c] = sum_u dz2[p][u] W2[u][c]: points 4 ty .. 4 ty + 3
-    {
-      float acc[4][8];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 8; ++c) acc[r][c] = 0.f;
-#pragma unroll 4
-      for (int u = 0; u < H; ++u) {
-        const float4 a = *reinterpret_cast<const float4*>(s_zT + u * kZT + 4 * ty);
-        const float4 w0 = *reinterpret_cast<const float4*>(s_w2 + u * H + 4 * tx);
-        const float4 w1 = *reinterpret_cast<const float4*>(s_w2 + u * H + 64 + 4 * tx);
-        const float av[4] = {a.x, a.y, a.z, a.w};
-        const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-          for (int c = 0; c < 8; ++c) acc[r][c] = fmaf(av[r], wv[c], acc[r][c]);
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int p = 4 * ty + r;
-        const float4 xv = *reinterpret_cast<const float4*>(s_x + 4 * p);
-        const float4 h0 = *reinterpret_cast<const float4*>(s_hP + p * kZP + 4 * tx);
-        const float4 h1 = *reinterpret_cast<const float4*>(s_hP + p * kZP + 64 + 4 * tx);
-        const float hv[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const float z1 = hv[c] > 0.f ? acc[r][c] : 0.f;
-          g1[c][0] = fmaf(z1, xv.x, g1[c][0]);
-          g1[c][1] = fmaf(z1, xv.y, g1[c][1]);
-          g1[c][2] = fmaf(z1, xv.z, g1[c][2]);
-          g1[c][3] += z1;
-        }
-      }
-    }
-    // dW2[u][c] += sum_p dz2[p][u] h1[p][c]
-    tile_gemm_8x8<kTileP, kZP, kZP>(s_zP, s_hP, ty, tx, acc2);
-    if (tid < H) {
-      float s = 0.f;
-#pragma unroll 8
-      for (int p = 0; p < kTileP; ++p) s += s_zP[p * kZP + tid];
-      gb2 += s;
-    }
-  }
-  const int stride = H * H + H * d + 2 * H;
-  float* out = part + (size_t)blockIdx.x * stride;
-#pragma unroll
-  for (int r = 0; r < 8; ++r)
-#pragma unroll
-    for (int c = 0; c < 8; ++c) out[(8 * ty + r) * H + 4 * tx + (c & 3) + 64 * (c >> 2)] = acc2[r][c];
-  // dW1 and db1: the 16 point groups' sums, added in order
-  __syncthreads();
-  float* s_g = sm;  // [16][128][4]
-#pragma unroll
-  for (int c = 0; c < 8; ++c)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) s_g[(ty * H + 4 * tx + (c & 3) + 64 * (c >> 2)) * 4 + j] = g1[c][j];
-  __syncthreads();
-  for (int q = tid; q < 4 * H; q += 256) {
-    float s = 0.f;
-    for (int g = 0; g < 16; ++g) s += s_g[g * 4 * H + q];
-    const int u = q >> 2, j = q & 3;
-    if (j == 3) out[H * H + H * d + u] = s;
-    else if (j < d) out[H * H + u * d + j] = s;
-  }
-  if (tid < H) out[H * H + H * d + H + tid] = gb2;
-}
-
 // The blocks' partial gradients added in order.
 __global__ void __launch_bounds__(64) sn_wgrad_reduce(const float* __restrict__ part, int nparts, int d, int k,
                                                       float* __restrict__ grads) {
@@ -634,20 +457,16 @@ cudaError_t launch_setnet_forward(const SetNetArgs& a, bool train, cudaStream_t 
   return cudaGetLastError();
 }
 
-static int bwd_blocks(int64_t P) { return (int)std::min<int64_t>(P / kTileP, kBwdBlocks); }
-
 cudaError_t launch_setnet_backward(const SetNetArgs& a, cudaStream_t st) {
-  const int64_t P = (int64_t)a.B * a.S;
-  const int nb = bwd_blocks(P);
-  cudaError_t e = cudaFuncSetAttribute(sn_bwd_points, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBwdSmem);
+  const int nb = setnet_bwd_blocks(a.B, a.S);
+  cudaError_t e = launch_setnet_bwd_points(a, nb, st);
   if (e != cudaSuccess) return e;
-  sn_bwd_points<<<nb, 256, kBwdSmem, st>>>(a.prm, a.d, a.k, a.S, P / kTileP, a.dG, a.xs, a.bits, a.part);
   const int stride = H * H + H * a.d + 2 * H;
   sn_wgrad_reduce<<<(stride + 63) / 64, 64, 0, st>>>(a.part, nb, a.d, a.k, a.grads);
   return cudaGetLastError();
 }
 
-int64_t setnet_part_floats(int64_t P, int d) { return (int64_t)bwd_blocks(P) * (H * H + H * d + 2 * H); }
+int64_t setnet_part_floats(int d) { return (int64_t)kSetBwdBlocks * (H * H + H * d + 2 * H); }
 
 cudaError_t launch_setnet_adam(float* prm, const float* grads, float* m, float* v, int n, float lr, float b1,
                                float b2, float eps, float c1, float c2, cudaStream_t st) {

@@ -81,7 +81,7 @@ km_status ensure(km_setnet* n, int B, int S) {
   KN_CUDA(n, nalloc(&n->dZ3, (size_t)B * kSetH));
   KN_CUDA(n, nalloc(&n->dP, (size_t)B * KD));
   KN_CUDA(n, nalloc(&n->set_loss, (size_t)B));
-  KN_CUDA(n, nalloc(&n->part, (size_t)setnet_part_floats(Pn, d)));
+  KN_CUDA(n, nalloc(&n->part, (size_t)setnet_part_floats(d)));
   KN_CUDA(n, nalloc(&n->cout, (size_t)B * KD));
   n->capB = B;
   n->capS = S;
@@ -95,6 +95,7 @@ SetNetArgs args(km_setnet* n, const float* x, const float* t, int B, int S) {
   a.xs = n->xs; a.ts = n->ts; a.ms = n->ms; a.w2t = n->w2t; a.bits = n->bits;
   a.tile_pool = n->tile_pool; a.G = n->G; a.P = n->P; a.dG = n->dG; a.loss = n->loss;
   a.A3 = n->A3; a.dZ3 = n->dZ3; a.dP = n->dP; a.set_loss = n->set_loss; a.part = n->part;
+  a.err = reinterpret_cast<int*>(n->loss + 1);
   return a;
 }
 
@@ -154,7 +155,8 @@ km_status km_setnet_create(km_setnet** out, int32_t d, int32_t k, void* stream) 
   KN_CUDA(n, nalloc(&n->m, (size_t)n->nparam));
   KN_CUDA(n, nalloc(&n->v, (size_t)n->nparam));
   KN_CUDA(n, nalloc(&n->w2t, (size_t)kSetH * kSetH));
-  KN_CUDA(n, nalloc(&n->loss, 1));
+  KN_CUDA(n, nalloc(&n->loss, 2));  // the loss and the error word of the backward kernel
+  KN_CUDA(n, cudaMemsetAsync(n->loss, 0, 2 * sizeof(float), n->st));
   KN_CUDA(n, cudaMemsetAsync(n->prm, 0, sizeof(float) * n->nparam, n->st));
   KN_CUDA(n, cudaMemsetAsync(n->grads, 0, sizeof(float) * n->nparam, n->st));
   KN_CUDA(n, cudaMemsetAsync(n->m, 0, sizeof(float) * n->nparam, n->st));
@@ -182,11 +184,20 @@ km_status km_setnet_get_params(km_setnet* n, float* params_out) {
   return KM_OK;
 }
 
+// The loss and the error word of the last backward pass (synchronizes).
+static km_status read_loss(km_setnet* n, float* loss_out) {
+  struct { float loss; int32_t err; } h{};
+  KN_CUDA(n, cudaMemcpyAsync(&h, n->loss, sizeof(h), cudaMemcpyDeviceToHost, n->st));
+  KN_CUDA(n, cudaStreamSynchronize(n->st));
+  if (h.err) return nfail(n, KM_ETIMEOUT, "a bounded device wait gave up (error word " + std::to_string(h.err) + ")");
+  if (loss_out) *loss_out = h.loss;
+  return KM_OK;
+}
+
 km_status km_setnet_get_grads(km_setnet* n, float* grads_out) {
   if (!n || !grads_out) return KM_EINVAL;
   KN_CUDA(n, cudaMemcpyAsync(grads_out, n->grads, sizeof(float) * n->nparam, cudaMemcpyDeviceToHost, n->st));
-  KN_CUDA(n, cudaStreamSynchronize(n->st));
-  return KM_OK;
+  return read_loss(n, nullptr);
 }
 
 km_status km_setnet_loss_grad(km_setnet* n, const float* x, const float* targets, int32_t B, int32_t S,
@@ -198,11 +209,7 @@ km_status km_setnet_loss_grad(km_setnet* n, const float* x, const float* targets
   SetNetArgs a = args(n, xd, td, B, S);
   KN_CUDA(n, launch_setnet_forward(a, true, n->st));
   KN_CUDA(n, launch_setnet_backward(a, n->st));
-  if (loss_out) {
-    KN_CUDA(n, cudaMemcpyAsync(loss_out, n->loss, sizeof(float), cudaMemcpyDeviceToHost, n->st));
-    KN_CUDA(n, cudaStreamSynchronize(n->st));
-  }
-  return KM_OK;
+  return loss_out ? read_loss(n, loss_out) : KM_OK;
 }
 
 km_status km_setnet_adam(km_setnet* n, float lr, float beta1, float beta2, float eps) {
@@ -221,11 +228,7 @@ km_status km_setnet_train_step(km_setnet* n, const float* x, const float* target
   if (s != KM_OK) return s;
   s = km_setnet_adam(n, lr, 0.9f, 0.999f, 1e-8f);
   if (s != KM_OK) return s;
-  if (loss_out) {
-    KN_CUDA(n, cudaMemcpyAsync(loss_out, n->loss, sizeof(float), cudaMemcpyDeviceToHost, n->st));
-    KN_CUDA(n, cudaStreamSynchronize(n->st));
-  }
-  return KM_OK;
+  return loss_out ? read_loss(n, loss_out) : KM_OK;
 }
 
 km_status km_setnet_predict(km_setnet* n, const float* x, int32_t B, int32_t S, int32_t mem, double* centroids_out) {
