@@ -75,6 +75,10 @@ static __device__ void fast_screen_tables(const double* mu, const float* shift, 
   // the largest sigma with 2^sigma P < 2^half, P in [2^e, 2^(e + 1))
   const float P = __fmul_ru(__fadd_ru(__fmul_ru(A_max, 1.f + 0x1p-20f), 2.f * bmax), 1.f + 0x1p-10f);
   const int e = (int)(__float_as_uint(P) >> 23) - 127;
+  // squares so large that the scale leaves FP32's range (|x| from about 1e10 at
+  // K = 8, 1e16 at K = 32 and 1e17 at K = 64): the values below leave the
+  // binade, so every point is flagged
+  const bool out = half - e - 1 < -120;
   const int sigma = max(-120, min(120, half - e - 1));
   auto pow2 = [](int x) {  // 2^x, +infinity or 0 outside the normal range
     return x > 127 ? __uint_as_float(0x7f800000u) : x < -126 ? 0.f : __uint_as_float((uint32_t)(x + 127) << 23);
@@ -87,7 +91,7 @@ static __device__ void fast_screen_tables(const double* mu, const float* shift, 
     ic.mul = 1u << L;
     ic.bitsM_low = __float_as_uint(M) & ((1u << (32 - L)) - 1u);
     ic.G = G;
-    ic.thr_c0 = ((float)(d + 3) + (8.002f * u + u64x * (float)(d + 1)) * bmax * G) * (1.f + 1.01e-4f);
+    ic.thr_c0 = out ? __uint_as_float(0x7f800000u) : ((float)(d + 3) + (8.002f * u + u64x * (float)(d + 1)) * bmax * G) * (1.f + 1.01e-4f);
     ic.thr_cA = (4.001f * u + u64x * (float)(d + 1)) * G * (1.f + 1.12e-4f);
     ic.tau = tau;
     ic.B_max = bmax;

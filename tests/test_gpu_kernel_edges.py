@@ -182,3 +182,23 @@ def test_tensor_run_and_step_after_it(km, oracle, n, k, ops):
     z, _, cnt, _ = oracle.step(x, r["centroids"])
     assert np.array_equal(g.labels(), z) and np.array_equal(g.counts(), cnt)
     g.close()
+
+
+
+# squared distances near FP32's overflow, for each packing width of the screen:
+# the labels stay the oracle's
+@pytest.mark.parametrize("scale", [1e9, 1e15, 1e18])
+@pytest.mark.parametrize("d,k", [(1, 3), (2, 8), (3, 20), (3, 33), (2, 64), (1, 100), (4, 200)])
+def test_large_magnitudes(km, oracle, d, k, scale):
+    n = 8193
+    x, _, _ = synth.iso_mixture(n, d, max(2, k // 2), sigma=1.5, box=8.0, seed=d + k)
+    x = (x.astype(np.float64) * scale).astype(np.float32)
+    mu0, _ = synth.init_distinct(x, k, seed=1)
+    ref = oracle.run(x, mu0, 12, 0.0)
+    for graph in (0, 1):
+        g = km.KMeans(n, d, k, use_graph=graph)
+        g.set_points(x)
+        g.set_init(mu0)
+        r = g.run(12, 0.0)
+        assert r["iters"] == ref["iters"] and np.array_equal(r["labels"], ref["labels"])
+        g.close()
