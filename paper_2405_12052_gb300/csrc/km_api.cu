@@ -113,7 +113,7 @@ struct km_ctx {
   int G0 = 0;
   // whole-run kernel (fused path)
   int run_state = 0;           // 0 not looked at yet, 1 in use, -1 not for this context (shape or memory)
-  int run_grid = 0, run_priv_sh = 0;
+  int run_grid = 0, run_priv_sh = 0, run_rep = 1;
   size_t run_smem = 0;
   float* slack = nullptr;
   uint8_t* zrun = nullptr;     // labels as bytes where the context keeps int32 labels
@@ -284,15 +284,18 @@ bool run_ready(km_ctx* c) {
   c->run_smem = sh ? base + priv : base;
   c->run_priv_sh = sh ? (int)base : 0;
   const int64_t ntiles = (c->n + kWarpTile - 1) / kWarpTile;
-  const int64_t g = std::min<int64_t>(ntiles, (int64_t)c->sms * b0);
+  // one block per SM while that leaves a warp at most four 256-point tiles,
+  // which it tests together: fewer blocks meet in the wait of each step
+  const int64_t g = ntiles <= (int64_t)c->sms * kWarps * 4 ? std::min<int64_t>(ntiles, c->sms) : (int64_t)c->sms * b0;
   const int64_t wtot = g * kWarps;
   if ((ntiles + wtot - 1) / wtot * kWarps * kWarpTile > kMaxPointsPerBlock) return false;
   c->run_grid = (int)g;
-  const size_t cols = (size_t)c->k * (c->d + 1);
+  c->run_rep = g > c->sms ? run_rep(c->d, c->k) : std::min(2, run_rep(c->d, c->k));
+  const size_t kd = (size_t)c->k * c->d;
   if (dalloc(&c->slack, (size_t)c->n) != cudaSuccess ||
       (!c->labels8 && dalloc(&c->zrun, (size_t)c->n) != cudaSuccess) ||
-      dalloc(&c->run_delta, run_delta_words(c->d, c->k)) != cudaSuccess ||
-      dalloc(&c->run_tot, (size_t)g * cols * 2) != cudaSuccess || dalloc(&c->run_tot0, cols * 2) != cudaSuccess ||
+      dalloc(&c->run_delta, run_delta_words(c->d, c->k, c->run_rep)) != cudaSuccess ||
+      dalloc(&c->run_tot, (size_t)g * kd * 4) != cudaSuccess || dalloc(&c->run_tot0, kd * 4) != cudaSuccess ||
       dalloc(&c->run_cum0, (size_t)c->k) != cudaSuccess ||
       (!sh && dalloc(&c->run_priv, (size_t)g * priv) != cudaSuccess)) {
     void* bufs[] = {c->slack, c->zrun, c->run_delta, c->run_tot, c->run_tot0, c->run_cum0, c->run_priv};
@@ -319,7 +322,7 @@ km_status run_whole(km_ctx* c) {
   r.z = c->labels8 ? c->labels8 : c->zrun;
   r.mu = c->mu; r.counts = c->counts;
   r.delta = c->run_delta;
-  r.bar = reinterpret_cast<unsigned int*>(c->run_delta + run_delta_words(c->d, c->k) - 1);
+  r.bar = reinterpret_cast<unsigned int*>(c->run_delta + run_delta_words(c->d, c->k, c->run_rep) - 1);
   r.tot = c->run_tot; r.tot0 = c->run_tot0; r.cum0 = c->run_cum0;
   r.priv = c->run_priv; r.priv_stride = run_priv_bytes(c->d, c->k); r.priv_sh = c->run_priv_sh;
   r.ctil_out = c->ctil4; r.ic_out = c->ic; r.tab_out = c->tab2;
@@ -327,7 +330,7 @@ km_status run_whole(km_ctx* c) {
   // FP64 distances are within 16 2^-53 relative of the exact ones; sqrt(D) <=
   // 2 sqrt(A_max) + 2^20 ulps of slack for centroids outside the data's range
   r.margin = (float)(1e-13 * (4.0 * std::sqrt((double)c->A_max) + 1e-20));
-  r.rep = run_rep(c->d, c->k);
+  r.rep = c->run_rep;
   r.steps = 64;
   // one pass over the points takes far less: K N evaluations at 1e11 a second
   r.wait_ns = 2000000000ull + (unsigned long long)((double)c->n * c->k * 0.01);

@@ -133,27 +133,6 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) assign_fast_kernel(FastArgs
 // memory have fixed bases (the layout of d = 3, K = 64), so instances of any
 // d follow one another without clearing: windows are zero after every flush.
 
-// Points of an instance are packed without padding, so the staging copies
-// are 4 bytes each (rows need not be 16-byte aligned); past N, zero-filled.
-template <int D>
-__device__ __forceinline__ void prefetch_tile_any(const FastArgs& a, float* xb, int64_t base, int lane) {
-#pragma unroll
-  for (int g = 0; g < kNG; ++g)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int off = g * kGS + 4 * lane + e;
-      const int64_t i = base + off;
-      const int bytes = i < a.n ? 4 : 0;
-#pragma unroll
-      for (int j = 0; j < D; ++j) {
-        const float* src = a.x + (int64_t)j * a.ld + (bytes ? i : 0);
-        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(xb + j * kWarpTile + off);
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes));
-      }
-    }
-  asm volatile("cp.async.commit_group;" ::: "memory");
-}
-
 constexpr int kBatchWinWords = 2 * (kBatchMaxK + 1) * 7;  // per warp: two windows of 65 bins of 7 words
 
 template <int D>

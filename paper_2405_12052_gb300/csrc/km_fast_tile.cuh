@@ -134,6 +134,8 @@ __device__ __forceinline__ float unpack_val(float w, const FastCtx& cx) {
   return __uint_as_float(__funnelshift_r(__float_as_uint(w), cx.ehi, LB > 0 ? LB : cx.L));
 }
 
+constexpr uint32_t kRecheck = 0x80000000u;  // whole-run queue entry that the screen has already flagged
+
 // What the whole-run kernel keeps per point besides the label: z and the
 // slack, a lower bound of sqrt(D2) - sqrt(D1) at the step that decided the
 // point plus the drift of its cluster up to that step (see km_run_fast.cu).
@@ -150,12 +152,18 @@ struct RunTile {
 // threshold T and A = ||x~||^2.  For every other centroid k the flag test's
 // bound gives D_k - D_1 >= dl = (v2 - v1 - T) 2^-sigma, and D_1 <= d1, so
 // sqrt(D_k) - sqrt(D_1) >= dl / (sqrt(d1 + dl) + sqrt(d1)) (decreasing in d1);
-// the factors cover the roundings here and of A.
+// the factors cover the roundings here (approximate roots and quotient, a few
+// ulps) and of A.
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
 __device__ __forceinline__ float screen_slack(float v1, float v2, float T, float A, float M, const RunTile& rt,
                                               int label) {
   const float dl = (v2 - v1 - T) * rt.invs * 0.9999f;
   const float d1 = fmaxf(fmaf(v1 - M + T, rt.invs, A * 1.0001f), 0.f) * 1.0001f + 1e-37f;
-  return __fadd_rd(dl * 0.9998f / (__fsqrt_rn(d1 + dl) + __fsqrt_rn(d1)) - rt.margin, rt.cum[label]);
+  return __fadd_rd(__fdividef(dl * 0.9998f, sqrt_approx(d1 + dl) + sqrt_approx(d1)) - rt.margin, rt.cum[label]);
 }
 
 // Screen of one group of 4 centroids (table rows tr) for this lane's 8
@@ -398,55 +406,58 @@ __device__ __forceinline__ void process_tile(const FastArgs& a, FastSmem<D>& sm,
     int at = qn + incl - nf;
     for (uint32_t fb = fbits; fb; fb &= fb - 1u) {
       const int p = __ffs(fb) - 1;
-      q[at++] = (uint32_t)(m << 8) | (uint32_t)((p >> 2) * kGS + 4 * lane + (p & 3));
+      q[at++] = (RUN ? kRecheck : 0u) | (uint32_t)(m << 8) | (uint32_t)((p >> 2) * kGS + 4 * lane + (p & 3));
     }
     qn += __shfl_sync(0xffffffffu, incl, 31);
   }
   if constexpr (RUN) {
+    const bool first = rt->first != 0;
 #pragma unroll
     for (int g = 0; g < kNG; ++g) {
       const int64_t i0 = base + g * kGS + 4 * lane;
-      // old labels of this lane's 4 points; the new word keeps a flagged point's
-      uint32_t ow = 0u;
-      if constexpr (FULL) ow = *reinterpret_cast<const uint32_t*>(rt->z + i0);
-      else {
+      // old labels of this lane's 4 points; the new word keeps a flagged
+      // point's (in the first step the queue writes it whatever it is)
+      uint32_t ow = 0u, nw = 0u;
+      if (!first) {
+        if constexpr (FULL) ow = *reinterpret_cast<const uint32_t*>(rt->z + i0);
+        else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) if (i0 + e < a.n) ow |= (uint32_t)rt->z[i0 + e] << (8 * e);
+          for (int e = 0; e < 4; ++e) if (i0 + e < a.n) ow |= (uint32_t)rt->z[i0 + e] << (8 * e);
+        }
       }
-      uint32_t nw = 0u;
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const int p = 4 * g + e;
-        const uint32_t old = (ow >> (8 * e)) & 255u;
-        const bool skip = (dbits >> p) & 1u;
-        const uint32_t kk = skip ? old : (uint32_t)lab[p];
-        nw |= kk << (8 * e);
-        if (!skip && (rt->first || kk != old)) {
-          uint32_t* wa = wmine + kk * WIN;
-          uint32_t* wo = wmine + old * WIN;
-          atomicAdd(&wa[0], 1u);
-          if (!rt->first) atomicSub(&wo[0], 1u);
-#pragma unroll
-          for (int j = 0; j < D; ++j) {
-            uint32_t bh, bl;
-            split_limbs(xcur[j * kWarpTile + g * kGS + 4 * lane + e], dup_lo(cx.chi2), dup_lo(cx.clo2), bh, bl);
-            atomicAdd(&wa[1 + j], bh);
-            atomicAdd(&wa[1 + D + j], bl);
-            if (!rt->first) {
-              atomicSub(&wo[1 + j], bh);
-              atomicSub(&wo[1 + D + j], bl);
-            }
-          }
-        }
+        nw |= (((dbits >> p) & 1u) ? ow & (255u << (8 * e)) : (uint32_t)lab[p] << (8 * e));
       }
       if constexpr (FULL) *reinterpret_cast<uint32_t*>(rt->z + i0) = nw;
       else {
 #pragma unroll
         for (int e = 0; e < 4; ++e) if (i0 + e < a.n) rt->z[i0 + e] = (uint8_t)(nw >> (8 * e));
       }
+      if (!first && nw != ow) {  // changed labels only (a flagged or padding point keeps its byte)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const uint32_t old = (ow >> (8 * e)) & 255u, now = (nw >> (8 * e)) & 255u;
+          if (now == old) continue;
+          uint32_t* wa = wmine + now * WIN;
+          uint32_t* wo = wmine + old * WIN;
+          atomicAdd(&wa[0], 1u);
+          atomicSub(&wo[0], 1u);
+#pragma unroll
+          for (int j = 0; j < D; ++j) {
+            uint32_t bh, bl;
+            split_limbs(xcur[j * kWarpTile + g * kGS + 4 * lane + e], dup_lo(cx.chi2), dup_lo(cx.clo2), bh, bl);
+            atomicAdd(&wa[1 + j], bh);
+            atomicAdd(&wa[1 + D + j], bl);
+            atomicSub(&wo[1 + j], bh);
+            atomicSub(&wo[1 + D + j], bl);
+          }
+        }
+      }
     }
-    return;
-  }
+    if (!first) return;
+  } else
   // labels (flagged points are overwritten by the re-check)
   if (a.store_labels) {
 #pragma unroll
@@ -570,6 +581,317 @@ __device__ __forceinline__ int screen_point(const float4* gtab, const FastCtx& c
   if (!(v2 - v1 > T) || lab >= cx.k) return -1;
   slack = screen_slack(v1, v2, T, A, cx.M, rt, lab);
   return lab;
+}
+
+// Points of an instance are packed without padding, so the staging copies
+// are 4 bytes each (rows need not be 16-byte aligned); past N, zero-filled.
+template <int D>
+__device__ __forceinline__ void prefetch_tile_any(const FastArgs& a, float* xb, int64_t base, int lane) {
+#pragma unroll
+  for (int g = 0; g < kNG; ++g)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int off = g * kGS + 4 * lane + e;
+      const int64_t i = base + off;
+      const int bytes = i < a.n ? 4 : 0;
+#pragma unroll
+      for (int j = 0; j < D; ++j) {
+        const float* src = a.x + (int64_t)j * a.ld + (bytes ? i : 0);
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(xb + j * kWarpTile + off);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes));
+      }
+    }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// A point's new label and slack; a changed label goes straight into the int64
+// totals (few points change).
+template <int D>
+__device__ __forceinline__ void run_commit(const RunTile& rt, long long* acc, const DataConst& dc, int64_t i,
+                                           const float (&xo)[D], int kk, int old, float sl) {
+  constexpr int DP = D + 1;
+  rt.slack[i] = sl;
+  if (rt.first || kk != old) {
+    rt.z[i] = (uint8_t)kk;
+    unsigned long long* ta = reinterpret_cast<unsigned long long*>(acc + kk * DP);
+    unsigned long long* to = reinterpret_cast<unsigned long long*>(acc + old * DP);
+    atomicAdd(ta + D, 1ull);
+    if (!rt.first) atomicAdd(to + D, ~0ull);
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+      uint32_t bh, bl;
+      split_limbs(xo[j], dc.C_hi, dc.C_lo, bh, bl);
+      const long long v = ((long long)(int)(bh - dc.bits_C_hi) << 22) + (long long)(int)(bl - dc.bits_C_lo);
+      atomicAdd(ta + j, (unsigned long long)v);
+      if (!rt.first) atomicAdd(to + j, (unsigned long long)(-v));
+    }
+  }
+}
+
+// Re-check of nr queued points, one per lane.  Not inlined: few points come
+// here, and the kernels' instructions should stay in the SM's cache.
+template <int D>
+__device__ __noinline__ int run_recheck(const float* x, int64_t ld, const float4* ctil, const double* mu, int k,
+                                        const uint32_t* q, int nr, int64_t wid, int wtot, long long* acc, DataConst dc,
+                                        float B_max, float tau, RunTile rt) {
+  int n64 = 0;
+  for (int e = threadIdx.x & 31; e < nr; e += 32) {
+    const uint32_t loc = q[e];
+    const int64_t i = (wid + (int64_t)((loc & ~kRecheck) >> 8) * wtot) * kWarpTile + (loc & 255u);
+    float xo[D];
+#pragma unroll
+    for (int j = 0; j < D; ++j) xo[j] = x[(int64_t)j * ld + i];
+    const int old = rt.z[i];
+    bool used64;
+    float sl;
+    const int kk = recheck_fast<D>(xo, dc.s, ctil, mu, k, B_max, tau, used64, &sl);
+    n64 += used64 ? 1 : 0;
+    sl = used64 ? -1.f : __fadd_rd(sl - rt.margin, rt.cum[kk]);
+    run_commit<D>(rt, acc, dc, i, xo, kk, old, sl);
+  }
+  return n64;
+}
+
+// Decide the queued points one per lane: by the screen, and the ones it flags
+// (with kRecheck set, or all in the first step: flagged before) by the
+// re-check.  The open points of a tile lie near cluster borders, where the
+// screen flags some of nearly every 32, and the re-check takes three times the
+// screen's instructions: so flagged points are gathered at the front of the
+// queue and re-checked side by side afterwards.
+template <int D, int KG>
+__device__ __forceinline__ void run_drain(const FastArgs& a, const float4* gtab, const FastCtx& cx, const float4* ctil,
+                                          const double* mu, uint32_t* q, int qn, int wid, int wtot, long long* acc,
+                                          int lane, const float* s, const DataConst& dc, float B_max,
+                                          const RunTile& rt, int& n64) {
+  __syncwarp();
+  int nr = 0;
+  for (int b = 0; b < qn; b += 32) {
+    const bool live = b + lane < qn;
+    const uint32_t loc = live ? q[b + lane] : 0u;
+    bool rec = live && (loc & kRecheck);
+    if (live && !rec) {
+      const int64_t i = ((int64_t)wid + (int64_t)(loc >> 8) * wtot) * kWarpTile + (loc & 255u);
+      float xo[D];
+#pragma unroll
+      for (int j = 0; j < D; ++j) xo[j] = a.x[(int64_t)j * a.ld + i];
+      const int old = rt.z[i];
+      float sl;
+      const int kk = screen_point<D, KG>(gtab, cx, s, xo, rt, sl);
+      if (kk < 0) rec = true;
+      else run_commit<D>(rt, acc, dc, i, xo, kk, old, sl);
+    }
+    const unsigned bal = __ballot_sync(0xffffffffu, rec);  // every lane holds its entry: the front may be written
+    if (rec) q[nr + __popc(bal & ((1u << lane) - 1u))] = loc;
+    nr += __popc(bal);
+  }
+  __syncwarp();
+  if (nr > 0) n64 += run_recheck<D>(a.x, a.ld, ctil, mu, a.k, q, nr, wid, wtot, acc, dc, B_max, cx.tau, rt);
+  __syncwarp();
+}
+
+// Open points of a 256-point tile: above kHeavy it is screened whole; above
+// kStage its points are copied to shared memory (3 KB in whole lines, where
+// gathering 12 bytes a point takes three 64-byte accesses) and the open ones
+// decided from there; below, they are queued across tiles and gathered.
+constexpr int kHeavy = 96, kStage = 16;
+constexpr int kQueueFull = kWarpQueue - 128;  // entries from which the queue is emptied (a tile adds at most kHeavy)
+
+// One warp's part of a step that skips points (see km_run_fast.cu): warp-tiles
+// wid, wid + wtot, ... below end of the points a.x (a.n of them).  Adds the
+// changes to acc (int64, k x (D + 1)); nflag and n64 count the points decided
+// again and those decided in FP64.  ANY: rows without 16-byte alignment.
+// Tiles are tested four at a time, their slacks and labels (5 KB a warp)
+// loaded together: 1e8 points that keep their labels took 150 us a step with
+// one tile loaded ahead, 97 us with four.
+template <int D, int KG, bool ANY>
+__device__ __forceinline__ void run_pass(const FastArgs& a, FastSmem<D>& sm, const FastCtx& cx,
+                                         const unsigned long long* s2, const float* s, const DataConst& dc,
+                                         const RunTile& rt, const float4* ctil, const double* mu, float B_max,
+                                         long long* acc, uint32_t* q, uint32_t* wwarp, uint32_t* wmine, float* xb,
+                                         int nbuf, int wid, int wtot, int end, int lane, int& nflag, int& n64) {
+  const int nwin = a.nwin;
+  int qn = 0, since_flush = 0, m = 0, tile = wid;
+  auto fetch = [&](float* dst, int t) {
+    if constexpr (ANY) prefetch_tile_any<D>(a, dst, (int64_t)t * kWarpTile, lane);
+    else prefetch_tile<D>(a, dst, (int64_t)t * kWarpTile, lane);
+  };
+  auto whole = [&](int t, int mt, const float* xcur) {
+    const int64_t base = (int64_t)t * kWarpTile;
+    if (base + kWarpTile <= a.n)
+      process_tile<D, KG, false, true, true>(a, sm, cx, s2, xcur, base, mt, lane, wmine, q, qn, &rt);
+    else
+      process_tile<D, KG, false, false, true>(a, sm, cx, s2, xcur, base, mt, lane, wmine, q, qn, &rt);
+    // at most 512 additions and 512 subtractions per bin between flushes
+    if (++since_flush == (nwin == 4 ? 8 : nwin == 2 ? 4 : 2)) {
+      flush_windows<D>(wwarp, acc, a.k, nwin, lane, dc.bits_C_hi, dc.bits_C_lo);
+      since_flush = 0;
+    }
+  };
+  if (rt.first) {
+    // every point; the queue holds the flagged ones
+    auto recheck = [&]() {
+      __syncwarp();
+      n64 += run_recheck<D>(a.x, a.ld, ctil, mu, a.k, q, qn, wid, wtot, acc, dc, B_max, cx.tau, rt);
+      __syncwarp();
+      nflag += qn;
+      qn = 0;
+    };
+    if (tile < end) fetch(xb, tile);
+    for (; tile < end; tile += wtot, ++m) {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      // each lane reads only the chunks it copied itself
+      if (nbuf == 2 && tile + wtot < end) fetch(xb + ((m + 1) & 1) * D * kWarpTile, tile + wtot);
+      whole(tile, m, xb + (nbuf == 2 ? (m & 1) : 0) * D * kWarpTile);
+      if (nbuf == 1 && tile + wtot < end) fetch(xb, tile + wtot);
+      if (qn > kWarpQueue - kWarpTile || (qn > 0 && tile + wtot >= end)) recheck();
+    }
+  } else {
+    // batches of four tiles; u: the next of the current batch's tiles with
+    // more than kStage open points (4: none left)
+    uint32_t open = 0u;       // this lane's open points of such tiles: 8 bits per tile
+    uint32_t n01 = 0u, n23 = 0u;  // open points of the batch's tiles, 16 bits each
+    int u = 4, tb = 0, mb = 0;
+    while (true) {
+      if (u == 4 && tile < end) {
+        open = 0u;
+        {
+          float4 sv[4][2];
+          uint32_t zv[4][2];
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            const int t = tile + v * wtot;
+            const int64_t base = (int64_t)t * kWarpTile;
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+              const int64_t i0 = base + g * kGS + 4 * lane;
+              sv[v][g] = make_float4(3.0e38f, 3.0e38f, 3.0e38f, 3.0e38f);  // past the end: never open
+              zv[v][g] = 0u;
+              if (t < end) {
+                if (base + kWarpTile <= a.n) {
+                  sv[v][g] = *reinterpret_cast<const float4*>(rt.slack + i0);
+                  zv[v][g] = *reinterpret_cast<const uint32_t*>(rt.z + i0);
+                } else {
+                  float* sp = reinterpret_cast<float*>(&sv[v][g]);
+#pragma unroll
+                  for (int e = 0; e < 4; ++e)
+                    if (i0 + e < a.n) {
+                      sp[e] = rt.slack[i0 + e];
+                      zv[v][g] |= (uint32_t)rt.z[i0 + e] << (8 * e);
+                    }
+                }
+              }
+            }
+          }
+#pragma unroll
+          for (int v = 0; v < 4; ++v)
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+              const float sp[4] = {sv[v][g].x, sv[v][g].y, sv[v][g].z, sv[v][g].w};
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                open |= (sp[e] > rt.cum[(zv[v][g] >> (8 * e)) & 255u] ? 0u : 1u) << (8 * v + 4 * g + e);
+            }
+        }
+        tb = tile;
+        mb = m;
+        tile += 4 * wtot;
+        m += 4;
+        if (__any_sync(0xffffffffu, open != 0u)) {
+          n01 = __reduce_add_sync(0xffffffffu, (unsigned)__popc(open & 0xffu) | (unsigned)__popc(open & 0xff00u) << 16);
+          n23 = __reduce_add_sync(0xffffffffu,
+                                  (unsigned)__popc(open & 0xff0000u) | (unsigned)__popc(open & 0xff000000u) << 16);
+          // the tiles with few open points, all four at once, into the queue
+          uint32_t few = 0u, nfew = 0u;
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            const uint32_t nv = ((v < 2 ? n01 : n23) >> (16 * (v & 1))) & 0xffffu;
+            if (nv <= kStage) { few |= 0xffu << (8 * v); nfew += nv; }
+            else u = min(u, v);
+          }
+          few &= open;
+          open &= ~few;
+          if (nfew) {  // at most 4 kStage: the queue has room (kQueueFull)
+            const int nf = __popc(few);
+            int incl = nf;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+              const int t = __shfl_up_sync(0xffffffffu, incl, o);
+              if (lane >= o) incl += t;
+            }
+            int at = qn + incl - nf;
+            for (; few; few &= few - 1u) {
+              const int p = __ffs((int)few) - 1;
+              q[at++] = (uint32_t)((mb + (p >> 3)) << 8) | (uint32_t)(((p >> 2) & 1) * kGS + 4 * lane + (p & 3));
+            }
+            qn += (int)nfew;
+          }
+        }
+      }
+      for (; u < 4; ++u) {
+        const int total = (int)(((u < 2 ? n01 : n23) >> (16 * (u & 1))) & 0xffffu);
+        if (total <= kStage) continue;
+        const int t = tb + u * wtot;
+        if (total > kHeavy) {
+          if (qn > kWarpQueue - kWarpTile) break;  // empty the queue first
+          fetch(xb, t);
+          asm volatile("cp.async.wait_group 0;" ::: "memory");
+          whole(t, mb + u, xb);
+          nflag += total;
+        } else {
+          if (qn > kQueueFull) break;
+          fetch(xb, t);
+          uint32_t fb = (open >> (8 * u)) & 255u;
+          const int nf = __popc(fb);
+          int incl = nf;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+          }
+          int at = qn + incl - nf;
+          for (; fb; fb &= fb - 1u) {
+            const int p = __ffs((int)fb) - 1;
+            q[at++] = (uint32_t)((mb + u) << 8) | (uint32_t)((p >> 2) * kGS + 4 * lane + (p & 3));
+          }
+          asm volatile("cp.async.wait_group 0;" ::: "memory");
+          __syncwarp();  // every lane's copies and queue entries
+          int nr = qn;
+          for (int b = qn; b < qn + total; b += 32) {
+            const bool live = b + lane < qn + total;
+            const uint32_t loc = live ? q[b + lane] : 0u;
+            bool rec = false;
+            if (live) {
+              const int off = (int)(loc & 255u);
+              const int64_t i = (int64_t)t * kWarpTile + off;
+              float xo[D];
+#pragma unroll
+              for (int j = 0; j < D; ++j) xo[j] = xb[j * kWarpTile + off];
+              const int old = rt.z[i];
+              float sl;
+              const int kk = screen_point<D, KG>(sm.gtab, cx, s, xo, rt, sl);
+              if (kk < 0) rec = true;
+              else run_commit<D>(rt, acc, dc, i, xo, kk, old, sl);
+            }
+            const unsigned bal = __ballot_sync(0xffffffffu, rec);
+            if (rec) q[nr + __popc(bal & ((1u << lane) - 1u))] = loc | kRecheck;
+            nr += __popc(bal);
+          }
+          nflag += total - (nr - qn);
+          qn = nr;
+          __syncwarp();  // the points are read no more
+        }
+      }
+      const bool last = u == 4 && tile >= end;
+      if (qn > 0 && (u < 4 || qn > kQueueFull || last)) {
+        run_drain<D, KG>(a, sm.gtab, cx, ctil, mu, q, qn, wid, wtot, acc, lane, s, dc, B_max, rt, n64);
+        nflag += qn;
+        qn = 0;
+      }
+      if (last) break;
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  if (since_flush) flush_windows<D>(wwarp, acc, a.k, nwin, lane, dc.bits_C_hi, dc.bits_C_lo);
 }
 
 }  // namespace

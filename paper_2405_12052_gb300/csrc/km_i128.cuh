@@ -1,5 +1,6 @@
-// 128-bit integer sums of the mean calculation: two's complement in a low and
-// a high 64-bit word, and the correctly rounded conversion to FP64.
+// Arithmetic of the mean calculation: 128-bit integer sums (two's complement in
+// a low and a high 64-bit word), their correctly rounded conversion to FP64,
+// and an upward-rounded root for the centroids' moves.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -38,6 +39,16 @@ __device__ __forceinline__ void add128p(unsigned long long& lo, long long& hi, u
   unsigned long long nl = lo + vl;
   hi += vh + (nl < lo ? 1ll : 0ll);
   lo = nl;
+}
+
+// sqrt(t), rounded up, for t >= 0: the FP32 root of t's significand and half
+// its exponent (an FP64 root is a long chain); at least 2^-120.
+__device__ __forceinline__ float sqrt_up(double t) {
+  if (!(t > 0.0)) return 0.f;
+  const int hi = __double2hiint(t), e = ((hi >> 20) - 1023) & ~1;
+  if (e < -240) return 0x1p-120f;
+  const float m = __double2float_ru(__hiloint2double(hi - (e << 20), __double2loint(t)));
+  return __fmul_ru(__fsqrt_ru(m), e > 252 ? __uint_as_float(0x7f800000u) : __uint_as_float((uint32_t)(127 + e / 2) << 23));
 }
 
 }  // namespace

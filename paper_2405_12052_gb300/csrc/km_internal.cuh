@@ -130,8 +130,8 @@ struct RunArgs {
   unsigned long long* delta;   // [3][rep][k (d + 1) + 2][2] changes of the column totals, flagged, FP64-decided; then
   unsigned int* bar;           // the arrival counter (cleared together)
   int rep;                     // copies of the table of changes
-  long long* tot;              // [grid][k (d + 1)][2] each block's running totals
-  long long* tot0;             // [k (d + 1)][2], [k]: totals and drift sums between launches
+  long long* tot;              // [grid][k d][4] each block's running totals (low, high word, the cluster's count)
+  long long* tot0;             // [k d][4], [k]: totals and drift sums between launches
   float* cum0;
   unsigned char* priv;         // per-block values in global memory, priv_stride bytes each
   size_t priv_stride;
@@ -145,7 +145,7 @@ struct RunArgs {
 };
 // words of delta including the arrival counter
 int run_rep(int d, int k);
-inline size_t run_delta_words(int d, int k) { return (size_t)3 * run_rep(d, k) * ((size_t)k * (d + 1) + 2) * 2 + 1; }
+inline size_t run_delta_words(int d, int k, int rep) { return (size_t)3 * rep * ((size_t)k * (d + 1) + 2) * 2 + 1; }
 size_t run_priv_bytes(int d, int k);
 int run_blocks_per_sm(int d, int kpad, size_t smem);
 cudaError_t launch_run_fast(int d, int grid, size_t smem, cudaStream_t st, const RunArgs& a);

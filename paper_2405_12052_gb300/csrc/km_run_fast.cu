@@ -32,7 +32,8 @@
 // 5 bytes a point (0.5 GB for 1e8 points: 75 us at the memory's rate).
 //
 // A 256-point warp-tile with more than kHeavy open points goes through the
-// fused kernel's screen whole; fewer are listed and decided one per lane.
+// fused kernel's screen whole; fewer are listed and decided one per lane
+// (run_pass in km_fast_tile.cuh, shared with the batched runs).
 #include <algorithm>
 
 #include "km_fast_tile.cuh"
@@ -43,22 +44,10 @@ namespace km {
 
 namespace {
 
-constexpr int kHeavy = 128;  // open points of a 256-point tile above which it is screened whole
-
 __device__ __forceinline__ unsigned long long run_clock() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
   return t;
-}
-
-// sqrt(t), rounded up, for t >= 0: the FP32 root of t's significand and half
-// its exponent (an FP64 root is a long chain); at least 2^-120.
-__device__ __forceinline__ float sqrt_up(double t) {
-  if (!(t > 0.0)) return 0.f;
-  const int hi = __double2hiint(t), e = ((hi >> 20) - 1023) & ~1;
-  if (e < -240) return 0x1p-120f;
-  const float m = __double2float_ru(__hiloint2double(hi - (e << 20), __double2loint(t)));
-  return __fmul_ru(__fsqrt_ru(m), e > 252 ? __uint_as_float(0x7f800000u) : __uint_as_float((uint32_t)(127 + e / 2) << 23));
 }
 
 // All blocks have arrived `target` times in all (monotone counter, one block's
@@ -84,51 +73,6 @@ __device__ bool grid_wait(unsigned int* bar, unsigned int target, unsigned long 
   return s_ok != 0;
 }
 
-// Decide the queued points one per lane: by the screen, or by the re-check
-// where that flags the point (in the first step only points that it flagged
-// are queued).  Few of them change clusters, so a change goes straight into
-// the block's int64 totals.
-template <int D, int KG>
-__device__ void run_drain(const FastArgs& a, const float4* gtab, const FastCtx& cx, const float4* ctil,
-                          const double* mu, const uint32_t* q, int qn, int wid, int wtot, long long* acc, int lane,
-                          const float* s, const DataConst& dc, float B_max, const RunTile& rt, int& n64) {
-  constexpr int DP = D + 1;
-  __syncwarp();
-  for (int e = lane; e < qn; e += 32) {
-    const uint32_t loc = q[e];
-    const int64_t i = ((int64_t)wid + (int64_t)(loc >> 8) * wtot) * kWarpTile + (loc & 255u);
-    float xo[D];
-#pragma unroll
-    for (int j = 0; j < D; ++j) xo[j] = a.x[(int64_t)j * a.ld + i];
-    const int old = rt.z[i];
-    float sl;
-    int kk = rt.first ? -1 : screen_point<D, KG>(gtab, cx, s, xo, rt, sl);
-    if (kk < 0) {
-      bool used64;
-      kk = recheck_fast<D>(xo, s, ctil, mu, a.k, B_max, cx.tau, used64, &sl);
-      n64 += used64 ? 1 : 0;
-      sl = used64 ? -1.f : __fadd_rd(sl - rt.margin, rt.cum[kk]);
-    }
-    rt.slack[i] = sl;
-    if (rt.first || kk != old) {
-      rt.z[i] = (uint8_t)kk;
-      unsigned long long* ta = reinterpret_cast<unsigned long long*>(acc + kk * DP);
-      unsigned long long* to = reinterpret_cast<unsigned long long*>(acc + old * DP);
-      atomicAdd(ta + D, 1ull);
-      if (!rt.first) atomicAdd(to + D, ~0ull);
-#pragma unroll
-      for (int j = 0; j < D; ++j) {
-        uint32_t bh, bl;
-        split_limbs(xo[j], dc.C_hi, dc.C_lo, bh, bl);
-        const long long v = ((long long)(int)(bh - dc.bits_C_hi) << 22) + (long long)(int)(bl - dc.bits_C_lo);
-        atomicAdd(ta + j, (unsigned long long)v);
-        if (!rt.first) atomicAdd(to + j, (unsigned long long)(-v));
-      }
-    }
-  }
-  __syncwarp();
-}
-
 // The block's own values: centroids, drift sums and tables (in shared memory
 // when they fit beside the fused kernel's layout without costing a resident
 // block, else in the block's slice of global memory).
@@ -150,6 +94,7 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
   constexpr int DP = D + 1, WIN = 2 * D + 1, GS = FastSmem<D>::GS;
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ IterConst s_ic;
+  __shared__ double s_e2;
   __shared__ int s_empty;
   const FastArgs& a = ra.f;
   if (a.ls->done) return;  // written by block 0 only behind a wait for every block
@@ -159,12 +104,12 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
   const int k = a.k, kpad = KG > 0 ? 4 * KG : a.kpad, nwin = a.nwin;
   const int cols = k * DP;
   RunPriv pv(ra.priv_sh ? smraw + ra.priv_sh : ra.priv + (size_t)blockIdx.x * ra.priv_stride, k, D);
-  long long* tot = ra.tot + (size_t)blockIdx.x * cols * 2;  // running totals: low word, high word
+  // running totals of (cluster, coordinate): low word, high word, the cluster's count, unused
+  long long* tot = ra.tot + (size_t)blockIdx.x * k * D * 4;
   // between the passes the point buffers hold the update's values
   double* s_df2 = reinterpret_cast<double*>(sm.xbuf);  // [k][D] squared moves
   double* sB = s_df2 + (size_t)k * D;                  // [k]
   double* s_red = sB + k;                              // [256]
-  long long* s_cnt = reinterpret_cast<long long*>(s_red + kThreads);  // [k]
 
   const DataConst dc = *a.dc;
   float s[D];
@@ -187,7 +132,7 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
 
   for (int c = tid; c < k * D; c += kThreads) pv.mu[c] = ra.mu[c];
   for (int c = tid; c < k; c += kThreads) pv.cum[c] = ra.resume ? ra.cum0[c] : 0.f;
-  for (int c = tid; c < 2 * cols; c += kThreads) tot[c] = ra.resume ? ra.tot0[c] : 0;
+  for (int c = tid; c < 4 * k * D; c += kThreads) tot[c] = ra.resume ? ra.tot0[c] : 0;
   for (int c = tid; c < cols; c += kThreads) acc[c] = 0;
   for (int c = tid; c < kWarps * nwin * (k + 1) * WIN; c += kThreads) sm.win[c] = 0u;
   if (tid < 2) sm.cnt[tid] = 0;
@@ -217,110 +162,9 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
     rt.slack = ra.slack; rt.z = ra.z; rt.cum = pv.cum; rt.margin = ra.margin;
     rt.first = !ra.resume && step == 0;
     const float B_max = s_ic.B_max;
-    int qn = 0, nflag = 0, n64 = 0, since_flush = 0, m = 0, tile = wid;
-    auto whole = [&](int64_t base, const float* xcur) {
-      if (base + kWarpTile <= a.n)
-        process_tile<D, KG, false, true, true>(a, sm, cx, s2, xcur, base, m, lane, wmine, q, qn, &rt);
-      else
-        process_tile<D, KG, false, false, true>(a, sm, cx, s2, xcur, base, m, lane, wmine, q, qn, &rt);
-      // at most 512 additions and 512 subtractions per bin between flushes
-      if (++since_flush == (nwin == 4 ? 8 : nwin == 2 ? 4 : 2)) {
-        flush_windows<D>(wwarp, acc, k, nwin, lane, dc.bits_C_hi, dc.bits_C_lo);
-        since_flush = 0;
-      }
-    };
-    auto drain = [&]() {
-      run_drain<D, KG>(a, sm.gtab, cx, pv.ctil, pv.mu, q, qn, wid, wtot, acc, lane, s, dc, B_max, rt, n64);
-      nflag += qn;
-      qn = 0;
-    };
-    // slack and labels of this lane's 8 points of a tile; points past N never open
-    auto load = [&](int t, float (&sl)[8], uint32_t (&zw)[2]) {
-      const int64_t base = (int64_t)t * kWarpTile;
-#pragma unroll
-      for (int g = 0; g < 2; ++g) {
-        const int64_t i0 = base + g * kGS + 4 * lane;
-        if (base + kWarpTile <= a.n) {
-          const float4 v = *reinterpret_cast<const float4*>(ra.slack + i0);
-          sl[4 * g] = v.x; sl[4 * g + 1] = v.y; sl[4 * g + 2] = v.z; sl[4 * g + 3] = v.w;
-          zw[g] = *reinterpret_cast<const uint32_t*>(ra.z + i0);
-        } else {
-          zw[g] = 0u;
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            sl[4 * g + e] = i0 + e < a.n ? ra.slack[i0 + e] : 3.0e38f;
-            if (i0 + e < a.n) zw[g] |= (uint32_t)ra.z[i0 + e] << (8 * e);
-          }
-        }
-      }
-    };
-    if (rt.first) {
-      if (tile < ntiles) prefetch_tile<D>(a, xb, (int64_t)tile * kWarpTile, lane);
-      for (; tile < ntiles; tile += wtot, ++m) {
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        // each lane reads only the chunks it copied itself
-        if (nbuf == 2 && tile + wtot < ntiles)
-          prefetch_tile<D>(a, xb + ((m + 1) & 1) * D * kWarpTile, (int64_t)(tile + wtot) * kWarpTile, lane);
-        whole((int64_t)tile * kWarpTile, xb + (nbuf == 2 ? (m & 1) : 0) * D * kWarpTile);
-        if (nbuf == 1 && tile + wtot < ntiles) prefetch_tile<D>(a, xb, (int64_t)(tile + wtot) * kWarpTile, lane);
-        if (qn > kWarpQueue - kWarpTile) drain();
-      }
-    } else {
-      while (tile < ntiles) {
-        // test tiles until one is to be screened whole or the queue is full
-        // enough; the next tile's values are loaded while this one is tested
-        bool heavy = false;
-        float sl[8], sn[8];
-        uint32_t zw[2], zn[2];
-        load(tile, sl, zw);
-        while (true) {
-          const int nt = tile + wtot;
-          if (nt < ntiles) load(nt, sn, zn);
-          uint32_t fb = 0u;
-#pragma unroll
-          for (int p = 0; p < 8; ++p) {
-            const uint32_t zz = (zw[p >> 2] >> (8 * (p & 3))) & 255u;
-            fb |= (sl[p] > pv.cum[zz] ? 0u : 1u) << p;
-          }
-          if (__any_sync(0xffffffffu, fb != 0u)) {
-            const int nf = __popc(fb);
-            int incl = nf;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-              const int t = __shfl_up_sync(0xffffffffu, incl, o);
-              if (lane >= o) incl += t;
-            }
-            const int total = __shfl_sync(0xffffffffu, incl, 31);
-            if (total > kHeavy) { heavy = true; break; }
-            int at = qn + incl - nf;
-            for (; fb; fb &= fb - 1u) {
-              const int p = __ffs(fb) - 1;
-              q[at++] = (uint32_t)(m << 8) | (uint32_t)((p >> 2) * kGS + 4 * lane + (p & 3));
-            }
-            qn += total;
-          }
-          tile = nt;
-          ++m;
-          if (tile >= ntiles || qn > kWarpQueue - kWarpTile) break;
-#pragma unroll
-          for (int p = 0; p < 8; ++p) sl[p] = sn[p];
-          zw[0] = zn[0];
-          zw[1] = zn[1];
-        }
-        if (heavy) {
-          const int64_t base = (int64_t)tile * kWarpTile;
-          prefetch_tile<D>(a, xb, base, lane);
-          asm volatile("cp.async.wait_group 0;" ::: "memory");
-          whole(base, xb);
-          tile += wtot;
-          ++m;
-        }
-        if (qn > kWarpQueue - kWarpTile) drain();
-      }
-    }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    if (qn > 0) drain();
-    if (since_flush) flush_windows<D>(wwarp, acc, k, nwin, lane, dc.bits_C_hi, dc.bits_C_lo);
+    int nflag = 0, n64 = 0;
+    run_pass<D, KG, false>(a, sm, cx, s2, s, dc, rt, pv.ctil, pv.mu, B_max, acc, q, wwarp, wmine, xb, nbuf, wid, wtot,
+                           ntiles, lane, nflag, n64);
     if (lane == 0 && nflag) atomicAdd(&sm.cnt[0], nflag);
     if (n64) atomicAdd(&sm.cnt[1], n64);
     __syncthreads();
@@ -353,9 +197,9 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
     // this step's table was the one before last's; the last step's is read
     // by no block any more (all have arrived) and is added to again only after
     // the next wait: clear it
-    if (blockIdx.x == 0) {
+    {
       unsigned long long* old = ra.delta + (size_t)((step + 2) % 3) * ra.rep * words;
-      for (int c = tid; c < ra.rep * words; c += kThreads) old[c] = 0ull;
+      for (int c = blockIdx.x * kThreads + tid; c < ra.rep * words; c += gridDim.x * kThreads) old[c] = 0ull;
     }
     // sum over the copies of the table's entry w: low and high words
     auto entry = [&](int w, long long& lo, long long& hi) {
@@ -368,39 +212,25 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
         hi += v.y;
       }
     };
-    // a thread's first column total is on its way while the counts are added
-    long long plo = 0, phi = 0;
-    ulonglong2 ptot = make_ulonglong2(0ull, 0ull);
-    if (tid < k * D) {
-      const int w = 2 * (tid / D * DP + tid % D);
-      entry(w, plo, phi);
-      ptot = *reinterpret_cast<const ulonglong2*>(tot + w);
-    }
-    int empty = 0;
-    for (int c = tid; c < k; c += kThreads) {
-      const int w = 2 * (c * DP + D);
-      long long lo, hi;
-      entry(w, lo, hi);
-      const long long nn = tot[w] + lo + (hi << 54);
-      tot[w] = nn;
-      s_cnt[c] = nn;
-      empty += nn == 0;
-    }
-    __syncthreads();
+    // centroids: a thread per (cluster, coordinate) keeps that column's running
+    // total and its own copy of the cluster's count, so one round of loads and
+    // one barrier do
     double e2p = 0.0;
+    int empty = 0;
     for (int qd = tid; qd < k * D; qd += kThreads) {
-      const int c = qd / D, j = qd - c * D, w = 2 * (c * DP + j);
-      if (qd != tid) {
-        entry(w, plo, phi);
-        ptot = *reinterpret_cast<const ulonglong2*>(tot + w);
-      }
-      unsigned long long tl = ptot.x;
-      long long th = (long long)ptot.y;
+      const int c = qd / D, j = qd - c * D;
+      long long plo, phi, clo, chi;
+      entry(2 * (c * DP + j), plo, phi);
+      entry(2 * (c * DP + D), clo, chi);
+      const ulonglong2 pt = *reinterpret_cast<const ulonglong2*>(tot + 4 * qd);
+      const long long nn = tot[4 * qd + 2] + clo + (chi << 54);
+      const double old = pv.mu[qd];
+      unsigned long long tl = pt.x;
+      long long th = (long long)pt.y;
       add128p(tl, th, (unsigned long long)phi << 54, phi >> 10);
       add128p(tl, th, (unsigned long long)plo, plo >> 63);
-      *reinterpret_cast<ulonglong2*>(tot + w) = make_ulonglong2(tl, (unsigned long long)th);
-      const long long nn = s_cnt[c];
-      const double old = pv.mu[qd];
+      *reinterpret_cast<ulonglong2*>(tot + 4 * qd) = make_ulonglong2(tl, (unsigned long long)th);
+      tot[4 * qd + 2] = nn;
       double nw = old;
       // 2^G0 is a normal number and the product exact, as the update kernel's ldexp
       if (nn > 0) nw = __ddiv_rn(i128_to_double((long long)tl, th) * grid_unit, (double)nn);
@@ -409,12 +239,13 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
       e2p = __dadd_rn(e2p, dd);
       s_df2[qd] = dd;
       pv.mu[qd] = nw;
+      empty += j == 0 && nn == 0;
     }
-    // E^2 by the update kernel's tree over 256 threads (levels that only add
-    // zeros left out)
     s_red[tid] = e2p;
     if (empty) atomicAdd(&s_empty, empty);
     __syncthreads();
+    // E^2 by the update kernel's tree over 256 threads (levels that only add
+    // zeros left out)
 #pragma unroll
     for (int w = kThreads / 2; w >= 32; w >>= 1) {
       if (k * D <= w) continue;
@@ -425,23 +256,19 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
       double t = s_red[tid];
 #pragma unroll
       for (int w = 16; w > 0; w >>= 1) t = __dadd_rn(t, __shfl_down_sync(0xffffffffu, t, w));
-      if (tid == 0) s_red[0] = t;
+      if (tid == 0) s_e2 = t;
     }
-    // moves per centroid, rounded up
-    float* s_mv = reinterpret_cast<float*>(sB);
-    for (int c = tid; c < k; c += kThreads) {
-      double t = 0.0;
-#pragma unroll
-      for (int j = 0; j < D; ++j) t = __dadd_ru(t, s_df2[c * D + j]);
-      s_mv[c] = sqrt_up(t);
-    }
-    __syncthreads();
     {
-      // the largest move, its centroid, and the second largest (every warp)
-      float m1 = -1.f, m2 = -1.f;
+      // every warp forms the centroids' moves, rounded up, the largest with its
+      // centroid and the second largest; thread c keeps centroid c's
+      float m1 = -1.f, m2 = -1.f, mine = 0.f;
       int i1 = -1;
       for (int c = lane; c < k; c += 32) {
-        const float v = s_mv[c];
+        double t = 0.0;
+#pragma unroll
+        for (int j = 0; j < D; ++j) t = __dadd_ru(t, s_df2[c * D + j]);
+        const float v = sqrt_up(t);
+        if (c == tid) mine = v;
         if (v > m1) { m2 = m1; m1 = v; i1 = c; }
         else if (v > m2) m2 = v;
       }
@@ -453,10 +280,10 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
         else m2 = fmaxf(m2, p1);
       }
       m2 = fmaxf(m2, 0.f);
-      for (int c = tid; c < k; c += kThreads)
-        pv.cum[c] = __fadd_ru(pv.cum[c], __fadd_ru(s_mv[c], c == i1 ? m2 : m1));
+      if (tid < k) pv.cum[tid] = __fadd_ru(pv.cum[tid], __fadd_ru(mine, tid == i1 ? m2 : m1));  // k <= 256 threads
     }
-    const double E2 = s_red[0];
+    tables();  // its barriers also publish s_e2 and the drift sums
+    const double E2 = s_e2;
     const int iter = iter0 + step + 1;
     // sqrt(E2) < tol; the root itself only where E2 is not clearly above tol^2
     const bool conv = e_mode == 1 ? E2 < tol : !(tol <= 0.0) && E2 <= tol * tol * 1.001 + 1e-300 && sqrt(E2) < tol;
@@ -464,10 +291,12 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
     if (done || step + 1 == ra.steps) {
       // block 0 leaves the state of a stopped (or paused) loop
       if (blockIdx.x != 0) return;
-      __syncthreads();
-      for (int c = tid; c < k * D; c += kThreads) ra.mu[c] = pv.mu[c];
-      for (int c = tid; c < k; c += kThreads) { ra.counts[c] = s_cnt[c]; ra.cum0[c] = pv.cum[c]; }
-      for (int c = tid; c < 2 * cols; c += kThreads) ra.tot0[c] = tot[c];
+      for (int c = tid; c < k * D; c += kThreads) {
+        ra.mu[c] = pv.mu[c];
+        if (c % D == 0) ra.counts[c / D] = tot[4 * c + 2];
+      }
+      for (int c = tid; c < k; c += kThreads) ra.cum0[c] = pv.cum[c];
+      for (int c = tid; c < 4 * k * D; c += kThreads) ra.tot0[c] = tot[c];
       if (tid == 0) {
         LoopState* ls = a.ls;
         ls->E2 = E2;
@@ -483,13 +312,12 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
         ls->last_overflowed = 0ull;
         ls->done = done ? 1 : 0;
       }
-      __syncthreads();
       // the step kernels' tables of the final centroids
-      fast_screen_tables(ra.mu, dc.s, dc.A_max, k, D, a.kpad, ra.tie_rel, ra.ctil_out, ra.ic_out, ra.tab_out, sB);
+      for (int c = tid; c < a.kpad * DP; c += kThreads) ra.tab_out[c] = sm.tab[c];
+      for (int c = tid; c < k; c += kThreads) ra.ctil_out[c] = pv.ctil[c];
+      if (tid == 0) *ra.ic_out = s_ic;
       return;
     }
-    __syncthreads();
-    tables();
   }
 }
 
@@ -538,7 +366,7 @@ int run_rep(int d, int k) { return (int)std::max<size_t>(1, std::min<size_t>(8, 
 int run_blocks_per_sm(int d, int kpad, size_t smem) { KM_RUN_DISPATCH(run_blocks, d, kpad, smem); }
 
 cudaError_t launch_run_fast(int d, int grid, size_t smem, cudaStream_t st, const RunArgs& a) {
-  cudaError_t e = cudaMemsetAsync(a.delta, 0, run_delta_words(d, a.f.k) * sizeof(unsigned long long), st);
+  cudaError_t e = cudaMemsetAsync(a.delta, 0, run_delta_words(d, a.f.k, a.rep) * sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
   KM_RUN_DISPATCH(run_launch, d, a.f.kpad, grid, smem, st, a);
 }
