@@ -121,6 +121,7 @@ struct FastArgs {
 };
 
 // A whole run in one cooperative kernel (km_run_fast.cu).
+constexpr float kDriftMax = 2.9e38f;  // drift sums stop here, below the "never open" (3e38) of what lies past the end
 struct RunArgs {
   FastArgs f;                  // points, sizes, constants and loop state (labels and partials unused)
   float* slack;                // [N]

@@ -280,7 +280,8 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
         else m2 = fmaxf(m2, p1);
       }
       m2 = fmaxf(m2, 0.f);
-      if (tid < k) pv.cum[tid] = __fadd_ru(pv.cum[tid], __fadd_ru(mine, tid == i1 ? m2 : m1));  // k <= 256 threads
+      if (tid < k)  // k <= 256 threads
+        pv.cum[tid] = fminf(__fadd_ru(pv.cum[tid], __fadd_ru(mine, tid == i1 ? m2 : m1)), kDriftMax);
     }
     tables();  // its barriers also publish s_e2 and the drift sums
     const double E2 = s_e2;

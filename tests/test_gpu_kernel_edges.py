@@ -202,3 +202,28 @@ def test_large_magnitudes(km, oracle, d, k, scale):
         r = g.run(12, 0.0)
         assert r["iters"] == ref["iters"] and np.array_equal(r["labels"], ref["labels"])
         g.close()
+
+
+
+# starting centroids so far out that every squared distance overflows FP64: the
+# lowest index takes the points, and the moves leave FP32's range
+@pytest.mark.parametrize("n,d,k", [(300, 2, 2), (1001, 3, 5), (9001, 1, 40)])
+def test_far_centroids(km, oracle, n, d, k):
+    x, _, _ = synth.iso_mixture(n, d, 3, sigma=1.0, box=8.0, seed=n)
+    mu0 = np.random.default_rng(k).normal(size=(k, d)) * 1e200
+    ref = oracle.run(x, mu0, 6, 0.0)
+    for graph in (0, 1):
+        g = km.KMeans(n, d, k, use_graph=graph)
+        g.set_points(x)
+        g.set_init(mu0)
+        r = g.run(6, 0.0)
+        assert np.array_equal(r["labels"], ref["labels"]) and np.allclose(r["centroids"], ref["centroids"], rtol=1e-6)
+        g.close()
+    for shape in ((8192, 256), (512, 128)):
+        b = km.KMeansBatch([n], [d], [k])
+        b.set_points([x])
+        b.set_init([mu0])
+        b.set_shape(*shape)
+        r = b.run(6, 0.0)
+        assert np.array_equal(r["labels"], ref["labels"])
+        b.close()
