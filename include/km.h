@@ -72,8 +72,13 @@ enum { KM_TC_BF16 = 0, KM_TC_F16 = 1 };                         /* tensor-core o
 typedef struct km_options {
   int32_t e_mode;  /* KM_E_NORM (default): stop when sqrt(E^2) < tol;
                       KM_E_SQUARED: the paper's E^2 = sum ||dmu||^2 < tol */
-  int32_t use_graph; /* 1 (default): km_run drives the loop from one CUDA graph
-                        with a device-side stop; 0: one host round trip per step */
+  int32_t use_graph; /* 1 (default): km_run keeps the loop on the device -- on the
+                        fused path (km_stats.path 1) one cooperative kernel for up to
+                        64 steps at a time, 5 (label_bytes 1: 4) more bytes of device
+                        memory per point from the first run on (without that memory,
+                        and on the other paths, a CUDA graph of steps with a
+                        device-side stop); 0: one host round trip per step.  Same
+                        results */
   double tie_rel;  /* relative near-tie threshold re-decided in FP64 (default 1e-5) */
   void* stream;    /* cudaStream_t for all work (NULL: the context creates one) */
   int32_t label_policy; /* KM_LABELS_EVERY_STEP (default): every step writes its labels
@@ -237,7 +242,8 @@ typedef struct km_stats {
   int32_t iters;          /* steps since km_set_init */
   int32_t converged;      /* 1 once the tolerance was met in km_run */
   double e, e2;           /* error of the last step */
-  int64_t flagged;        /* points re-checked past the FP32 screen in the last step */
+  int64_t flagged;        /* points re-checked past the FP32 screen in the last step (of a
+                             km_run in one kernel: points decided again in its last step) */
   int64_t fp64_decided;   /* of those, points decided in FP64 */
   int32_t empty_clusters; /* clusters with no points in the last step */
   int64_t overflowed;     /* tensor-core path: points whose candidate list overflowed (all K re-ranked) */
@@ -331,14 +337,18 @@ km_status km_batch_set_init(km_batch* b, const double* mu0);
  * km_batch_run does this when it was not called): the batch kernel's tile
  * sizes (512, 1024 points) x block sizes (128, 256, 512 threads), then the
  * fused kernel's tile machinery (8 points per lane, 256 threads) on tiles of
- * 8192 and 32768 points.  Every shape gives the same results.  Leaves
- * centroids and iteration counts unchanged.  Outputs may be NULL. */
+ * 8192 and 32768 points, which decide a point again only when its label can
+ * have changed (timed as one first step and two without such points, per
+ * step).  Every shape gives the same results.  Leaves centroids and iteration
+ * counts unchanged.  Outputs may be NULL. */
 km_status km_batch_tune(km_batch* b, int32_t* tile_out, int32_t* threads_out);
 
 /* Use a launch shape without timing (one the tuner times: tile_points 512 or
  * 1024 with threads 128, 256 or 512, or tile_points 8192 or 32768 with 256
  * threads for the fused kernel), e.g. a shape a previous km_batch_tune chose
- * for the same instances, kept in a cache.  Errors: KM_EINVAL (another
+ * for the same instances, kept in a cache.  (The fused shapes keep 5 bytes a
+ * point; a batch that could not allocate them runs the batch kernel's 1024
+ * points instead.)  Errors: KM_EINVAL (another
  * shape), KM_ESTATE (no points). */
 km_status km_batch_set_shape(km_batch* b, int32_t tile_points, int32_t threads);
 
@@ -349,7 +359,7 @@ km_status km_batch_set_shape(km_batch* b, int32_t tile_points, int32_t threads);
 km_status km_batch_objective(km_batch* b, double* out);
 
 /* Run every instance until its selected error is < tol or max_iter more
- * steps have run; the steps are replayed from a captured CUDA graph (4 steps
+ * steps have run; the steps are replayed from a captured CUDA graph (8 steps
  * per launch; stopped instances do no work) until no instance is active.
  * Outputs (host or device pointers, each may be NULL): labels_out (sum N_i),
  * centroids_out (sum K_i d_i), and per instance iters_out (steps since
@@ -362,7 +372,7 @@ km_status km_batch_run(km_batch* b, int32_t max_iter, double tol, int32_t* label
 km_status km_batch_get_counts(km_batch* b, int64_t* counts_out);
 
 typedef struct km_batch_info {
-  int64_t flagged;        /* points re-checked past the FP32 screen, all steps so far */
+  int64_t flagged;        /* points re-checked past the FP32 screen (fused shapes: or decided again), all steps so far */
   int64_t fp64_decided;   /* of those, decided in FP64 */
   int32_t tile_points;    /* launch shape in use */
   int32_t threads;

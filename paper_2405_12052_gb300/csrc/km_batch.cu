@@ -23,6 +23,7 @@
 // Stopped instances are skipped by both kernels, so a captured run of U
 // steps can be replayed until no instance is active.
 #include "km_internal.cuh"
+#include "km_i128.cuh"
 #include "km_tables.cuh"
 
 #include <algorithm>
@@ -41,25 +42,6 @@ __device__ __forceinline__ double bd64(const float* xo, const double* mu_k, int 
     acc = __dadd_rn(acc, __dmul_rn(t, t));
   }
   return acc;
-}
-
-__device__ __forceinline__ double i128_to_double(unsigned long long lo, long long hs) {
-  unsigned long long hi = (unsigned long long)hs;
-  const bool neg = hs < 0;
-  if (neg) {
-    lo = ~lo + 1ull;
-    hi = ~hi + (lo == 0ull ? 1ull : 0ull);
-  }
-  double r;
-  if (hi == 0ull) {
-    r = __ull2double_rn(lo);
-  } else {
-    const int sh = 64 - __clzll((long long)hi);
-    unsigned long long top = (hi << (64 - sh)) | (lo >> sh);
-    if (lo << (64 - sh)) top |= 1ull;  // sticky bit: one rounding in the conversion
-    r = ldexp(__ull2double_rn(top), sh);
-  }
-  return neg ? -r : r;
 }
 
 __device__ __forceinline__ unsigned long long bfma2(unsigned long long a, unsigned long long b,
@@ -284,51 +266,103 @@ __global__ void __launch_bounds__(kBatchMaxThreads) batch_assign_kernel(BatchArg
   }
 }
 
-// One block (256 threads) per instance.
-__global__ void __launch_bounds__(256) batch_update_kernel(BatchArgs a) {
+// One block per instance.  The column totals: with steps that skip points,
+// the instance's running totals; else the sums over its tiles' rows, dealt
+// over the block's groups of 256 threads (integers: any order).  From there on
+// 256 threads, in the order of the single-context update.
+constexpr int kUpdThreads = 512;
+__global__ void __launch_bounds__(kUpdThreads) batch_update_kernel(BatchArgs a) {
   __shared__ double s_red[256];
   __shared__ double s_bmax[256];
-  __shared__ int s_empty;
+  __shared__ unsigned long long s_lo[kUpdThreads / 256][256];
+  __shared__ long long s_hi[kUpdThreads / 256][256];
+  __shared__ double s_df2[kBatchMaxK * 3];
+  __shared__ float s_mv[kBatchMaxK];
+  __shared__ int s_empty, s_at;
   const int inst = blockIdx.x, tid = threadIdx.x;
   BatchState* st = a.state + inst;
   if (st->done) return;
-  const BatchInst bi = a.inst[inst];
-  const int d = bi.d, k = bi.k, dp = d + 1;
+  const BatchInst& bi = a.inst[inst];
+  const int d = bi.d, k = bi.k, dp = d + 1, cols = k * dp;  // cols <= 256
   if (tid == 0) s_empty = 0;
+  {
+    const int col = tid & 255, g = tid >> 8;
+    unsigned long long lo = 0ull;
+    long long hi = 0ll;
+    if (a.cum) {
+      if (g == 0 && col < cols) {
+        unsigned long long* t = a.totals + 2 * (bi.tot_off + col);
+        const unsigned long long tl = t[0];
+        const long long th = (long long)t[1] + (long long)(tl >> 32);  // carry what the steps' additions left over
+        t[0] = tl & 0xffffffffull;
+        t[1] = (unsigned long long)th;
+        lo = ((unsigned long long)th << 32) | (tl & 0xffffffffull);
+        hi = th >> 32;
+      }
+    } else if (col < cols) {
+      const long long* p0 = a.partials + a.tile_poff[bi.tile0] + col;  // an instance's rows follow one another
+#pragma unroll 8
+      for (int t = g; t < bi.ntiles; t += kUpdThreads / 256) {
+        const long long v = p0[(size_t)t * cols];
+        const unsigned long long nl = lo + (unsigned long long)v;
+        hi += (v < 0 ? -1ll : 0ll) + (nl < lo ? 1ll : 0ll);
+        lo = nl;
+      }
+    }
+    s_lo[g][col] = lo;
+    s_hi[g][col] = hi;
+  }
+  __syncthreads();
+  if (tid < cols) {
+    unsigned long long lo = s_lo[0][tid];
+    long long hi = s_hi[0][tid];
+    for (int g = 1; g < kUpdThreads / 256; ++g) add128p(lo, hi, s_lo[g][tid], s_hi[g][tid]);
+    s_lo[0][tid] = lo;
+    s_hi[0][tid] = hi;
+  }
   __syncthreads();
   double* mu = a.mu + bi.mu_off;
   double e2p = 0.0;
   int empty = 0;
-  for (int q = tid; q < k * d; q += blockDim.x) {
-    const int c = q / d, j = q - c * d;
-    unsigned long long lo = 0ull;
-    long long hi = 0ll, cnt = 0;
-    for (int t = 0; t < bi.ntiles; ++t) {
-      const long long* prow = a.partials + a.tile_poff[bi.tile0 + t] + (size_t)c * dp;
-      const long long v = prow[j];
-      const unsigned long long nl = lo + (unsigned long long)v;
-      hi += (v < 0 ? -1ll : 0ll) + (nl < lo ? 1ll : 0ll);
-      lo = nl;
-      cnt += prow[d];
-    }
+  if (tid < k * d) {
+    const int q = tid, c = q / d, j = q - c * d;
+    const long long cnt = (long long)s_lo[0][c * dp + d];
     const double old = mu[q];
     double nw = old;
-    if (cnt > 0) nw = __ddiv_rn(ldexp(i128_to_double(lo, hi), bi.G0), (double)cnt);
+    if (cnt > 0) nw = __ddiv_rn(ldexp(i128_to_double((long long)s_lo[0][c * dp + j], s_hi[0][c * dp + j]), bi.G0), (double)cnt);
     const double df = __dsub_rn(nw, old);
-    e2p = __dadd_rn(e2p, __dmul_rn(df, df));
+    const double dd = __dmul_rn(df, df);
+    e2p = __dadd_rn(e2p, dd);
+    s_df2[q] = dd;
     mu[q] = nw;
     if (j == 0) {
       a.counts[bi.k_off + c] = cnt;
       empty += cnt == 0;
     }
   }
-  s_red[tid] = e2p;
+  if (tid < 256) s_red[tid] = e2p;
+  if (empty) atomicAdd(&s_empty, empty);
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+  for (int w = 128; w > 0; w >>= 1) {
     if (tid < w) s_red[tid] = __dadd_rn(s_red[tid], s_red[tid + w]);
     __syncthreads();
   }
-  if (empty) atomicAdd(&s_empty, empty);
+  if (a.cum) {
+    // the drift sums of the steps that skip points (see km_run_fast.cu)
+    if (tid < k) {
+      double t = 0.0;
+      for (int j = 0; j < d; ++j) t = __dadd_ru(t, s_df2[tid * d + j]);
+      s_mv[tid] = sqrt_up(t);
+    }
+    __syncthreads();
+    if (tid < k) {
+      float oth = 0.f;  // the largest move of the other centroids
+      for (int c = 0; c < k; ++c)
+        if (c != tid) oth = fmaxf(oth, s_mv[c]);
+      float* cu = a.cum + bi.k_off + tid;
+      *cu = fminf(__fadd_ru(st->first ? 0.f : *cu, __fadd_ru(s_mv[tid], oth)), kDriftMax);
+    }
+  }
   // next step's FP32 table c~ = fl32(mu - s) and max ||mu - s||^2
   double bm = 0.0;
   for (int c = tid; c < k; c += blockDim.x) {
@@ -340,9 +374,9 @@ __global__ void __launch_bounds__(256) batch_update_kernel(BatchArgs a) {
     }
     bm = fmax(bm, B);
   }
-  s_bmax[tid] = bm;
+  if (tid < 256) s_bmax[tid] = bm;  // k <= 64 threads have values
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+  for (int w = 32; w > 0; w >>= 1) {
     if (tid < w) s_bmax[tid] = fmax(s_bmax[tid], s_bmax[tid + w]);
     __syncthreads();
   }
@@ -355,6 +389,7 @@ __global__ void __launch_bounds__(256) batch_update_kernel(BatchArgs a) {
     st->E2 = E2;
     st->E = E;
     st->iter += 1;
+    st->first = 0;
     st->empty = s_empty;
     st->B_max = (float)(s_bmax[0] * (1.0 + 1e-6));
     const double esel = a.e_mode == 1 ? E2 : E;
@@ -363,6 +398,12 @@ __global__ void __launch_bounds__(256) batch_update_kernel(BatchArgs a) {
       st->done = 1;
       atomicSub(a.active, 1);
     }
+    s_at = a.list && !st->done ? atomicAdd(a.work, bi.ntiles) : -1;
+  }
+  if (a.list) {  // the next step's tiles
+    __syncthreads();
+    if (s_at >= 0)
+      for (int t = tid; t < bi.ntiles; t += kUpdThreads) a.list[s_at + t] = bi.tile0 + t;
   }
 }
 
@@ -484,7 +525,7 @@ cudaError_t launch_batch_assign(const BatchArgs& a, int grid, int threads, cudaS
 }
 
 cudaError_t launch_batch_update(const BatchArgs& a, int count, cudaStream_t st) {
-  batch_update_kernel<<<count, 256, 0, st>>>(a);
+  batch_update_kernel<<<count, kUpdThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -39,7 +39,13 @@ struct km_batch {
   unsigned long long* tab2 = nullptr;   // fused kernel: per-instance screen tables
   float4* ctil4 = nullptr;
   IterConst* ic = nullptr;
-  int64_t total_tab = 0;
+  float* slack = nullptr;               // fused kernel's tiles: per point, instances at 256-point boundaries
+  uint8_t* z8 = nullptr;
+  float* cum = nullptr;                 // [total_k]
+  unsigned long long* totals = nullptr; // [total_cols][2]
+  int* list = nullptr;                  // tiles of the step
+  int* work = nullptr;                  // [3]
+  int64_t total_tab = 0, total_p = 0, total_cols = 0;
   int kind = 0;                         // assign kernel: 0 the batch kernel, 1 the fused kernel's tiles
   int* active = nullptr;
   int64_t max_tiles = 0, max_partials = 0;
@@ -59,7 +65,7 @@ constexpr int kTileCand[2] = {512, 1024};
 constexpr int kThreadCand[3] = {128, 256, 512};
 // the fused kernel's tiles (a multiple of its 256-point warp-tiles; 256 threads)
 constexpr int kFastTileCand[2] = {8192, 32768};
-constexpr int kGraphSteps = 4;
+constexpr int kGraphSteps = 8;
 
 km_status bfail(km_batch* b, km_status s, const std::string& m) {
   b->err = m;
@@ -86,6 +92,9 @@ BatchArgs bargs(km_batch* b) {
   a.counts = b->counts; a.flagged = b->stats; a.fp64 = b->stats + 1; a.active = b->active;
   a.tau = (float)(b->opt.tie_rel * (1.0 + 1e-4)); a.e_mode = b->opt.e_mode; a.tol = 0.0;
   a.tab2 = b->tab2; a.ctil4 = b->ctil4; a.ic = b->ic; a.tie_rel = b->opt.tie_rel;
+  if (b->kind == 1) {
+    a.slack = b->slack; a.z8 = b->z8; a.cum = b->cum; a.totals = b->totals; a.list = b->list; a.work = b->work;
+  }
   return a;
 }
 
@@ -129,13 +138,13 @@ void drop_graph(km_batch* b) {
 }
 
 int grid_for(km_batch* b, int threads) {
-  const int per_sm = b->kind == 1 ? batch_fast_blocks_per_sm() : batch_blocks_per_sm(threads);
+  const int per_sm = b->kind == 1 ? batch_run_blocks_per_sm() : batch_blocks_per_sm(threads);
   const int64_t g = std::min<int64_t>(b->ntiles, (int64_t)b->sms * per_sm);
   return (int)std::max<int64_t>(1, g);
 }
 
 cudaError_t launch_assign_kind(km_batch* b, const BatchArgs& a) {
-  return b->kind == 1 ? launch_batch_fast(a, b->grid, b->st) : launch_batch_assign(a, b->grid, b->threads, b->st);
+  return b->kind == 1 ? launch_batch_run(a, b->grid, 0, b->st) : launch_batch_assign(a, b->grid, b->threads, b->st);
 }
 
 }  // namespace
@@ -166,6 +175,10 @@ km_status km_batch_create(km_batch** out, int32_t count, const int64_t* n, const
     bi.x_off = xo; bi.lab_off = lo; bi.mu_off = (int32_t)mo; bi.k_off = (int32_t)ko;
     bi.kpad = (k[i] + 7) / 8 * 8;
     bi.tab_off = (int32_t)b->total_tab;
+    bi.p_off = b->total_p;
+    b->total_p += (n[i] + 255) / 256 * 256;
+    bi.tot_off = b->total_cols;
+    b->total_cols += (int64_t)k[i] * (d[i] + 1);
     b->total_tab += (int64_t)bi.kpad * (d[i] + 1);
     xo += n[i] * d[i]; lo += n[i]; mo += (int64_t)k[i] * d[i]; ko += k[i];
     const int64_t nt = (n[i] + kTileCand[0] - 1) / kTileCand[0];
@@ -198,6 +211,18 @@ km_status km_batch_create(km_batch** out, int32_t count, const int64_t* n, const
   KB_CUDA(b, balloc(&b->ctil4, (size_t)ko));
   KB_CUDA(b, balloc(&b->ic, (size_t)count));
   KB_CUDA(b, balloc(&b->active, 1));
+  // the buffers of the steps that skip points; without the memory for them
+  // the batch kernel's tiles run every shape
+  if (balloc(&b->slack, (size_t)b->total_p) != cudaSuccess || balloc(&b->z8, (size_t)b->total_p) != cudaSuccess ||
+      balloc(&b->cum, (size_t)ko) != cudaSuccess || balloc(&b->totals, (size_t)b->total_cols * 2) != cudaSuccess ||
+      balloc(&b->list, (size_t)tiles_max) != cudaSuccess || balloc(&b->work, 3) != cudaSuccess) {
+    cudaGetLastError();
+    void* bufs[] = {b->slack, b->z8, b->cum, b->totals, b->list, b->work};
+    for (void* p : bufs)
+      if (p) cudaFree(p);
+    b->slack = nullptr; b->z8 = nullptr; b->cum = nullptr; b->totals = nullptr; b->list = nullptr;
+    b->work = nullptr;
+  }
   KB_CUDA(b, cudaMemcpyAsync(b->inst, b->hinst.data(), sizeof(BatchInst) * count, cudaMemcpyHostToDevice, b->st));
   KB_CUDA(b, cudaMemsetAsync(b->state, 0, sizeof(BatchState) * count, b->st));
   KB_CUDA(b, cudaMemsetAsync(b->labels, 0, sizeof(int32_t) * (size_t)lo, b->st));
@@ -256,9 +281,12 @@ km_status km_batch_tune(km_batch* b, int32_t* tile_out, int32_t* threads_out) {
   float best = 3.0e38f;
   int bt = kTileCand[1], bth = 256, bkind = 0;
   b->tune_ms.clear();
-  // the assign kernel writes labels, partials and counters only: timing it
-  // leaves the centroids and the loop state untouched.  Candidates: the
-  // batch kernel's tiles x block sizes, then the fused kernel's tiles.
+  // the assign kernels write labels, slacks, partials and counters only:
+  // timing them leaves the centroids and the loop state untouched.
+  // Candidates: the batch kernel's tiles x block sizes, then the fused kernel's
+  // tiles.  The latter compare every point in the first step only and mostly
+  // skip afterwards, so theirs is the time of one such step and two in which
+  // no point is open, per step.
   auto time_shape = [&](int kind, int tp, int th) -> km_status {
     km_status s = build_tiles(b, tp);
     if (s != KM_OK) return s;
@@ -266,9 +294,15 @@ km_status km_batch_tune(km_batch* b, int32_t* tile_out, int32_t* threads_out) {
     b->threads = th;
     b->grid = grid_for(b, th);
     BatchArgs a = bargs(b);
-    KB_CUDA(b, launch_assign_kind(b, a));  // warm-up
+    auto launch = [&](int r) {
+      if (kind == 0) return launch_batch_assign(a, b->grid, th, b->st);
+      cudaError_t e = launch_batch_list(a, 1, b->st);
+      return e != cudaSuccess ? e : launch_batch_run(a, b->grid, r == 0 ? 1 : -1, b->st);
+    };
+    if (kind == 1) KB_CUDA(b, cudaMemsetAsync(b->cum, 0, sizeof(float) * (size_t)b->total_k, b->st));
+    KB_CUDA(b, launch(0));  // warm-up
     KB_CUDA(b, cudaEventRecord(e0, b->st));
-    for (int r = 0; r < 3; ++r) KB_CUDA(b, launch_assign_kind(b, a));
+    for (int r = 0; r < 3; ++r) KB_CUDA(b, launch(r));
     KB_CUDA(b, cudaEventRecord(e1, b->st));
     KB_CUDA(b, cudaEventSynchronize(e1));
     float ms = 0.f;
@@ -282,10 +316,11 @@ km_status km_batch_tune(km_batch* b, int32_t* tile_out, int32_t* threads_out) {
       km_status s = time_shape(0, tp, th);
       if (s != KM_OK) return s;
     }
-  for (int tp : kFastTileCand) {
-    km_status s = time_shape(1, tp, 256);
-    if (s != KM_OK) return s;
-  }
+  if (b->slack)
+    for (int tp : kFastTileCand) {
+      km_status s = time_shape(1, tp, 256);
+      if (s != KM_OK) return s;
+    }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   km_status s = build_tiles(b, bt);
@@ -310,6 +345,11 @@ km_status km_batch_set_shape(km_batch* b, int32_t tile_points, int32_t threads) 
   for (int th : kThreadCand) ok_th = ok_th || th == threads;
   for (int tp : kFastTileCand) fast = fast || (tp == tile_points && threads == 256);
   if (!fast && (!ok_t || !ok_th)) return bfail(b, KM_EINVAL, "tile_points or threads is not one the tuner times");
+  if (fast && !b->slack) {
+    // no memory for the buffers these tiles need: the batch kernel's instead
+    fast = false;
+    tile_points = kTileCand[1];
+  }
   km_status s = build_tiles(b, tile_points);
   if (s != KM_OK) return s;
   b->kind = fast ? 1 : 0;
@@ -338,6 +378,7 @@ km_status km_batch_run(km_batch* b, int32_t max_iter, double tol, int32_t* label
   for (auto& s : b->hstate) {
     s.max_iter = s.iter + max_iter;
     s.converged = 0;
+    s.first = 1;
     s.done = max_iter == 0 ? 1 : 0;
     act += !s.done;
   }
@@ -345,6 +386,10 @@ km_status km_batch_run(km_batch* b, int32_t max_iter, double tol, int32_t* label
   KB_CUDA(b, cudaMemcpyAsync(b->active, &act, sizeof(int), cudaMemcpyHostToDevice, b->st));
   BatchArgs a = bargs(b);
   a.tol = tol;
+  if (b->kind == 1) {
+    KB_CUDA(b, cudaMemsetAsync(b->totals, 0, sizeof(unsigned long long) * 2 * (size_t)b->total_cols, b->st));
+    KB_CUDA(b, launch_batch_list(a, 0, b->st));
+  }
   // the tolerance is a kernel argument: the graph is rebuilt when it changes
   if (b->graph && b->graph_tol != tol) drop_graph(b);
   if (b->opt.use_graph && !b->graph) {
@@ -376,6 +421,7 @@ km_status km_batch_run(km_batch* b, int32_t max_iter, double tol, int32_t* label
     KB_CUDA(b, cudaStreamSynchronize(b->st));
   }
   KB_CUDA(b, cudaMemcpyAsync(b->hstate.data(), b->state, sizeof(BatchState) * b->count, cudaMemcpyDeviceToHost, b->st));
+  if (b->kind == 1 && max_iter > 0) KB_CUDA(b, launch_batch_labels(a, b->count, b->sms, b->st));
   if (labels_out)
     KB_CUDA(b, cudaMemcpyAsync(labels_out, b->labels, sizeof(int32_t) * (size_t)b->total_n, cudaMemcpyDefault, b->st));
   if (centroids_out)
@@ -437,7 +483,8 @@ void km_batch_destroy(km_batch* b) {
   if (!b) return;
   drop_graph(b);
   void* bufs[] = {b->x, b->labels, b->mu, b->ctil, b->counts, b->inst, b->state, b->tiles,
-                  b->tile_poff, b->partials, b->stats, b->active, b->tab2, b->ctil4, b->ic};
+                  b->tile_poff, b->partials, b->stats, b->active, b->tab2, b->ctil4, b->ic,
+                  b->slack, b->z8, b->cum, b->totals, b->list, b->work};
   for (void* p : bufs)
     if (p) cudaFree(p);
   if (b->own_stream && b->st) cudaStreamDestroy(b->st);

@@ -119,11 +119,25 @@ __device__ int recheck_fast(const float* xo, const float* s, const float4* ctil,
     // lo2 <= D2 and hi1 >= D1; the factor covers the roundings here
     if (slack) *slack = clear ? (lo2 - hi1) * 0.9999f / (__fsqrt_rn(lo2) + __fsqrt_rn(fmaxf(hi1, 0.f)) + 1e-37f) : -1.f;
     if (!clear) {
+      // only centroids whose lower bound is not above the best's upper bound
+      // can be the oracle's argmin (the bounds cover its own rounding): mostly
+      // two, where K FP64 distances one after another, each behind a load of
+      // its centroid, took a warp about 30 us at K = 64
       used64 = true;
-      double bd = d64_fixed<D>(xo, mu);
+      const float lim = best < 3.0e38f ? hi1 : __int_as_float(0x7f800000);  // no FP32 distance: all K
+      double bd = __longlong_as_double(0x7ff0000000000000ll);
       kb = 0;
-      for (int c = 1; c < k; ++c) {
-        double dd = d64_fixed<D>(xo, mu + (int64_t)c * D);
+      for (int c = 0; c < k; ++c) {
+        const float4 cc = ctil[c];
+        const float cv[4] = {cc.x, cc.y, cc.z, cc.w};
+        float dv = 0.f;
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+          const float t = __fsub_rn(xt[j], cv[j]);
+          dv = __fmaf_rn(t, t, dv);
+        }
+        if (dv - direct_bound(dv, sA, sB, AB, D) > lim) continue;  // an infinity or NaN stays a candidate
+        const double dd = d64_fixed<D>(xo, mu + (int64_t)c * D);
         if (dd < bd) { bd = dd; kb = c; }
       }
     }

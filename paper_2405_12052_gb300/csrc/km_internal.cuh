@@ -272,11 +272,13 @@ struct BatchInst {        // per instance, written at set_points (scan kernel) a
   int32_t G0;                      // fixed-point grid exponent
   float C_hi, C_lo;
   uint32_t bits_C_hi, bits_C_lo;
+  int64_t p_off;                   // offset of the points' slacks and byte labels (a multiple of 256)
+  int64_t tot_off;                 // offset of the running totals (K_i (d_i + 1) columns)
 };
 
 struct BatchState {       // per instance, advanced on the device
   int32_t done, iter, converged, empty;
-  int32_t max_iter, pad;
+  int32_t max_iter, first;         // first: 1 until the run's first step is done
   double E, E2;
   float B_max, pad2;
 };
@@ -304,15 +306,28 @@ struct BatchArgs {
   float4* ctil4;                  // [sum K_i] fl32(mu - s)
   IterConst* ic;                  // [count] screen constants
   double tie_rel;
+  // steps that skip points (fused kernel's tiles; null where they are not run)
+  float* slack;                   // [p_off of the last instance + its points]
+  uint8_t* z8;
+  float* cum;                     // [sum K] drift per cluster in this run, rounded up
+  int* list;                      // [tiles] the step's tiles, in any order
+  int* work;                      // [3] tiles listed, tiles taken, blocks done
+  unsigned long long* totals;     // [sum K_i (d_i + 1)][2] running column totals of this run: low (below 2^32
+                                  // between steps) and high word, value = high 2^32 + low
 };
 
 cudaError_t launch_batch_scan(const float* x, BatchInst* inst, int count, unsigned long long* bad, cudaStream_t st);
 cudaError_t launch_batch_tables(const BatchArgs& a, int count, cudaStream_t st);
 cudaError_t launch_batch_assign(const BatchArgs& a, int grid, int threads, cudaStream_t st);
-// The batch through the fused kernel's tile machinery (256 threads per block;
-// tiles of a multiple of 256 points).
-cudaError_t launch_batch_fast(const BatchArgs& a, int grid, cudaStream_t st);
-int batch_fast_blocks_per_sm();
+// The batch through the fused kernel's tile machinery, skipping points (256
+// threads per block; tiles of a multiple of 2048 points): the listed tiles'
+// step, and the list at the start of a run (a step's update lists the next
+// step's).  mode: 0 as the instances' states say, 1 every instance in its first
+// step, -1 none.
+cudaError_t launch_batch_list(const BatchArgs& a, int mode, cudaStream_t st);
+cudaError_t launch_batch_run(const BatchArgs& a, int grid, int mode, cudaStream_t st);
+int batch_run_blocks_per_sm();
+cudaError_t launch_batch_labels(const BatchArgs& a, int count, int sms, cudaStream_t st);
 cudaError_t launch_batch_update(const BatchArgs& a, int count, cudaStream_t st);
 int batch_blocks_per_sm(int threads);
 cudaError_t launch_batch_objective(const float* x, const BatchInst* inst, const int32_t* labels, const double* mu,

@@ -227,3 +227,48 @@ def test_far_centroids(km, oracle, n, d, k):
         r = b.run(6, 0.0)
         assert np.array_equal(r["labels"], ref["labels"])
         b.close()
+
+
+# many steps of a batch whose tiles are skipped, taken from the lists of open
+# points (few, many) or screened whole, against the shape that compares every
+# point in every step: whole numbers and centroids are the same.  Instances of
+# one point up to past the largest tile, at its edges and the 256-point ones;
+# repeated points and a duplicated centroid are exact ties, some in FP64 every
+# step; a second run continues the first
+@pytest.mark.parametrize("scale", [1.0, 1e18])
+@pytest.mark.parametrize("tile", [8192, 32768])
+def test_batch_skipping_equals_every_point(km, oracle, tile, scale):
+    sizes = [1, 2, 255, 256, 257, 1023, 1025, 2049, 8191, 8192, 8193, 32_767, 32_769, 70_001]
+    ks = [1, 2, 7, 8, 33, 64]
+    xs, mus = [], []
+    for q, n in enumerate(sizes * 3):
+        d, k = 1 + q // len(sizes), min(n, ks[q % len(ks)])
+        x, _, _ = synth.iso_mixture(n, d, max(2, k // 2), sigma=1.5, box=8.0, seed=q)
+        if q % 4 == 1:
+            x = np.round(x)                          # a grid: exact ties
+        x[:, n // 2:n // 2 + n // 20] = x[:, :n // 20]
+        x = (x.astype(np.float64) * scale).astype(np.float32)
+        mu = x[:, np.random.default_rng(q).permutation(n)[:k]].T.astype(np.float64)
+        if k > 2 and q % 3 == 0:
+            mu[1] = mu[0]
+        xs.append(x)
+        mus.append(mu)
+    got = []
+    for shape in ((tile, 256), (512, 128)):
+        b = km.KMeansBatch([x.shape[1] for x in xs], [x.shape[0] for x in xs], [m.shape[0] for m in mus])
+        b.set_points(xs)
+        b.set_init(mus)
+        b.set_shape(*shape)
+        r = b.run(35, 0.0)
+        r2 = b.run(12, 0.0)
+        got.append([np.asarray(v) for s in (r, r2) for v in (s["labels"], s["centroids"], s["iters"], s["E"])]
+                   + [b.counts()])
+        b.close()
+    for p, q in zip(*got):
+        assert np.array_equal(p, q)
+    off = 0
+    for q, (x, m) in enumerate(zip(xs, mus)):
+        if q % 5 == 0:
+            ref = oracle.run(x, m, 35, 0.0)
+            assert np.array_equal(got[0][0][off:off + x.shape[1]], ref["labels"]) and got[0][2][q] == ref["iters"]
+        off += x.shape[1]
