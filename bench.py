@@ -35,9 +35,6 @@ if ROOT not in sys.path:
 METRIC = "point-centroid distance evals/s per Lloyd iter"
 UNIT = "evals/s"
 FP32_LANES_PER_SM = 128  # FFMA lanes per SM per clock (2 flops each)
-# FP64 add or multiply lane-operations per SM per cycle, measured on GB300
-# (independent DADD and DMUL chains, 32 warps per SM, clock64 timing): 1.89.
-FP64_ADDMUL_PER_SM_CYCLE = 1.89
 
 
 def parse():
@@ -169,7 +166,7 @@ class ClockSampler:
 
 
 KERNEL_SOURCES = {
-    "assign_fast_kernel<3>": ("km_assign.cu", "km_fast_common.cuh", "km_internal.cuh"),
+    "assign_fast_kernel<3>": ("km_assign.cu", "km_fast_tile.cuh", "km_fast_common.cuh", "km_internal.cuh"),
     "gemm_assign_kernel": ("km_gemm.cu", "km_tcgen05.cuh", "km_internal.cuh"),
 }
 
@@ -456,7 +453,7 @@ def run_ours(args, ws, rank, local):
                       "labels": "one pass after the last step (inside the timed region)" if final_pass
                                 else "written every step",
                       "label_bytes": lb},
-           "clocks": clk, "e2e": e2e, "gpu_launches": (11 if stats["path"] == 3 else 2) * K + int(final_pass),
+           "clocks": clk, "e2e": e2e, "gpu_launches": ((12 if n >= 1 << 20 else 11) if stats["path"] == 3 else 2) * K + int(final_pass),
            "roofline": roof,
            "assign_ms": assign_ms, "update_ms": ms_step - assign_ms,
            "flagged_per_step": stats["flagged"], "fp64_decided_per_step": stats["fp64_decided"],
@@ -571,13 +568,11 @@ def kmeanspp_record(km, xt, k, dev, reps=3):
         times.append(time.perf_counter() - t0)
     g.close()
     t = statistics.median(times)
-    mhz = float(peaks()[0].get("sm_max_mhz", 2070.0))
-    sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    peak_ops = FP64_ADDMUL_PER_SM_CYCLE * sms * mhz * 1e6 / 1e12
-    ach = 3.0 * d * n * k / t / 1e12
+    # the points and their D^2 are read once per round after the first pick
+    hbm = float(peaks()[0].get("hbm_gbs", 6800.0))
+    ach = n * (4 * d + 8) * (k - 1) / t / 1e9
     return {"n": n, "d": d, "k": k, "ms_per_seeding": 1e3 * t, "evals_per_s": n * k / t,
-            "roofline": {"bound": "alu", "achieved": ach, "peak": peak_ops, "unit": "Tops/s (FP64 add/mul)",
-                         "frac": ach / peak_ops}}
+            "roofline": {"bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm}}
 
 
 def batch_ttc(count, dev):
@@ -688,17 +683,19 @@ def run_batch(args, ws, rank, local):
     e2e_s = time.perf_counter() - t0
     b2.close()
     # roofline of the assign kernel with every instance active: sum_i 3 N_i K_i d_i
-    # flops per launch over the tuner's time of the chosen launch shape
+    # flops per launch over the tuner's best time of the batch kernel, the one
+    # that compares every point in every step (the fused kernel's tiles skip
+    # points whose label cannot have changed)
     pk, src = peaks()
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     fp32_peak = sms * FP32_LANES_PER_SM * 2 * float(pk.get("sm_max_mhz", 2070.0)) * 1e6 / 1e12
-    assign_ms = min(info["tune_ms"]) if info["tune_ms"] else None
+    assign_ms = min(info["tune_ms"][:6]) if info["tune_ms"] else None
     flops = float(np.sum(3.0 * ns * ks * ds))
     roof = None
     if assign_ms:
         ach = flops / (assign_ms / 1e3) / 1e12
         roof = {"bound": "alu", "achieved": ach, "peak": fp32_peak, "unit": "TFLOP/s", "frac": ach / fp32_peak,
-                "traffic": None, "kernel": "batch_fast_kernel" if tile > 1024 else "batch_assign_kernel",
+                "traffic": None, "kernel": "batch_assign_kernel",
                 "kernel_ms": assign_ms,
                 "peak_source": f"{sms} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 flops x sm_max_mhz ({src} peaks); "
                                "algorithmic sum_i 3 N_i K_i d_i flops per launch with every instance active"}
@@ -738,7 +735,7 @@ def run_batch(args, ws, rank, local):
            "e2e": {"value": evals / e2e_s, "unit": UNIT, "h2d_bytes_per_step": int(flat.nbytes + mus.nbytes),
                    "d2h_bytes_per_step": int(ns.sum() * 4 + mus.nbytes), "time_to_converge_s": e2e_s,
                    "note": "one 'step' here is the whole batch run to convergence"},
-           "gpu_launches": int(2 * 4 * ((int(iters.max()) + 3) // 4)), "roofline": roof,
+           "gpu_launches": int(2 * 8 * ((int(iters.max()) + 7) // 8)) + (2 if tile > 1024 else 0), "roofline": roof,
            "time_to_converge_s": batch_s, "plain_sequential_s": plain_s * scale,
            "plain_sequential_warm_graph_s": plain_warm_s * scale,
            "plain_timed_instances": len(sel), "speedup_vs_plain": plain_s * scale / batch_s,
@@ -842,30 +839,21 @@ def run_kmeanspp(args, ws, rank, local):
     clk = clocks.stop()
     g.close()
     t = statistics.median(times)
-    # Per point and round the oracle's expression takes d FP64 subtractions,
-    # d products and d additions (unfused: fusing would change the sums and
-    # hence the picks).  Its ceiling is the FP64 add/multiply issue rate:
-    # FP64_ADDMUL_PER_SM_CYCLE lane-operations per SM cycle, measured on GB300
-    # with independent DADD/DMUL chains timed by clock64().
-    ops = 3.0 * d * n * k
-    mhz = float(peaks()[0].get("sm_max_mhz", 2070.0))
-    sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    peak_ops = FP64_ADDMUL_PER_SM_CYCLE * sms * mhz * 1e6 / 1e12
-    ach = ops / t / 1e12
+    # Each round after the first pick reads the points and their D^2 once; the
+    # D^2 that shrink (decided by an FP32 bound) are written back.  The exact FP64
+    # work is on those points only, so the reads are the floor.
+    ach = n * (4 * d + 8) * (k - 1) / t / 1e9
+    hbm = float(peaks()[0].get("hbm_gbs", 6800.0))
     out = {"metric": METRIC, "value": n * k / t, "unit": UNIT, "n_gpus": 1, "steps": args.steps,
            "warmup": args.warmup, "ms_per_step": 1e3 * t, "higher_is_better": True, "scaling": "weak",
            "vs_baseline": None, "dtype": "f64", "data": "synthetic",
            "config": {"workload": f"kmeanspp_3d_n{n}_k{k}", "n": n, "d": d, "k": k,
                       "step": "one k-means++ seeding (K rounds), host wall time around the call",
                       "parallelism": "single"},
-           "clocks": clk, "e2e": None, "gpu_launches": 2 * k - 1,
-           "roofline": {"bound": "alu", "achieved": ach, "peak": peak_ops, "unit": "Tops/s (FP64 add/mul)",
-                        "frac": ach / peak_ops,
-                        "traffic": None, "kernel": "kpp_d2_kernel + kpp_pick_kernel",
-                        "peak_source": f"measured FP64 DADD/DMUL issue rate, {FP64_ADDMUL_PER_SM_CYCLE} lane-ops "
-                                       f"per SM cycle x {sms} SMs x {mhz:.0f} MHz; 3 N K d FP64 operations "
-                                       "per seeding",
-                        "hbm_frac_of_measured": (n * (4 * d + 16) * k / t / 1e9) / float(peaks()[0].get("hbm_gbs", 6800.0))}}
+           "clocks": clk, "e2e": None, "gpu_launches": k,
+           "roofline": {"bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm,
+                        "traffic": None, "kernel": "kpp_d2_kernel",
+                        "peak_source": "measured copy bandwidth; (4 d + 8) N bytes read per round after the first pick"}}
     print(json.dumps(out), flush=True)
     return 0
 
