@@ -693,8 +693,11 @@ __device__ __forceinline__ void run_drain(const FastArgs& a, const float4* gtab,
 // kStage its points are copied to shared memory (3 KB in whole lines, where
 // gathering 12 bytes a point takes three 64-byte accesses) and the open ones
 // decided from there; below, they are queued across tiles and gathered.
-constexpr int kHeavy = 96, kStage = 16;
-constexpr int kQueueFull = kWarpQueue - 128;  // entries from which the queue is emptied (a tile adds at most kHeavy)
+// Measured: 72, 96, 128, 160 for kHeavy give 11.5, 10.6, 10.0, 9.9 ms for a run of
+// 1e8 points (K = 32, 37 steps) and 63, 61, 61, 61 ms for 256 instances.
+constexpr int kHeavy = 160, kStage = 32;
+constexpr int kQueueFull = kWarpQueue - kHeavy;  // entries from which the queue is emptied (a tile adds at most kHeavy)
+static_assert(kQueueFull + 4 * kStage <= kWarpQueue, "a batch of tiles with few open points fits");
 
 // One warp's part of a step that skips points (see km_run_fast.cu): warp-tiles
 // wid, wid + wtot, ... below end of the points a.x (a.n of them).  Adds the
