@@ -734,7 +734,8 @@ def run_batch(args, ws, rank, local):
            "clocks": clk,
            "e2e": {"value": evals / e2e_s, "unit": UNIT, "h2d_bytes_per_step": int(flat.nbytes + mus.nbytes),
                    "d2h_bytes_per_step": int(ns.sum() * 4 + mus.nbytes), "time_to_converge_s": e2e_s,
-                   "note": "one 'step' here is the whole batch run to convergence"},
+                   "note": "one 'step' here is the whole batch run to convergence; evals count N K per step, with those "
+                           "that the kept bounds make unnecessary"},
            "gpu_launches": int(2 * 8 * ((int(iters.max()) + 7) // 8)) + (2 if tile > 1024 else 0), "roofline": roof,
            "time_to_converge_s": batch_s, "plain_sequential_s": plain_s * scale,
            "plain_sequential_warm_graph_s": plain_warm_s * scale,
