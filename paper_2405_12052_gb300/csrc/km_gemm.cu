@@ -54,7 +54,7 @@ constexpr int kPtStride = kSlots * kHalf * 2 + 16;  // bytes per point (padding 
 constexpr int kTileBytes = kGM * kGemmD * 2;   // 16 KB of 16-bit operands per point tile
 constexpr int kTieMax = 20;       // candidates per near-tie list entry (48 bytes)
 constexpr int64_t kRescueTileMin = int64_t(1) << 20;  // points from which the rescue list is taken in tiles
-constexpr int kTieChunk = 64;     // near-tie entries an epilogue warp reserves at a time
+constexpr int kTieChunk = 64;     // near-tie entries an epilogue warp reserves at a time, at most
 // shared-memory layout (bytes from the 1024-aligned base)
 constexpr int kOffStore = 0;                                  // [128][kPtStride] bytes
 constexpr int kOffSk = kOffStore + kGM * kPtStride;           // [128][kSlots] int16
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_assign_kernel(GemmArgs a) {
     int gcount = 0;
     int nflag = 0, nresc = 0;
     // this warp's reserved near-tie entries [tnext, tend): one global atomic
-    // per kTieChunk entries instead of one per warp and tile (every warp of
+    // per tie_chunk entries instead of one per warp and tile (every warp of
     // the grid adds to the same counter)
     unsigned tnext = 0, tend = 0;
     // per-point inputs of the next tile are loaded one tile ahead: z and
@@ -495,10 +495,10 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_assign_kernel(GemmArgs a) {
         const unsigned ntie = (unsigned)__popc(btie), rem = tend - tnext, t0 = tnext;
         unsigned t1 = 0, base_r = 0;
         if (ntie > rem) {  // warp-uniform
-          if (lane == 0) t1 = atomicAdd(a.tie_count, (unsigned)kTieChunk);
+          if (lane == 0) t1 = atomicAdd(a.tie_count, a.tie_chunk);
           t1 = __shfl_sync(0xffffffffu, t1, 0);
           tnext = t1 + (ntie - rem);
-          tend = t1 + kTieChunk;
+          tend = t1 + a.tie_chunk;
         } else {
           tnext += ntie;
         }
@@ -1090,7 +1090,15 @@ size_t gemm_smem_bytes(int kpad) {
 
 int64_t gemm_xb_rows(int64_t n) { return (n + kGM - 1) / kGM * kGM; }
 
-cudaError_t launch_gemm_assign(int grid, cudaStream_t st, const GemmArgs& a) {
+cudaError_t launch_gemm_assign(int grid, cudaStream_t st, const GemmArgs& args) {
+  GemmArgs a = args;
+  // a sixteenth of a warp's points, 8 (a tile's near ties of a warp) to
+  // kTieChunk: the tie kernel also walks over the unused entries of every
+  // warp's last chunk, with 64 of them four times the entries in use at 2e5
+  // points, K = 100 (tie kernel 42 -> 36 us)
+  const int64_t share = a.n / ((int64_t)grid * kEpiWarps * 16);
+  a.tie_chunk = 8;
+  while (a.tie_chunk < (unsigned)kTieChunk && (int64_t)a.tie_chunk < share) a.tie_chunk *= 2;
   const size_t smem = gemm_smem_bytes(a.kpad);
   cudaError_t e = cudaFuncSetAttribute(gemm_assign_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

@@ -203,6 +203,7 @@ struct GemmArgs {
   unsigned* rescue_count;  // [0] rescue entries, [1] near-tie entries, [2] second rescue list
   unsigned* rescue_count2; // = rescue_count + 2
   unsigned* tie_count;     // = rescue_count + 1
+  unsigned tie_chunk;      // entries reserved at a time (set at the launch)
   int64_t n;
   int k, kpad, ntiles;
   int f16;               // operands are FP16 (scaled by powers of two), else BF16

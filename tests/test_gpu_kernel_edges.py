@@ -164,10 +164,11 @@ def test_generic_tile_edges(km, oracle, n, d, k, kw):
     g.close()
 
 
-# the sorted sums' small and large chunks (2^21 points), several steps past
-# the stop inside one graph, and a step after a converged run (its tables must
-# be the final centroids')
-@pytest.mark.parametrize("n,k,ops", [(5, 3, "bf16"), (20_001, 40, "f16"), (60_000, 300, "bf16"), (2_100_000, 16, "bf16")])
+# the sorted sums' small and large chunks (2^21 points), each reservation of
+# near-tie entries, several steps past the stop inside one graph, and a step
+# after a converged run (its tables must be the final centroids')
+@pytest.mark.parametrize("n,k,ops", [(5, 3, "bf16"), (20_001, 40, "f16"), (60_000, 300, "bf16"), (700_001, 32, "bf16"),
+                                     (2_100_000, 16, "bf16")])
 def test_tensor_run_and_step_after_it(km, oracle, n, k, ops):
     x, _, _ = synth.iso_mixture(n, 64, max(2, k // 2), sigma=1.0, box=6.0, seed=n)
     mu0, _ = synth.init_distinct(x, k, seed=5)
