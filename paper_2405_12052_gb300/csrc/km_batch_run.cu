@@ -20,7 +20,7 @@
 // Bound by issue while many points are open (0.67 ms the first step), by the
 // latency of a tile's dependent loads afterwards (about 90 us a step over 4.6e7
 // points, 35 us at the memory's rate).  256 instances, 4.6e7 points, K 4 to 64,
-// 300 steps: 150 -> 55 ms without the copy of the labels.  Slower: a separate
+// 300 steps: 150 -> 52 ms without the copy of the labels.  Slower: a separate
 // kernel with 48 warps an SM that tests the bounds and lists open points for two
 // more (69 ms: the points' second pass costs more than the first one gains); a
 // warp per tile of an eighth (100 ms: the warps of an SM then run the tables and
