@@ -484,8 +484,12 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_assign_kernel(GemmArgs a) {
         // candidates of the point's threads with a lower sub
         const int before = sub == 0 ? 0 : sub == 1 ? n1 : sub == 2 ? n2 + n3 : n1 + n2 + n3;
         const bool live = ii < a.n;
+        // no finite threshold: the screen says nothing (values past its binade,
+        // see the consts kernel), and the point goes to the rescue list whatever
+        // was stored (NaN halves are not, padding columns may be)
+        const bool open = tb >= 0x7f800000u;
         // kind: 1 = decided here, 2 = near tie, 3 = rescue
-        const int kind = !live ? 0 : (over || tot == 0 || tot > kTieMax) ? 3 : tot == 1 ? 1 : 2;
+        const int kind = !live ? 0 : (open || over || tot == 0 || tot > kTieMax) ? 3 : tot == 1 ? 1 : 2;
         // list slots: near ties from the warp's reserved entries (a new
         // chunk when they run out; the rest of the old one is used first),
         // rescues by one atomic per warp (rare)
@@ -874,13 +878,14 @@ __global__ void __launch_bounds__(256) gemm_rescue_kernel(GemmArgs a) {
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
-    const float hi1 = best + bound64(best, sA, sB, AB);
+    // no FP32 distance below the start value: every centroid is a candidate
+    const float hi1 = best < 3.0e38f ? best + bound64(best, sA, sB, AB) : __int_as_float(0x7f800000);
     double bd = 0.0;
     int k64 = -1;
 #pragma unroll
     for (int t = 0; t < kGemmMaxK / 32; ++t) {
       const int c = lane + 32 * t;
-      if (c < a.k && dv[t] - bound64(dv[t], sA, sB, AB) <= hi1) {
+      if (c < a.k && !(dv[t] - bound64(dv[t], sA, sB, AB) > hi1)) {  // an infinity or NaN stays a candidate
         const double dd = d64row(xr, a.mu + (size_t)c * kGemmD);
         if (k64 < 0 || dd < bd || (dd == bd && c < k64)) { bd = dd; k64 = c; }
       }
@@ -1000,6 +1005,10 @@ __global__ void __launch_bounds__(256) gemm_consts_kernel(GemmPrepArgs a) {
     const float P = __fmul_ru(1.02f, __fadd_ru(a.A_max, 2.f * bmax));
     // binade [1, 2): M = 1.5, |2^sigma (h - 2S)| < 0.5; P in [2^e, 2^(e+1))
     const int e = (int)(__float_as_uint(P) >> 23) - 127;
+    // squares so large that the scale leaves FP32's range (|x| from about 1e17):
+    // values leave the binade, so an infinite window sends every point to the
+    // rescue kernels
+    const bool out = -2 - e < -120;
     const int sigma = max(-120, min(120, -2 - e));
     s_sigma = sigma;
     const float u = 0x1p-24f, tw = gpow2(sigma), tr = (float)a.tie_rel;
@@ -1033,7 +1042,8 @@ __global__ void __launch_bounds__(256) gemm_consts_kernel(GemmPrepArgs a) {
     // each, the oracle's FP64 error, tie_rel * D2 with D2 <= (||x~|| + ||c~||)^2,
     // four ulps of the binade
     const float up = 1.f + 1.01e-3f;
-    g.c0 = (tw * ((2.f * u + gam + tr) * bmax + 4.f * (8.f * (1.f + v) * ax * sB + 64.f * ax * ac)) + 8.f * 0x1p-23f) * up;
+    g.c0 = out ? __uint_as_float(0x7f800000u)
+               : (tw * ((2.f * u + gam + tr) * bmax + 4.f * (8.f * (1.f + v) * ax * sB + 64.f * ax * ac)) + 8.f * 0x1p-23f) * up;
     g.c1 = tw * ((4.f * epsS + 2.f * tr) * sB + 32.f * (1.f + v) * ac) * up;
     g.cA = tw * (gam + tr) * up;
     // start estimate: |r_est - r_tc| <= 2^(sigma+1) (2^-16 + 2^-18) ||x_b|| ||c_b|| (two FP32
