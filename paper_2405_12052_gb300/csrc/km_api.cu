@@ -26,6 +26,15 @@ bool inject_alloc_failure() {
   }
   return false;
 }
+cudaError_t max_dynamic_smem(const void* fn, int* bytes) {
+  int dev = 0, optin = 0;
+  cudaFuncAttributes fa{};
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fn);
+  if (e == cudaSuccess) *bytes = optin - (int)fa.sharedSizeBytes;
+  return e;
+}
 // The fused kernel's constant-bank screen table exists once per device (a
 // module-level __constant__ array), so at most one context per device may use
 // it at a time: the context that claims it at km_create keeps it until

@@ -137,7 +137,7 @@ size_t fast_smem_bytes(int d, int kpad, int k, int nwin) {
 template <int D, int KG, bool CT>
 static cudaError_t launch_fast_dk(int grid, size_t smem, cudaStream_t st, const FastArgs& a) {
   auto fn = assign_fast_kernel<D, KG, CT>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_max_smem<assign_fast_kernel<D, KG, CT>>();
   if (e != cudaSuccess) return e;
   if constexpr (CT) {
     e = cudaMemcpyToSymbolAsync(c_screen_tab, a.tab2, (size_t)a.kpad * (D + 1) * sizeof(unsigned long long), 0,
@@ -151,7 +151,7 @@ static cudaError_t launch_fast_dk(int grid, size_t smem, cudaStream_t st, const 
 template <int D, int KG, bool CT>
 static int blocks_dk(size_t smem) {
   int nb = 0;
-  cudaFuncSetAttribute(assign_fast_kernel<D, KG, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_max_smem<assign_fast_kernel<D, KG, CT>>();
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, assign_fast_kernel<D, KG, CT>, kThreads, smem) !=
       cudaSuccess)
     return 1;

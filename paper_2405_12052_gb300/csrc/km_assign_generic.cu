@@ -296,8 +296,7 @@ GenericPlan generic_plan(int d, int k) {
 int64_t generic_grid(int64_t n, int d, int k, int sms) {
   const GenericPlan g = generic_plan(d, k);
   int nb = 0;
-  if (cudaFuncSetAttribute(assign_generic_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem) !=
-          cudaSuccess ||
+  if (allow_max_smem<assign_generic_kernel>() != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, assign_generic_kernel, kThreads, g.smem) != cudaSuccess ||
       nb < 1)
     nb = 1;
@@ -306,7 +305,7 @@ int64_t generic_grid(int64_t n, int d, int k, int sms) {
 
 cudaError_t launch_assign_generic(int grid, cudaStream_t st, const GenericArgs& a) {
   const GenericPlan g = generic_plan(a.d, a.k);
-  cudaError_t e = cudaFuncSetAttribute(assign_generic_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+  cudaError_t e = allow_max_smem<assign_generic_kernel>();
   if (e != cudaSuccess) return e;
   assign_generic_kernel<<<grid, kThreads, g.smem, st>>>(a, g.use_win, g.tot_sh);
   return cudaGetLastError();

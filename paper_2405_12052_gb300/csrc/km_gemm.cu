@@ -1110,7 +1110,7 @@ cudaError_t launch_gemm_assign(int grid, cudaStream_t st, const GemmArgs& args) 
   a.tie_chunk = 8;
   while (a.tie_chunk < (unsigned)kTieChunk && (int64_t)a.tie_chunk < share) a.tie_chunk *= 2;
   const size_t smem = gemm_smem_bytes(a.kpad);
-  cudaError_t e = cudaFuncSetAttribute(gemm_assign_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_max_smem<gemm_assign_kernel>();
   if (e != cudaSuccess) return e;
   // the three list lengths are adjacent: one memset clears them
   e = cudaMemsetAsync(a.rescue_count, 0, 3 * sizeof(unsigned), st);

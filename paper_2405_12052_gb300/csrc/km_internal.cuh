@@ -28,6 +28,7 @@
 // partials are reduced in a fixed order in int128 and converted once.
 #pragma once
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -379,6 +380,25 @@ int64_t objective_chunks(int64_t n);
 cudaError_t launch_widen_labels(const uint8_t* z8, int32_t* z, int64_t n, cudaStream_t st);
 cudaError_t launch_objective(const float* x, int64_t ld, int64_t n, int d, const double* mu, const int32_t* z,
                              const uint8_t* z8, double* part, double* out, cudaStream_t st);
+
+// The limit on a kernel's dynamic shared memory belongs to the function, not to
+// a launch: a limit set to one context's size can be lowered by another
+// thread's context between the call that sets it and the launch that needs it.
+// So kernels whose size depends on K, d or the padding get the device's largest
+// limit, the same value from every caller.  max_dynamic_smem: that limit for fn
+// (the opt-in maximum less its static shared memory).
+cudaError_t max_dynamic_smem(const void* fn, int* bytes);
+template <auto Fn>
+cudaError_t allow_max_smem() {
+  static std::atomic<int> limit{0};
+  int v = limit.load(std::memory_order_relaxed);
+  if (v == 0) {
+    cudaError_t e = max_dynamic_smem(reinterpret_cast<const void*>(Fn), &v);
+    if (e != cudaSuccess) return e;
+    limit.store(v, std::memory_order_relaxed);
+  }
+  return cudaFuncSetAttribute(reinterpret_cast<const void*>(Fn), cudaFuncAttributeMaxDynamicSharedMemorySize, v);
+}
 
 // Host-side launchers (defined in the .cu files).
 cudaError_t launch_assign_fast(int d, int grid, size_t smem, cudaStream_t st, const FastArgs& a);

@@ -325,8 +325,7 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
 template <int D, int KG>
 int run_blocks(size_t smem) {
   int nb = 0;
-  if (cudaFuncSetAttribute(run_fast_kernel<D, KG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-          cudaSuccess ||
+  if (allow_max_smem<run_fast_kernel<D, KG>>() != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, run_fast_kernel<D, KG>, kThreads, smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
@@ -336,7 +335,7 @@ int run_blocks(size_t smem) {
 
 template <int D, int KG>
 cudaError_t run_launch(int grid, size_t smem, cudaStream_t st, const RunArgs& a) {
-  cudaError_t e = cudaFuncSetAttribute(run_fast_kernel<D, KG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_max_smem<run_fast_kernel<D, KG>>();
   if (e != cudaSuccess) return e;
   void* args[] = {const_cast<RunArgs*>(&a)};
   return cudaLaunchCooperativeKernel(reinterpret_cast<void*>(run_fast_kernel<D, KG>), dim3(grid), dim3(kThreads), args,

@@ -446,7 +446,7 @@ cudaError_t launch_setnet_forward(const SetNetArgs& a, bool train, cudaStream_t 
                                               : launch_fwd_points<64>(a, train, P, st);
   if (e != cudaSuccess) return e;
   const size_t hs = sizeof(float) * (size_t)std::max(H, a.k * a.d) * kWS;
-  e = cudaFuncSetAttribute(sn_head, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hs);
+  e = allow_max_smem<sn_head>();
   if (e != cudaSuccess) return e;
   sn_head<<<a.B, 256, hs, st>>>(a.prm, a.tile_pool, a.S / kTileP, a.S, a.B, a.d, a.k, train ? a.ts : nullptr, a.G, a.P,
                                 a.A3, a.dZ3, a.dP, a.dG, a.set_loss);
