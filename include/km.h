@@ -415,9 +415,11 @@ km_status km_setnet_set_params(km_setnet* net, const float* params);
 km_status km_setnet_get_params(km_setnet* net, float* params_out);
 /* Forward, loss and backward on a batch of B sets; the gradients stay on the
  * device (km_setnet_get_grads copies them).  loss_out (host) may be NULL
- * (then nothing synchronizes).  KM_ETIMEOUT, here or from km_setnet_get_grads:
- * a bounded wait of the backward kernel gave up; the gradients are not to be
- * used. */
+ * (then nothing synchronizes).  KM_ETIMEOUT, here or from km_setnet_get_grads or
+ * km_setnet_train_step: a bounded wait of the backward kernel gave up in this
+ * pass, whose gradients are not to be used, or in an earlier one whose loss was
+ * not read (reported once).  An Adam step on such a pass changes nothing, and
+ * the next pass starts afresh. */
 km_status km_setnet_loss_grad(km_setnet* net, const float* x, const float* targets, int32_t B, int32_t S,
                               int32_t mem, float* loss_out);
 km_status km_setnet_get_grads(km_setnet* net, float* grads_out);
@@ -429,6 +431,8 @@ km_status km_setnet_train_step(km_setnet* net, const float* x, const float* targ
 /* Centres for each of B sets: centroids_out [B][K][d] doubles (host or device). */
 km_status km_setnet_predict(km_setnet* net, const float* x, int32_t B, int32_t S, int32_t mem,
                             double* centroids_out);
+/* Testing hook: marks the last backward pass as one whose bounded wait gave up. */
+km_status km_debug_setnet_pass_gave_up(km_setnet* net);
 const char* km_setnet_last_error(const km_setnet* net);
 void km_setnet_destroy(km_setnet* net);
 

@@ -162,6 +162,8 @@ def lib(path: str | None = None):
     L.km_setnet_train_step.restype = st
     L.km_setnet_predict.argtypes = [P, P, i32, i32, i32, P]
     L.km_setnet_predict.restype = st
+    L.km_debug_setnet_pass_gave_up.argtypes = [P]
+    L.km_debug_setnet_pass_gave_up.restype = st
     L.km_setnet_last_error.argtypes = [P]
     L.km_setnet_last_error.restype = ctypes.c_char_p
     L.km_setnet_destroy.argtypes = [P]
@@ -758,6 +760,11 @@ class SetNet:
         self._check(self._L.km_setnet_train_step(self._h, px, pt, B, S, mx, float(lr),
                                                  ctypes.byref(loss) if want_loss else None))
         return float(loss.value) if want_loss else None
+
+    def debug_pass_gave_up(self):
+        """Testing hook: marks the last backward pass as one whose bounded
+        wait gave up."""
+        self._check(self._L.km_debug_setnet_pass_gave_up(self._h))
 
     def predict(self, x) -> np.ndarray:
         B, S = int(x.shape[0]), int(x.shape[1])

@@ -353,7 +353,7 @@ struct SetNetArgs {
   float* w2t; uint32_t* bits; float* tile_pool; float* G; float* P; float* dG; float* loss;
   float* A3; float* dZ3; float* dP; float* set_loss;  // [B][H], [B][H], [B][K d], [B]: head values of each set
   float* part;
-  int* err;           // set to 3 when a bounded wait of the backward kernel gives up
+  int* err;           // [2] set to 3 when a bounded wait of the backward kernel gives up
 };
 constexpr int kSetBwdBlocks = 152;  // backward blocks at most: one per SM
 int setnet_param_count(int d, int k);
@@ -363,7 +363,7 @@ cudaError_t launch_setnet_bwd_points(const SetNetArgs& a, int blocks, cudaStream
 cudaError_t launch_setnet_forward(const SetNetArgs& a, bool train, cudaStream_t st);
 cudaError_t launch_setnet_backward(const SetNetArgs& a, cudaStream_t st);
 cudaError_t launch_setnet_adam(float* prm, const float* grads, float* m, float* v, int n, float lr, float b1,
-                               float b2, float eps, float c1, float c2, cudaStream_t st);
+                               float b2, float eps, float c1, float c2, const int* err, int* skipped, cudaStream_t st);
 cudaError_t launch_setnet_sample(const float* x, int64_t ld, int64_t n, int d, int S, unsigned long long seed,
                                  float* out, cudaStream_t st);
 // Set transforms of the learned initialiser: per-set FP64 means, and

@@ -377,9 +377,14 @@ __global__ void __launch_bounds__(64) sn_wgrad_reduce(const float* __restrict__ 
   grads[dst] = s;
 }
 
+// The gradients of a pass that gave up (*err) are not taken.
 __global__ void sn_adam(float* prm, const float* grads, float* m, float* v, int n, float lr, float b1, float b2,
-                        float eps, float c1, float c2) {
+                        float eps, float c1, float c2, const int* err, int* skipped) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (*err) {
+    if (q == 0) *skipped += 1;
+    return;
+  }
   if (q >= n) return;
   const float g = grads[q];
   const float mq = b1 * m[q] + (1.f - b1) * g;
@@ -469,8 +474,9 @@ cudaError_t launch_setnet_backward(const SetNetArgs& a, cudaStream_t st) {
 int64_t setnet_part_floats(int d) { return (int64_t)kSetBwdBlocks * (H * H + H * d + 2 * H); }
 
 cudaError_t launch_setnet_adam(float* prm, const float* grads, float* m, float* v, int n, float lr, float b1,
-                               float b2, float eps, float c1, float c2, cudaStream_t st) {
-  sn_adam<<<(n + 255) / 256, 256, 0, st>>>(prm, grads, m, v, n, lr, b1, b2, eps, c1, c2);
+                               float b2, float eps, float c1, float c2, const int* err, int* skipped,
+                               cudaStream_t st) {
+  sn_adam<<<(n + 255) / 256, 256, 0, st>>>(prm, grads, m, v, n, lr, b1, b2, eps, c1, c2, err, skipped);
   return cudaGetLastError();
 }
 

@@ -29,6 +29,13 @@ struct km_setnet {
 
 namespace {
 
+// Words behind the loss: set to 3 by the backward kernel when a bounded wait
+// gives up in this pass (cleared before each pass); the same until it has been
+// reported (a pass whose loss nobody reads is reported by the next call that
+// reads a result); Adam steps not taken on a pass that gave up.
+enum { kErrPass = 1, kErrAny = 2, kErrSkipped = 3, kLossWords = 4 };
+int* err_word(km_setnet* n, int w) { return reinterpret_cast<int*>(n->loss) + w; }
+
 km_status nfail(km_setnet* n, km_status s, const std::string& m) {
   n->err = m;
   return s;
@@ -95,7 +102,7 @@ SetNetArgs args(km_setnet* n, const float* x, const float* t, int B, int S) {
   a.xs = n->xs; a.ts = n->ts; a.ms = n->ms; a.w2t = n->w2t; a.bits = n->bits;
   a.tile_pool = n->tile_pool; a.G = n->G; a.P = n->P; a.dG = n->dG; a.loss = n->loss;
   a.A3 = n->A3; a.dZ3 = n->dZ3; a.dP = n->dP; a.set_loss = n->set_loss; a.part = n->part;
-  a.err = reinterpret_cast<int*>(n->loss + 1);
+  a.err = err_word(n, kErrPass);
   return a;
 }
 
@@ -155,8 +162,8 @@ km_status km_setnet_create(km_setnet** out, int32_t d, int32_t k, void* stream) 
   KN_CUDA(n, nalloc(&n->m, (size_t)n->nparam));
   KN_CUDA(n, nalloc(&n->v, (size_t)n->nparam));
   KN_CUDA(n, nalloc(&n->w2t, (size_t)kSetH * kSetH));
-  KN_CUDA(n, nalloc(&n->loss, 2));  // the loss and the error word of the backward kernel
-  KN_CUDA(n, cudaMemsetAsync(n->loss, 0, 2 * sizeof(float), n->st));
+  KN_CUDA(n, nalloc(&n->loss, kLossWords));  // the loss and the error words
+  KN_CUDA(n, cudaMemsetAsync(n->loss, 0, kLossWords * sizeof(float), n->st));
   KN_CUDA(n, cudaMemsetAsync(n->prm, 0, sizeof(float) * n->nparam, n->st));
   KN_CUDA(n, cudaMemsetAsync(n->grads, 0, sizeof(float) * n->nparam, n->st));
   KN_CUDA(n, cudaMemsetAsync(n->m, 0, sizeof(float) * n->nparam, n->st));
@@ -172,6 +179,7 @@ km_status km_setnet_set_params(km_setnet* n, const float* params) {
   KN_CUDA(n, cudaMemcpyAsync(n->prm, params, sizeof(float) * n->nparam, cudaMemcpyHostToDevice, n->st));
   KN_CUDA(n, cudaMemsetAsync(n->m, 0, sizeof(float) * n->nparam, n->st));
   KN_CUDA(n, cudaMemsetAsync(n->v, 0, sizeof(float) * n->nparam, n->st));
+  KN_CUDA(n, cudaMemsetAsync(err_word(n, kErrSkipped), 0, sizeof(int), n->st));
   KN_CUDA(n, cudaStreamSynchronize(n->st));
   n->adam_t = 0;
   return KM_OK;
@@ -184,12 +192,20 @@ km_status km_setnet_get_params(km_setnet* n, float* params_out) {
   return KM_OK;
 }
 
-// The loss and the error word of the last backward pass (synchronizes).
+// The loss and the error words (synchronizes): of the last backward pass, and of
+// any before it that has not been reported.
 static km_status read_loss(km_setnet* n, float* loss_out) {
-  struct { float loss; int32_t err; } h{};
+  struct { float loss; int32_t pass, any, skipped; } h{};
+  static_assert(sizeof(h) == kLossWords * sizeof(float), "the words behind the loss");
   KN_CUDA(n, cudaMemcpyAsync(&h, n->loss, sizeof(h), cudaMemcpyDeviceToHost, n->st));
   KN_CUDA(n, cudaStreamSynchronize(n->st));
-  if (h.err) return nfail(n, KM_ETIMEOUT, "a bounded device wait gave up (error word " + std::to_string(h.err) + ")");
+  if (h.pass || h.any) {
+    n->adam_t -= h.skipped;  // those steps were not taken
+    KN_CUDA(n, cudaMemsetAsync(err_word(n, kErrAny), 0, 2 * sizeof(int), n->st));
+    return nfail(n, KM_ETIMEOUT, std::string("a bounded device wait gave up in ") +
+                                     (h.pass ? "the last backward pass" : "an earlier backward pass") + " (error word " +
+                                     std::to_string(h.pass ? h.pass : h.any) + ")");
+  }
   if (loss_out) *loss_out = h.loss;
   return KM_OK;
 }
@@ -208,6 +224,7 @@ km_status km_setnet_loss_grad(km_setnet* n, const float* x, const float* targets
   if (s != KM_OK) return s;
   SetNetArgs a = args(n, xd, td, B, S);
   KN_CUDA(n, launch_setnet_forward(a, true, n->st));
+  KN_CUDA(n, cudaMemsetAsync(a.err, 0, sizeof(int), n->st));
   KN_CUDA(n, launch_setnet_backward(a, n->st));
   return loss_out ? read_loss(n, loss_out) : KM_OK;
 }
@@ -218,7 +235,15 @@ km_status km_setnet_adam(km_setnet* n, float lr, float beta1, float beta2, float
   const double c1 = 1.0 - std::pow((double)beta1, (double)n->adam_t);
   const double c2 = 1.0 - std::pow((double)beta2, (double)n->adam_t);
   KN_CUDA(n, launch_setnet_adam(n->prm, n->grads, n->m, n->v, n->nparam, lr, beta1, beta2, eps, (float)c1,
-                                (float)c2, n->st));
+                                (float)c2, err_word(n, kErrPass), err_word(n, kErrSkipped), n->st));
+  return KM_OK;
+}
+
+km_status km_debug_setnet_pass_gave_up(km_setnet* n) {
+  if (!n) return KM_EINVAL;
+  const int32_t w[2] = {3, 3};
+  KN_CUDA(n, cudaMemcpyAsync(err_word(n, kErrPass), w, sizeof(w), cudaMemcpyHostToDevice, n->st));
+  KN_CUDA(n, cudaStreamSynchronize(n->st));
   return KM_OK;
 }
 

@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kBwThreads, 1) sn_bwd_points(const float* __re
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");  // the accumulators may be rewritten
     if (__syncthreads_or(bad ? 1 : 0)) {
-      if (tid == 0) *err = 3;  // a wait gave up
+      if (tid == 0) { err[0] = 3; err[1] = 3; }  // a wait gave up: in this pass, and not yet reported
       break;
     }
   }
