@@ -281,6 +281,15 @@ cudaError_t launch_step(km_ctx* c) {
 // Shape and buffers of the whole-run kernel, at the context's first graph-
 // driven run.  Without the memory for them the step kernels' graph runs
 // instead, as it does for more points than a resident grid's int64 sums take.
+void release_run(km_ctx* c) {
+  void* bufs[] = {c->slack, c->zrun, c->run_delta, c->run_tot, c->run_tot0, c->run_cum0, c->run_priv};
+  for (void* b : bufs)
+    if (b) cudaFree(b);
+  c->slack = nullptr; c->zrun = nullptr; c->run_delta = nullptr; c->run_tot = nullptr; c->run_tot0 = nullptr;
+  c->run_cum0 = nullptr; c->run_priv = nullptr;
+  cudaGetLastError();
+}
+
 bool run_ready(km_ctx* c) {
   if (c->run_state) return c->run_state > 0;
   c->run_state = -1;
@@ -309,12 +318,7 @@ bool run_ready(km_ctx* c) {
       dalloc(&c->run_tot, (size_t)g * kd * 4) != cudaSuccess || dalloc(&c->run_tot0, kd * 4) != cudaSuccess ||
       dalloc(&c->run_cum0, (size_t)c->k) != cudaSuccess ||
       (!sh && dalloc(&c->run_priv, (size_t)g * priv) != cudaSuccess)) {
-    void* bufs[] = {c->slack, c->zrun, c->run_delta, c->run_tot, c->run_tot0, c->run_cum0, c->run_priv};
-    for (void* b : bufs)
-      if (b) cudaFree(b);
-    c->slack = nullptr; c->zrun = nullptr; c->run_delta = nullptr; c->run_tot = nullptr; c->run_tot0 = nullptr;
-    c->run_cum0 = nullptr; c->run_priv = nullptr;
-    cudaGetLastError();
+    release_run(c);
     return false;
   }
   c->run_state = 1;
@@ -323,9 +327,12 @@ bool run_ready(km_ctx* c) {
 
 // The steps of a run: launches of the whole-run kernel until the stop rule
 // has fired, each of at most 64 steps (so that the host keeps control of long
-// runs); then the labels.
+// runs); then the labels.  *ran is false when the kernel cannot be launched on
+// the context's stream (one that owns fewer SMs than its grid needs, for
+// instance): nothing has run then, and the context keeps to the step kernels.
 km_status read_state(km_ctx* c);
-km_status run_whole(km_ctx* c) {
+km_status run_whole(km_ctx* c, bool* ran) {
+  *ran = true;
   RunArgs r{};
   r.f.x = c->x; r.f.ld = c->ld; r.f.n = c->n; r.f.k = c->k; r.f.kpad = c->kpad;
   r.f.dc = c->dc; r.f.ls = c->ls; r.f.ntiles = (c->n + kWarpTile - 1) / kWarpTile; r.f.nwin = c->nwin;
@@ -346,7 +353,14 @@ km_status run_whole(km_ctx* c) {
   // one pass over the points takes far less: K N evaluations at 1e11 a second
   r.wait_ns = 2000000000ull + (unsigned long long)((double)c->n * c->k * 0.01);
   while (true) {
-    KM_CUDA(c, launch_run_fast(c->d, c->run_grid, c->run_smem, c->st, r));
+    const cudaError_t e = launch_run_fast(c->d, c->run_grid, c->run_smem, c->st, r);
+    if (e != cudaSuccess && !r.resume) {
+      release_run(c);
+      c->run_state = -1;
+      *ran = false;
+      return KM_OK;
+    }
+    KM_CUDA(c, e);
     r.resume = 1;
     km_status s = read_state(c);
     if (s != KM_OK) return s;
@@ -831,11 +845,13 @@ km_status km_run(km_ctx* c, int32_t max_iter, double tol, int32_t* labels_out,
     s = write_control(c, 0, start + max_iter, tol);
     if (s != KM_OK) return s;
     if (c->opt.use_graph && run_ready(c)) {
-      s = run_whole(c);
+      s = run_whole(c, &ran);
       if (s != KM_OK) return s;
-    } else if (c->opt.use_graph) {
+    }
+    if (!ran && c->opt.use_graph) {
       if (!c->graph) {
         cudaGraph_t g = nullptr;
+    bool ran = false;
         KM_CUDA(c, cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal));
         cudaError_t e = cudaSuccess;
         // the tensor-core path's steps are many kernels, so fewer of them run
@@ -855,7 +871,7 @@ km_status km_run(km_ctx* c, int32_t max_iter, double tol, int32_t* labels_out,
         if (s != KM_OK) return s;
         if (c->host_ls.done) break;
       }
-    } else {
+    } else if (!ran) {
       while (true) {
         KM_CUDA(c, launch_step(c));
         s = read_state(c);

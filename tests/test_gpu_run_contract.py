@@ -1,0 +1,61 @@
+"""What calls around a whole run (km_run in one kernel) see: its last step's sums,
+its counters, and streams its grid does not fit on."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def km():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2405_12052_gb300 as m
+    m.build()
+    return m
+
+
+def _green_stream(dev, sms):
+    """A stream that owns at least `sms` SMs of the device (a green context), or None."""
+    try:
+        cu = ctypes.CDLL("libcuda.so.1")
+        split, gen, create, stream = (getattr(cu, f) for f in ("cuDevSmResourceSplitByCount", "cuDevResourceGenerateDesc",
+                                                              "cuGreenCtxCreate", "cuGreenCtxStreamCreate"))
+    except (OSError, AttributeError):
+        return None
+    res, part, rest = (ctypes.create_string_buffer(256) for _ in range(3))  # CUdevResource: 144 bytes
+    groups = ctypes.c_uint(1)
+    desc, ctx, st = ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_void_p()
+    if cu.cuDeviceGetDevResource(dev, res, 1) or split(part, ctypes.byref(groups), res, rest, 0, sms):
+        return None
+    if gen(ctypes.byref(desc), part, 1) or create(ctypes.byref(ctx), desc, dev, 1):
+        return None
+    return None if stream(ctypes.byref(st), ctx, 1, 0) else st.value
+
+
+# a stream on part of the GPU: the run's grid, sized for all of it, is not resident
+# there, and the step kernels' graph runs instead
+@pytest.mark.parametrize("n,d,k,kw", [(200_000, 3, 11, {}), (3_000_000, 2, 8, {"label_bytes": 1})])
+def test_run_on_a_stream_with_fewer_sms(km, oracle, n, d, k, kw):
+    import torch
+    torch.cuda.init()
+    torch.zeros(1, device="cuda")
+    st = _green_stream(0, 16)
+    if st is None:
+        pytest.skip("no green contexts here")
+    x, _, _ = synth.iso_mixture(n, d, k, sigma=1.0, box=8.0, seed=n)
+    mu0, _ = synth.init_distinct(x, k, seed=3)
+    ref = oracle.run(x, mu0, 6, 0.0)
+    g = km.KMeans(n, d, k, stream=st, **kw)
+    g.set_points(x)
+    for _ in range(2):
+        g.set_init(mu0)
+        r = g.run(6, 0.0)
+        assert r["iters"] == ref["iters"] and np.array_equal(r["labels"], ref["labels"])
+        assert np.allclose(r["centroids"], ref["centroids"], rtol=1e-6, atol=1e-6)
+    g.close()
