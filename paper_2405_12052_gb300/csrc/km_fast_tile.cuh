@@ -838,8 +838,9 @@ __device__ __forceinline__ void run_pass(const FastArgs& a, FastSmem<D>& sm, con
           if (qn > kWarpQueue - kWarpTile) break;  // empty the queue first
           fetch(xb, t);
           asm volatile("cp.async.wait_group 0;" ::: "memory");
+          nflag += total + qn;
           whole(t, mb + u, xb);
-          nflag += total;
+          nflag -= qn;  // what it queued is counted when the queue is emptied
         } else {
           if (qn > kQueueFull) break;
           fetch(xb, t);

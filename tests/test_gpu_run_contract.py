@@ -20,6 +20,33 @@ def km():
     return m
 
 
+# no point is counted twice in a step.  At this magnitude the screen flags every
+# point it decides; the start lies in a corner of the data, so the first moves open
+# whole tiles again
+@pytest.mark.parametrize("how", ["run", "batch"])
+def test_flagged_points_are_counted_once(km, how):
+    n, k, steps = 20_000, 20, 2
+    x, _, _ = synth.iso_mixture(n, 3, 10, sigma=1.0, box=8.0, seed=5)
+    x = (x.astype(np.float64) * 1e17).astype(np.float32)
+    mu0, _ = synth.init_distinct(x, k, seed=6)
+    mu0 = mu0.min(0) + 0.05 * (mu0 - mu0.min(0))
+    if how == "run":
+        g = km.KMeans(n, 3, k)
+        g.set_points(x)
+        g.set_init(mu0)
+        g.run(steps, 0.0)
+        assert 0 < g.stats()["flagged"] <= n
+        g.close()
+    else:
+        b = km.KMeansBatch([n], [3], [k])
+        b.set_points([x])
+        b.set_init([mu0])
+        b.set_shape(8192, 256)
+        b.run(steps, 0.0)
+        assert 0 < b.info()["flagged"] <= steps * n
+        b.close()
+
+
 def _green_stream(dev, sms):
     """A stream that owns at least `sms` SMs of the device (a green context), or None."""
     try:
