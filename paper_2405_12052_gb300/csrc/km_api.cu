@@ -130,6 +130,8 @@ struct km_ctx {
   long long *run_tot = nullptr, *run_tot0 = nullptr;
   float* run_cum0 = nullptr;
   unsigned char* run_priv = nullptr;
+  bool run_totals = false;     // the last step's sums are in run_tot0 (a whole run), not in partials
+  bool armed = false;          // the stop flag has been cleared since then: an assignment writes partials
   // loop
   cudaGraphExec_t graph = nullptr;
   int graph_unroll = 16;
@@ -219,6 +221,7 @@ cudaError_t launch_tables(km_ctx* c) {
 cudaError_t launch_assign(km_ctx* c, bool labels_pass = false) {
   cudaError_t e;
   const int store = (c->opt.label_policy == KM_LABELS_EVERY_STEP || labels_pass) ? 1 : 0;
+  if (labels_pass || c->armed) c->run_totals = false;
   if (c->path == 3) {
     GemmArgs g{};
     g.xb = c->xb; g.xa = c->xa_pt; g.xaos = c->xaos; g.cb = c->cbf; g.nprime = c->nprime; g.ctil = c->ctil;
@@ -278,9 +281,6 @@ cudaError_t launch_step(km_ctx* c) {
   return launch_update_all(c);
 }
 
-// Shape and buffers of the whole-run kernel, at the context's first graph-
-// driven run.  Without the memory for them the step kernels' graph runs
-// instead, as it does for more points than a resident grid's int64 sums take.
 void release_run(km_ctx* c) {
   void* bufs[] = {c->slack, c->zrun, c->run_delta, c->run_tot, c->run_tot0, c->run_cum0, c->run_priv};
   for (void* b : bufs)
@@ -290,6 +290,9 @@ void release_run(km_ctx* c) {
   cudaGetLastError();
 }
 
+// Shape and buffers of the whole-run kernel, at the context's first graph-
+// driven run.  Without the memory for them the step kernels' graph runs
+// instead, as it does for more points than a resident grid's int64 sums take.
 bool run_ready(km_ctx* c) {
   if (c->run_state) return c->run_state > 0;
   c->run_state = -1;
@@ -366,6 +369,8 @@ km_status run_whole(km_ctx* c, bool* ran) {
     if (s != KM_OK) return s;
     if (c->host_ls.done) break;
   }
+  c->run_totals = true;
+  c->armed = false;
   if (c->zrun && c->opt.label_policy == KM_LABELS_EVERY_STEP)
     KM_CUDA(c, launch_widen_labels(c->zrun, c->labels, c->n, c->st));
   return KM_OK;
@@ -379,6 +384,7 @@ km_status write_control(km_ctx* c, int done, int max_iter_abs, double tol) {
   lc.converged = 0;
   lc.tol = tol;
   KM_CUDA(c, cudaMemcpyAsync(c->ls, &lc, sizeof(lc), cudaMemcpyHostToDevice, c->st));
+  c->armed = !done;
   return KM_OK;
 }
 
@@ -844,6 +850,7 @@ km_status km_run(km_ctx* c, int32_t max_iter, double tol, int32_t* labels_out,
   if (max_iter > 0) {
     s = write_control(c, 0, start + max_iter, tol);
     if (s != KM_OK) return s;
+    bool ran = false;
     if (c->opt.use_graph && run_ready(c)) {
       s = run_whole(c, &ran);
       if (s != KM_OK) return s;
@@ -851,7 +858,6 @@ km_status km_run(km_ctx* c, int32_t max_iter, double tol, int32_t* labels_out,
     if (!ran && c->opt.use_graph) {
       if (!c->graph) {
         cudaGraph_t g = nullptr;
-    bool ran = false;
         KM_CUDA(c, cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal));
         cudaError_t e = cudaSuccess;
         // the tensor-core path's steps are many kernels, so fewer of them run
@@ -915,6 +921,11 @@ km_status km_assign_async(km_ctx* c) {
 km_status km_update_async(km_ctx* c) {
   km_status s = ready(c);
   if (s != KM_OK) return s;
+  if (c->run_totals) {  // the sums a whole run left, as one shard's totals
+    KM_CUDA(c, launch_run_totals(c->d, c->k, c->run_tot0, c->s128, c->st));
+    KM_CUDA(c, launch_shard_update(c->st, update_args(c), c->s128, 1));
+    return KM_OK;
+  }
   KM_CUDA(c, launch_update_all(c));
   return KM_OK;
 }
@@ -959,9 +970,10 @@ km_status km_shard_totals(km_ctx* c, int64_t* out, int32_t mem) {
     dst = c->shard_out;
   }
   // the tensor-core path sums by the sorted mean calculation; the FP32 paths
-  // add their per-block partials
-  KM_CUDA(c, c->path == 3 ? launch_msort_shard_totals(msort_args(c), dst, c->st)
-                          : launch_shard_totals(c->st, update_args(c), dst));
+  // add their per-block partials, which a whole run does not write
+  KM_CUDA(c, c->path == 3   ? launch_msort_shard_totals(msort_args(c), dst, c->st)
+             : c->run_totals ? launch_run_totals(c->d, c->k, c->run_tot0, dst, c->st)
+                             : launch_shard_totals(c->st, update_args(c), dst));
   if (mem == KM_HOST) {
     KM_CUDA(c, cudaMemcpyAsync(out, dst, words * sizeof(long long), cudaMemcpyDeviceToHost, c->st));
     KM_CUDA(c, cudaStreamSynchronize(c->st));

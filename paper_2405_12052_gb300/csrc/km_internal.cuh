@@ -151,6 +151,8 @@ inline size_t run_delta_words(int d, int k, int rep) { return (size_t)3 * rep * 
 size_t run_priv_bytes(int d, int k);
 int run_blocks_per_sm(int d, int kpad, size_t smem);
 cudaError_t launch_run_fast(int d, int grid, size_t smem, cudaStream_t st, const RunArgs& a);
+// tot0 as the column totals of a shard, [k][d+1] of (low, high word)
+cudaError_t launch_run_totals(int d, int k, const long long* tot0, long long* out, cudaStream_t st);
 
 struct GenericArgs {
   const float* x; int64_t ld; int64_t n; int d; int k;

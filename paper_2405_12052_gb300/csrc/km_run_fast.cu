@@ -322,6 +322,15 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
   }
 }
 
+__global__ void run_totals_kernel(int d, int k, const long long* __restrict__ tot0, long long* __restrict__ out) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= k * (d + 1)) return;
+  const int c = q / (d + 1), j = q - c * (d + 1);
+  const long long* t = tot0 + 4 * ((size_t)c * d + (j < d ? j : 0));
+  out[2 * (size_t)q] = j < d ? t[0] : t[2];
+  out[2 * (size_t)q + 1] = j < d ? t[1] : 0;
+}
+
 template <int D, int KG>
 int run_blocks(size_t smem) {
   int nb = 0;
@@ -364,6 +373,11 @@ size_t run_priv_bytes(int d, int k) { return ((size_t)k * (16 + 8 * d + 4) + 15)
 int run_rep(int d, int k) { return (int)std::max<size_t>(1, std::min<size_t>(8, 1024 / ((size_t)k * (d + 1) + 2))); }
 
 int run_blocks_per_sm(int d, int kpad, size_t smem) { KM_RUN_DISPATCH(run_blocks, d, kpad, smem); }
+
+cudaError_t launch_run_totals(int d, int k, const long long* tot0, long long* out, cudaStream_t st) {
+  run_totals_kernel<<<(k * (d + 1) + 255) / 256, 256, 0, st>>>(d, k, tot0, out);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_run_fast(int d, int grid, size_t smem, cudaStream_t st, const RunArgs& a) {
   cudaError_t e = cudaMemsetAsync(a.delta, 0, run_delta_words(d, a.f.k, a.rep) * sizeof(unsigned long long), st);

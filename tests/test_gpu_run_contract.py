@@ -20,6 +20,33 @@ def km():
     return m
 
 
+# the sums after a run are the last step's, whichever driver ran it; an update
+# without an assignment before it divides them again
+@pytest.mark.parametrize("n,d,k,steps,kw", [(5000, 1, 3, 4, {}), (30_011, 2, 40, 70, {}), (20_000, 3, 256, 9, {"label_bytes": 1}),
+                                            (9000, 4, 7, 5, {"label_policy": "final"}), (4_500_001, 3, 6, 12, {})])
+def test_sums_after_a_run(km, n, d, k, steps, kw):
+    x, _, _ = synth.iso_mixture(n, d, max(2, k // 2), sigma=1.5, box=8.0, seed=n, offset=50.0)
+    mu0, _ = synth.init_distinct(x, k, seed=3)
+    got = []
+    for graph in (True, False):
+        g = km.KMeans(n, d, k, use_graph=graph, **kw)
+        g.set_points(x)
+        g.set_init(mu0)
+        g.run(steps, 0.0)
+        t0 = g.shard_totals()
+        g.begin(1, 0.0)
+        t1 = g.shard_totals()
+        g.update_async()
+        g.sync()
+        mu1, cnt1 = g.centroids(), g.counts()
+        g.begin(1, 0.0)
+        g.assign_async()
+        got.append((t0, t1, mu1, cnt1, g.shard_totals()))
+        g.close()
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
+
+
 # no point is counted twice in a step.  At this magnitude the screen flags every
 # point it decides; the start lies in a corner of the data, so the first moves open
 # whole tiles again
