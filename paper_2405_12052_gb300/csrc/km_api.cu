@@ -281,6 +281,13 @@ cudaError_t launch_step(km_ctx* c) {
   return launch_update_all(c);
 }
 
+// E below which most points keep their label without a look (kSettled).  At
+// least 1e-150: data without extent and a tolerance of zero settle as well.
+double settled_e(const km_ctx* c) {
+  const double f = kSettled * std::min(1.0, 0.5 * c->d);
+  return std::max(1e-150, f * std::sqrt((double)c->A_max * c->k) / std::pow((double)c->k, 1.0 / c->d));
+}
+
 void release_run(km_ctx* c) {
   void* bufs[] = {c->slack, c->zrun, c->run_delta, c->run_tot, c->run_tot0, c->run_cum0, c->run_priv};
   for (void* b : bufs)
@@ -363,6 +370,7 @@ km_status run_whole(km_ctx* c, bool* ran) {
       *ran = false;
       return KM_OK;
     }
+  r.restart_e2 = settled_e(c) * settled_e(c);
     KM_CUDA(c, e);
     r.resume = 1;
     km_status s = read_state(c);
@@ -387,6 +395,35 @@ km_status write_control(km_ctx* c, int done, int max_iter_abs, double tol) {
   c->armed = !done;
   return KM_OK;
 }
+km_status write_control(km_ctx* c, int done, int max_iter_abs, double tol);
+// The first steps of a run by the step kernels, which compare every point and
+// keep no slacks: all of a one-step run, and in large sets those until the
+// centroids' moves are small enough for skipping.  *left: the run goes on.
+km_status run_plain(km_ctx* c, int stop, double tol, bool* left) {
+  const double se = settled_e(c), sw = c->opt.e_mode == KM_E_SQUARED ? se * se : se;
+  km_status s = write_control(c, 0, stop, tol > sw ? tol : sw);
+  if (s != KM_OK) return s;
+  // launched ahead of the look at the state: 1, 2, 4, 8, ... steps (those past
+  // the stop return at once)
+  double e = 0.0;
+  for (int ahead = 1;; ahead = std::min(16, 2 * ahead)) {
+    for (int q = std::min(ahead, stop - c->host_ls.iter); q > 0; --q) KM_CUDA(c, launch_step(c));
+    s = read_state(c);
+    if (s != KM_OK) return s;
+    e = c->opt.e_mode == KM_E_SQUARED ? c->host_ls.E2 : c->host_ls.E;
+    if (!c->host_ls.done) continue;
+    if (e < tol || c->host_ls.iter != stop - 1) break;
+    s = write_control(c, 0, stop, tol);  // one more step does not pay for a first step with slacks
+    if (s != KM_OK) return s;
+  }
+  *left = !(e < tol) && c->host_ls.iter < stop;
+  if (!*left && (e < tol || !c->host_ls.converged)) return KM_OK;
+  s = write_control(c, *left ? 0 : 1, stop, tol);  // the step kernels stopped at the larger tolerance
+  if (s != KM_OK) return s;
+  c->host_ls.converged = 0;
+  return KM_OK;
+}
+
 
 km_status read_state(km_ctx* c) {
   KM_CUDA(c, cudaMemcpyAsync(&c->host_ls, c->ls, sizeof(LoopState), cudaMemcpyDeviceToHost, c->st));
@@ -848,10 +885,15 @@ km_status km_run(km_ctx* c, int32_t max_iter, double tol, int32_t* labels_out,
   if (s != KM_OK) return s;
   const int start = c->host_ls.iter;
   if (max_iter > 0) {
-    s = write_control(c, 0, start + max_iter, tol);
+    bool ran = false, left = true;
+    if (c->opt.use_graph && c->path == 1 && (max_iter == 1 || c->n >= kPlainMin)) {
+      s = run_plain(c, start + max_iter, tol, &left);
+    } else {
+      s = write_control(c, 0, start + max_iter, tol);
+    }
     if (s != KM_OK) return s;
-    bool ran = false;
-    if (c->opt.use_graph && run_ready(c)) {
+    ran = !left;
+    if (!ran && c->opt.use_graph && run_ready(c)) {
       s = run_whole(c, &ran);
       if (s != KM_OK) return s;
     }

@@ -122,6 +122,27 @@ struct FastArgs {
 };
 
 // A whole run in one cooperative kernel (km_run_fast.cu).
+// Runs that skip points.  A point is open after a step when its slack is less
+// than its own centroid's move and the largest other one together, so while the
+// moves are a good part of the spacing of the centroids nearly all points are,
+// and taking them back one by one costs more than screening all of them.  So
+// while E (a norm over K moves) exceeds
+//   kSettled min(1, d / 2) sqrt(K) sqrt(A_max) / K^(1/d)
+// -- sqrt(A_max) bounds the data's radius, divided by K^(1/d) the spacing -- a
+// step is followed by a first step again (every point screened, the sums from
+// zero).  Screening costs more for larger K and d; on mixtures, overlapping ones
+// and evenly spread points, K 4 to 200, 3 to 100 steps, 0.018 lay between limits
+// that skip too early (N = 5e7, K = 4, overlapping: 3.6 ms for five steps, 1.7
+// with every point compared) and too late (evenly spread, K = 200, 40 steps: 86
+// ms with a limit of 0.03 without the root, 53 with 0.3).
+constexpr double kSettled = 0.018;
+// Points from which those steps are the step kernels', which keep no slacks
+// (1e8 points, K = 32: 0.88 ms a step against 1.19).  Going over costs a launch, a
+// look at the state and a first step with slacks: at 5e6 points about 50 us, as
+// much as two steps' difference (2 to 10 steps, K 4 to 200, against comparing every
+// point in every step: 0.88-1.1 with the step kernels, 0.97-1.3 without), at 2e7 a
+// part of one step (0.97-1.1 with them, 0.86-1.0 without).
+constexpr int64_t kPlainMin = int64_t(1) << 23;
 constexpr float kDriftMax = 2.9e38f;  // drift sums stop here, below the "never open" (3e38) of what lies past the end
 struct RunArgs {
   FastArgs f;                  // points, sizes, constants and loop state (labels and partials unused)
@@ -140,6 +161,7 @@ struct RunArgs {
   int priv_sh;                 // their offset in shared memory (0: global)
   float4* ctil_out; IterConst* ic_out; unsigned long long* tab_out;  // tables of the final centroids
   double tie_rel;
+  double restart_e2;           // E^2 above which the next step is a first step again
   float margin;                // least slack that FP64 rounding of the distances cannot turn around
   int steps;                   // steps of this launch at most
   int resume;                  // 1: continues the launch before (slack, labels, totals kept)

@@ -143,6 +143,7 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
   };
   tables();
 
+  bool first = !ra.resume;  // this step adds every point (the totals start from zero)
   for (int step = 0;; ++step) {
     FastCtx cx;
     RunTile rt;
@@ -160,7 +161,7 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
       rt.invs = 1.f / (ic.G * ulp);  // powers of two: exact
     }
     rt.slack = ra.slack; rt.z = ra.z; rt.cum = pv.cum; rt.margin = ra.margin;
-    rt.first = !ra.resume && step == 0;
+    rt.first = first;
     const float B_max = s_ic.B_max;
     int nflag = 0, n64 = 0;
     run_pass<D, KG, false>(a, sm, cx, s2, s, dc, rt, pv.ctil, pv.mu, B_max, acc, q, wwarp, wmine, xb, nbuf, wid, wtot,
@@ -222,8 +223,10 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
       long long plo, phi, clo, chi;
       entry(2 * (c * DP + j), plo, phi);
       entry(2 * (c * DP + D), clo, chi);
-      const ulonglong2 pt = *reinterpret_cast<const ulonglong2*>(tot + 4 * qd);
-      const long long nn = tot[4 * qd + 2] + clo + (chi << 54);
+      ulonglong2 pt = *reinterpret_cast<const ulonglong2*>(tot + 4 * qd);
+      long long nn = tot[4 * qd + 2];
+      if (first) { pt.x = 0ull; pt.y = 0ull; nn = 0; }
+      nn += clo + (chi << 54);
       const double old = pv.mu[qd];
       unsigned long long tl = pt.x;
       long long th = (long long)pt.y;
@@ -318,6 +321,12 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
       for (int c = tid; c < k; c += kThreads) ra.ctil_out[c] = pv.ctil[c];
       if (tid == 0) *ra.ic_out = s_ic;
       return;
+    }
+    first = E2 > ra.restart_e2;  // the same in every block
+    if (first) {
+      // the next step reads no label and no slack: the drift starts over
+      for (int c = tid; c < k; c += kThreads) pv.cum[c] = 0.f;
+      __syncthreads();
     }
   }
 }
