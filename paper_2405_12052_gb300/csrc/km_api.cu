@@ -120,7 +120,8 @@ struct km_ctx {
   float A_max = 0.f;
   int tc_ex = 0;           // FP16 tensor-core operands: points scaled by 2^tc_ex
   int G0 = 0;
-  // whole-run kernel (fused path)
+  // whole-run kernel (fused path); run_mem holds its buffers but slack and zrun
+  unsigned char* run_mem = nullptr;
   int run_state = 0;           // 0 not looked at yet, 1 in use, -1 not for this context (shape or memory)
   int run_grid = 0, run_priv_sh = 0, run_rep = 1;
   size_t run_smem = 0;
@@ -170,8 +171,7 @@ void free_all(km_ctx* c) {
                   c->scan, c->scan_bad, c->xb, c->xa_pt, c->xaos, c->cbf, c->nprime, c->gc,
                   c->ms_counts, c->ms_offsets, c->ms_cfirst, c->ms_cursor, c->ms_chunks, c->ms_nchunks,
                   c->ms_chunk_sums, c->ms_perm, c->rescue_list, c->tie_list, c->rescue_count, c->ms_df2, c->bnorm,
-                  c->shard_out, c->shard_in, c->slack, c->zrun, c->run_delta, c->run_tot, c->run_tot0, c->run_cum0,
-                  c->run_priv};
+                  c->shard_out, c->shard_in, c->slack, c->zrun, c->run_mem};
   for (void* b : bufs)
     if (b) cudaFree(b);
   if (c->own_stream && c->st) cudaStreamDestroy(c->st);
@@ -289,11 +289,10 @@ double settled_e(const km_ctx* c) {
 }
 
 void release_run(km_ctx* c) {
-  void* bufs[] = {c->slack, c->zrun, c->run_delta, c->run_tot, c->run_tot0, c->run_cum0, c->run_priv};
+  void* bufs[] = {c->slack, c->zrun, c->run_mem};
   for (void* b : bufs)
     if (b) cudaFree(b);
-  c->slack = nullptr; c->zrun = nullptr; c->run_delta = nullptr; c->run_tot = nullptr; c->run_tot0 = nullptr;
-  c->run_cum0 = nullptr; c->run_priv = nullptr;
+  c->slack = nullptr; c->zrun = nullptr; c->run_mem = nullptr;
   cudaGetLastError();
 }
 
@@ -322,15 +321,27 @@ bool run_ready(km_ctx* c) {
   // (1e6 points, K = 11: 1.74 ms with two copies, 1.69 with one)
   c->run_rep = g > c->sms ? run_rep(c->d, c->k) : 1;
   const size_t kd = (size_t)c->k * c->d;
+  // one allocation for the small ones (five of them: 30 us of a first run of 3e6
+  // points); the per-point ones apart, as one of 0.6 MB (1e5 points) takes a new
+  // block of memory where the parts fit beside the context's: 90 us
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    const size_t o = at;
+    at += (bytes + 255) & ~size_t(255);
+    return o;
+  };
+  const size_t o_delta = take(run_delta_words(c->d, c->k, c->run_rep) * 8), o_tot = take((size_t)g * kd * 32),
+               o_tot0 = take(kd * 32), o_cum0 = take((size_t)c->k * sizeof(float)), o_priv = take(sh ? 0 : (size_t)g * priv);
   if (dalloc(&c->slack, (size_t)c->n) != cudaSuccess ||
-      (!c->labels8 && dalloc(&c->zrun, (size_t)c->n) != cudaSuccess) ||
-      dalloc(&c->run_delta, run_delta_words(c->d, c->k, c->run_rep)) != cudaSuccess ||
-      dalloc(&c->run_tot, (size_t)g * kd * 4) != cudaSuccess || dalloc(&c->run_tot0, kd * 4) != cudaSuccess ||
-      dalloc(&c->run_cum0, (size_t)c->k) != cudaSuccess ||
-      (!sh && dalloc(&c->run_priv, (size_t)g * priv) != cudaSuccess)) {
+      (!c->labels8 && dalloc(&c->zrun, (size_t)c->n) != cudaSuccess) || dalloc(&c->run_mem, at) != cudaSuccess) {
     release_run(c);
     return false;
   }
+  c->run_delta = reinterpret_cast<unsigned long long*>(c->run_mem + o_delta);
+  c->run_tot = reinterpret_cast<long long*>(c->run_mem + o_tot);
+  c->run_tot0 = reinterpret_cast<long long*>(c->run_mem + o_tot0);
+  c->run_cum0 = reinterpret_cast<float*>(c->run_mem + o_cum0);
+  c->run_priv = sh ? nullptr : c->run_mem + o_priv;
   c->run_state = 1;
   return true;
 }
@@ -359,6 +370,7 @@ km_status run_whole(km_ctx* c, bool* ran) {
   // 2 sqrt(A_max) + 2^20 ulps of slack for centroids outside the data's range
   r.margin = (float)(1e-13 * (4.0 * std::sqrt((double)c->A_max) + 1e-20));
   r.rep = c->run_rep;
+  r.restart_e2 = settled_e(c) * settled_e(c);
   r.steps = 64;
   // one pass over the points takes far less: K N evaluations at 1e11 a second
   r.wait_ns = 2000000000ull + (unsigned long long)((double)c->n * c->k * 0.01);
@@ -370,7 +382,6 @@ km_status run_whole(km_ctx* c, bool* ran) {
       *ran = false;
       return KM_OK;
     }
-  r.restart_e2 = settled_e(c) * settled_e(c);
     KM_CUDA(c, e);
     r.resume = 1;
     km_status s = read_state(c);
@@ -384,17 +395,6 @@ km_status run_whole(km_ctx* c, bool* ran) {
   return KM_OK;
 }
 
-km_status write_control(km_ctx* c, int done, int max_iter_abs, double tol) {
-  LoopControl lc{};
-  lc.done = done;
-  lc.max_iter = max_iter_abs;
-  lc.e_mode = c->opt.e_mode;
-  lc.converged = 0;
-  lc.tol = tol;
-  KM_CUDA(c, cudaMemcpyAsync(c->ls, &lc, sizeof(lc), cudaMemcpyHostToDevice, c->st));
-  c->armed = !done;
-  return KM_OK;
-}
 km_status write_control(km_ctx* c, int done, int max_iter_abs, double tol);
 // The first steps of a run by the step kernels, which compare every point and
 // keep no slacks: all of a one-step run, and in large sets those until the
@@ -424,6 +424,17 @@ km_status run_plain(km_ctx* c, int stop, double tol, bool* left) {
   return KM_OK;
 }
 
+km_status write_control(km_ctx* c, int done, int max_iter_abs, double tol) {
+  LoopControl lc{};
+  lc.done = done;
+  lc.max_iter = max_iter_abs;
+  lc.e_mode = c->opt.e_mode;
+  lc.converged = 0;
+  lc.tol = tol;
+  KM_CUDA(c, cudaMemcpyAsync(c->ls, &lc, sizeof(lc), cudaMemcpyHostToDevice, c->st));
+  c->armed = !done;
+  return KM_OK;
+}
 
 km_status read_state(km_ctx* c) {
   KM_CUDA(c, cudaMemcpyAsync(&c->host_ls, c->ls, sizeof(LoopState), cudaMemcpyDeviceToHost, c->st));
