@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(kUpdThreads) batch_update_kernel(BatchArgs a) 
   __shared__ long long s_hi[kUpdThreads / 256][256];
   __shared__ double s_df2[kBatchMaxK * 3];
   __shared__ float s_mv[kBatchMaxK];
-  __shared__ int s_empty, s_at;
+  __shared__ int s_empty, s_at, s_first;
   const int inst = blockIdx.x, tid = threadIdx.x;
   BatchState* st = a.state + inst;
   if (st->done) return;
@@ -389,7 +389,12 @@ __global__ void __launch_bounds__(kUpdThreads) batch_update_kernel(BatchArgs a) 
     st->E2 = E2;
     st->E = E;
     st->iter += 1;
-    st->first = 0;
+    // with steps that skip points: moves that open most points again make the
+    // next step a first one (every point screened, the totals from zero), which
+    // costs less than taking those points back one by one
+    s_first = a.cum && E > (double)((float)kSettled * fminf(1.f, 0.5f * (float)d) * sqrtf(bi.A_max * (float)k) *
+                                    powf((float)k, -1.f / (float)d));
+    st->first = s_first;
     st->empty = s_empty;
     st->B_max = (float)(s_bmax[0] * (1.0 + 1e-6));
     const double esel = a.e_mode == 1 ? E2 : E;
@@ -404,6 +409,11 @@ __global__ void __launch_bounds__(kUpdThreads) batch_update_kernel(BatchArgs a) 
     __syncthreads();
     if (s_at >= 0)
       for (int t = tid; t < bi.ntiles; t += kUpdThreads) a.list[s_at + t] = bi.tile0 + t;
+    if (s_first && tid < cols) {
+      unsigned long long* t = a.totals + 2 * (bi.tot_off + tid);
+      t[0] = 0ull;
+      t[1] = 0ull;
+    }
   }
 }
 

@@ -390,9 +390,11 @@ km_status km_batch_run(km_batch* b, int32_t max_iter, double tol, int32_t* label
     KB_CUDA(b, cudaMemsetAsync(b->totals, 0, sizeof(unsigned long long) * 2 * (size_t)b->total_cols, b->st));
     KB_CUDA(b, launch_batch_list(a, 0, b->st));
   }
-  // the tolerance is a kernel argument: the graph is rebuilt when it changes
+  // the tolerance is a kernel argument: the graph is rebuilt when it changes.
+  // Fewer steps than it holds are launched one by one: a step past the limit
+  // costs two launches (4096 small instances, one step: 0.39 -> 0.33 ms)
   if (b->graph && b->graph_tol != tol) drop_graph(b);
-  if (b->opt.use_graph && !b->graph) {
+  if (b->opt.use_graph && !b->graph && max_iter >= kGraphSteps) {
     cudaGraph_t g = nullptr;
     KB_CUDA(b, cudaStreamBeginCapture(b->st, cudaStreamCaptureModeThreadLocal));
     for (int r = 0; r < kGraphSteps; ++r) {
@@ -409,13 +411,16 @@ km_status km_batch_run(km_batch* b, int32_t max_iter, double tol, int32_t* label
   }
   int remaining = act;
   for (int done_steps = 0; remaining > 0 && done_steps < max_iter;) {
-    if (b->graph) {
+    if (b->graph && max_iter - done_steps >= b->graph_steps) {
       KB_CUDA(b, cudaGraphLaunch(b->graph, b->st));
       done_steps += b->graph_steps;
     } else {
-      KB_CUDA(b, launch_assign_kind(b, a));
-      KB_CUDA(b, launch_batch_update(a, b->count, b->st));
-      done_steps += 1;
+      const int q = b->opt.use_graph ? std::min(kGraphSteps, max_iter - done_steps) : 1;
+      for (int r = 0; r < q; ++r) {
+        KB_CUDA(b, launch_assign_kind(b, a));
+        KB_CUDA(b, launch_batch_update(a, b->count, b->st));
+      }
+      done_steps += q;
     }
     KB_CUDA(b, cudaMemcpyAsync(&remaining, b->active, sizeof(int), cudaMemcpyDeviceToHost, b->st));
     KB_CUDA(b, cudaStreamSynchronize(b->st));
