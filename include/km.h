@@ -483,10 +483,15 @@ km_status km_selftest_bounded_wait(int32_t* gave_up, double* elapsed_ms);
 
 /* Testing hook (allocation-failure injection, process-wide): after n more
  * successful device allocations by the library, the next one fails as if
- * the device were out of memory, and the call making it returns KM_ENOMEM
+ * the device were out of memory.  The call making it returns KM_ENOMEM
  * (the context then only accepts km_destroy, which frees what was
- * allocated).  n < 0 turns the injection off (the default). */
+ * allocated), except where the memory only serves to skip points: km_run then
+ * keeps to the step kernels and a batch to the shapes that compare all points,
+ * with the same results.  n < 0 turns the injection off (the default). */
 void km_debug_fail_alloc_after(int64_t n);
+/* Allocations left before the injected failure; -1 once it has happened, or
+ * when the injection is off. */
+int64_t km_debug_allocs_left(void);
 
 #ifdef __cplusplus
 }

@@ -170,6 +170,8 @@ def lib(path: str | None = None):
     L.km_setnet_destroy.restype = None
     L.km_debug_fail_alloc_after.argtypes = [i64]
     L.km_debug_fail_alloc_after.restype = None
+    L.km_debug_allocs_left.argtypes = []
+    L.km_debug_allocs_left.restype = i64
     L.km_selftest_bounded_wait.argtypes = [ctypes.POINTER(i32), ctypes.POINTER(f64)]
     L.km_selftest_bounded_wait.restype = st
     L.km_get_labels_u8.argtypes = [P, P, i32]
@@ -221,6 +223,12 @@ def debug_fail_alloc_after(n: int):
     """Testing hook: after n more device allocations by the library, the next
     one fails as out of memory (n < 0: off)."""
     lib().km_debug_fail_alloc_after(int(n))
+
+
+def debug_allocs_left() -> int:
+    """Testing hook: allocations left before the injected failure (-1: it has
+    happened, or the injection is off)."""
+    return int(lib().km_debug_allocs_left())
 
 
 def header_symbols(header: str = HEADER) -> list[str]:

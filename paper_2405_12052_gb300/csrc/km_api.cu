@@ -472,6 +472,7 @@ void km_default_options(km_options* opt) {
 const char* km_version(void) { return "libkm 0.1 (sm_103a)"; }
 
 void km_debug_fail_alloc_after(int64_t n) { g_alloc_countdown.store(n < 0 ? -1 : n); }
+int64_t km_debug_allocs_left(void) { return g_alloc_countdown.load(); }
 
 km_status km_selftest_bounded_wait(int32_t* gave_up, double* elapsed_ms) {
   if (!gave_up || !elapsed_ms) return KM_EINVAL;
