@@ -397,7 +397,7 @@ def run_ours(args, ws, rank, local):
                        label_bytes=lb, dist_path=args.dist_path)
         g3.set_points(xt, borrow=True)
         ttc_runs = []
-        for rep in range(2):  # the first run also builds the context's step graph
+        for rep in range(2):  # the first run also allocates the buffers of runs
             g3.set_init(mu0)
             torch.cuda.synchronize(dev)
             t0 = time.perf_counter()
@@ -409,8 +409,8 @@ def run_ours(args, ws, rank, local):
                "converged": bool(r["converged"]), "E": r["E"], "objective": g3.objective(),
                "ms_per_iter": 1e3 * wall / max(1, r["iters"]), "tol": 1e-6, "max_iter": 300,
                "evals_per_s": n * k * r["iters"] / wall,
-               "note": "km_run from the same k-means++ start; wall clock of the call (second run: the step "
-                       "graph already built); centroids copied out, labels left on the device"}
+               "note": "km_run from the same k-means++ start; wall clock of the call (second run: its buffers "
+                       "already allocated); centroids copied out, labels left on the device"}
         g3.close()
 
     pk, src = peaks()
@@ -579,7 +579,7 @@ def batch_ttc(count, dev):
     """Time to converge of the first `count` instances of the batch recipe
     (tol 1e-6, max 300): one KMeansBatch run (launch shape from the tuner,
     tuning not timed) against the same instances run one after another with
-    plain km_run (each context's step graph already built: its second run is
+    plain km_run (each context's buffers already allocated: its second run is
     timed)."""
     import numpy as np
     import torch
@@ -608,7 +608,7 @@ def batch_ttc(count, dev):
         g = km.KMeans(w["n"], w["d"], w["k"])
         g.set_points(w["x"])
         g.set_init(w["mu0"])
-        g.run(300, 1e-6, want_labels=False)  # builds the step graph
+        g.run(300, 1e-6, want_labels=False)  # allocates the run's buffers
         g.set_init(w["mu0"])
         torch.cuda.synchronize(dev)
         t1 = time.perf_counter()
@@ -628,8 +628,8 @@ def run_batch(args, ws, rank, local):
     """Batched form: all instances to convergence (tol 1e-6, max 300) in one
     batch, against the same instances run one after another with plain
     km_run on the same GPU (setup of each context not timed; each plain run
-    timed twice: the first builds the context's step graph, the second
-    reuses it)."""
+    timed twice: the first allocates the run's buffers, the second reuses
+    them)."""
     import numpy as np
     t0 = time.perf_counter()
     insts = gen_batch(args.batch_count)
@@ -682,23 +682,32 @@ def run_batch(args, ws, rank, local):
     torch.cuda.synchronize(dev)
     e2e_s = time.perf_counter() - t0
     b2.close()
-    # roofline of the assign kernel with every instance active: sum_i 3 N_i K_i d_i
-    # flops per launch over the tuner's best time of the batch kernel, the one
-    # that compares every point in every step (the fused kernel's tiles skip
-    # points whose label cannot have changed)
+    # Roofline of the timed run.  Shapes that compare every point: sum_i 3 N_i K_i d_i
+    # flops per step over the tuner's time of the shape in use.  Shapes that skip
+    # points: the 5 bytes a point (slack, label) that every step of an instance
+    # reads, over the whole run (the points decided again come on top).  Beside it
+    # the batch kernel's, which compares every point, from the tuner.
     pk, src = peaks()
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     fp32_peak = sms * FP32_LANES_PER_SM * 2 * float(pk.get("sm_max_mhz", 2070.0)) * 1e6 / 1e12
     assign_ms = min(info["tune_ms"][:6]) if info["tune_ms"] else None
     flops = float(np.sum(3.0 * ns * ks * ds))
-    roof = None
+    roof = full = None
     if assign_ms:
         ach = flops / (assign_ms / 1e3) / 1e12
-        roof = {"bound": "alu", "achieved": ach, "peak": fp32_peak, "unit": "TFLOP/s", "frac": ach / fp32_peak,
+        full = {"bound": "alu", "achieved": ach, "peak": fp32_peak, "unit": "TFLOP/s", "frac": ach / fp32_peak,
                 "traffic": None, "kernel": "batch_assign_kernel",
                 "kernel_ms": assign_ms,
                 "peak_source": f"{sms} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 flops x sm_max_mhz ({src} peaks); "
                                "algorithmic sum_i 3 N_i K_i d_i flops per launch with every instance active"}
+    if tile > 1024:
+        hbm = float(pk.get("hbm_gbs", 6800.0))
+        ach = 5.0 * float(np.sum(ns * iters)) / batch_s / 1e9
+        roof = {"bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm, "traffic": None,
+                "kernel": "batch_run_kernel", "kernel_ms": None,
+                "note": "whole run, updates included: 5 bytes a point and step"}
+    else:
+        roof = full
     # plain km_run, one instance after another
     sel = list(range(0, len(insts), max(1, args.plain_every)))
     plain_s = 0.0
@@ -712,11 +721,11 @@ def run_batch(args, ws, rank, local):
         g.set_init(w["mu0"])
         torch.cuda.synchronize(dev)
         t1 = time.perf_counter()
-        rr = g.run(300, 1e-6, want_labels=False)  # includes building the context's step graph
+        rr = g.run(300, 1e-6, want_labels=False)  # includes allocating the run's buffers
         plain_s += time.perf_counter() - t1
         same = same and rr["iters"] == int(iters[i]) and np.array_equal(rr["centroids"], mu_batch[i])
         plain_iters += rr["iters"]
-        g.set_init(w["mu0"])  # the same run again, its graph already built
+        g.set_init(w["mu0"])  # the same run again, its buffers allocated
         torch.cuda.synchronize(dev)
         t1 = time.perf_counter()
         rr2 = g.run(300, 1e-6, want_labels=False)
@@ -736,7 +745,9 @@ def run_batch(args, ws, rank, local):
                    "d2h_bytes_per_step": int(ns.sum() * 4 + mus.nbytes), "time_to_converge_s": e2e_s,
                    "note": "one 'step' here is the whole batch run to convergence; evals count N K per step, with those "
                            "that the kept bounds make unnecessary"},
-           "gpu_launches": int(2 * 8 * ((int(iters.max()) + 7) // 8)) + (2 if tile > 1024 else 0), "roofline": roof,
+           # two a step, eight steps at a time as far as the limit of 300 allows
+           "gpu_launches": 2 * min(300, 8 * ((int(iters.max()) + 7) // 8)) + (2 if tile > 1024 else 0),
+           "roofline": roof, "roofline_every_point": full,
            "time_to_converge_s": batch_s, "plain_sequential_s": plain_s * scale,
            "plain_sequential_warm_graph_s": plain_warm_s * scale,
            "plain_timed_instances": len(sel), "speedup_vs_plain": plain_s * scale / batch_s,

@@ -6,6 +6,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
+#include <limits>
 #include <new>
 #include <string>
 #include <vector>
@@ -288,6 +289,16 @@ double settled_e(const km_ctx* c) {
   return std::max(1e-150, f * std::sqrt((double)c->A_max * c->k) / std::pow((double)c->k, 1.0 / c->d));
 }
 
+// The squares of the data's extent take the fused screen's scale out of FP32's
+// range (see fast_screen_tables): it then flags every point.
+bool screen_out(const km_ctx* c) {
+  int L = 1;
+  while ((1 << L) < c->kpad) ++L;
+  const int base = 1 << (7 - L), step = 1 << (9 - L);
+  const int half = L <= 6 ? base + (127 - base) / step * step - 128 : -4;
+  return !(3.0 * c->A_max < std::ldexp(1.0, half + 120));
+}
+
 void release_run(km_ctx* c) {
   void* bufs[] = {c->slack, c->zrun, c->run_mem};
   for (void* b : bufs)
@@ -370,7 +381,9 @@ km_status run_whole(km_ctx* c, bool* ran) {
   // 2 sqrt(A_max) + 2^20 ulps of slack for centroids outside the data's range
   r.margin = (float)(1e-13 * (4.0 * std::sqrt((double)c->A_max) + 1e-20));
   r.rep = c->run_rep;
-  r.restart_e2 = settled_e(c) * settled_e(c);
+  // where the screen decides nothing, taking every point afresh costs a re-check
+  // each: never (1e6 points of magnitude 1e17, K = 20, 20 steps: 1.47 -> 0.98 ms)
+  r.restart_e2 = screen_out(c) ? std::numeric_limits<double>::infinity() : settled_e(c) * settled_e(c);
   r.steps = 64;
   // one pass over the points takes far less: K N evaluations at 1e11 a second
   r.wait_ns = 2000000000ull + (unsigned long long)((double)c->n * c->k * 0.01);
