@@ -75,10 +75,12 @@ typedef struct km_options {
   int32_t use_graph; /* 1 (default): km_run keeps the loop on the device -- on the
                         fused path (km_stats.path 1) one cooperative kernel for up to
                         64 steps at a time, 5 (label_bytes 1: 4) more bytes of device
-                        memory per point from the first run on (without that memory,
-                        and on the other paths, a CUDA graph of steps with a
-                        device-side stop); 0: one host round trip per step.  Same
-                        results */
+                        memory per point from the first run of several steps on, in
+                        sets of 2^23 points and more after as many single steps as
+                        move the centroids far (without that memory, on a stream with
+                        fewer SMs than the kernel needs, and on the other paths, a
+                        CUDA graph of steps with a device-side stop); 0: one host
+                        round trip per step.  Same results */
   double tie_rel;  /* relative near-tie threshold re-decided in FP64 (default 1e-5) */
   void* stream;    /* cudaStream_t for all work (NULL: the context creates one) */
   int32_t label_policy; /* KM_LABELS_EVERY_STEP (default): every step writes its labels
@@ -156,7 +158,10 @@ km_status km_step(km_ctx* ctx, double* e_out, double* e2_out);
  * (K x d doubles, host), iters_out (steps run, including the one that met the
  * tolerance), e_out (E of the last step).  Returns KM_OK when converged,
  * KM_NOT_CONVERGED when max_iter was reached.  The iteration count restarts
- * at km_set_init; a second km_run continues from the current centroids. */
+ * at km_set_init; a second km_run continues from the current centroids.
+ * Errors: KM_ESTATE, KM_EINVAL (max_iter < 0), KM_ENOMEM, KM_ECUDA, KM_ETIMEOUT
+ * (a wait of the run's kernel for its other blocks, two seconds and more, or a
+ * bounded wait of the tensor-core path gave up). */
 km_status km_run(km_ctx* ctx, int32_t max_iter, double tol, int32_t* labels_out,
                  double* centroids_out, int32_t* iters_out, double* e_out);
 
@@ -188,9 +193,10 @@ km_status km_sync(km_ctx* ctx, int32_t* iters_out, double* e_out, int32_t* done_
  * centroids on every shard, and km_begin as for the asynchronous pieces.
  *
  * Each step on each shard: km_assign_async; km_shard_totals writes this
- * shard's column totals -- for every centre k and column j (0..d-1 the
- * coordinate sums on the fixed-point grid, d the count) one exact int128 as
- * two int64 words, low word first: K * (d+1) * 2 int64 in total, row-major
+ * shard's column totals (after a km_run those of its last step) -- for every
+ * centre k and column j (0..d-1 the coordinate sums on the fixed-point grid, d
+ * the count) one exact int128 as two int64 words, low word first:
+ * K * (d+1) * 2 int64 in total, row-major
  * [k][j][word]; the caller all-gathers the R tables in rank order
  * (R * K * (d+1) * 2 int64) and passes them to km_shard_update, which adds
  * them in rank order (exact integers), divides, forms E, applies the stop
@@ -242,8 +248,8 @@ typedef struct km_stats {
   int32_t iters;          /* steps since km_set_init */
   int32_t converged;      /* 1 once the tolerance was met in km_run */
   double e, e2;           /* error of the last step */
-  int64_t flagged;        /* points re-checked past the FP32 screen in the last step (of a
-                             km_run in one kernel: points decided again in its last step) */
+  int64_t flagged;        /* points re-checked past the FP32 screen in the last step (where a
+                             km_run skips points: points decided again in its last step) */
   int64_t fp64_decided;   /* of those, points decided in FP64 */
   int32_t empty_clusters; /* clusters with no points in the last step */
   int64_t overflowed;     /* tensor-core path: points whose candidate list overflowed (all K re-ranked) */
@@ -360,7 +366,8 @@ km_status km_batch_objective(km_batch* b, double* out);
 
 /* Run every instance until its selected error is < tol or max_iter more
  * steps have run; the steps are replayed from a captured CUDA graph (8 steps
- * per launch; stopped instances do no work) until no instance is active.
+ * per launch, the last max_iter mod 8 one by one; stopped instances do no work)
+ * until no instance is active.
  * Outputs (host or device pointers, each may be NULL): labels_out (sum N_i),
  * centroids_out (sum K_i d_i), and per instance iters_out (steps since
  * km_batch_set_init), e_out (E, or E^2 when e_mode = 1), converged_out.

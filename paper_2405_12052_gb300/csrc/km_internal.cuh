@@ -179,7 +179,7 @@ cudaError_t launch_run_totals(int d, int k, const long long* tot0, long long* ou
 struct GenericArgs {
   const float* x; int64_t ld; int64_t n; int d; int k;
   const float* ctil;               // [k][d] fp32 (mu - s)
-  const float* cnorm;              // [k] ||c~||^2 fp32 (unused by the direct form)
+  const float* cnorm;              // [k] ||c~||^2 fp32, rounded up
   const double* mu;                // [k][d]
   const float* shift;              // [d]
   const DataConst* dc;

@@ -29,7 +29,9 @@
 // argmin as in every step.  The sums are exact integers, so taking a point
 // out of its old cluster and adding it to the new one gives the same totals
 // as adding all points again.  A step over points that keep their labels reads
-// 5 bytes a point (0.5 GB for 1e8 points: 75 us at the memory's rate).
+// 5 bytes a point (0.5 GB for 1e8 points: 75 us at the memory's rate).  While the
+// centroids move far nearly every point is open; the next step is then a first
+// step again, in large sets the step kernels' (kSettled, kPlainMin).
 //
 // A 256-point warp-tile with more than kHeavy open points goes through the
 // fused kernel's screen whole; fewer are listed and decided one per lane
@@ -363,6 +365,8 @@ cudaError_t run_launch(int grid, size_t smem, cudaStream_t st, const RunArgs& a)
 }  // namespace
 
 // The instances of the fused kernel that read their table from shared memory.
+// With the group count at run time in place of kpad = 32 and 256 (d = 3) a run is
+// up to 3 % (K = 32; N = 1e5 to 4e6, 10 and 40 steps) and 1 % (K = 250) slower.
 #define KM_RUN_DISPATCH(FN, d, kpad, ...)             \
   do {                                                \
     switch (d) {                                      \
