@@ -496,6 +496,10 @@ km_status km_selftest_bounded_wait(int32_t* gave_up, double* elapsed_ms);
  * keeps to the step kernels and a batch to the shapes that compare all points,
  * with the same results.  n < 0 turns the injection off (the default). */
 void km_debug_fail_alloc_after(int64_t n);
+/* Testing hook: the waits of the context's whole-run kernel wait for an arrival
+ * that nothing makes and give up after ns nanoseconds (< 0: off, the default), so
+ * a km_run that uses that kernel returns KM_ETIMEOUT. */
+km_status km_debug_run_wait_fails(km_ctx* ctx, int64_t ns);
 /* Allocations left before the injected failure; -1 once it has happened, or
  * when the injection is off. */
 int64_t km_debug_allocs_left(void);

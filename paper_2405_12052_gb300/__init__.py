@@ -170,6 +170,8 @@ def lib(path: str | None = None):
     L.km_setnet_destroy.restype = None
     L.km_debug_fail_alloc_after.argtypes = [i64]
     L.km_debug_fail_alloc_after.restype = None
+    L.km_debug_run_wait_fails.argtypes = [P, i64]
+    L.km_debug_run_wait_fails.restype = st
     L.km_debug_allocs_left.argtypes = []
     L.km_debug_allocs_left.restype = i64
     L.km_selftest_bounded_wait.argtypes = [ctypes.POINTER(i32), ctypes.POINTER(f64)]
@@ -434,6 +436,11 @@ class KMeans:
                     centroids=self.centroids(), records=recs)
 
     # -- asynchronous pieces of a step (no synchronization) ---------------
+    def debug_run_wait_fails(self, ns: int):
+        """Testing hook: the whole-run kernel's waits give up after ns
+        nanoseconds (< 0: off)."""
+        self._check(self._L.km_debug_run_wait_fails(self._h, int(ns)))
+
     def begin(self, max_iter: int, tol: float):
         self._check(self._L.km_begin(self._h, int(max_iter), float(tol)))
 

@@ -132,6 +132,7 @@ struct km_ctx {
   long long *run_tot = nullptr, *run_tot0 = nullptr;
   float* run_cum0 = nullptr;
   unsigned char* run_priv = nullptr;
+  int64_t run_wait_fails = -1;  // testing: the run kernel's waits give up after so many ns (< 0: off)
   bool run_totals = false;     // the last step's sums are in run_tot0 (a whole run), not in partials
   bool armed = false;          // the stop flag has been cleared since then: an assignment writes partials
   // loop
@@ -387,6 +388,10 @@ km_status run_whole(km_ctx* c, bool* ran) {
   r.steps = 64;
   // one pass over the points takes far less: K N evaluations at 1e11 a second
   r.wait_ns = 2000000000ull + (unsigned long long)((double)c->n * c->k * 0.01);
+  if (c->run_wait_fails >= 0) {
+    r.wait_ns = (unsigned long long)c->run_wait_fails;
+    r.wait_more = 1;
+  }
   while (true) {
     const cudaError_t e = launch_run_fast(c->d, c->run_grid, c->run_smem, c->st, r);
     if (e != cudaSuccess && !r.resume) {
@@ -486,6 +491,12 @@ const char* km_version(void) { return "libkm 0.1 (sm_103a)"; }
 
 void km_debug_fail_alloc_after(int64_t n) { g_alloc_countdown.store(n < 0 ? -1 : n); }
 int64_t km_debug_allocs_left(void) { return g_alloc_countdown.load(); }
+
+km_status km_debug_run_wait_fails(km_ctx* c, int64_t ns) {
+  if (!c) return KM_EINVAL;
+  c->run_wait_fails = ns < 0 ? -1 : ns;
+  return KM_OK;
+}
 
 km_status km_selftest_bounded_wait(int32_t* gave_up, double* elapsed_ms) {
   if (!gave_up || !elapsed_ms) return KM_EINVAL;

@@ -166,6 +166,7 @@ struct RunArgs {
   int steps;                   // steps of this launch at most
   int resume;                  // 1: continues the launch before (slack, labels, totals kept)
   unsigned long long wait_ns;  // limit of one wait for the other blocks
+  unsigned int wait_more;      // arrivals waited for beyond the grid's (testing: none comes)
 };
 // words of delta including the arrival counter
 int run_rep(int d, int k);

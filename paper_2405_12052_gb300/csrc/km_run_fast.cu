@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(kThreads, KM_MINB) run_fast_kernel(RunArgs ra)
       sm.cnt[tid] = 0;
     }
     if (tid == 0) s_empty = 0;
-    if (!grid_wait(ra.bar, (unsigned)(step + 1) * gridDim.x, ra.wait_ns)) {
+    if (!grid_wait(ra.bar, (unsigned)(step + 1) * gridDim.x + ra.wait_more, ra.wait_ns)) {
       if (tid == 0) a.ls->error = 3;
       return;
     }
