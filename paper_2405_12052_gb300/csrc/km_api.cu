@@ -286,7 +286,7 @@ cudaError_t launch_step(km_ctx* c) {
 // E below which most points keep their label without a look (kSettled).  At
 // least 1e-150: data without extent and a tolerance of zero settle as well.
 double settled_e(const km_ctx* c) {
-  const double f = kSettled * std::min(1.0, 0.5 * c->d);
+  const double f = kSettled * std::max(1.0, c->k / 32.0);
   return std::max(1e-150, f * std::sqrt((double)c->A_max * c->k) / std::pow((double)c->k, 1.0 / c->d));
 }
 

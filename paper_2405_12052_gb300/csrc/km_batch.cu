@@ -392,8 +392,7 @@ __global__ void __launch_bounds__(kUpdThreads) batch_update_kernel(BatchArgs a) 
     // with steps that skip points: moves that open most points again make the
     // next step a first one (every point screened, the totals from zero), which
     // costs less than taking those points back one by one
-    s_first = a.cum && E > (double)((float)kSettled * fminf(1.f, 0.5f * (float)d) * sqrtf(bi.A_max * (float)k) *
-                                    powf((float)k, -1.f / (float)d));
+    s_first = a.cum && E > (double)bi.settled;
     st->first = s_first;
     st->empty = s_empty;
     st->B_max = (float)(s_bmax[0] * (1.0 + 1e-6));
@@ -514,7 +513,11 @@ __global__ void __launch_bounds__(256) batch_scan_kernel(const float* __restrict
     if (tid < w) s_a[tid] = fmaxf(s_a[tid], s_a[tid + w]);
     __syncthreads();
   }
-  if (tid == 0) bi.A_max = s_a[0];
+  if (tid == 0) {
+    const float k = (float)bi.k;
+    bi.A_max = s_a[0];
+    bi.settled = (float)kSettled * fmaxf(1.f, k / 32.f) * sqrtf(s_a[0] * k) * powf(k, -1.f / (float)bi.d);
+  }
 }
 
 }  // namespace

@@ -127,14 +127,15 @@ struct FastArgs {
 // moves are a good part of the spacing of the centroids nearly all points are,
 // and taking them back one by one costs more than screening all of them.  So
 // while E (a norm over K moves) exceeds
-//   kSettled min(1, d / 2) sqrt(K) sqrt(A_max) / K^(1/d)
+//   kSettled max(1, K / 32) sqrt(K) sqrt(A_max) / K^(1/d)
 // -- sqrt(A_max) bounds the data's radius, divided by K^(1/d) the spacing -- a
 // step is followed by a first step again (every point screened, the sums from
-// zero).  Screening costs more for larger K and d; on mixtures, overlapping ones
-// and evenly spread points, K 4 to 200, 3 to 100 steps, 0.018 lay between limits
-// that skip too early (N = 5e7, K = 4, overlapping: 3.6 ms for five steps, 1.7
-// with every point compared) and too late (evenly spread, K = 200, 40 steps: 86
-// ms with a limit of 0.03 without the root, 53 with 0.3).
+// zero).  Screening costs more for larger K, so the limit grows with it; on
+// mixtures, overlapping ones and evenly spread points, K 2 to 256, 3 to 100 steps,
+// it lies between limits that skip too early (N = 5e7, K = 4, overlapping: 3.6 ms
+// for five steps, 1.7 with every point compared; K = 32 with three times the limit
+// x0.87-0.92) and too late (N = 2e7, K = 200, evenly spread, 30 steps: 21.4 ms
+// without the factor K / 32, 17.9 with it).
 constexpr double kSettled = 0.018;
 // Points from which those steps are the step kernels', which keep no slacks
 // (1e8 points, K = 32: 0.88 ms a step against 1.19).  Going over costs a launch, a
@@ -301,6 +302,7 @@ struct BatchInst {        // per instance, written at set_points (scan kernel) a
   uint32_t bits_C_hi, bits_C_lo;
   int64_t p_off;                   // offset of the points' slacks and byte labels (a multiple of 256)
   int64_t tot_off;                 // offset of the running totals (K_i (d_i + 1) columns)
+  float settled;                   // E above which the next step is a first one (kSettled)
 };
 
 struct BatchState {       // per instance, advanced on the device
