@@ -300,9 +300,9 @@ struct BatchInst {        // per instance, written at set_points (scan kernel) a
   int32_t G0;                      // fixed-point grid exponent
   float C_hi, C_lo;
   uint32_t bits_C_hi, bits_C_lo;
+  float settled;                   // E above which the next step is a first one (kSettled)
   int64_t p_off;                   // offset of the points' slacks and byte labels (a multiple of 256)
   int64_t tot_off;                 // offset of the running totals (K_i (d_i + 1) columns)
-  float settled;                   // E above which the next step is a first one (kSettled)
 };
 
 struct BatchState {       // per instance, advanced on the device
